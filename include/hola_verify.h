@@ -62,7 +62,7 @@ typedef enum {
 /* Storage of W_lm.  HOLA_W_INT8 is the 8-bit case of the Lo-Bi quantiser applied to the LM head (Lo-Bi Optimization
  * section; the paper leaves the quantiser's format open): int8 [V][H] plus one fp32 scale per vocabulary row,
  * W8[v][h] = w_scale[v] * q[v][h].  The weights are streamed at half the bytes, expanded exactly to bf16 on chip, and
- * the scale multiplies the fp32 accumulators.  At most 256 verify rows go into one pass over W_lm in this mode. */
+ * the scale multiplies the fp32 accumulators.  At most 192 verify rows go into one pass over W_lm in this mode. */
 typedef enum {
   HOLA_W_BF16 = 0,
   HOLA_W_INT8 = 1, /* int8 weights, bf16 activations: the weights are expanded exactly on chip (W8A16)             */
@@ -77,7 +77,7 @@ typedef enum {
                     * At most 256 verify rows per pass over W_lm.  Needs a context. */
   HOLA_W_MIXED = 4 /* the Lo-Bi section's mixed precision on the LM head: groups of 256 vocabulary rows stored at 4, 8 or 16
                     * bits (hola_wmix below), all expanded exactly to bf16 on chip, bf16 activations as given.  W_lm of
-                    * the arguments is not read.  At most 256 verify rows per pass; H a multiple of 128. */
+                    * the arguments is not read.  At most 192 verify rows per pass; H a multiple of 128. */
 } hola_w_dtype;
 
 /* The weights of HOLA_W_MIXED (args->wmix points to one of these, in HOST memory; its pointers are DEVICE pointers).
@@ -160,9 +160,9 @@ typedef enum {
   HOLA_OPT_HOST_IN_PLACE = 7,       /* hola_verify_host with rows on demand: 1 = where draft_q is pinned host memory the
                                      * device can address, the accept/sample kernel reads the rows not sent ahead in
                                      * place over the bus (default), 0 = they are copied after a read-back of accept_len */
-  HOLA_OPT_CONVERTER_GROUP = 8,     /* on-chip expansion (HOLA_W_INT8, HOLA_W_MIXED): converter warps that share one K
-                                     * block, 1..8; groups of that many of the eight converter warps take whole blocks
-                                     * in turn.  0 = the default (2)                                                  */
+  HOLA_OPT_CONVERTER_GROUP = 8,     /* on-chip expansion (HOLA_W_INT8, HOLA_W_MIXED): a K block takes four converter
+                                     * warps, one per quarter of the tensor-memory lanes; 1..4 or 0 (default) = both
+                                     * groups of four take blocks in turn, 5..8 = one group takes them all            */
   HOLA_OPT_FUSED_PASSES = 9,        /* more verify rows than one pass over W_lm holds: 1 = all passes in one launch, in
                                      * which as many neighbouring CTA pairs as there are passes walk the same vocabulary
                                      * tiles together and keep in step (default), 2 = the same without keeping in

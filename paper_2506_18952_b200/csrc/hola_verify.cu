@@ -17,8 +17,8 @@
 //       With 257..384 verify rows the accumulators rotate over the four 128-column units of the tensor memory and a
 //       unit is handed back as soon as its chunk has gone to the logits buffer and a staging buffer.  In its
 //       on-chip-expansion mode the kernel streams groups of 256 vocabulary rows stored at 4, 8 or 16 bits and
-//       converter warps (groups of two, each owning whole K blocks) expand the codes exactly to bf16 (mixed-precision
-//       quantiser of the Lo-Bi Optimization section).
+//       converter warps (groups of four, each owning whole K blocks) expand the codes exactly to bf16 in tensor memory,
+//       from where the MMA reads them (mixed-precision quantiser of the Lo-Bi Optimization section).
 //   quantize_rows_int8_kernel   8-bit case of the Lo-Bi quantiser, per row (W_lm ahead of time, hidden rows per call).
 //   quantize_rows_w4_kernel     4-bit case: codes in [-7, 7] with one shared exponent per sub-block of 128 channels.
 //   bounded_wait_selftest_kernel  a wait that is made to run out, to exercise the give-up path without breaking anything.
@@ -66,14 +66,20 @@ constexpr int kK1Threads = kK1Warps * 32;
 constexpr int kEpiSlots = 4;                     // 32-column chunks of a tile one epilogue warp handles at most
 constexpr int kTransRows = 16;                   // verify rows per transposition step of an epilogue warp
 constexpr int kTransBytes = kTransRows * 32 * 4; // its staging buffer: [16 rows][32 vocabulary entries] fp32
-// 8-bit W_lm, expanded on chip (mode 1): the int8 tile of a K block lands in a raw block of the ring slot and
-// converter warps expand it to the bf16 tile the MMA reads.  Warps 2..9 are epilogue warps, warps 10..17 convert (and
-// the first lane of a group also fetches the hidden blocks of the K blocks the group owns).
-constexpr int kRawBlockBytes = kLanes * kBlockK;  // int8 [128][64]
+// 8-bit and 4-bit W_lm, expanded on chip (mode 1): the codes of a K block land in the ring slot and converter warps
+// expand them, through registers, into the bf16 operand in TENSOR MEMORY that the MMA reads (64 columns hold the 128
+// channels of a K block, one lane per vocabulary row).  Warps 2..9 are epilogue warps, warps 10..17 convert: two groups
+// of four warps (one per quarter of the tensor-memory lanes) take the K blocks in turn.
+constexpr int kExpandK = 128;                     // channels per K block of 4- and 8-bit rows (16-bit rows: kBlockK)
+constexpr int kExpandMaxN = 192;                  // two accumulators of 192 columns leave 128 columns for the operand
+constexpr int kOperandCols = kExpandK / 2;        // tensor-memory columns of one K block of the expanded operand
 constexpr int kSubBlock = 128;                    // hidden channels per 4-bit sub-block (one shared exponent each)
-constexpr int kGroupRows = 256;                   // vocabulary rows per group of one width
 constexpr int kW8EpiWarps = 8;
-constexpr int kConvWarps = kK1Warps - 2 - kW8EpiWarps;   // 8
+constexpr int kConvGroup = 4;                     // converter warps per K block: one per tensor-memory lane quarter
+constexpr int kConvGroups = (kK1Warps - 2 - kW8EpiWarps) / kConvGroup;   // 2
+// What the expansion leaves in the operand is the code times a power of two (see expand_*); the epilogue takes it out
+// of the accumulators together with the row's scale.  Both are exact.
+constexpr float kExpandUnscale8 = 64.f, kExpandUnscale4 = 1024.f;
 constexpr int kTmemCols = 512;
 constexpr int kMaxStages = 12;
 constexpr int kMaxPaceGroups = 128;              // groups of CTA pairs of a launch that holds all passes
@@ -103,7 +109,9 @@ struct K1Params {
   int n_sub, N;   // MMAs per K step and their N (verify rows each; multiple of 16)
   int rot;        // 1: three MMAs of N <= 128 per K step whose accumulators rotate over the four 128-column units
   int pair256;    // rot with N = 128 exactly: two of the three units of a tile are adjacent and take ONE MMA of N = 256
-  int conv_group; // (on-chip expansion) converter warps that share one K block
+  int acc_cols;   // tensor-memory columns from one accumulator buffer to the next
+  int conv_groups, a_slots;   // (on-chip expansion) groups of converter warps that take part, K blocks of expanded operand
+                              // that tensor memory holds (at most as many as ring slots)
   int tile_rows;  // vocabulary rows per CTA per tile (<= 128, multiple of 4): balances the tiles over the pairs
   int ldl;        // row pitch of the logits buffer, in floats
   const float* w_scale;   // 8-bit W_lm: fp32 scale per vocabulary row, applied to the accumulators
@@ -243,6 +251,28 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same for a converged warp that polls together: no lane is singled out and nothing has to be handed round, which
+// takes a wait that is satisfied already from about 300 to about 50 cycles.
+__device__ __forceinline__ bool mbar_wait_together(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                                   unsigned* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  long long t0 = 0;
+  uint32_t spins = 0;
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((++spins & 255u) == 0u) {
+      const long long now = clock64();
+      if (t0 == 0) t0 = now;
+      const bool late = now - t0 > kWaitLimitCycles;
+      if (late) {
+        *abort_flag = 1u;
+        if (status) atomicOr(status, HOLA_FLAG_TIMEOUT);
+      }
+      if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+    }
+  }
+}
+
 // Whole-warp form: lane 0 polls, every lane gets the same answer (and, through the shuffle, the same ordering).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag,
                                                unsigned* status, long long limit_cycles = kWaitLimitCycles) {
@@ -328,6 +358,15 @@ __device__ __forceinline__ void umma(uint32_t tmem_d, uint64_t adesc, uint64_t b
         : "memory");
   }
 }
+// The same with A in tensor memory: lane i of each CTA holds row i of its half of A, two bf16 channels per column.
+__device__ __forceinline__ void umma_tmem_a(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 // The mbarrier at this shared-memory offset in BOTH CTAs of the pair gets one arrival once every MMA issued so far
 // by this thread has completed.
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
@@ -354,6 +393,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// 32 words into 32 consecutive columns of this thread's tensor-memory lane (tmem_st_wait: they are there).
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),
+        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
+        "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 16 consecutive 32-bit columns of this thread's tensor-memory lane, as raw words (no wait: the caller waits once
 // for all loads it has issued).
@@ -524,62 +577,43 @@ __device__ __forceinline__ void stats_fold16_packed(const float* v, int vocab0, 
   st.t += fmaf(-m, sc, aa + ab);
 }
 
-// Integer codes to bf16 without conversion instructions: 0x4300 | n is the bf16 number 128 + n for 0 <= n < 128 (seven
-// mantissa bits, unit steps), two such numbers sit in one register, and one packed bf16 subtraction or multiply-add
-// (exact: every intermediate is an integer of at most eight bits) leaves the codes themselves.
-__device__ __forceinline__ uint32_t bf16x2_sub(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
+// Integer codes to bf16 without conversion instructions.  A byte u in the low half of a 16-bit lane, high half zero, IS
+// the bf16 number u * 2^-133 (subnormal below 128, first binade above: the spacing is the same on both sides), so one
+// packed multiply-add per two codes scales and centres them; every result is an integer of at most eight bits times a
+// power of two, exact in bf16.
 __device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
 
-// Sixteen int8 values (one 16-byte piece of a row of the raw block) -> sixteen bf16 values, written as the two 16-byte
-// chunks d0, d1 of the 128-byte-swizzled K-major tile that the caller has located.
-__device__ __forceinline__ void expand_int8x16(const uint4 x, uint8_t* d0, uint8_t* d1) {
+// Sixteen int8 codes -> sixteen bf16 values code / 64, in channel order, two per word: with the sign bit flipped a byte
+// is u = code + 128, and u 2^-133 * 2^127 - 2 = code / 64.  Three integer-pipe instructions and two multiply-adds per
+// four codes.
+__device__ __forceinline__ void expand_int8x16(const uint4 x, uint32_t* o) {
   const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-  uint32_t o[8];
-  // byte b = (128 + its low seven bits) - (256 if its sign bit is set, else 128); as bf16 bit patterns the minuend is
-  // 0x4300 | low bits and the subtrahend 0x4300 | sign bit (0x4380 = 256), so one byte permutation each puts two of
-  // them in a register next to the constant high byte 0x43
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const uint32_t lo = w[j] & 0x7F7F7F7Fu, sg = w[j] & 0x80808080u;
-    o[2 * j] = bf16x2_sub(__byte_perm(lo, 0x43434343u, 0x4140), __byte_perm(sg, 0x43434343u, 0x4140));       // bytes 0, 1
-    o[2 * j + 1] = bf16x2_sub(__byte_perm(lo, 0x43434343u, 0x4342), __byte_perm(sg, 0x43434343u, 0x4342));   // bytes 2, 3
+    const uint32_t u = w[j] ^ 0x80808080u;
+    o[2 * j] = bf16x2_fma(__byte_perm(u, 0u, 0x4140), 0x7F007F00u, 0xC000C000u);
+    o[2 * j + 1] = bf16x2_fma(__byte_perm(u, 0u, 0x4342), 0x7F007F00u, 0xC000C000u);
   }
-  *reinterpret_cast<uint4*>(d0) = make_uint4(o[0], o[1], o[2], o[3]);
-  *reinterpret_cast<uint4*>(d1) = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
-// Thirty-two 4-bit codes (one 16-byte piece of a row of the raw block; two's complement nibbles, even entry in the low
-// nibble) -> thirty-two bf16 values  code << shift, written as four 16-byte chunks of the 128-byte-swizzled K-major
-// tile: chunk j goes to d + ((16 j) ^ x3), d and x3 = 16 (row % 4) located by the caller.  Every value (magnitude
-// <= 7 * 2^4) is exact in bf16.
-__device__ __forceinline__ void expand_int4x32(const uint4 x, uint8_t* d, uint32_t x3, int shift) {
+// Thirty-two 4-bit codes (two's complement nibbles, even channel in the low one) -> thirty-two bf16 values
+// code * 2^(shift - 10): a byte goes into both 16-bit lanes, the low lane keeps its low nibble and the high lane its high
+// nibble (sixteen times the code, which that lane's multiplier takes out), both with the sign bit flipped (code + 8).
+// Two integer-pipe instructions and one multiply-add per two codes.
+__device__ __forceinline__ void expand_int4x32(const uint4 x, uint32_t* o, uint32_t shift) {
   const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-  // nibble n with its sign bit flipped is code + 8; (128 + code + 8) * 2^shift - 136 * 2^shift = code * 2^shift
-  const uint32_t mul1 = static_cast<uint32_t>(127 + shift) << 7;           // bf16 bits of 2^shift
-  const uint32_t mul = mul1 | (mul1 << 16);
-  const uint32_t sub1 = 0xC308u + (static_cast<uint32_t>(shift) << 7);     // bf16 bits of -136 * 2^shift
-  const uint32_t sub = sub1 | (sub1 << 16);
+  const uint32_t mul = ((250u + shift) << 7) | ((246u + shift) << 23);     // 2^(123 + shift), 2^(119 + shift)
+  const uint32_t add1 = 0x8000u | ((120u + shift) << 7);                    // -2^(shift - 7) = -8 * 2^(shift - 10)
+  const uint32_t add = add1 | (add1 << 16);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    // entries (0,4), (1,5), (2,6), (3,7) of this word side by side in 16-bit lanes; flipping the sign bit of the nibble
-    // and setting the bits of 128 are one exclusive-or with 0x4308 (the masked nibble has no bits there)
-    const uint32_t u = w[j];
-    const uint32_t r0 = bf16x2_fma((u & 0x000F000Fu) ^ 0x43084308u, mul, sub);
-    const uint32_t r1 = bf16x2_fma(((u >> 4) & 0x000F000Fu) ^ 0x43084308u, mul, sub);
-    const uint32_t r2 = bf16x2_fma(((u >> 8) & 0x000F000Fu) ^ 0x43084308u, mul, sub);
-    const uint32_t r3 = bf16x2_fma(((u >> 12) & 0x000F000Fu) ^ 0x43084308u, mul, sub);
-    // back into channel order: (0,1) (2,3) (4,5) (6,7)
-    *reinterpret_cast<uint4*>(d + ((16u * j) ^ x3)) =
-        make_uint4(__byte_perm(r0, r1, 0x5410), __byte_perm(r2, r3, 0x5410), __byte_perm(r0, r1, 0x7632),
-                   __byte_perm(r2, r3, 0x7632));
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      o[4 * j + b] = bf16x2_fma((__byte_perm(w[j], 0u, 0x4040 + 0x101 * b) & 0x00F0000Fu) ^ 0x00800008u, mul, add);
   }
 }
 
@@ -610,8 +644,9 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
 //   tempty[4]  @208  leader's copy: all epilogue warps of the pair have read their accumulators (per buffer; per
 //                    128-column unit when the accumulators rotate)
 //   tensor-memory base @256, abort flag @260
-//   8-bit W_lm only: rawfull[12] @272 per CTA: the int8 tile of the slot has landed; rawempty[12] @368 per CTA: the
-//   converter warps have expanded it.  full[] then collects, besides the hidden bytes, one arrival per converter warp.
+//   on-chip expansion only: rawfull[12] @272 per CTA: the codes of the slot have landed (full[] then counts the hidden
+//   bytes and, for 16-bit rows, their bytes); operand[8] @368 leader's copy: the eight converter warps of the pair that
+//   own a K block have put it into tensor memory.
 // After the barrier area: one 2 KB transposition buffer per epilogue warp (reused for the final merge of the
 // statistics of the four tensor-memory lane quarters).
 // kMode 3 is kMode 2 with every verify row present twice in the hidden operand (coarse 8-bit plane and the plane of
@@ -647,15 +682,14 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   const int rows = p.n_pass > 1 ? min(p.rows_per_pass, p.M - row0) : p.rows;
   const int half_n = p.N >> 1;                           // hidden rows this CTA supplies per MMA
   const uint32_t hid_block_bytes = static_cast<uint32_t>(half_n) * 128u;
-  const uint32_t raw_off = kWBlockBytes + p.n_sub * hid_block_bytes;     // int8 block of the slot (8-bit W_lm only)
-  const uint32_t stage_bytes = raw_off + (kW8 ? kRawBlockBytes : 0);
+  const uint32_t stage_bytes = kWBlockBytes + (kW8 ? 2 : p.n_sub) * hid_block_bytes;
   const uint32_t hid_tx_bytes = p.n_sub * hid_block_bytes;
   const uint32_t tx_bytes = static_cast<uint32_t>(p.tile_rows) * 128u + hid_tx_bytes;   // bf16 W_lm: per CTA and slot
-  const uint32_t raw_tx_bytes = static_cast<uint32_t>(p.tile_rows) * 64u;
+  const int code_blocks = (p.n_kblocks + 1) >> 1;        // (on-chip expansion) K blocks of a tile of 4- or 8-bit rows
   const int pair_rows = 2 * p.tile_rows;                 // vocabulary rows of a pair's tile
   const uint32_t bar_base = base + p.stages * stage_bytes;
   const uint32_t full_bar = bar_base, empty_bar = bar_base + 96, tfull_bar = bar_base + 192,
-                 tempty_bar = bar_base + 208, rawfull_bar = bar_base + 272, rawempty_bar = bar_base + 368;
+                 tempty_bar = bar_base + 208, rawfull_bar = bar_base + 272, operand_bar = bar_base + 368;
   constexpr int kNumEpi = kW8 ? kW8EpiWarps : kEpiWarps;      // epilogue warps 2 .. 2 + kNumEpi - 1
   constexpr int kGroups = kNumEpi / 4;                        // warps per tensor-memory lane quarter
   constexpr int kWarpTransBytes = kRot ? 2 * kTransBytes : kTransBytes;   // rotating units: a whole 32-row chunk at once
@@ -665,13 +699,12 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.stages; ++i) {
-      mbar_init(full_bar + 8 * i, kW8 ? 2 + 2 * p.conv_group : 2);   // + the converter warps of a K block, both CTAs
+      mbar_init(full_bar + 8 * i, 2);
       mbar_init(empty_bar + 8 * i, 1);
-      if (kW8) {
-        mbar_init(rawfull_bar + 8 * i, 1);
-        mbar_init(rawempty_bar + 8 * i, p.conv_group);
-      }
+      if (kW8) mbar_init(rawfull_bar + 8 * i, 1);
     }
+    if (kW8)
+      for (int i = 0; i < p.a_slots; ++i) mbar_init(operand_bar + 8 * i, 2 * kConvGroup);
     for (int i = 0; i < 2; ++i) mbar_init(tfull_bar + 8 * i, 1);
     for (int i = 0; i < 4; ++i) mbar_init(tempty_bar + 8 * i, 2 * kNumEpi);
     *abort_flag = 0u;
@@ -710,10 +743,8 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       bool ok = true;
       grid_dependency_wait();                            // W_lm and the hidden rows may come from the kernel before
       if (kW8) {
-        // On-chip expansion: only the raw W_lm blocks.  The raw block of a slot may be refilled as soon as the
-        // converters have read it (16-bit rows, which go straight into the tile the MMA reads: once the MMAs of the
-        // slot's previous use are done as well).  The hidden blocks of a slot are fetched by the converter group that
-        // owns the K block, which waits for those MMAs anyway.
+        // On-chip expansion: codes (or 16-bit rows as they are) and hidden rows of a K block into one slot, which is free
+        // again once the MMAs of its previous use are done: those have waited for the converters.
         for (int t = 0; t < my_tiles && ok; ++t) {
           if (p.n_pass > 1 && p.pace && t > 0) keep_pace(p.pace + pair, static_cast<unsigned>(2 * p.n_pass * t));
           int tile_width = 8;                              // width of this tile's rows and where they are stored
@@ -723,21 +754,31 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
             tile_width = p.group_width[g];
             w_row = p.group_row[g] + static_cast<int>(rank) * p.tile_rows;
           }
+          const int h_row = row0 + static_cast<int>(rank) * half_n;
+          const int n_blocks = tile_width == 16 ? p.n_kblocks : code_blocks;
           int kx = 0;
-          for (int kb = 0; kb < p.n_kblocks; ++kb, kx += kKStep) {
-            if (!mbar_wait(rawempty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+          for (int kb = 0; kb < n_blocks; ++kb) {
+            if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
             const uint32_t sa = base + stage * stage_bytes;
-            const uint32_t rb = own_rawfull + 8 * stage;
-            if (tile_width == 8) {
-              mbar_expect_tx_cluster(rb, raw_tx_bytes);
-              tma_load_2d(sa + raw_off, &tmap_w, rb, kx, w_row, pol_w);
-            } else if (tile_width == 4) {                  // two codes per byte: 32 bytes per row and K block
-              mbar_expect_tx_cluster(rb, raw_tx_bytes >> 1);
-              tma_load_2d(sa + raw_off, &tmap_w4, rb, kx >> 1, w_row, pol_w);
+            const uint32_t rb = own_rawfull + 8 * stage, fb = leader_full + 8 * stage;
+            if (tile_width == 16) {                        // 16-bit rows: the tile the MMA reads from shared memory
+              mbar_arrive(rawfull_bar + 8 * stage);        // (every barrier moves on by one phase per use of the slot)
+              mbar_expect_tx_cluster(fb, tx_bytes);
+              tma_load_2d(sa, &tmap_w16, fb, kx, w_row, pol_w);
+              tma_load_2d(sa + kWBlockBytes, &tmap_hidden, fb, kx, h_row, pol_h);
+              kx += kBlockK;
             } else {
-              if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-              mbar_expect_tx_cluster(rb, raw_tx_bytes << 1);
-              tma_load_2d(sa, &tmap_w16, rb, kx, w_row, pol_w);
+              if (tile_width == 8) {                       // a byte per code: 128 bytes per row and K block
+                mbar_expect_tx_cluster(rb, static_cast<uint32_t>(p.tile_rows) * 128u);
+                tma_load_2d(sa, &tmap_w, rb, kx, w_row, pol_w);
+              } else {                                     // two codes per byte: 64 bytes
+                mbar_expect_tx_cluster(rb, static_cast<uint32_t>(p.tile_rows) * 64u);
+                tma_load_2d(sa, &tmap_w4, rb, kx >> 1, w_row, pol_w);
+              }
+              mbar_expect_tx_cluster(fb, 2 * hid_block_bytes);
+              tma_load_2d(sa + kWBlockBytes, &tmap_hidden, fb, kx, h_row, pol_h);
+              tma_load_2d(sa + kWBlockBytes + hid_block_bytes, &tmap_hidden, fb, kx + kBlockK, h_row, pol_h);
+              kx += kExpandK;
             }
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
           }
@@ -839,6 +880,51 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           if (ok) umma_commit_pair(tfull_bar);           // all three units of this tile are complete in both CTAs
         }
       } else
+      if (kW8) {
+        // A K block's operand is in tensor memory (4- and 8-bit rows) or in the slot's shared memory (16-bit rows); in
+        // either case the converters report for it, so that all barriers move on block by block.
+        const uint32_t operand0 = tmem_base + 2 * p.acc_cols;
+        int aslot = 0;
+        uint32_t aphase = 0;
+        if (p.group_width) grid_dependency_wait();         // the width table may come from the kernel before
+        int width_next = p.group_width && my_tiles > 0 ? p.group_width[pair] : 8;
+        for (int t = 0; t < my_tiles && ok; ++t) {
+          const int buf = t & 1;
+          const uint32_t acc_phase = static_cast<uint32_t>(t >> 1) & 1u;
+          const bool in_smem = width_next == 16;
+          if (p.group_width && t + 1 < my_tiles) width_next = p.group_width[pair + (t + 1) * npairs];
+          if (!mbar_wait(tempty_bar + 8 * buf, acc_phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d0 = tmem_base + buf * p.acc_cols;
+          const int n_blocks = in_smem ? p.n_kblocks : code_blocks;
+          for (int kb = 0; kb < n_blocks; ++kb) {
+            if (!mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status)) { ok = false; break; }
+            if (!mbar_wait(operand_bar + 8 * aslot, aphase, abort_flag, p.status)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t adesc = desc0 + ((stage * stage_bytes) >> 4);
+            const uint64_t bdesc = adesc + (kWBlockBytes >> 4);
+            const uint32_t acc = kb != 0 ? 1u : 0u;
+            if (in_smem) {
+              umma<false>(d0, adesc, bdesc, idesc, acc);
+#pragma unroll
+              for (int kk = 1; kk < kBlockK / 16; ++kk) umma<false>(d0, adesc + 2 * kk, bdesc + 2 * kk, idesc, 1u);
+            } else {
+              const uint32_t a = operand0 + aslot * kOperandCols;
+              umma_tmem_a(d0, a, bdesc, idesc, acc);
+#pragma unroll
+              for (int kk = 1; kk < kBlockK / 16; ++kk) umma_tmem_a(d0, a + 8 * kk, bdesc + 2 * kk, idesc, 1u);
+              const uint64_t bdesc2 = bdesc + (hid_block_bytes >> 4);
+#pragma unroll
+              for (int kk = 0; kk < kBlockK / 16; ++kk)
+                umma_tmem_a(d0, a + kBlockK / 2 + 8 * kk, bdesc2 + 2 * kk, idesc, 1u);
+            }
+            umma_commit_pair(empty_bar + 8 * stage);
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+            if (++aslot == p.a_slots) { aslot = 0; aphase ^= 1u; }
+          }
+          if (ok) umma_commit_pair(tfull_bar + 8 * buf);
+        }
+      } else
       for (int t = 0; t < my_tiles && ok; ++t) {
         const int buf = t % p.nbuf;
         const uint32_t acc_phase = static_cast<uint32_t>(t / p.nbuf) & 1u;
@@ -889,7 +975,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                               : (group < n_chunks ? (n_chunks - 1 - group) / kGroups + 1 : 0);
     float* tbuf = trans_base + (warp - 2) * (kWarpTransBytes / 4);
     const int trow = lane & 15, thalf = lane >> 4;       // row of a transposition step; which 16 of the 32 entries
-    constexpr int kSlots = kRot ? 3 : kEpiSlots;         // chunks per tile this warp keeps statistics for
+    constexpr int kSlots = (kRot || kW8) ? 3 : kEpiSlots;   // chunks per tile this warp keeps statistics for
     Stats st[kSlots][2];
 #pragma unroll
     for (int i = 0; i < kSlots; ++i) { st[i][0] = stats_empty(); st[i][1] = stats_empty(); }
@@ -908,7 +994,11 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       const int nv = max(0, min(32, min(p.tile_rows, p.V - vbase) - quarter * 32));
       const int n16 = max(0, min(16, nv - thalf * 16));
       const int vocab16 = vbase + quarter * 32 + thalf * 16;
-      const float w_scale = ((kW8 || kI8) && vocab_ok) ? p.w_scale[vocab] : 1.f;   // 8-bit W_lm: the row's scale
+      float w_scale = ((kW8 || kI8) && vocab_ok) ? p.w_scale[vocab] : 1.f;   // 8-bit W_lm: the row's scale
+      if (kW8) {                                         // and the power of two the expansion put in (exact)
+        const int width = p.group_width ? p.group_width[pair + t * npairs] : 8;
+        w_scale *= width == 8 ? kExpandUnscale8 : (width == 4 ? kExpandUnscale4 : 1.f);
+      }
       const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
       if (kTwoPlane) {
         // Two planes: 64 consecutive accumulator columns hold the coarse-plane sums (first 32) and the remainder-plane
@@ -1077,7 +1167,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           const int unit = (3 * t + slot) & 3;           // (rotating accumulators only)
           float v[32];
           __syncwarp();                                  // tcgen05.ld is warp-collective: reconverge first
-          tmem_ld32(lane_addr + (rot ? unit * 128 : buf * 256 + sub * 256) + j * 32, v);
+          tmem_ld32(lane_addr + (rot ? unit * 128 : kW8 ? buf * p.acc_cols : buf * 256 + sub * 256) + j * 32, v);
           if (rot || slot == my_chunks - 1) {            // this warp's accumulators (of this unit) may be overwritten
             tc_fence_before();
             __syncwarp();
@@ -1164,128 +1254,99 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       }
     }
   } else if (kW8) {
-    // ------------------------------------------------------------------ 8-bit W_lm: converter warps
-    // int8 [tile_rows][64] (row pitch 64 bytes) -> bf16 [tile_rows][64] in the 128-byte-swizzled K-major layout the
-    // MMA reads: 16-byte chunk c of row r sits at chunk position c ^ (r % 8) of its 128-byte row.  Every int8 value is
-    // exact in bf16; the row's scale is applied to the accumulators by the epilogue warps.
-    // The converter warps form groups of conv_group warps; each group owns whole K blocks, every ngroups-th one of the
-    // CTA's sequence of blocks.  The waits, the expansion and the fence of one block are a chain of dependent steps:
-    // several groups run such chains side by side (ring slots permitting), several warps in a group shorten the chain.
-    const int cw = warp - (2 + kW8EpiWarps);
-    const uint32_t leader_full = map_to_cta(full_bar, 0);
-    const int units = p.tile_rows * 4;                   // 16-byte pieces of the int8 tile
-    const uint64_t pol_h = l2_policy_evict_last();       // hidden is re-read for every tile
-    const int total_blocks = my_tiles * p.n_kblocks;
+    // ------------------------------------------------------------------ on-chip expansion: converter warps
+    // Codes of a K block, [tile_rows][128] in the slot -> bf16 operand in tensor memory, thread = vocabulary row = lane:
+    // 128 (8-bit) or 64 (4-bit) bytes of the row come in as 16-byte pieces (the TMA swizzle of 128 / 64 bytes spreads
+    // eight neighbouring rows over all banks), are expanded in registers and go out 32 columns per tcgen05.st.  The
+    // expanded operand never touches shared memory.  Two groups of four warps (a warp reaches only its own quarter of the
+    // lanes) take the blocks in turn.
+    // What bounds it: with few verify rows the chain of one block, ~1600 cycles per group (expansion 570, waits and loop
+    // the rest), against ~690 cycles per block and two groups that HBM allows at 8 bits; with 129..192 rows the MMAs (768
+    // cycles per block), of whose operand tensor memory then holds only two blocks.  Measured against the form before
+    // (bf16 tile written to shared memory by groups of two warps, K blocks of 64; three byte permutes or more per two
+    // codes): whole step of one sequence, H = 4096, V = 32000, widths 20/70/10 % 68.3 -> 44.0 us, all 8-bit 58.1 -> 39.2;
+    // 192 rows, V = 128256 331 -> 236 us, 120 rows 277 -> 184.  K blocks of 64 with the same warps: 81 us (the waits
+    // cost as much per block as the expansion does).
+    const int quarter = warp & 3;
+    const int grp = (warp - (2 + kW8EpiWarps)) / kConvGroup;
+    const int row = quarter * 32 + lane;
+    const int G = p.conv_groups;
+    const uint32_t leader_operand = map_to_cta(operand_bar, 0);
+    const uint32_t operand_lane = tmem_base + 2 * p.acc_cols + (static_cast<uint32_t>(quarter * 32) << 16);
     grid_dependency_wait();                              // the width table and the exponents may come from the kernel before
-    // No more groups than ring slots take part: a group that starts block i has finished block i - ngroups, whose slot
-    // had been freed by the MMAs of block i - ngroups - stages, so with ngroups <= stages every barrier it waits on is at
-    // most one phase behind and the parity waits below cannot mistake "two trips round the ring ago" for "done".
-    const int G = p.conv_group;
-    const int ngroups = min(kConvWarps / G, p.stages);
-    const int grp = cw / G, mem = cw - grp * G;          // warps beyond ngroups * G groups stay idle
-    const int step = 32 * G;                             // pieces the group expands per trip of its loops
-    const int first = mem * 32 + lane;                   // this lane's first piece
-    int t = 0, kb = grp;                                 // block i = t * n_kblocks + kb of the sequence, i % ngroups == grp
-    while (kb >= p.n_kblocks && t < my_tiles) { kb -= p.n_kblocks; ++t; }
-    // Where this lane's pieces go does not change from block to block.  8-bit: piece u is the 16 bytes c = u % 4 of row
-    // u / 4 and becomes chunks 2c, 2c+1 of the row's 128 bytes in the tile, each XOR-ed with row % 8 (128-byte swizzle;
-    // the row itself starts at row * 128); a step of the loop moves on by a multiple of 8 rows.  4-bit: piece u is half
-    // c = u % 2 of row u / 2 and becomes chunks 4c .. 4c+3.
-    const uint32_t off8 = static_cast<uint32_t>(first >> 2) * 128u + (((2u * (first & 3)) ^ ((first >> 2) & 7u)) << 4);
-    const uint32_t off4 = static_cast<uint32_t>(first >> 1) * 128u + (((4u * (first & 1)) ^ ((first >> 1) & 4u)) << 4);
-    const uint32_t x3 = ((first >> 1) & 3u) << 4;
-    const uint32_t raw_step = static_cast<uint32_t>(step) * 16u;          // bytes of the raw block per step
-    const uint32_t tile_step8 = static_cast<uint32_t>(step) * 32u;        // 8 G rows of the tile
-    const uint32_t tile_step4 = static_cast<uint32_t>(step) * 64u;        // 16 G rows of the tile
-    // Width of a tile's rows and where they start in the buffer of that width (4-bit: for the exponents).
-    auto tile_info = [&](int tt, int& width, int& wrow) {
-      width = 8; wrow = 0;
-      if (p.group_width) {
-        const int g = pair + tt * npairs;
-        width = p.group_width[g];
-        wrow = p.group_row[g] + static_cast<int>(rank) * p.tile_rows;
+    // Where this lane's row starts in the slot, and what the swizzle does to the index of its 16-byte pieces.
+    const uint32_t off8 = static_cast<uint32_t>(row) * 128u, x8 = (static_cast<uint32_t>(row) & 7u) << 4;
+    const uint32_t off4 = static_cast<uint32_t>(row) * 64u, x4 = (static_cast<uint32_t>(row >> 1) & 3u) << 4;
+    // Ring slot and phase of block i of the CTA's sequence; operand slot of block i; ring slot and phase of block
+    // i - a_slots, whose MMAs must be done before the operand slot is overwritten.  a_slots <= stages, so having waited
+    // for that block implies that the slot's previous codes have been used up, and no wait is more than a phase behind.
+    int stage = grp, aslot = grp;                        // (grp < conv_groups <= a_slots <= stages)
+    int old_stage = (grp - p.a_slots) & (G - 1);         // first block >= a_slots of this group, less a_slots
+    uint32_t phase = 0, old_phase = 0;
+    int i = grp, kb = grp;                               // block i is block kb of tile t
+    bool ok = grp < G;
+    for (int t = 0; t < my_tiles && ok; ++t) {
+      const int g = pair + t * npairs;
+      const int width = p.group_width ? p.group_width[g] : 8;
+      const int n_blocks = width == 16 ? p.n_kblocks : code_blocks;
+      // (4-bit) exponents of this lane's row, one per K block, fetched two of the group's blocks ahead
+      const uint8_t* sh = nullptr;
+      if (width == 4) {
+        const int r4 = p.group_row[g] + static_cast<int>(rank) * p.tile_rows + row;
+        if (r4 < p.rows4) sh = p.shift4 + r4;
       }
-    };
-    // (4-bit) the exponents of this lane's rows in K block kkb: a sub-block of 128 hidden channels spans two K blocks
-    auto fetch_shifts = [&](int kkb, int width, int wrow, uint32_t (&e)[8]) {
-      const uint8_t* sh = p.shift4 + static_cast<size_t>(kkb >> 1) * p.rows4;
-#pragma unroll
-      for (int n = 0; n < 8; ++n) {
-        const int row = (first + step * n) >> 1;
-        const int r4 = wrow + row;
-        e[n] = (width == 4 && row < p.tile_rows && r4 >= 0 && r4 < p.rows4) ? sh[r4] : 0u;
-      }
-    };
-    int tile_width, w_row;
-    uint32_t e[8];
-    if (grp < ngroups && grp < total_blocks) {
-      tile_info(t, tile_width, w_row);
-      if (tile_width == 4) fetch_shifts(kb, tile_width, w_row, e);
-    }
-    int stage = grp;                                     // ring slot and phase of block i (grp < ngroups <= stages)
-    uint32_t phase = 0;
-    for (int i = grp; i < total_blocks && grp < ngroups; i += ngroups) {
-      uint8_t* slot = smem + stage * stage_bytes;
-      uint32_t shifts = 0;                               // one nibble per step
-      if (tile_width == 4) {
-#pragma unroll
-        for (int n = 0; n < 8; ++n) shifts |= min(e[n], 4u) << (4 * n);
-      }
-      // the group's next block: its exponents are fetched while this block is waited for and expanded
-      int t2 = t, kb2 = kb + ngroups, width2 = tile_width, w_row2 = w_row;
-      while (kb2 >= p.n_kblocks) { kb2 -= p.n_kblocks; ++t2; }
-      if (i + ngroups < total_blocks) {
-        if (t2 != t) tile_info(t2, width2, w_row2);
-        if (width2 == 4) fetch_shifts(kb2, width2, w_row2, e);
-      }
-      // first the slot's previous use (which implies that its raw block's previous phase is over), then this block's bytes
-      if (!mbar_wait_warp(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) break;
-      if (mem == 0 && lane == 0) {                       // the slot is free: its hidden blocks arrive while the W_lm block is expanded
-        const uint32_t sa = base + stage * stage_bytes;
-        const uint32_t fb = leader_full + 8 * stage;
-        mbar_expect_tx_cluster(fb, hid_tx_bytes);
-        for (int sb = 0; sb < p.n_sub; ++sb)
-          tma_load_2d(sa + kWBlockBytes + sb * hid_block_bytes, &tmap_hidden, fb, kb * kKStep,
-                      row0 + sb * p.N + static_cast<int>(rank) * half_n, pol_h);
-      }
-      if (!mbar_wait_warp(rawfull_bar + 8 * stage, phase, abort_flag, p.status)) break;
-      // Two pieces per trip of a loop that is kept rolled: the expansion of a whole block written out is some ten
-      // thousand bytes of straight-line code per width, which a warp would fetch anew for every block (measured: rolled
-      // is faster, and four pieces per trip are no faster than two).
-      const uint8_t* src = slot + raw_off + first * 16;
-      if (tile_width == 8) {
-        uint32_t o = off8;
-#pragma unroll 1
-        for (int u0 = first; u0 < units; u0 += 2 * step, src += 2 * raw_step, o += 2 * tile_step8) {
-          const bool two = u0 + step < units;
-          const uint4 x0 = *reinterpret_cast<const uint4*>(src);
-          const uint4 x1 = two ? *reinterpret_cast<const uint4*>(src + raw_step) : make_uint4(0u, 0u, 0u, 0u);
-          expand_int8x16(x0, slot + o, slot + (o ^ 16u));
-          if (two) expand_int8x16(x1, slot + o + tile_step8, slot + ((o + tile_step8) ^ 16u));
+      uint32_t sh0 = sh && kb < n_blocks ? sh[static_cast<size_t>(kb) * p.rows4] : 0u;
+      uint32_t sh1 = sh && kb + G < n_blocks ? sh[static_cast<size_t>(kb + G) * p.rows4] : 0u;
+      for (; kb < n_blocks; kb += G, i += G) {
+        const uint32_t sh2 = sh && kb + 2 * G < n_blocks ? sh[static_cast<size_t>(kb + 2 * G) * p.rows4] : 0u;
+        if (i >= p.a_slots) {
+          if (!mbar_wait_together(empty_bar + 8 * old_stage, old_phase, abort_flag, p.status)) { ok = false; break; }
+          tc_fence_after();
+          old_stage += G;
+          if (old_stage >= p.stages) { old_stage -= p.stages; old_phase ^= 1u; }
         }
-      } else if (tile_width == 4) {
-        uint32_t o = off4;
-#pragma unroll 1
-        for (int n = 0; n < 8; n += 2, src += 2 * raw_step, o += 2 * tile_step4) {   // 32-byte rows: two pieces per row
-          const int u0 = first + step * n;
-          if (u0 >= (units >> 1)) break;
-          const bool two = u0 + step < (units >> 1);
-          const uint4 x0 = *reinterpret_cast<const uint4*>(src);
-          const uint4 x1 = two ? *reinterpret_cast<const uint4*>(src + raw_step) : make_uint4(0u, 0u, 0u, 0u);
-          expand_int4x32(x0, slot + o, x3, static_cast<int>((shifts >> (4 * n)) & 15u));
-          if (two) expand_int4x32(x1, slot + o + tile_step4, x3, static_cast<int>((shifts >> (4 * n + 4)) & 15u));
+        if (width != 16) {
+          if (!mbar_wait_together(rawfull_bar + 8 * stage, phase, abort_flag, p.status)) { ok = false; break; }
+          const uint8_t* slot = smem + stage * stage_bytes;
+          const uint32_t dst = operand_lane + aslot * kOperandCols;
+          if (width == 8) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              uint4 x[4];
+              uint32_t o[32];
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                x[c] = *reinterpret_cast<const uint4*>(slot + off8 + ((16u * (4 * half + c)) ^ x8));
+#pragma unroll
+              for (int c = 0; c < 4; ++c) expand_int8x16(x[c], o + 8 * c);
+              tmem_st32(dst + 32 * half, o);
+            }
+          } else {
+            const uint32_t shift = min(sh0, 4u);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              uint4 x[2];
+              uint32_t o[32];
+#pragma unroll
+              for (int c = 0; c < 2; ++c)
+                x[c] = *reinterpret_cast<const uint4*>(slot + off4 + ((16u * (2 * half + c)) ^ x4));
+#pragma unroll
+              for (int c = 0; c < 2; ++c) expand_int4x32(x[c], o + 16 * c, shift);
+              tmem_st32(dst + 32 * half, o);
+            }
+          }
+          tmem_st_wait();
+          tc_fence_before();
         }
+        __syncwarp();
+        if (elect_one()) mbar_arrive_cluster(leader_operand + 8 * aslot);
+        sh0 = sh1; sh1 = sh2;
+        stage += G;
+        if (stage >= p.stages) { stage -= p.stages; phase ^= 1u; }
+        aslot += G;
+        if (aslot >= p.a_slots) aslot -= p.a_slots;
       }
-      // (16-bit rows were loaded into the tile as they are)
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // generic-proxy writes, read by the MMA
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive_cluster(leader_full + 8 * stage);    // this warp's share of the bf16 tile is in place
-        mbar_arrive(rawempty_bar + 8 * stage);           // and the raw block may be refilled
-      }
-      t = t2; kb = kb2; tile_width = width2; w_row = w_row2;
-      stage += ngroups;
-      if (stage >= p.stages) { stage -= p.stages; phase ^= 1u; }
+      kb -= n_blocks;                                    // where this group starts in the next tile
     }
   }
 
@@ -2161,8 +2222,8 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   Plan best{};
   double best_cost = 1e300;
   const int rows = M > 0 ? M : 1;
-  // 8-bit W_lm: one MMA per K step (at most 256 rows per pass), and the slot also holds the int8 block
-  const int max_rows_per_pass = (w8 || two) ? kMaxN : kMaxRowsPerPass;
+  // expanded on chip: one MMA per K step, and tensor memory also holds the operand; two planes: two MMAs hold 256 rows
+  const int max_rows_per_pass = w8 ? kExpandMaxN : two ? kMaxN : kMaxRowsPerPass;
   const int p_min = (rows + max_rows_per_pass - 1) / max_rows_per_pass;
   const double t_hbm = (w8 || i8 ? 1.0 : 2.0) * ctx->V * static_cast<double>(ctx->H) / 6.4e12;
   const int p_max = ctx->force_passes > p_min + 3 ? ctx->force_passes : p_min + 3;
@@ -2188,7 +2249,7 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   }
   // a pass may end up empty when rows_per_pass * (passes - 1) already covers M
   best.passes = (rows + best.rows_per_pass - 1) / best.rows_per_pass;
-  const int stage_bytes = kWBlockBytes + best.n_sub * (best.N / 2) * 128 + (w8 ? kRawBlockBytes : 0);
+  const int stage_bytes = kWBlockBytes + (w8 ? 2 : best.n_sub) * (best.N / 2) * 128;
   // (rotating units: every epilogue warp stages a whole 32-row chunk, twice the bytes)
   const int trans_bytes = (w8 ? kW8EpiWarps : kEpiWarps) * kTransBytes * (best.n_sub == 3 ? 2 : 1);
   int stages = (kSmemBudget - 1024 - kBarrierBytes - trans_bytes) / stage_bytes;
@@ -2230,21 +2291,19 @@ const Plan& plan_for(hola_ctx* ctx, int M, int w_dtype) {
   return e.pl;
 }
 
-// K-major 2-D tensor map with a box of 64 elements x box_rows.  bf16: 128-byte swizzle (the layout the MMA reads);
-// int8: plain rows of 64 bytes (the converter warps read them).
-// int8 with swizzle (8-bit MMA): box of 128 elements = 128 bytes, 128-byte swizzle, the same bytes as a bf16 block.
-// `packed4`: rows of cols / 2 bytes holding two 4-bit codes each; box of 32 bytes (64 codes) x box_rows, plain rows.
+// K-major 2-D tensor map.  bf16: box of 64 elements x box_rows; int8: box of 128 elements; both 128 bytes per row with
+// the 128-byte swizzle that the MMA reads (and that spreads the rows of 8-bit codes over the banks for the converter
+// warps).  `packed4`: rows of cols / 2 bytes holding two 4-bit codes each; box of 64 bytes (128 codes), 64-byte swizzle.
 hola_status encode_map(hola_ctx* ctx, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
-                       uint32_t box_rows, bool int8 = false, bool int8_swizzled = false, bool packed4 = false) {
-  if (packed4) { cols /= 2; int8 = true; int8_swizzled = false; }
+                       uint32_t box_rows, bool int8 = false, bool packed4 = false) {
+  if (packed4) { cols /= 2; int8 = true; }
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {cols * (int8 ? 1u : 2u)};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(packed4 ? kBlockK / 2 : (int8_swizzled ? 2 * kBlockK : kBlockK)),
-                             box_rows};
+  const cuuint32_t box[2] = {static_cast<cuuint32_t>(int8 && !packed4 ? 2 * kBlockK : kBlockK), box_rows};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = ctx->encode(map, int8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                                  const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                 (int8 && !int8_swizzled) ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+                                 packed4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     snprintf(ctx->last_error, sizeof ctx->last_error, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
@@ -2308,17 +2367,17 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     me->valid = 0;
     if (two)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(2 * round_up(M, 32)), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, true);
+                     static_cast<uint32_t>(pl.N / 2), true);
     else if (i8)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, true);
+                     static_cast<uint32_t>(pl.N / 2), true);
     else
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
                      static_cast<uint32_t>(pl.N / 2));
     if (s != HOLA_OK) return s;
     const uint32_t trows = static_cast<uint32_t>(pl.tile_rows);
     if (!mixed) {
-      s = encode_map(ctx, &me->tw, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, w8 || i8, i8);
+      s = encode_map(ctx, &me->tw, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, w8 || i8);
       if (s != HOLA_OK) return s;
       me->tw4 = me->tw; me->tw16 = me->tw;               // (never read outside the mixed-width form)
       me->W4 = nullptr; me->W16 = nullptr;
@@ -2332,7 +2391,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
       }
       if (mx->rows4 > 0) {
         s = encode_map(ctx, &me->tw4, mx->W4, static_cast<uint64_t>(mx->rows4), static_cast<uint64_t>(a->H), trows, true,
-                       false, true);
+                       true);
         if (s != HOLA_OK) return s;
         if (!have) me->tw = me->tw4;
         have = true;
@@ -2356,7 +2415,10 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   K1Params kp;
   kp.M = M; kp.V = a->V; kp.n_ptiles = pl.n_ptiles; kp.n_kblocks = pl.n_kblocks;
   kp.pair256 = (pl.rot && pl.N == 128 && !ctx->no_pair256) ? 1 : 0;
-  kp.conv_group = ctx->conv_group > 0 ? ctx->conv_group : 2;
+  kp.acc_cols = !w8 ? 256 : (pl.N <= 128 ? 128 : kExpandMaxN);
+  kp.conv_groups = ctx->conv_group > kConvGroup ? 1 : kConvGroups;
+  const int a_slots = (kTmemCols - 2 * kp.acc_cols) / kOperandCols;
+  kp.a_slots = a_slots < pl.stages ? a_slots : pl.stages;
   kp.stages = pl.stages; kp.nbuf = pl.nbuf; kp.rot = pl.rot; kp.n_sub = pl.n_sub; kp.N = pl.N; kp.tile_rows = pl.tile_rows; kp.ldl = ldl;
   kp.logits = logits; kp.partials = ctx->partials; kp.part_stride = ctx->max_rows;
   kp.status = a->status_word ? a->status_word : ctx->status;
@@ -2692,7 +2754,7 @@ hola_status hola_set_option(hola_ctx* ctx, int option, int value) {
       ctx->no_pace = value == 2;
       break;
     case HOLA_OPT_CONVERTER_GROUP:
-      if (value < 0 || value > kConvWarps) return HOLA_ERR_INVALID_ARG;
+      if (value < 0 || value > kConvGroup * kConvGroups) return HOLA_ERR_INVALID_ARG;
       ctx->conv_group = value;
       break;
     case HOLA_OPT_PASSES:

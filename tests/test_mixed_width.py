@@ -184,3 +184,33 @@ def test_converter_group_size_changes_speed_not_results(binding):
     rep = compare.compare(orc, _np(w.draft_q), _np(w.uniforms), _np(base.accept_len), _np(base.next_tok),
                           _np(base.entropy), _np(base.logZ), _np(base.logits))
     assert rep.ok, rep.summary()
+
+
+@pytest.mark.parametrize("B,k,H,V,pattern", [
+    (32, 3, 128, 1100, [4, 8]),                # 128 rows, one K block of codes per tile, four operand slots
+    (43, 2, 384, 2100, [16, 4, 8]),            # 129 rows: wider accumulators, two operand slots
+    (64, 2, 640, 2500, [8, 16, 4, 4]),         # 192 rows, the most one pass holds; an odd number of K blocks
+    (193, 0, 256, 900, [4, 16]),               # 193 rows: two passes
+    (3, 4, 176, 1100, None), (64, 2, 112, 37000, None),   # all 8-bit (no width table): ragged last K block, many tiles
+])
+def test_expansion_at_the_edges_of_its_tiles(binding, B, k, H, V, pattern):
+    """Row counts around the switch of the accumulator layout and of the pass count, K extents around the 128-channel
+    blocks of codes and the 64-channel blocks of 16-bit rows: logits against an fp64 product of the dequantised weights
+    (fp32 accumulation, one rounding or truncation of 2^-23 per step of sixteen products and per product within a step:
+    an error below (H / 16 + 16) 2^-23 of sum |terms|)."""
+    w = workloads.gaussian_head("edges", B, k, H, V, seed=B + H, device=DEV, w_std=0.3)
+    if pattern is None:
+        head, scale = binding.hola_quantize_w8(w.W_lm)
+        Wd = head.double() * scale.double()[:, None]
+    else:
+        head, scale = binding.hola_quantize_mixed(w.W_lm, _widths(V, pattern)), None
+        W32 = ref.bf16_bits_to_f64(_np(w.W_lm)).astype(np.float32)
+        Wd = torch.from_numpy(lobi.dequantize_mixed(W32, _widths(V, pattern))).to(DEV)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        out = ctx.hola_verify(w.hidden, head, w.draft_tok, w.draft_q, w.uniforms, w.tau, want_logits=True, w_scale=scale)
+        torch.cuda.synchronize()
+    assert int(out.status.item()) == 0
+    h = w.hidden.double()
+    want = h @ Wd.T
+    bound = (H / 16 + 16) * 2.0 ** -23 * (h.abs() @ Wd.abs().T)
+    assert torch.all((out.logits.double() - want).abs() <= bound)
