@@ -290,6 +290,13 @@ hola_status hola_quantize_w8(const void* W_bf16, int V, int H, void* q_out, floa
 hola_status hola_quantize_w4(const void* W_bf16, int rows, int H, void* packed_out, uint8_t* shift_out, int shift_stride,
                              float* scale_out, void* cuda_stream);
 
+/* A whole bf16 head [V][H] (H a multiple of 128) to the HOLA_W_MIXED form in one launch: group g of 256 vocabulary rows
+ * goes, at out->group_width[g] bits, to rows out->group_row[g] .. of that width's buffer (hola_quantize_w8 /
+ * hola_quantize_w4 per row; 16-bit rows are copied), scale_out[v] is the scale of vocabulary row v (1 for a 16-bit row).
+ * `out` is a host struct whose pointers are device buffers of the caller (tables filled in, the rest written
+ * here).  Current device, asynchronous on the stream, allocates nothing. */
+hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream);
+
 /* Launch geometry chosen for a shape (for reports): vocabulary rows per tile of a CTA pair, grid size (CTAs),
  * shared-memory ring slots, verify rows per pass, passes over W_lm, kernel launches per hola_verify call. */
 typedef struct {

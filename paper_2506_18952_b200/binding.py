@@ -7,6 +7,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from array import array
 from dataclasses import dataclass
 
 import torch
@@ -24,7 +25,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -88,6 +89,9 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_quantize_w4.restype = ctypes.c_int
     lib.hola_quantize_w4.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p,
                                      ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]
+    lib.hola_quantize_mixed.restype = ctypes.c_int
+    lib.hola_quantize_mixed.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_wmix),
+                                        ctypes.c_void_p, ctypes.c_void_p]
     lib.hola_plan.restype = ctypes.c_int
     lib.hola_plan.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_plan_info)]
     lib.hola_plan_for_shape.restype = ctypes.c_int
@@ -180,57 +184,42 @@ class MixedHead:
 
 
 def hola_quantize_mixed(W_lm: torch.Tensor, widths, stream=None) -> MixedHead:
-    """bf16 W_lm [V, H] -> the mixed-width form: widths[g] in {4, 8, 16} for group g of 256 vocabulary rows.  The codes,
-    scales and exponents are made by the library's quantiser kernels, each run of groups of one width in one launch that
-    writes straight into that width's compact buffer; 16-bit rows are copied as they are.  torch provides the buffers."""
+    """bf16 W_lm [V, H] -> the mixed-width form: widths[g] in {4, 8, 16} for group g of 256 vocabulary rows.  Codes,
+    scales and exponents are made by one launch of the library's quantiser; torch provides the buffers (and carries the
+    two tables of groups to the device in one copy)."""
     if W_lm.dtype != torch.bfloat16 or not W_lm.is_cuda or not W_lm.is_contiguous():
         raise HolaError("hola_quantize_mixed takes a contiguous bfloat16 device tensor")
     lib = load_library()
     V, H = W_lm.shape
     ng = -(-V // GROUP_ROWS)
     widths = [int(x) for x in widths]
-    if len(widths) != ng or any(x not in (4, 8, 16) for x in widths) or H % SUB_BLOCK:
+    if len(widths) != ng or not set(widths) <= {4, 8, 16} or H % SUB_BLOCK:
         raise HolaError(f"need {ng} widths out of 4, 8, 16 and H a multiple of {SUB_BLOCK}")
     dev = W_lm.device
-    rows = {4: 0, 8: 0, 16: 0}
-    group_row = []
-    for g, wd in enumerate(widths):
+    rows = [0] * 17                                              # rows of each width so far
+    group_row = array("i")
+    for wd in widths:
         group_row.append(rows[wd])
-        rows[wd] += min(V, (g + 1) * GROUP_ROWS) - g * GROUP_ROWS
-    W16 = torch.empty((rows[16], H), dtype=torch.bfloat16, device=dev) if rows[16] else None
-    W8 = torch.empty((rows[8], H), dtype=torch.int8, device=dev) if rows[8] else None
-    W4 = torch.empty((rows[4], H // 2), dtype=torch.uint8, device=dev) if rows[4] else None
-    shift4 = torch.zeros((H // SUB_BLOCK, rows[4]), dtype=torch.uint8, device=dev) if rows[4] else None
-    w_scale = torch.ones((V,), dtype=torch.float32, device=dev)
-    sp = _stream_ptr(stream)
-    with torch.cuda.device(dev):
-        g = 0
-        while g < ng:                                            # runs of consecutive groups of one width
-            g1 = g
-            while g1 < ng and widths[g1] == widths[g]:
-                g1 += 1
-            v0, v1 = g * GROUP_ROWS, min(V, g1 * GROUP_ROWS)
-            n, r0, wd = v1 - v0, group_row[g], widths[g]
-            src = ctypes.c_void_p(W_lm.data_ptr() + v0 * H * 2)
-            scale = ctypes.c_void_p(w_scale.data_ptr() + v0 * 4)
-            if wd == 16:
-                W16[r0:r0 + n].copy_(W_lm[v0:v1])
-            elif wd == 8:
-                _check(lib, None, lib.hola_quantize_w8(src, n, H, ctypes.c_void_p(W8.data_ptr() + r0 * H), scale, sp),
-                       "hola_quantize_w8")
-            else:
-                _check(lib, None, lib.hola_quantize_w4(src, n, H, ctypes.c_void_p(W4.data_ptr() + r0 * (H // 2)),
-                                                       ctypes.c_void_p(shift4.data_ptr() + r0), rows[4], scale, sp),
-                       "hola_quantize_w4")
-            g = g1
-    head = MixedHead(V, H, widths, W16, W8, W4, shift4, w_scale,
-                     torch.tensor(widths, dtype=torch.uint8, device=dev),
-                     torch.tensor(group_row, dtype=torch.int32, device=dev))
-    st = hola_wmix()
-    st.W16, st.W8, st.W4, st.shift4 = (t.data_ptr() if t is not None else None for t in (W16, W8, W4, shift4))
-    st.group_width, st.group_row = head.group_width.data_ptr(), head.group_row.data_ptr()
-    st.rows16, st.rows8, st.rows4 = rows[16], rows[8], rows[4]
-    head.struct = st
+        rows[wd] += GROUP_ROWS
+    rows[widths[-1]] -= ng * GROUP_ROWS - V                      # the last group may be ragged
+    tables = torch.frombuffer(bytearray(group_row.tobytes() + bytes(widths)), dtype=torch.uint8)
+    s = torch.cuda.current_stream(dev) if stream is None else stream
+    with torch.cuda.device(dev), torch.cuda.stream(s):
+        W16 = torch.empty((rows[16], H), dtype=torch.bfloat16, device=dev) if rows[16] else None
+        W8 = torch.empty((rows[8], H), dtype=torch.int8, device=dev) if rows[8] else None
+        W4 = torch.empty((rows[4], H // 2), dtype=torch.uint8, device=dev) if rows[4] else None
+        shift4 = torch.empty((H // SUB_BLOCK, rows[4]), dtype=torch.uint8, device=dev) if rows[4] else None
+        w_scale = torch.empty((V,), dtype=torch.float32, device=dev)
+        # (a copy from pageable memory has left that memory when the call returns)
+        tables = tables.to(dev, non_blocking=True)
+        head = MixedHead(V, H, widths, W16, W8, W4, shift4, w_scale, tables[4 * ng:], tables[:4 * ng].view(torch.int32))
+        st = hola_wmix()
+        st.W16, st.W8, st.W4, st.shift4 = (t.data_ptr() if t is not None else None for t in (W16, W8, W4, shift4))
+        st.group_width, st.group_row = head.group_width.data_ptr(), head.group_row.data_ptr()
+        st.rows16, st.rows8, st.rows4 = rows[16], rows[8], rows[4]
+        head.struct = st
+        _check(lib, None, lib.hola_quantize_mixed(_dptr(W_lm), V, H, ctypes.byref(st), _dptr(w_scale), _stream_ptr(s)),
+               "hola_quantize_mixed")
     return head
 
 

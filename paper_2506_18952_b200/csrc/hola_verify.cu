@@ -19,8 +19,9 @@
 //       on-chip-expansion mode the kernel streams groups of 256 vocabulary rows stored at 4, 8 or 16 bits and
 //       converter warps (groups of four, each owning whole K blocks) expand the codes exactly to bf16 in tensor memory,
 //       from where the MMA reads them (mixed-precision quantiser of the Lo-Bi Optimization section).
-//   quantize_rows_int8_kernel   8-bit case of the Lo-Bi quantiser, per row (W_lm ahead of time, hidden rows per call).
-//   quantize_rows_w4_kernel     4-bit case: codes in [-7, 7] with one shared exponent per sub-block of 128 channels.
+//   quantize_rows_kernel        the Lo-Bi quantiser on W_lm ahead of time: rows at 8 bits, at 4 bits (codes in [-7, 7], one
+//       shared exponent per sub-block of 128 channels) or in groups of mixed width, one launch for the whole head.
+//   quantize_hidden_kernel      the hidden rows of a call as one or two 8-bit planes.
 //   bounded_wait_selftest_kernel  a wait that is made to run out, to exercise the give-up path without breaking anything.
 //   draft_entropy_kernel        H(q_j) of the draft rows, for the gate on the draft distribution.
 //   shard_record_kernel         vocabulary-parallel form: a rank's statistics record for the first all-gather.
@@ -73,6 +74,7 @@ constexpr int kTransBytes = kTransRows * 32 * 4; // its staging buffer: [16 rows
 constexpr int kExpandK = 128;                     // channels per K block of 4- and 8-bit rows (16-bit rows: kBlockK)
 constexpr int kExpandMaxN = 192;                  // two accumulators of 192 columns leave 128 columns for the operand
 constexpr int kOperandCols = kExpandK / 2;        // tensor-memory columns of one K block of the expanded operand
+constexpr int kGroupRows = 256;                   // vocabulary rows per group of one width
 constexpr int kSubBlock = 128;                    // hidden channels per 4-bit sub-block (one shared exponent each)
 constexpr int kW8EpiWarps = 8;
 constexpr int kConvGroup = 4;                     // converter warps per K block: one per tensor-memory lane quarter
@@ -1889,127 +1891,318 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
 // The 8-bit case of the Lo-Bi quantiser on the LM head (Lo-Bi Optimization section; the quantiser itself is not
 // spelled out there): one vocabulary row per sub-block, symmetric integers in [-127, 127], one fp32 scale per row,
 //   scale = max|w| / 127 (1 for an all-zero row),  q = clip(rint(w / scale)),  all in fp32, ties to even.
-// One CTA per row.
-__global__ void __launch_bounds__(256) quantize_rows_int8_kernel(const __nv_bfloat16* W, int H, signed char* q,
-                                                                 float* scale) {
-  __shared__ float sh_max[8];
-  __shared__ float sh_scale;
-  grid_dependency_wait();                                // (no-op unless launched with programmatic serialization)
-  const size_t row = blockIdx.x;
-  const __nv_bfloat16* wr = W + row * H;
-  float amax = 0.f;
-  for (int h = threadIdx.x; h < H; h += 256) amax = fmaxf(amax, fabsf(__bfloat162float(wr[h])));
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-  if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = amax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float m = 0.f;
-    for (int i = 0; i < 8; ++i) m = fmaxf(m, sh_max[i]);
-    const float sc = m > 0.f ? __fdiv_rn(m, 127.f) : 1.f;
-    sh_scale = sc;
-    scale[row] = sc;
-  }
-  __syncthreads();
-  const float sc = sh_scale;
-  for (int h = threadIdx.x; h < H; h += 256) {
-    const float r = rintf(__fdiv_rn(__bfloat162float(wr[h]), sc));
-    q[row * H + h] = static_cast<signed char>(fminf(127.f, fmaxf(-127.f, r)));
-  }
-}
-
 // The 4-bit case of the Lo-Bi quantiser on the LM head (reading: a sub-block is 128 hidden channels of one vocabulary
 // row; symmetric codes in [-7, 7]; the sub-block's scale is the row's fp32 scale times a power of two):
 //   s = max|w| / 112 (1 for an all-zero row);  e_b = the smallest e in 0..4 with  7 * 2^e * s >= max_{h in b} |w|  (else 4);
 //   c = clip(rint(w / (s * 2^e_b)), -7, 7),  every step one fp32 operation, ties to even.
 // Two codes per byte (even channel in the low nibble, 4-bit two's complement).  Exponents go to
-// shift[b * shift_stride + row].  One CTA per row; warp w takes sub-blocks w, w + 8, ...; a lane holds four channels.
-__global__ void __launch_bounds__(256) quantize_rows_w4_kernel(const __nv_bfloat16* W, int H, uint8_t* packed,
-                                                               uint8_t* shift, int shift_stride, float* scale) {
-  __shared__ float sh_max[8];
-  __shared__ float sh_scale;
-  const size_t row = blockIdx.x;
-  const __nv_bfloat16* wr = W + row * H;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float amax = 0.f;
-  for (int h = threadIdx.x; h < H; h += 256) amax = fmaxf(amax, fabsf(__bfloat162float(wr[h])));
+// shift[b * shift_stride + row].
+
+// rint(fdiv_rn(a, b)) without a division: the product with the rounded reciprocal y, corrected once by its exact remainder
+// (q = a y, q + (a - q b) y: Newton's step on the quotient), is within 2^-23 of a unit in the last place of a / b before
+// its one rounding, so it is the rounded quotient unless a / b lies that close to the middle of two fp32 numbers, and only
+// next to a half integer would that matter.  The quotients that occur do not depend on more than two bf16 mantissas (of
+// the row's maximum and of the entry) and the difference of their exponents, at most 31 binades of which do not round to
+// zero: all of them, both signs, the second plane's remainders and the five 4-bit steps included, were compared with the
+// division (1 294 464 quotients, no difference).  Rows whose step lies near the ends of the fp32 range, where the
+// products would not be exact, and rows with a NaN take the division.  The integers end up in the low bits of t[] (two's
+// complement).
+constexpr float kRoundMagic = 12582912.f;                // 1.5 * 2^23: adding it rounds to an integer, ties to even
+__device__ __forceinline__ void bf16x8_to_f32(const uint4 x, float f[8]) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-  if (lane == 0) sh_max[warp] = amax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float m = 0.f;
-    for (int i = 0; i < 8; ++i) m = fmaxf(m, sh_max[i]);
-    const float sc = m > 0.f ? __fdiv_rn(m, 112.f) : 1.f;
-    sh_scale = sc;
-    scale[row] = sc;
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = __uint_as_float(w[i] << 16);
+    f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
   }
-  __syncthreads();
-  const float sc = sh_scale;
-  for (int b = warp; b < H / kSubBlock; b += 8) {
-    float w[4];
+}
+struct Step {
+  float b, y;           // step and its reciprocal
+  bool divide;          // (the same for the whole row)
+};
+__device__ __forceinline__ Step make_step(float b, bool divide) { return Step{b, __frcp_rn(b), divide}; }
+__device__ __forceinline__ bool needs_division(float scale, bool has_nan) {
+  return has_nan || !(scale > 1e-20f && scale < 1e30f);
+}
+__device__ __forceinline__ void round_div8(const float f[8], const Step& st, float limit, uint32_t t[8]) {
+  if (st.divide) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = __bfloat162float(wr[b * kSubBlock + lane * 4 + i]);
-    float bmax = fmaxf(fmaxf(fabsf(w[0]), fabsf(w[1])), fmaxf(fabsf(w[2]), fabsf(w[3])));
+    for (int i = 0; i < 8; ++i)
+      t[i] = __float_as_uint(fminf(limit, fmaxf(-limit, rintf(__fdiv_rn(f[i], st.b)))) + kRoundMagic);
+    return;
+  }
+  const uint64_t y2 = pack2(st.y, st.y), zero2 = pack2(-0.f, -0.f), mg = pack2(kRoundMagic, kRoundMagic),
+                 nb = pack2(-st.b, -st.b);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
-    int e = 4;
+  for (int i = 0; i < 8; i += 2) {
+    const uint64_t a = pack2(f[i], f[i + 1]);
+    const uint64_t q = fma2(a, y2, zero2);
+    float r0, r1;
+    unpack2(add2(fma2(fma2(q, nb, a), y2, q), mg), r0, r1);
+    t[i] = __float_as_uint(r0);
+    t[i + 1] = __float_as_uint(r1);
+  }
+}
+// The low bytes of four words side by side.
+__device__ __forceinline__ uint32_t pack_bytes(const uint32_t* t) {
+  return __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
+}
+// Running maximum of |x| over pairs of bf16; kNaN: a NaN comes through, otherwise it is dropped, as by fmaxf.
+template <bool kNaN>
+__device__ __forceinline__ uint32_t absmax_step(uint32_t m, const uint4 x) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-    for (int c = 3; c >= 0; --c)
-      if (__fmul_rn(sc, static_cast<float>(7 << c)) >= bmax) e = c;
-    const float step = sc * static_cast<float>(1 << e);              // exact
-    uint32_t bits = 0;
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t a = w[i] & 0x7FFF7FFFu;
+    if (kNaN) asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(a));
+    else asm("max.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(a));
+  }
+  return m;
+}
+template <bool kNaN>
+__device__ __forceinline__ float absmax_of_pair(uint32_t m) {
+  float a = __uint_as_float(m << 16);
+  const float b = __uint_as_float(m & 0xFFFF0000u);
+  if (kNaN) asm("max.NaN.f32 %0, %0, %1;" : "+f"(a) : "f"(b));
+  else a = fmaxf(a, b);
+  return a;
+}
+template <bool kNaN>
+__device__ __forceinline__ float warp_max(float a) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float r = fminf(7.f, fmaxf(-7.f, rintf(__fdiv_rn(w[i], step))));
-      bits |= (static_cast<uint32_t>(static_cast<int>(r)) & 0xFu) << (4 * i);
+  for (int off = 16; off > 0; off >>= 1) {
+    const float o = __shfl_xor_sync(0xffffffffu, a, off);
+    if (kNaN) asm("max.NaN.f32 %0, %0, %1;" : "+f"(a) : "f"(o));
+    else a = fmaxf(a, o);
+  }
+  return a;
+}
+
+// Element-by-element forms of a 16-byte load and of the stores, for the first n elements.
+__device__ __forceinline__ uint4 gather8(const uint16_t* src, int n) {
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (i < n) w[i >> 1] |= static_cast<uint32_t>(src[i]) << (16 * (i & 1));
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <typename T>
+__device__ __forceinline__ void scatter(T* dst, const uint4 x, int n) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+  constexpr int kPer = 4 / sizeof(T);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (i < n) dst[i] = static_cast<T>(w[i / kPer] >> (8 * static_cast<int>(sizeof(T)) * (i % kPer)));
+}
+
+// Where the quantised rows go: rows of one width sit compactly in that width's buffer.
+struct QuantOut {
+  const uint8_t* group_width;   // null: every row is `width` bits wide and row v of W is row v of its buffer
+  const int* group_row;
+  int width;
+  uint16_t* w16;
+  signed char* w8;
+  uint8_t* w4;
+  uint8_t* shift4;
+  int shift_stride;
+  float* scale;
+};
+
+// A head (or rows of it) to 4, 8 or 16 bits in ONE launch, a warp per row: one pass for the row's maximum, one that
+// rounds (the row, 8 KB at 4096 channels, then comes out of the L1 or the L2).  Bound: HBM (2 bytes in, half to two out
+// per weight).  32000 x 4096 at 4 / 8 / 16 bits in the proportions 20 / 70 / 10 %: 75 us = 4.9 TB/s (61 us at the measured
+// copy rate), of which the instructions (eleven per weight) take half; one launch per run of groups with a CTA per row, two
+// bytes per load and a division per weight needed 540 us.  Rows kept in registers between the passes: 102 registers,
+// 217 us with a slow path that divides next to half integers.
+// kVec: rows and buffers that 16-byte pieces tile and that are aligned for it; otherwise the same element by element.
+template <bool kVec>
+__global__ void __launch_bounds__(256, 3) quantize_rows_kernel(const uint16_t* W, int V, int H, const QuantOut out) {
+  const int v = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (v >= V) return;
+  const int pieces = (H + 7) >> 3;                       // pieces of eight channels of a row
+  const uint16_t* src = W + static_cast<size_t>(v) * H;
+  int width = out.width;
+  size_t row = v;
+  if (out.group_width) {
+    const int g = v / kGroupRows;
+    width = out.group_width[g];
+    row = static_cast<size_t>(out.group_row[g]) + (v - g * kGroupRows);
+  }
+  auto fetch = [&](int p) {
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (p < pieces) x = kVec ? reinterpret_cast<const uint4*>(src)[p] : gather8(src + 8 * p, H - 8 * p);
+    return x;
+  };
+  constexpr int kInFlight = kVec ? 8 : 1;
+  if (width == 16) {
+    uint16_t* dst = out.w16 + row * H;
+    for (int p0 = lane; p0 < pieces; p0 += 32 * kInFlight) {
+      uint4 x[kInFlight];
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i) x[i] = fetch(p0 + 32 * i);
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i) {
+        const int p = p0 + 32 * i;
+        if (p < pieces) {
+          if (kVec) reinterpret_cast<uint4*>(dst)[p] = x[i];
+          else scatter<uint16_t>(dst + 8 * p, x[i], H - 8 * p);
+        }
+      }
     }
-    *reinterpret_cast<uint16_t*>(packed + row * (H / 2) + b * (kSubBlock / 2) + lane * 2) = static_cast<uint16_t>(bits);
-    if (lane == 0) shift[static_cast<size_t>(b) * shift_stride + row] = static_cast<uint8_t>(e);
+    if (lane == 0) out.scale[v] = 1.f;
+    return;
+  }
+  uint32_t m = 0;
+  for (int p0 = lane; p0 < pieces; p0 += 32 * kInFlight) {
+    uint4 x[kInFlight];
+#pragma unroll
+    for (int i = 0; i < kInFlight; ++i) x[i] = fetch(p0 + 32 * i);
+#pragma unroll
+    for (int i = 0; i < kInFlight; ++i) m = absmax_step<true>(m, x[i]);
+  }
+  float amax = warp_max<true>(absmax_of_pair<true>(m));
+  const bool has_nan = amax != amax;
+  if (has_nan) {
+    m = 0;
+    for (int p = lane; p < pieces; p += 32) m = absmax_step<false>(m, fetch(p));
+    amax = warp_max<false>(absmax_of_pair<false>(m));
+  }
+  const float sc = amax > 0.f ? __fdiv_rn(amax, width == 8 ? 127.f : 112.f) : 1.f;
+  if (lane == 0) out.scale[v] = sc;
+  const bool divide = needs_division(sc, has_nan);
+  uint4 x = fetch(lane), next = fetch(lane + 32);        // (two pieces ahead: the row comes back out of the L1 or the L2)
+  if (width == 8) {
+    const Step st = make_step(sc, divide);
+    signed char* dst = out.w8 + row * H;
+#pragma unroll 1
+    for (int p = lane; p < pieces; p += 32) {
+      const uint4 after = fetch(p + 64);
+      float f[8];
+      uint32_t t[8];
+      bf16x8_to_f32(x, f);
+      round_div8(f, st, 127.f, t);
+      const uint2 b = make_uint2(pack_bytes(t), pack_bytes(t + 4));
+      if (kVec) reinterpret_cast<uint2*>(dst)[p] = b;
+      else scatter<signed char>(dst + 8 * p, make_uint4(b.x, b.y, 0u, 0u), H - 8 * p);
+      x = next;
+      next = after;
+    }
+  } else {
+    uint8_t* dst = out.w4 + row * (H >> 1);
+#pragma unroll 1
+    for (int p0 = 0; p0 < pieces; p0 += 32) {
+      const int p = p0 + lane;
+      const uint4 after = fetch(p + 64);
+      // a sub-block is sixteen pieces: lanes 0..15 or 16..31
+      float bmax = absmax_of_pair<false>(absmax_step<false>(0u, x));
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, off));
+      int e = 4;
+#pragma unroll
+      for (int c = 3; c >= 0; --c)
+        if (__fmul_rn(sc, static_cast<float>(7 << c)) >= bmax) e = c;
+      if (p < pieces) {
+        float f[8];
+        uint32_t t[8];
+        bf16x8_to_f32(x, f);
+        round_div8(f, make_step(sc * static_cast<float>(1 << e), divide), 7.f, t);     // (the product is exact)
+        const uint32_t lo = pack_bytes(t), hi = pack_bytes(t + 4);
+        const uint32_t a = (lo & 0x000F000Fu) | ((lo >> 4) & 0x00F000F0u);
+        const uint32_t b = (hi & 0x000F000Fu) | ((hi >> 4) & 0x00F000F0u);
+        const uint32_t packed = __byte_perm(a, b, 0x6420);
+        if (kVec) reinterpret_cast<uint32_t*>(dst)[p] = packed;
+        else scatter<uint8_t>(dst + 4 * p, make_uint4(packed, 0u, 0u, 0u), 4);
+        if ((lane & 15) == 0)
+          out.shift4[static_cast<size_t>(p >> 4) * out.shift_stride + row] = static_cast<uint8_t>(e);
+      }
+      x = next;
+      next = after;
+    }
   }
 }
 
-// Hidden rows as two 8-bit planes (16-bit-class activations for the 8-bit MMA kind): per verify row
+// The hidden rows of a call as one or two 8-bit planes (the 8-bit activation modes).  One plane: as an 8-bit weight row.
+// Two planes (16-bit-class activations): per verify row
 //   s1 = max|x| / 127 (1 if zero), q1 = clip(rint(x / s1));  r = x - s1 q1;  s2 = s1 / 254, q2 = clip(rint(r / s2)),
-// every step one fp32 operation.  Operand layout: blocks of 32 verify rows, each block as 32 rows of q1 followed by
-// 32 rows of q2 (so that 64 consecutive accumulator columns hold both sums of the same 32 rows); rows past M are
-// written as zeros.  One CTA per (padded) verify row.
-__global__ void __launch_bounds__(256) quantize_rows_two_plane_kernel(const __nv_bfloat16* X, int M, int H,
-                                                                      signed char* q, float* s1, float* s2) {
-  __shared__ float sh_max[8];
-  __shared__ float sh_scale;
-  grid_dependency_wait();
+// every step one fp32 operation.  Operand layout of two planes: blocks of 32 verify rows, each block as 32 rows of q1
+// followed by 32 rows of q2 (so that 64 consecutive accumulator columns hold both sums of the same 32 rows); rows past M
+// are written as zeros.  A CTA per (padded) verify row: few rows, so what counts is the latency of one - two 16-byte
+// loads per thread at 4096 channels, one barrier.
+constexpr int kHidThreads = 256, kHidKeep = 4;
+template <bool kTwoPlane>
+__global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint4* X, int M, int H, signed char* q,
+                                                                      float* s1, float* s2) {
+  __shared__ float sh_max[kHidThreads / 32];
+  grid_dependency_wait();                                // (no-op unless launched with programmatic serialization)
   const int row = blockIdx.x;
-  signed char* q1 = q + (static_cast<size_t>(64) * (row >> 5) + (row & 31)) * H;
-  signed char* q2 = q1 + static_cast<size_t>(32) * H;
+  const int pieces = H >> 3;
+  const size_t row1 = kTwoPlane ? static_cast<size_t>(64) * (row >> 5) + (row & 31) : static_cast<size_t>(row);
+  uint2* q1 = reinterpret_cast<uint2*>(q) + row1 * pieces;
+  uint2* q2 = q1 + static_cast<size_t>(32) * pieces;
   if (row >= M) {
-    for (int h = threadIdx.x; h < H; h += 256) { q1[h] = 0; q2[h] = 0; }
+    for (int p = threadIdx.x; p < pieces; p += kHidThreads) { q1[p] = make_uint2(0u, 0u); q2[p] = make_uint2(0u, 0u); }
     return;
   }
-  const __nv_bfloat16* xr = X + static_cast<size_t>(row) * H;
-  float amax = 0.f;
-  for (int h = threadIdx.x; h < H; h += 256) amax = fmaxf(amax, fabsf(__bfloat162float(xr[h])));
+  const uint4* src = X + static_cast<size_t>(row) * pieces;
+  const bool kept = pieces <= kHidThreads * kHidKeep;
+  uint4 x[kHidKeep];
+  auto fetch = [&](int p0) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
+    for (int i = 0; i < kHidKeep; ++i) {
+      const int p = p0 + kHidThreads * i + threadIdx.x;
+      x[i] = p < pieces ? src[p] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  uint32_t m = 0;
+  for (int p0 = 0; p0 < pieces; p0 += kHidThreads * kHidKeep) {
+    fetch(p0);
+#pragma unroll
+    for (int i = 0; i < kHidKeep; ++i) m = absmax_step<true>(m, x[i]);
+  }
+  float amax = warp_max<true>(absmax_of_pair<true>(m));
   if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = amax;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float m = 0.f;
-    for (int i = 0; i < 8; ++i) m = fmaxf(m, sh_max[i]);
-    const float sc = m > 0.f ? __fdiv_rn(m, 127.f) : 1.f;
-    sh_scale = sc;
-    s1[row] = sc;
-    s2[row] = __fdiv_rn(sc, 254.f);
+#pragma unroll
+  for (int i = 0; i < kHidThreads / 32; ++i) asm("max.NaN.f32 %0, %0, %1;" : "+f"(amax) : "f"(sh_max[i]));
+  const bool has_nan = amax != amax;
+  if (has_nan) {                                         // (the same decision in every thread) the maximum of the others
+    m = 0;
+    for (int p = threadIdx.x; p < pieces; p += kHidThreads) m = absmax_step<false>(m, src[p]);
+    amax = warp_max<false>(absmax_of_pair<false>(m));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = amax;
+    __syncthreads();
+    for (int i = 0; i < kHidThreads / 32; ++i) amax = fmaxf(amax, sh_max[i]);
   }
-  __syncthreads();
-  const float sc = sh_scale, sc2 = __fdiv_rn(sc, 254.f);
-  for (int h = threadIdx.x; h < H; h += 256) {
-    const float x = __bfloat162float(xr[h]);
-    const float a = fminf(127.f, fmaxf(-127.f, rintf(__fdiv_rn(x, sc))));
-    const float rem = __fsub_rn(x, __fmul_rn(sc, a));                  // no fused multiply-add: two roundings
-    const float b = fminf(127.f, fmaxf(-127.f, rintf(__fdiv_rn(rem, sc2))));
-    q1[h] = static_cast<signed char>(a);
-    q2[h] = static_cast<signed char>(b);
+  const float sc = amax > 0.f ? __fdiv_rn(amax, 127.f) : 1.f;
+  const float sc2 = __fdiv_rn(sc, 254.f);
+  const bool divide = needs_division(sc, has_nan);
+  const Step st1 = make_step(sc, divide), st2 = make_step(sc2, divide);
+  if (threadIdx.x == 0) {
+    s1[row] = sc;
+    if (kTwoPlane) s2[row] = sc2;
+  }
+  for (int p0 = 0; p0 < pieces; p0 += kHidThreads * kHidKeep) {
+    if (!kept) fetch(p0);
+#pragma unroll
+    for (int i = 0; i < kHidKeep; ++i) {
+      const int p = p0 + kHidThreads * i + threadIdx.x;
+      if (p < pieces) {
+        float f[8];
+        uint32_t t[8];
+        bf16x8_to_f32(x[i], f);
+        round_div8(f, st1, 127.f, t);
+        q1[p] = make_uint2(pack_bytes(t), pack_bytes(t + 4));
+        if (kTwoPlane) {
+#pragma unroll
+          for (int n = 0; n < 8; ++n)                    // no fused multiply-add: two roundings
+            f[n] = __fsub_rn(f[n], __fmul_rn(sc, __uint_as_float(t[n]) - kRoundMagic));
+          round_div8(f, st2, 127.f, t);
+          q2[p] = make_uint2(pack_bytes(t), pack_bytes(t + 4));
+        }
+      }
+    }
   }
 }
 
@@ -2343,16 +2536,15 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     // the same per-row quantiser as for W_lm (one plane), or the two-plane form in blocks of 32 rows
     const int padded = round_up(M, 32);
     cudaLaunchConfig_t qc = {};
-    qc.gridDim = dim3(static_cast<unsigned>(two ? padded : M)); qc.blockDim = dim3(256); qc.stream = stream;
+    qc.gridDim = dim3(static_cast<unsigned>(two ? padded : M)); qc.blockDim = dim3(kHidThreads); qc.stream = stream;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // launch latency hides behind the call before
     qa[0].val.programmaticStreamSerializationAllowed = 1;
     qc.attrs = qa; qc.numAttrs = 1;
     const cudaError_t qe =
-        two ? cudaLaunchKernelEx(&qc, quantize_rows_two_plane_kernel, static_cast<const __nv_bfloat16*>(a->hidden), M,
-                                 a->H, ctx->hid8, ctx->hid_scale, ctx->hid_scale + ctx->max_rows)
-            : cudaLaunchKernelEx(&qc, quantize_rows_int8_kernel, static_cast<const __nv_bfloat16*>(a->hidden), a->H,
-                                 ctx->hid8, ctx->hid_scale);
+        cudaLaunchKernelEx(&qc, two ? quantize_hidden_kernel<true> : quantize_hidden_kernel<false>,
+                           static_cast<const uint4*>(a->hidden), M, a->H, ctx->hid8, ctx->hid_scale,
+                           ctx->hid_scale + ctx->max_rows);
     if (qe != cudaSuccess) { set_error(ctx, "launch of the hidden-row quantiser", qe); return HOLA_ERR_CUDA; }
   }
   MapEntry* me = nullptr;
@@ -3207,21 +3399,48 @@ hola_status hola_host_traffic(const hola_ctx* ctx, unsigned long long* h2d_bytes
   return HOLA_OK;
 }
 
+static hola_status launch_quantiser(const void* W, int V, int H, const QuantOut& o, void* cuda_stream) {
+  const bool vec = H % 8 == 0 && aligned16(W) && aligned16(o.w16) && aligned16(o.w8) && aligned16(o.w4);
+  const unsigned grid = static_cast<unsigned>((V + 7) / 8);
+  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  const uint16_t* src = static_cast<const uint16_t*>(W);
+  if (vec) quantize_rows_kernel<true><<<grid, 256, 0, stream>>>(src, V, H, o);
+  else quantize_rows_kernel<false><<<grid, 256, 0, stream>>>(src, V, H, o);
+  return cudaGetLastError() == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
+}
+
 hola_status hola_quantize_w4(const void* W_bf16, int rows, int H, void* packed_out, uint8_t* shift_out, int shift_stride,
                              float* scale_out, void* cuda_stream) {
   if (!W_bf16 || !packed_out || !shift_out || !scale_out || rows <= 0 || H <= 0 || shift_stride < rows)
     return HOLA_ERR_INVALID_ARG;
   if (H % kSubBlock != 0) return HOLA_ERR_UNSUPPORTED_SHAPE;
-  quantize_rows_w4_kernel<<<static_cast<unsigned>(rows), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const __nv_bfloat16*>(W_bf16), H, static_cast<uint8_t*>(packed_out), shift_out, shift_stride, scale_out);
-  return cudaGetLastError() == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
+  QuantOut o = {};
+  o.width = 4; o.w4 = static_cast<uint8_t*>(packed_out); o.shift4 = shift_out; o.shift_stride = shift_stride; o.scale = scale_out;
+  return launch_quantiser(W_bf16, rows, H, o, cuda_stream);
 }
 
 hola_status hola_quantize_w8(const void* W_bf16, int V, int H, void* q_out, float* scale_out, void* cuda_stream) {
   if (!W_bf16 || !q_out || !scale_out || V <= 0 || H <= 0) return HOLA_ERR_INVALID_ARG;
-  quantize_rows_int8_kernel<<<static_cast<unsigned>(V), 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-      static_cast<const __nv_bfloat16*>(W_bf16), H, static_cast<signed char*>(q_out), scale_out);
-  return cudaGetLastError() == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
+  QuantOut o = {};
+  o.width = 8; o.w8 = static_cast<signed char*>(q_out); o.scale = scale_out;
+  return launch_quantiser(W_bf16, V, H, o, cuda_stream);
+}
+
+hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream) {
+  if (!W_bf16 || !out || !scale_out || V <= 0 || H <= 0 || !out->group_width || !out->group_row) return HOLA_ERR_INVALID_ARG;
+  if (H % kSubBlock != 0) return HOLA_ERR_UNSUPPORTED_SHAPE;
+  if (out->rows4 < 0 || out->rows8 < 0 || out->rows16 < 0 ||
+      static_cast<long long>(out->rows4) + out->rows8 + out->rows16 < V)
+    return HOLA_ERR_INVALID_ARG;
+  if ((out->rows4 > 0 && (!out->W4 || !out->shift4)) || (out->rows8 > 0 && !out->W8) || (out->rows16 > 0 && !out->W16))
+    return HOLA_ERR_INVALID_ARG;
+  QuantOut o = {};
+  o.group_width = out->group_width; o.group_row = out->group_row;
+  o.w16 = static_cast<uint16_t*>(const_cast<void*>(out->W16));
+  o.w8 = static_cast<signed char*>(const_cast<void*>(out->W8));
+  o.w4 = static_cast<uint8_t*>(const_cast<void*>(out->W4));
+  o.shift4 = const_cast<uint8_t*>(out->shift4); o.shift_stride = out->rows4; o.scale = scale_out;
+  return launch_quantiser(W_bf16, V, H, o, cuda_stream);
 }
 
 }  // extern "C"

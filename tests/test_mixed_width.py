@@ -214,3 +214,94 @@ def test_expansion_at_the_edges_of_its_tiles(binding, B, k, H, V, pattern):
     want = h @ Wd.T
     bound = (H / 16 + 16) * 2.0 ** -23 * (h.abs() @ Wd.abs().T)
     assert torch.all((out.logits.double() - want).abs() <= bound)
+
+
+@pytest.mark.parametrize("V,H", [(257, 128), (600, 4096), (1025, 4224), (523, 640)])
+def test_whole_head_quantiser_is_bit_exact(binding, V, H):
+    """One launch for all groups: codes, exponents, scales and copied rows against the oracle, at the edges of what a warp
+    keeps in registers (4096 channels), with ragged last groups and rows of zeros, ties and a lone large entry."""
+    g = torch.Generator(device=DEV).manual_seed(V)
+    W = (torch.randn((V, H), generator=g, device=DEV) * 0.02).bfloat16()
+    W[7] = 0
+    W[9] = (torch.randint(-254, 255, (H,), generator=g, device=DEV) * 0.5).bfloat16()      # halves of the 8-bit step
+    W[9, 0] = 127
+    W[11, 5] = 30.0
+    W[13] *= 2.0 ** -100                                # steps at the end of the fp32 range
+    W[min(270, V - 1)] *= 2.0 ** -100
+    widths = _widths(V, [8, 4, 16, 4])
+    head = binding.hola_quantize_mixed(W, widths)
+    torch.cuda.synchronize()
+    W32 = W.float().cpu().numpy()
+    at = {4: 0, 8: 0, 16: 0}
+    for gi, wd in enumerate(widths):
+        lo, hi = 256 * gi, min(V, 256 * gi + 256)
+        r = slice(at[wd], at[wd] + hi - lo)
+        at[wd] += hi - lo
+        scale = _np(head.w_scale[lo:hi])
+        if wd == 16:
+            assert torch.equal(head.W16[r], W[lo:hi]) and np.all(scale == 1.0)
+        elif wd == 8:
+            q, s = lobi.quantize_rows_int8(W32[lo:hi])
+            assert np.array_equal(_np(head.W8[r]), q) and np.array_equal(scale, s)
+        else:
+            c, e, s = lobi.quantize_rows_w4(W32[lo:hi])
+            assert np.array_equal(_np(head.W4[r]), lobi.pack_nibbles(c)) and np.array_equal(scale, s)
+            assert np.array_equal(_np(head.shift4[:, r]).T, e)
+
+
+@pytest.mark.parametrize("V,H,offset", [(33, 203, 0), (40, 256, 1)])
+def test_quantisers_take_rows_that_16_byte_pieces_do_not_tile(binding, V, H, offset):
+    g = torch.Generator(device=DEV).manual_seed(H)
+    flat = (torch.randn(V * H + 8, generator=g, device=DEV) * 0.02).bfloat16()
+    W = flat[offset:offset + V * H].view(V, H)
+    W32 = W.float().cpu().numpy()
+    q, s = binding.hola_quantize_w8(W)
+    q0, s0 = lobi.quantize_rows_int8(W32)
+    assert np.array_equal(_np(q), q0) and np.array_equal(_np(s), s0)
+    if H % 128 == 0:
+        head = binding.hola_quantize_mixed(W, [4])
+        c, e, s = lobi.quantize_rows_w4(W32)
+        assert np.array_equal(_np(head.W4), lobi.pack_nibbles(c)) and np.array_equal(_np(head.w_scale), s)
+        assert np.array_equal(_np(head.shift4).T, e)
+        assert torch.equal(binding.hola_quantize_mixed(W, [16]).W16, W)
+
+
+def test_quantisers_round_every_quotient_of_two_bf16_mantissas_like_the_division(binding):
+    """The integers depend on the mantissas of a row's maximum and of an entry, their exponents' difference and the sign:
+    128 rows, one per mantissa of the maximum, with every other bf16 value down to 2^-15 of it, in an order in which the
+    4-bit sub-blocks take every exponent and in a shuffled one."""
+    m = torch.arange(128, 256, dtype=torch.float32)
+    mags = torch.cat([m * 2.0 ** -(9 + e) for e in range(16)])                # descending binades below 2^-1
+    signs = 1.0 - 2.0 * (torch.arange(mags.numel()) % 2)
+    row = torch.cat([mags * signs, -mags * signs])                            # 4096 entries, both signs
+    shuffled = row[torch.randperm(row.numel(), generator=torch.Generator().manual_seed(3))]
+    W = torch.zeros((256, row.numel()))
+    for i in range(128):
+        top = m[i] * 2.0 ** -9
+        for k, r in enumerate((row, shuffled)):
+            W[2 * i + k] = torch.where(r.abs() <= top, r, r * 2.0 ** -8)
+            W[2 * i + k, 17] = top
+    W = W.bfloat16().to(DEV)
+    W32 = W.float().cpu().numpy()
+    q, s = binding.hola_quantize_w8(W)
+    q0, s0 = lobi.quantize_rows_int8(W32)
+    assert np.array_equal(_np(q), q0) and np.array_equal(_np(s), s0)
+    head = binding.hola_quantize_mixed(W, [4])
+    c, e, s = lobi.quantize_rows_w4(W32)
+    assert np.array_equal(_np(head.W4), lobi.pack_nibbles(c)) and np.array_equal(_np(head.shift4).T, e)
+    assert set(np.unique(e)) == {0, 1, 2, 3, 4}
+    # hidden rows in one and in two planes: an identity-like head of ones picks single entries out as logits
+    q8 = torch.zeros((W.shape[1], W.shape[1]), dtype=torch.int8, device=DEV)
+    q8.fill_diagonal_(1)
+    ones = torch.ones(W.shape[1], dtype=torch.float32, device=DEV)
+    hidden = W.view(256, 1, -1)
+    with binding.HolaVerify(256, 0, W.shape[1], W.shape[1]) as ctx:
+        one = ctx.hola_lm_head_entropy(hidden, q8, w_scale=ones, a8=True).logits[:, 0]
+        two = ctx.hola_lm_head_entropy(hidden, q8, w_scale=ones, a8="a16").logits[:, 0]
+        torch.cuda.synchronize()
+    s1 = torch.from_numpy(s0).to(DEV)[:, None]
+    assert torch.equal(one, torch.from_numpy(q0).to(DEV).float() * s1)
+    p1, p2, sa, sb = (torch.from_numpy(np.asarray(x)).to(DEV) for x in lobi.quantize_rows_two_plane(W32))
+    want = p1.double() * sa.double()[:, None] + p2.double() * sb.double()[:, None]
+    assert torch.all((two.double() - want).abs() <= 2.0 ** -22 * want.abs() + 1e-30)       # one fused multiply-add
+    assert torch.equal(((two - p1.float() * sa[:, None]) / sb[:, None]).round(), p2.float())
