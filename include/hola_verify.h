@@ -108,6 +108,10 @@ typedef struct hola_wmix {
 #define HOLA_FLAG_TIMEOUT 4u     /* an on-chip wait ran out of iterations; outputs of this call are invalid  */
 #define HOLA_FLAG_R_ZERO 8u      /* residual mass was zero (p <= q everywhere): token drawn from p instead   */
 
+/* Bits of hola_verify_args::flags. */
+#define HOLA_ARG_CLEAR_STATUS 1 /* the call stores 0 to status_word before it OR-s anything in, so the caller need not  */
+                                /* (calls that run the LM head; one stream operation less per call)                   */
+
 typedef struct {
   int32_t B; /* sequences, >= 0 */
   int32_t k; /* draft tokens per sequence, >= 0; k = 0 is a plain draw from p_0 */
@@ -130,7 +134,7 @@ typedef struct {
   int32_t fallback;        /* hola_fallback; 0 = speculative sampling.  With GREEDY the uniforms are not read  */
   float* draft_entropy;    /* out fp32 [B][k], optional: H(q_j), written when gate_source = DRAFT_ENTROPY       */
   int32_t w_dtype;         /* hola_w_dtype; 0 = W_lm is bf16, otherwise W_lm is int8 [V][H] and H % 16 == 0     */
-  int32_t reserved_;       /* must be 0                                                                        */
+  int32_t flags;           /* HOLA_ARG_* bits, 0 = none                                                         */
   const float* w_scale;    /* fp32 [V], required with an int8 W_lm (w_dtype != 0): scale of each vocabulary row  */
   const hola_wmix* wmix;   /* HOST pointer, required with w_dtype = HOLA_W_MIXED, else ignored                   */
 } hola_verify_args;

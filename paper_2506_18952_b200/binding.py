@@ -19,6 +19,7 @@ HOLA_Q_BF16, HOLA_Q_F32 = 0, 1
 HOLA_GATE_TARGET_ENTROPY, HOLA_GATE_DRAFT_ENTROPY = 0, 1
 HOLA_FALLBACK_SAMPLE, HOLA_FALLBACK_GREEDY = 0, 1
 HOLA_W_BF16, HOLA_W_INT8, HOLA_W8A8, HOLA_W8A16, HOLA_W_MIXED = 0, 1, 2, 3, 4
+HOLA_ARG_CLEAR_STATUS = 1
 GROUP_ROWS, SUB_BLOCK = 256, 128
 FLAG_BAD_TOKEN, FLAG_BAD_UNIFORM, FLAG_TIMEOUT, FLAG_R_ZERO = 1, 2, 4, 8
 HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HOST_ROWS_ON_DEMAND, HOLA_OPT_PASSES, HOLA_OPT_PAIR_MMA, HOLA_OPT_HOST_IN_PLACE, HOLA_OPT_CONVERTER_GROUP, HOLA_OPT_FUSED_PASSES = 1, 2, 3, 4, 5, 6, 7, 8, 9
@@ -40,7 +41,7 @@ class hola_verify_args(ctypes.Structure):
                 ("tau", ctypes.c_float), ("accept_len", ctypes.c_void_p), ("next_tok", ctypes.c_void_p),
                 ("entropy", ctypes.c_void_p), ("logZ", ctypes.c_void_p), ("logits_out", ctypes.c_void_p),
                 ("status_word", ctypes.c_void_p), ("gate_source", ctypes.c_int32), ("fallback", ctypes.c_int32),
-                ("draft_entropy", ctypes.c_void_p), ("w_dtype", ctypes.c_int32), ("reserved_", ctypes.c_int32),
+                ("draft_entropy", ctypes.c_void_p), ("w_dtype", ctypes.c_int32), ("flags", ctypes.c_int32),
                 ("w_scale", ctypes.c_void_p), ("wmix", ctypes.c_void_p)]
 
 
@@ -139,9 +140,10 @@ def _dptr(t: torch.Tensor | None):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
 
-def _stream_ptr(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_ptr(stream) -> int:
+    """cudaStream_t of a torch stream; None: the current stream of the current device, without making a Stream object
+    for it (a quarter of what a call costs on the host)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def hola_quantize_w8(W_lm: torch.Tensor, stream=None):
@@ -256,6 +258,37 @@ class VerifyOutputs:
     draft_entropy: torch.Tensor | None = None   # fp32 [B, k], filled when the gate looks at the draft rows
 
 
+class _FreshOutputs(VerifyOutputs):
+    """Outputs a call makes for itself: only the tensors that it fills are allocated (one allocation costs the host as
+    much as a fifth of a call), the others when somebody asks for them.  The status word is cleared by the call
+    (HOLA_ARG_CLEAR_STATUS); an empty batch launches nothing."""
+
+    def __init__(self, ctx: "HolaVerify", B: int, k: int, want_logits: bool, draws: bool, draft_gate: bool):
+        dev = self._dev = ctx._dev
+        self._B, self._k = B, k
+        self.entropy = torch.empty((B, k + 1), dtype=torch.float32, device=dev)
+        self.logZ = torch.empty((B, k + 1), dtype=torch.float32, device=dev)
+        self.logits = torch.empty((B, k + 1, ctx.V), dtype=torch.float32, device=dev) if want_logits else None
+        self.status = (torch.empty if B else torch.zeros)(1, dtype=torch.int32, device=dev)
+        self._lazy = {"draft_entropy": torch.empty((B, k), dtype=torch.float32, device=dev)} if draft_gate else {}
+        if draws:
+            self._lazy["accept_len"] = torch.empty(B, dtype=torch.int32, device=dev)
+            self._lazy["next_tok"] = torch.empty(B, dtype=torch.int32, device=dev)
+
+    def _get(self, name, make):
+        t = self._lazy.get(name)
+        if t is None:
+            t = self._lazy[name] = make()
+        return t
+
+    accept_len = property(lambda self: self._get("accept_len", lambda: torch.empty(self._B, dtype=torch.int32, device=self._dev)),
+                          lambda self, t: self._lazy.__setitem__("accept_len", t))
+    next_tok = property(lambda self: self._get("next_tok", lambda: torch.empty(self._B, dtype=torch.int32, device=self._dev)),
+                        lambda self, t: self._lazy.__setitem__("next_tok", t))
+    draft_entropy = property(lambda self: self._get("draft_entropy", lambda: torch.zeros((self._B, self._k), device=self._dev)),
+                             lambda self, t: self._lazy.__setitem__("draft_entropy", t))
+
+
 class HolaVerify:
     """Owns one hola_ctx.  Methods are named after the C entry points they call."""
 
@@ -264,6 +297,7 @@ class HolaVerify:
             raise HolaError("hola_create: no CUDA device; this library has no CPU path")
         self.lib = load_library()
         self.device = torch.cuda.current_device() if device is None else int(device)
+        self._dev = torch.device("cuda", self.device)
         self.maxB, self.maxK, self.H, self.V = maxB, maxK, H, V
         self._ctx = ctypes.c_void_p()
         st = self.lib.hola_create(ctypes.byref(self._ctx), self.device, maxB, maxK, H, V)
@@ -332,7 +366,7 @@ class HolaVerify:
 
     def _args(self, hidden, W_lm, draft_tok, draft_q, uniforms, tau, out: VerifyOutputs, B, k,
               gate_source: int = HOLA_GATE_TARGET_ENTROPY, fallback: int = HOLA_FALLBACK_SAMPLE, w_scale=None,
-              a8: bool = False):
+              a8: bool = False, draws: bool = True):
         mixed = W_lm if isinstance(W_lm, MixedHead) else None
         if mixed is not None:
             if mixed.V != self.V or mixed.H != self.H or w_scale is not None or a8:
@@ -347,29 +381,41 @@ class HolaVerify:
         for t in (hidden, W_lm, draft_tok, draft_q, uniforms):
             if t is not None and not t.is_contiguous():
                 raise HolaError("all inputs must be contiguous")
+        # (plain integers into the pointer fields: a c_void_p object for each would cost as much as the call itself)
         a = hola_verify_args()
         a.B, a.k, a.H, a.V = B, k, self.H, self.V
-        a.hidden, a.W_lm = _dptr(hidden), _dptr(W_lm)
-        a.draft_tok = _dptr(draft_tok) if k > 0 else None
-        a.draft_q = _dptr(draft_q) if k > 0 else None
-        a.q_dtype = HOLA_Q_F32 if (draft_q is not None and draft_q.dtype == torch.float32) else HOLA_Q_BF16
-        a.uniforms = _dptr(uniforms)
+        a.hidden = hidden.data_ptr()
+        if k > 0:
+            if draft_tok is not None:
+                a.draft_tok = draft_tok.data_ptr()
+            if draft_q is not None:
+                a.draft_q = draft_q.data_ptr()
+        if draft_q is not None and draft_q.dtype == torch.float32:
+            a.q_dtype = HOLA_Q_F32
+        if uniforms is not None:
+            a.uniforms = uniforms.data_ptr()
         a.tau = float(tau)
-        a.accept_len, a.next_tok = _dptr(out.accept_len), _dptr(out.next_tok)
-        a.entropy, a.logZ = _dptr(out.entropy), _dptr(out.logZ)
-        a.logits_out = _dptr(out.logits)
-        a.status_word = _dptr(out.status)
+        if draws:
+            a.accept_len, a.next_tok = out.accept_len.data_ptr(), out.next_tok.data_ptr()
+        a.entropy, a.logZ = out.entropy.data_ptr(), out.logZ.data_ptr()
+        if out.logits is not None:
+            a.logits_out = out.logits.data_ptr()
+        if out.status is not None:
+            a.status_word = out.status.data_ptr()
         a.gate_source, a.fallback = int(gate_source), int(fallback)
-        a.draft_entropy = _dptr(out.draft_entropy)
+        if a.gate_source == HOLA_GATE_DRAFT_ENTROPY and out.draft_entropy is not None:
+            a.draft_entropy = out.draft_entropy.data_ptr()
         # a8: True = one 8-bit plane per hidden row (W8A8); "a16" = two planes (16-bit-class activations, W8A16)
         if a8 and w_scale is None:
             raise HolaError("8-bit activation planes (a8) go with an int8 W_lm and its scales")
-        act = HOLA_W8A16 if a8 == "a16" else (HOLA_W8A8 if a8 else HOLA_W_INT8)
-        a.w_dtype = act if w_scale is not None else HOLA_W_BF16
-        a.w_scale = _dptr(w_scale)
+        if w_scale is not None:
+            a.w_scale = w_scale.data_ptr()
         if mixed is not None:
-            a.w_dtype, a.W_lm = HOLA_W_MIXED, None
-            a.wmix = ctypes.addressof(mixed.struct)
+            a.w_dtype, a.wmix = HOLA_W_MIXED, ctypes.addressof(mixed.struct)
+        else:
+            a.W_lm = W_lm.data_ptr()
+            if w_scale is not None:
+                a.w_dtype = HOLA_W8A16 if a8 == "a16" else (HOLA_W8A8 if a8 else HOLA_W_INT8)
         return a
 
     def alloc_outputs(self, B: int, k: int, want_logits: bool = False, device=None) -> VerifyOutputs:
@@ -389,19 +435,30 @@ class HolaVerify:
         """The whole verify step on device tensors, asynchronous on the stream.  With w_scale, W_lm is the int8 form
         made by hola_quantize_w8; with a8 as well, the hidden rows are quantised on the fly and the products run on
         the 8-bit tensor-core kind."""
-        B, k = hidden.shape[0], hidden.shape[1] - 1
-        out = out or self.alloc_outputs(B, k, want_logits)
-        a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k, gate_source, fallback, w_scale, a8)
-        _check(self.lib, self._ctx, self.lib.hola_verify(self._ctx, ctypes.byref(a), _stream_ptr(stream)), "hola_verify")
+        B, k1 = hidden.shape[:2]
+        fresh = not out
+        if fresh:
+            out = _FreshOutputs(self, B, k1 - 1, want_logits, True, gate_source == HOLA_GATE_DRAFT_ENTROPY)
+        a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k1 - 1, gate_source, fallback, w_scale, a8)
+        if fresh:
+            a.flags = HOLA_ARG_CLEAR_STATUS
+        st = self.lib.hola_verify(self._ctx, ctypes.byref(a), _stream_ptr(stream))
+        if st:
+            _check(self.lib, self._ctx, st, "hola_verify")
         return out
 
     def hola_lm_head_entropy(self, hidden, W_lm, out: VerifyOutputs | None = None, want_logits: bool = True,
                              stream=None, w_scale=None, a8: bool = False) -> VerifyOutputs:
-        B, k = hidden.shape[0], hidden.shape[1] - 1
-        out = out or self.alloc_outputs(B, k, want_logits)
-        a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k, w_scale=w_scale, a8=a8)
-        _check(self.lib, self._ctx, self.lib.hola_lm_head_entropy(self._ctx, ctypes.byref(a), _stream_ptr(stream)),
-               "hola_lm_head_entropy")
+        B, k1 = hidden.shape[:2]
+        fresh = not out
+        if fresh:
+            out = _FreshOutputs(self, B, k1 - 1, want_logits, False, False)
+        a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k1 - 1, w_scale=w_scale, a8=a8, draws=False)
+        if fresh:
+            a.flags = HOLA_ARG_CLEAR_STATUS
+        st = self.lib.hola_lm_head_entropy(self._ctx, ctypes.byref(a), _stream_ptr(stream))
+        if st:
+            _check(self.lib, self._ctx, st, "hola_lm_head_entropy")
         return out
 
     def hola_accept_sample(self, logits, entropy, logZ, draft_tok, draft_q, uniforms, tau, stream=None) -> VerifyOutputs:

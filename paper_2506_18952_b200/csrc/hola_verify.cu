@@ -126,6 +126,8 @@ struct K1Params {
   const int* group_row;
   const uint8_t* shift4;
   int rows4;
+  int clear_status;       // 1: the status word holds anything; CTA 0 clears it (what sets bits comes seconds later, when a
+                          // wait runs out, or in a later kernel)
   int stream_logits;      // 1: store the logits with the streaming hint (they exceed what the L2 keeps until they are read)
   float* logits;
   float4* partials;   // [grid][part_stride] (m, s, t, arg-max index)
@@ -744,6 +746,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       uint32_t phase = 0;
       bool ok = true;
       grid_dependency_wait();                            // W_lm and the hidden rows may come from the kernel before
+      if (p.clear_status && blockIdx.x == 0) *p.status = 0u;
       if (kW8) {
         // On-chip expansion: codes (or 16-bit rows as they are) and hidden rows of a K block into one slot, which is free
         // again once the MMAs of its previous use are done: those have waited for the converters.
@@ -2651,6 +2654,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     kp.row0 = pass * pl.rows_per_pass;
     kp.rows = M - kp.row0 < pl.rows_per_pass ? M - kp.row0 : pl.rows_per_pass;
     if (kp.rows <= 0) break;
+    kp.clear_status = pass == 0 && (a->flags & HOLA_ARG_CLEAR_STATUS) && a->status_word;
     e = two ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<3, false>, th, tw, tw4, tw16, kp)
       : i8 ? (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, true>, th, tw, tw4, tw16, kp)
                      : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, false>, th, tw, tw4, tw16, kp))
@@ -2781,12 +2785,15 @@ cudaError_t configure_kernels() {
 
 struct DeviceGuard {
   int prev = -1;
-  bool ok = true;
+  bool ok = true, changed = false;
   explicit DeviceGuard(int dev) {
     if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-    if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+    if (prev != dev) {
+      changed = true;
+      if (cudaSetDevice(dev) != cudaSuccess) ok = false;
+    }
   }
-  ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+  ~DeviceGuard() { if (changed) cudaSetDevice(prev); }
 };
 
 }  // namespace
@@ -3027,15 +3034,15 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   const bool prof = ctx->prof_on && ctx->prof_n < ctx->prof_cap;
   cudaEvent_t* ev = prof ? ctx->prof_ev + 3 * ctx->prof_n : nullptr;
   if (prof) cudaEventRecord(ev[0], stream);
+  const bool draft_gate = a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
+  if (draft_gate && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
   // The pass over the draft rows (draft-entropy gate) depends on nothing the GEMM makes, and its small CTAs fit on the
   // SMs beside the GEMM's: it runs on the context's side stream (behind the copy of the draft tensor, when the host
   // entry put one there), branching off the caller's stream before the GEMM and joining it again before the
   // accept/sample kernel.  It is launched AFTER the GEMM so that the GEMM's CTAs get their SMs first.
   // (While the caller records a graph everything stays on the caller's stream.)
-  const bool side = a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0 &&
-                    (before_sample || capturing == cudaStreamCaptureStatusNone);
+  const bool side = draft_gate && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream);
   if (s != HOLA_OK) return s;
@@ -3114,7 +3121,6 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
   memcpy(ctx->h_small + ctx->small_u_off, a->uniforms, rows * 4);
   h2d(ctx->st_tok, ctx->h_small, ctx->small_qtok_off + static_cast<size_t>(B) * k * 4, stream);
   const OutBlock ob = out_block(B, k);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->st_out, 0, 4, stream);
   const size_t seq_pitch = static_cast<size_t>(k) * row_bytes;   // from row (b, 0) to row (b + 1, 0)
   ahead = ahead < 1 ? 1 : (ahead > k ? k : ahead);
   const size_t ahead_bytes = static_cast<size_t>(ahead) * row_bytes;     // rows 0 .. ahead-1 of a sequence are adjacent
@@ -3139,6 +3145,7 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
   d.entropy = reinterpret_cast<float*>(ctx->st_out + ob.entropy);
   d.logZ = reinterpret_cast<float*>(ctx->st_out + ob.logZ);
   d.logits_out = nullptr; d.status_word = reinterpret_cast<uint32_t*>(ctx->st_out); d.draft_entropy = nullptr;
+  d.flags = HOLA_ARG_CLEAR_STATUS;
   hola_status s = check_lm_head_args(ctx, &d);
   if (s != HOLA_OK) return s;
   const Plan& pl = plan_for(ctx, B * (k + 1), a->w_dtype);
@@ -3293,7 +3300,6 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
     h2d(ctx->st_q, a->draft_q, q_bytes);
   }
   const OutBlock ob = out_block(a->B, a->k);
-  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->st_out, 0, 4, stream);
   if (e != cudaSuccess) { set_error(ctx, "host-to-device copy", e); return HOLA_ERR_CUDA; }
   hola_verify_args d = *a;
   d.hidden = ctx->st_hidden; d.draft_tok = ctx->st_tok; d.draft_q = ctx->st_q; d.uniforms = ctx->st_u;
@@ -3302,6 +3308,7 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   d.entropy = reinterpret_cast<float*>(ctx->st_out + ob.entropy);
   d.logZ = reinterpret_cast<float*>(ctx->st_out + ob.logZ);
   d.logits_out = nullptr; d.status_word = reinterpret_cast<uint32_t*>(ctx->st_out);
+  d.flags = HOLA_ARG_CLEAR_STATUS;
   const bool want_dent = a->draft_entropy && a->gate_source == HOLA_GATE_DRAFT_ENTROPY;
   d.draft_entropy = a->draft_entropy ? reinterpret_cast<float*>(ctx->st_out + ob.dent) : nullptr;
   if ((s = check_lm_head_args(ctx, &d)) != HOLA_OK) return s;

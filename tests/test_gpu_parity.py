@@ -973,3 +973,30 @@ def test_split_entry_points_on_a_shape_with_several_passes(binding):
     assert int((~same).sum().item()) <= 1
     assert torch.equal(second.next_tok[same], whole.next_tok[same])
     check_against_oracle(binding, w, out=whole, seqs=range(0, w.B, 9))
+
+
+def test_fresh_outputs_start_with_a_clear_status_word_and_hold_every_field(binding):
+    """Outputs that a call allocates itself: flags of an earlier call must not show up in recycled memory, and fields the
+    call does not fill are there all the same."""
+    w = workloads.gaussian_head("fresh", 5, 3, 64, 700, seed=21, device=DEV, w_std=0.3)
+    bad = w.draft_tok.clone()
+    bad[:] = w.V + 5
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        ref_out = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, 0.0, out=ctx.alloc_outputs(w.B, w.k))
+        for _ in range(4):
+            dirty = ctx.hola_verify(w.hidden, w.W_lm, bad, w.draft_q, w.uniforms, 0.0)
+            torch.cuda.synchronize()
+            assert int(dirty.status.item()) == binding.FLAG_BAD_TOKEN
+            del dirty
+            out = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, 0.0)
+            lm = ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
+            torch.cuda.synchronize()
+            assert int(out.status.item()) == 0 and int(lm.status.item()) == 0
+            for f in ("accept_len", "next_tok", "entropy", "logZ"):
+                assert torch.equal(getattr(out, f), getattr(ref_out, f)), f
+            assert torch.equal(lm.entropy, ref_out.entropy) and lm.accept_len.shape == (w.B,) and lm.next_tok.dtype == torch.int32
+            assert out.logits is None and lm.logits.shape == (w.B, w.k + 1, w.V)
+            assert torch.equal(out.draft_entropy, torch.zeros((w.B, w.k), device=DEV))
+        gated = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, 1.0, gate_source=1)
+        want = -(w.draft_q.double() * w.draft_q.double().clamp_min(1e-300).log()).sum(-1)
+        assert torch.allclose(gated.draft_entropy.double(), want, atol=2e-3)
