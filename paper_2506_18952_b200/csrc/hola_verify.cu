@@ -111,6 +111,10 @@ struct K1Params {
   int n_sub, N;   // MMAs per K step and their N (verify rows each; multiple of 16)
   int rot;        // 1: three MMAs of N <= 128 per K step whose accumulators rotate over the four 128-column units
   int pair256;    // rot with N = 128 exactly: two of the three units of a tile are adjacent and take ONE MMA of N = 256
+  int kpb;        // K blocks per ring slot (1, 2 or 4); > 1: the tensor maps are three-dimensional and one copy brings them all;
+                  // a K block that H fills only in part then has a slot of its own, through two-dimensional maps (tmap_w4 of
+                  // W_lm, tmap_w16 of the hidden rows)
+  int k_tail;     // kpb > 1: 1 if there is such a block
   int acc_cols;   // tensor-memory columns from one accumulator buffer to the next
   int conv_groups, a_slots;   // (on-chip expansion) groups of converter warps that take part, K blocks of expanded operand
                               // that tensor memory holds (at most as many as ring slots)
@@ -133,6 +137,7 @@ struct K1Params {
   float4* partials;   // [grid][part_stride] (m, s, t, arg-max index)
   int part_stride;
   unsigned* status;
+  int prefetch_blocks;  // K blocks of its first tile a CTA asks into the L2 before it waits for the kernel before
   unsigned* pace;     // n_pass > 1: one counter per group of pairs (zero at launch), by which the group keeps in step
 };
 
@@ -306,6 +311,40 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       " [%0], [%1, {%3, %4}], [%2], %5;"
       ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(x), "r"(y), "l"(policy)
       : "memory");
+}
+
+// Three-dimensional form: (element of a K block, row, K block).
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int row, int kb,
+                                            uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(0), "r"(row), "r"(kb), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int row, int kb, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile.L2::cache_hint [%0, {%1, %2, %3}], %4;"
+               ::"l"(map), "r"(0), "r"(row), "r"(kb), "l"(policy)
+               : "memory");
+}
+// The same box into the L2 only.  A hint: it moves nothing that the program can see, so it may run ahead of the kernel
+// that this grid depends on even if that kernel writes the lines (the L2 is where writes land).
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y, uint64_t policy) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile.L2::cache_hint [%0, {%1, %2}], %3;"
+               ::"l"(map), "r"(x), "r"(y), "l"(policy)
+               : "memory");
+}
+// A table entry that the kernel before may still be writing, past the L1 (which must not keep what is read ahead of the
+// dependency wait).
+__device__ __forceinline__ int load_past_l1(const int* p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int load_past_l1(const uint8_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return static_cast<int>(v);
 }
 
 // All passes in one launch: the pairs of a group read the same tile of W_lm, and only those that read it within the
@@ -686,7 +725,12 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   const int rows = p.n_pass > 1 ? min(p.rows_per_pass, p.M - row0) : p.rows;
   const int half_n = p.N >> 1;                           // hidden rows this CTA supplies per MMA
   const uint32_t hid_block_bytes = static_cast<uint32_t>(half_n) * 128u;
-  const uint32_t stage_bytes = kWBlockBytes + (kW8 ? 2 : p.n_sub) * hid_block_bytes;
+  // Bytes of a K block's rows of W_lm in the slot (the MMA reads 128 rows from its start: what follows only reaches lanes
+  // that hold nothing) and of the slot.
+  const uint32_t w_block_bytes = kW8 || kRot ? kWBlockBytes : (static_cast<uint32_t>(p.tile_rows) * 128u + 1023u) & ~1023u;
+  const uint32_t stage_bytes = kW8 ? kWBlockBytes + 2 * hid_block_bytes : p.kpb * (w_block_bytes + p.n_sub * hid_block_bytes);
+  const int n_slots = kRot || kW8 || p.kpb == 1 ? p.n_kblocks        // slots' worth of K blocks per tile
+                                                : (p.n_kblocks - p.k_tail + p.kpb - 1) / p.kpb + p.k_tail;
   const uint32_t hid_tx_bytes = p.n_sub * hid_block_bytes;
   const uint32_t tx_bytes = static_cast<uint32_t>(p.tile_rows) * 128u + hid_tx_bytes;   // bf16 W_lm: per CTA and slot
   const int code_blocks = (p.n_kblocks + 1) >> 1;        // (on-chip expansion) K blocks of a tile of 4- or 8-bit rows
@@ -745,6 +789,21 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      // While the kernel before still runs (in a loop of calls: the accept/sample kernel, some 10 us of latency in which
+      // HBM would idle), the first blocks of this CTA's rows move into the L2.
+      if (p.prefetch_blocks > 0 && my_tiles > 0) {
+        int width = 0, w_row = pair * pair_rows + static_cast<int>(rank) * p.tile_rows;
+        if (kW8 && p.group_width) {
+          width = load_past_l1(p.group_width + pair);
+          w_row = load_past_l1(p.group_row + pair) + static_cast<int>(rank) * p.tile_rows;
+        }
+        const CUtensorMap* map = width == 4 ? &tmap_w4 : width == 16 ? &tmap_w16 : &tmap_w;
+        const int step = width == 4 || width == 16 ? kBlockK : (kW8 ? kExpandK : kKStep);   // box width, in map elements
+        if (!kRot && !kW8 && p.kpb > 1) {
+          for (int kb = 0; kb < p.prefetch_blocks; kb += p.kpb) tma_prefetch_3d(map, w_row, kb, pol_w);
+        } else
+        for (int kb = 0; kb < p.prefetch_blocks; ++kb) tma_prefetch_2d(map, kb * step, w_row, pol_w);
+      }
       grid_dependency_wait();                            // W_lm and the hidden rows may come from the kernel before
       if (p.clear_status && blockIdx.x == 0) *p.status = 0u;
       if (kW8) {
@@ -792,6 +851,29 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       for (int t = 0; t < my_tiles && ok; ++t) {
         const int v0 = (pair + t * npairs) * pair_rows + static_cast<int>(rank) * p.tile_rows;
         if (p.n_pass > 1 && p.pace && t > 0) keep_pace(p.pace + pair, static_cast<unsigned>(2 * p.n_pass * t));
+        if (!kRot && p.kpb > 1) {
+          // Several K blocks per slot: one wait, one announcement and two copies for all of them.  A producer that does
+          // this per K block needs some 450 cycles for it, which bounds narrow tiles (and tiles that are in the L2).
+          const uint32_t hid_off = p.kpb * w_block_bytes;
+          for (int i = 0; i < n_slots; ++i) {
+            const uint32_t sa = base + stage * stage_bytes;
+            if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+            const uint32_t fb = leader_full + 8 * stage;
+            const int h_row = (kTwoPlane ? 2 : 1) * row0 + static_cast<int>(rank) * half_n;
+            if (p.k_tail && i == n_slots - 1) {
+              const int kx = (p.n_kblocks - 1) * kKStep;
+              mbar_expect_tx_cluster(fb, tx_bytes);
+              tma_load_2d(sa, &tmap_w4, fb, kx, v0, pol_w);
+              tma_load_2d(sa + hid_off, &tmap_w16, fb, kx, h_row, pol_h);
+            } else {
+              mbar_expect_tx_cluster(fb, p.kpb * tx_bytes);
+              tma_load_3d(sa, &tmap_w, fb, v0, i * p.kpb, pol_w);
+              tma_load_3d(sa + hid_off, &tmap_hidden, fb, h_row, i * p.kpb, pol_h);
+            }
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+          }
+          continue;
+        }
         int kx = 0;                                      // K coordinate of the block, in elements
         for (int kb = 0; kb < p.n_kblocks; ++kb, kx += kKStep) {
           const uint32_t sa = base + stage * stage_bytes;
@@ -811,7 +893,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
             tma_load_2d(sa + kWBlockBytes + 2 * hid_block_bytes, &tmap_hidden, fb, kx, row0 + single_row, pol_h);
           } else {
             for (int s = 0; s < p.n_sub; ++s)
-              tma_load_2d(sa + kWBlockBytes + s * hid_block_bytes, &tmap_hidden, fb, kx,
+              tma_load_2d(sa + w_block_bytes + s * hid_block_bytes, &tmap_hidden, fb, kx,
                           (kTwoPlane ? 2 : 1) * row0 + s * p.N + static_cast<int>(rank) * half_n, pol_h);
           }
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -936,12 +1018,12 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         if (!mbar_wait(tempty_bar + 8 * buf, acc_phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + buf * 256;
-        for (int kb = 0; kb < p.n_kblocks; ++kb) {
+        for (int kb = 0; kb < n_slots; ++kb) {
           if (!mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status)) { ok = false; break; }
           tc_fence_after();
           // descriptors of this slot: only the 14-bit address field changes (16-byte units)
           const uint64_t adesc = desc0 + ((stage * stage_bytes) >> 4);
-          const uint64_t bdesc0 = adesc + (kWBlockBytes >> 4);
+          const uint64_t bdesc0 = adesc + ((p.kpb * w_block_bytes) >> 4);
           const uint32_t acc = kb != 0 ? 1u : 0u;
           // 16 bf16 = 32 bytes further along K inside the swizzled row: +2 in 16-byte address units
           if (two_mmas) {
@@ -957,6 +1039,13 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
             umma<kI8>(d0, adesc, bdesc0, idesc, acc);
 #pragma unroll
             for (int kk = 1; kk < kBlockK / 16; ++kk) umma<kI8>(d0, adesc + 2 * kk, bdesc0 + 2 * kk, idesc, 1u);
+            // (whole K blocks past the last one are zeros in both operands)
+            const int blocks = p.k_tail && kb == n_slots - 1 ? 1 : p.kpb;
+            for (int n = 1; n < blocks; ++n) {
+              const uint64_t an = adesc + n * (w_block_bytes >> 4), bn = bdesc0 + n * (hid_block_bytes >> 4);
+#pragma unroll
+              for (int kk = 0; kk < kBlockK / 16; ++kk) umma<kI8>(d0, an + 2 * kk, bn + 2 * kk, idesc, 1u);
+            }
           }
           umma_commit_pair(empty_bar + 8 * stage);       // frees the slot in both CTAs once these MMAs have read it
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -1465,8 +1554,11 @@ __device__ __forceinline__ void stats_to_outputs(Stats st, float* logZ, float* H
 
 __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, int nparts, int part_stride, int M,
                                                        float* logZ, float* entropy) {
+  // (launched like the accept/sample kernel: the next kernel in the stream may be put in place behind this one)
+  grid_dependency_release();
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  grid_dependency_wait();
   if (row >= M) return;
   Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
   if (lane == 0) stats_to_outputs(st, &logZ[row], &entropy[row]);
@@ -2290,6 +2382,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 struct Plan {
   int n_sub, N, rows_per_pass, passes, grid, stages, nbuf, rot, n_ptiles, n_kblocks, smem_bytes, tile_rows;
   int fused;            // all passes in one launch, groups of `passes` CTA pairs sharing the vocabulary tiles
+  int kpb, k_tail;      // K blocks per ring slot; a partial last K block in a slot of its own
   double est_seconds;   // rough duration of all passes (the cost the split was chosen by)
 };
 
@@ -2445,13 +2538,6 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   }
   // a pass may end up empty when rows_per_pass * (passes - 1) already covers M
   best.passes = (rows + best.rows_per_pass - 1) / best.rows_per_pass;
-  const int stage_bytes = kWBlockBytes + (w8 ? 2 : best.n_sub) * (best.N / 2) * 128;
-  // (rotating units: every epilogue warp stages a whole 32-row chunk, twice the bytes)
-  const int trans_bytes = (w8 ? kW8EpiWarps : kEpiWarps) * kTransBytes * (best.n_sub == 3 ? 2 : 1);
-  int stages = (kSmemBudget - 1024 - kBarrierBytes - trans_bytes) / stage_bytes;
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (ctx->force_stages && ctx->force_stages < stages) stages = ctx->force_stages;
-  best.stages = stages;
   best.nbuf = best.n_sub == 1 ? 2 : 1;
   best.rot = best.n_sub == 3 ? 1 : 0;
   // Vocabulary rows per CTA per tile: the smallest multiple of 4 that covers V in the fewest whole rounds over
@@ -2464,6 +2550,7 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int pairs = best.fused ? all_pairs / best.passes : all_pairs;     // pairs that divide the tiles among them
   const int rounds = (ctx->V + pairs * kPairTile - 1) / (pairs * kPairTile);
   int tile_rows = round_up((ctx->V + 2 * pairs * rounds - 1) / (2 * pairs * rounds), 4);
+  if (tile_rows < 104) tile_rows = round_up(tile_rows, 8);         // whole swizzle patterns: several K blocks per slot
   if (tile_rows < 8) tile_rows = 8;
   if (tile_rows > kLanes) tile_rows = kLanes;
   if (mixed) tile_rows = kLanes;                 // a pair's tile is one group of 256 rows of one width
@@ -2471,6 +2558,26 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   best.n_ptiles = (ctx->V + 2 * tile_rows - 1) / (2 * tile_rows);
   best.grid = 2 * (best.n_ptiles < pairs ? best.n_ptiles : pairs) * (best.fused ? best.passes : 1);
   best.n_kblocks = i8 ? (ctx->H + 2 * kBlockK - 1) / (2 * kBlockK) : (ctx->H + kBlockK - 1) / kBlockK;
+  // Ring slots.  Narrow tiles and few rows: several K blocks per slot, so that the producer's cost per slot (some 450
+  // cycles whatever the size) is spread over 30 to 40 KB.  Wide tiles (or 225 rows and more) take longer than that for a
+  // K block in HBM (or on the tensor cores) anyway.
+  const int w_block = w8 || best.rot ? kWBlockBytes : round_up(best.tile_rows * 128, 1024);
+  const int k_elems = i8 ? 2 * kBlockK : kBlockK;
+  const int block_bytes = w_block + best.n_sub * (best.N / 2) * 128;
+  const int whole_blocks = ctx->H / k_elems;
+  best.kpb = 1;
+  if (!w8 && best.n_sub == 1 && best.N <= 224 && best.tile_rows % 8 == 0) {
+    if (whole_blocks >= 4 && 4 * block_bytes <= 40 * 1024) best.kpb = 4;
+    else if (whole_blocks >= 2 && 2 * block_bytes <= 48 * 1024) best.kpb = 2;
+  }
+  best.k_tail = best.kpb > 1 && ctx->H % k_elems != 0 ? 1 : 0;
+  const int stage_bytes = w8 ? kWBlockBytes + 2 * (best.N / 2) * 128 : best.kpb * block_bytes;
+  // (rotating units: every epilogue warp stages a whole 32-row chunk, twice the bytes)
+  const int trans_bytes = (w8 ? kW8EpiWarps : kEpiWarps) * kTransBytes * (best.n_sub == 3 ? 2 : 1);
+  int stages = (kSmemBudget - 1024 - kBarrierBytes - trans_bytes) / stage_bytes;
+  if (stages > kMaxStages) stages = kMaxStages;
+  if (ctx->force_stages && ctx->force_stages < stages) stages = ctx->force_stages;
+  best.stages = stages;
   best.smem_bytes = stages * stage_bytes + kBarrierBytes + trans_bytes + 1024;
   return best;
 }
@@ -2491,14 +2598,21 @@ const Plan& plan_for(hola_ctx* ctx, int M, int w_dtype) {
 // the 128-byte swizzle that the MMA reads (and that spreads the rows of 8-bit codes over the banks for the converter
 // warps).  `packed4`: rows of cols / 2 bytes holding two 4-bit codes each; box of 64 bytes (128 codes), 64-byte swizzle.
 hola_status encode_map(hola_ctx* ctx, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
-                       uint32_t box_rows, bool int8 = false, bool packed4 = false) {
+                       uint32_t box_rows, bool int8 = false, bool packed4 = false, int kpb = 1) {
   if (packed4) { cols /= 2; int8 = true; }
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {cols * (int8 ? 1u : 2u)};
   const cuuint32_t box[2] = {static_cast<cuuint32_t>(int8 && !packed4 ? 2 * kBlockK : kBlockK), box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = ctx->encode(map, int8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                                 const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  // `kpb` > 1: the same memory as (element of a K block, row, K block), kpb K blocks per box; needs whole K blocks
+  const cuuint64_t dims3[3] = {box[0], rows, cols / box[0]};
+  const cuuint64_t strides3[2] = {strides[0], 128};
+  const cuuint32_t box3[3] = {box[0], box_rows, static_cast<cuuint32_t>(kpb)};
+  const cuuint32_t estr3[3] = {1, 1, 1};
+  const bool three = kpb > 1;
+  const CUresult r = ctx->encode(map, int8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                                 three ? 3 : 2, const_cast<void*>(ptr), three ? dims3 : dims, three ? strides3 : strides,
+                                 three ? box3 : box, three ? estr3 : estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                  packed4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
@@ -2521,9 +2635,18 @@ hola_status check_common(const hola_ctx* ctx, const hola_verify_args* a) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Cluster size of the accept/sample launch (CTAs per sequence): as many as keep the grid within one wave of the SMs.
+int sample_cluster(const hola_ctx* ctx, int B, int V) {
+  const int nchunks = (V + kChunk - 1) / kChunk;
+  int S = 8;
+  while (S > 1 && (B * S > kK3MaxPerSm * ctx->num_sms || nchunks / S < 8)) S >>= 1;
+  return S;
+}
+
 // Steps 1-2: the LM-head GEMM with fused statistics, one launch (clusters of two CTAs) per pass over W_lm.
+// `few_before`: the kernel in front is expected to be this context's accept/sample kernel on a few SMs.
 hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits, int ldl, const Plan& pl,
-                        cudaStream_t stream) {
+                        cudaStream_t stream, bool few_before = false) {
   const int M = a->B * (a->k + 1);
   const bool mixed = a->w_dtype == HOLA_W_MIXED;
   const bool w8 = a->w_dtype == HOLA_W_INT8 || mixed, two = a->w_dtype == HOLA_W8A16,
@@ -2562,19 +2685,27 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     me->valid = 0;
     if (two)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(2 * round_up(M, 32)), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true);
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb);
     else if (i8)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true);
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb);
     else
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2));
+                     static_cast<uint32_t>(pl.N / 2), false, false, pl.kpb);
     if (s != HOLA_OK) return s;
     const uint32_t trows = static_cast<uint32_t>(pl.tile_rows);
     if (!mixed) {
-      s = encode_map(ctx, &me->tw, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, w8 || i8);
+      s = encode_map(ctx, &me->tw, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, w8 || i8,
+                     false, pl.kpb);
       if (s != HOLA_OK) return s;
-      me->tw4 = me->tw; me->tw16 = me->tw;               // (never read outside the mixed-width form)
+      me->tw4 = me->tw; me->tw16 = me->tw;               // (read for a partial last K block only)
+      if (pl.k_tail) {
+        s = encode_map(ctx, &me->tw4, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, i8);
+        if (s != HOLA_OK) return s;
+        s = encode_map(ctx, &me->tw16, hid_src, static_cast<uint64_t>(two ? 2 * round_up(M, 32) : M),
+                       static_cast<uint64_t>(a->H), static_cast<uint32_t>(pl.N / 2), i8);
+        if (s != HOLA_OK) return s;
+      }
       me->W4 = nullptr; me->W16 = nullptr;
     } else {
       // one map per width that occurs; a width that does not occur gets a copy of one that does (never used)
@@ -2610,6 +2741,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   K1Params kp;
   kp.M = M; kp.V = a->V; kp.n_ptiles = pl.n_ptiles; kp.n_kblocks = pl.n_kblocks;
   kp.pair256 = (pl.rot && pl.N == 128 && !ctx->no_pair256) ? 1 : 0;
+  kp.kpb = pl.kpb; kp.k_tail = pl.k_tail;
   kp.acc_cols = !w8 ? 256 : (pl.N <= 128 ? 128 : kExpandMaxN);
   kp.conv_groups = ctx->conv_group > kConvGroup ? 1 : kConvGroups;
   const int a_slots = (kTmemCols - 2 * kp.acc_cols) / kOperandCols;
@@ -2642,6 +2774,16 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
+  // Ahead of the dependency wait: 32 MB, about what HBM moves while the accept/sample kernel of the call before runs, where
+  // that kernel leaves nearly all SMs to this one's CTAs.  V = 32000, H = 4096, one sequence, none / 16 / 32 / 48 MB: bf16
+  // 52.2 / 50.9 / 50.0 / 49.7 us, mixed widths 43.9 / 42.2 / 42.6 / 43.2, 8-bit 37.2 / 36.3 / 36.5 / 36.8; with 16
+  // sequences (128 CTAs of the accept/sample kernel in the way) 61.6 / 61.5 / 62.5 / 63.3, hence the limit.
+  kp.prefetch_blocks = 0;
+  if (few_before) {
+    const int per_tile = w8 ? (pl.n_kblocks + 1) / 2 : pl.n_kblocks - pl.k_tail;
+    const int blocks = static_cast<int>(32e6 / (static_cast<double>(pl.grid) * pl.tile_rows * 128.0));
+    kp.prefetch_blocks = (blocks < per_tile ? blocks : per_tile) / pl.kpb * pl.kpb;
+  }
   kp.n_pass = pl.fused ? pl.passes : 1;
   kp.rows_per_pass = pl.rows_per_pass;
   kp.pace = nullptr;
@@ -2664,6 +2806,17 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     if (e != cudaSuccess) { set_error(ctx, "launch lm_head_entropy_kernel", e); return HOLA_ERR_CUDA; }
   }
   return HOLA_OK;
+}
+
+cudaError_t launch_finalize(const hola_ctx* ctx, const hola_verify_args* a, int M, int nparts, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>((M + 7) / 8)); cfg.blockDim = dim3(256); cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, finalize_kernel, static_cast<const float4*>(ctx->partials), nparts, ctx->max_rows, M,
+                            a->logZ, a->entropy);
 }
 
 // What the accept/sample kernel needs to know in the vocabulary-parallel form.
@@ -2708,11 +2861,8 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     if (combine) { kp.partials = sh->stats_all; kp.nparts = sh->world; kp.part_stride = sh->rec_floats / 4; }
   }
   const bool vec = (a->V % 4 == 0) && (ldl % 4 == 0) && aligned16(logits) && (a->k == 0 || aligned16(a->draft_q));
-  // cluster size: as many CTAs per sequence as keeps the grid within a few waves of the SMs
   const int nchunks = (a->V + kChunk - 1) / kChunk;
-  int S = 8;
-  while (S > 1 && (a->B * S > kK3MaxPerSm * ctx->num_sms || nchunks / S < 8)) S >>= 1;   // one wave of CTAs
-  if (phase == 1) S = 1;                                 // no vocabulary pass: one CTA per sequence
+  const int S = phase == 1 ? 1 : sample_cluster(ctx, a->B, a->V);    // (phase 1: no vocabulary pass)
   const int cpc = (nchunks + S - 1) / S;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(a->B * S));
@@ -3003,9 +3153,8 @@ hola_status hola_lm_head_entropy(hola_ctx* ctx, const hola_verify_args* a, void*
   const Plan& pl = plan_for(ctx, M, a->w_dtype);
   float* logits = a->logits_out ? a->logits_out : ctx->logits;
   const int ldl = a->logits_out ? a->V : ctx->ldl;
-  if ((s = run_lm_head(ctx, a, logits, ldl, pl, stream)) != HOLA_OK) return s;
-  finalize_kernel<<<(M + 7) / 8, 256, 0, stream>>>(ctx->partials, pl.grid, ctx->max_rows, M, a->logZ, a->entropy);
-  const cudaError_t e = cudaGetLastError();
+  if ((s = run_lm_head(ctx, a, logits, ldl, pl, stream, M <= 256)) != HOLA_OK) return s;
+  const cudaError_t e = launch_finalize(ctx, a, M, pl.grid, stream);
   if (e != cudaSuccess) { set_error(ctx, "launch finalize_kernel", e); return HOLA_ERR_CUDA; }
   return HOLA_OK;
 }
@@ -3044,7 +3193,8 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   // (While the caller records a graph everything stays on the caller's stream.)
   const bool side = draft_gate && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
-  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream);
+  const bool few_before = a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
+  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
   if (side) {
@@ -3536,6 +3686,5 @@ extern "C" hola_status hola_lm_head_entropy_static(const hola_verify_args* a, vo
   // call before they are read; the internal status word is the one thing that must start at zero.
   if (cudaMemsetAsync(local.status, 0, sizeof(unsigned), stream) != cudaSuccess) return HOLA_ERR_CUDA;
   if ((s = run_lm_head(&local, a, a->logits_out, a->V, pl, stream)) != HOLA_OK) return s;
-  finalize_kernel<<<(M + 7) / 8, 256, 0, stream>>>(local.partials, pl.grid, local.max_rows, M, a->logZ, a->entropy);
-  return cudaGetLastError() == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
+  return launch_finalize(&local, a, M, pl.grid, stream) == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
 }

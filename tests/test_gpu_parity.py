@@ -1000,3 +1000,43 @@ def test_fresh_outputs_start_with_a_clear_status_word_and_hold_every_field(bindi
         gated = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, 1.0, gate_source=1)
         want = -(w.draft_q.double() * w.draft_q.double().clamp_min(1e-300).log()).sum(-1)
         assert torch.allclose(gated.draft_entropy.double(), want, atol=2e-3)
+
+
+@pytest.mark.parametrize("B,k,H,V,weights", [
+    (3, 4, 256, 4736, "bf16"),        # 32 rows per CTA, four K blocks per slot, one slot per tile
+    (3, 4, 704, 5003, "bf16"),        # eleven K blocks: the last slot is partly past the end
+    (23, 3, 1032, 9001, "bf16"),      # a K block that H fills in part: its own slot
+    (40, 4, 136, 14000, "bf16"),      # two whole K blocks and a part
+    (44, 4, 320, 23680, "bf16"),      # 220 rows: two K blocks per slot
+    (1, 4, 1040, 30000, "w8a8"), (9, 3, 1168, 9001, "w8a8"),      # K blocks of 128: a part of 16 channels; one of 16 beyond nine
+    (5, 2, 528, 6000, "w8a16"), (30, 2, 256, 3000, "w8a16"),
+])
+def test_several_k_blocks_per_slot(binding, B, k, H, V, weights):
+    """Narrow tiles take two or four K blocks per ring slot.  Logits against fp64 products of the operands as the mode
+    defines them (fp32 accumulation: one rounding or truncation of 2^-23 per step of sixteen products and per product in a
+    step, hence below (H / 16 + 16) 2^-23 of sum |terms|; the 8-bit modes accumulate exactly), twice over so that a slot's
+    stale contents would show."""
+    w = workloads.gaussian_head("slots", B, k, H, V, seed=B + H, device=DEV, w_std=0.3)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        head, scale, a8 = w.W_lm, None, False
+        h = w.hidden.double().reshape(-1, H)
+        if weights == "bf16":
+            Wd, bound = head.double(), (H / 16 + 16) * 2.0 ** -23
+        else:
+            from oracle import lobi
+            head, scale = binding.hola_quantize_w8(w.W_lm)
+            Wd, bound = head.double() * scale.double()[:, None], 2.0 ** -21
+            a8 = True if weights == "w8a8" else "a16"
+            h32 = w.hidden.float().reshape(-1, H).cpu().numpy()
+            deq = lobi.dequantize_rows(*lobi.quantize_rows_int8(h32)) if a8 is True else \
+                lobi.dequantize_two_plane(*lobi.quantize_rows_two_plane(h32))
+            h = torch.from_numpy(np.asarray(deq)).to(DEV)
+        want = h @ Wd.T
+        limit = bound * (h.abs() @ Wd.abs().T)
+        for _ in range(2):
+            out = ctx.hola_lm_head_entropy(w.hidden, head, w_scale=scale, a8=a8)
+            torch.cuda.synchronize()
+            assert int(out.status.item()) == 0
+            assert torch.all((out.logits.double().reshape(-1, V) - want).abs() <= limit)
+            full = ctx.hola_verify(w.hidden, head, w.draft_tok, w.draft_q, w.uniforms, w.tau, w_scale=scale, a8=a8)
+            assert torch.allclose(full.logZ.double().reshape(-1), torch.logsumexp(want, -1), atol=2e-3)
