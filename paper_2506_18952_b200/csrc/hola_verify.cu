@@ -95,6 +95,7 @@ constexpr int kK3MaxPerSm = 4;                   // CTAs of the accept/sample ke
 constexpr int kChunk = 128;                      // vocabulary entries per warp step (32 lanes x 4)
 constexpr int kMaxChunks = 4096;                 // => V <= 524288
 constexpr int kMaxK1 = 64;                       // k + 1 <= 64
+constexpr int kK3MaxDynSmem = 200 * 1024;        // rows staged in shared memory, see K3Params::staged
 constexpr int kK3Unroll = 4;                     // vocabulary chunks a warp has in flight per step
 
 constexpr int kHqSlices = 8;                     // CTAs that share one draft row in draft_entropy_kernel
@@ -137,6 +138,14 @@ struct K1Params {
   float4* partials;   // [grid][part_stride] (m, s, t, arg-max index)
   int part_stride;
   unsigned* status;
+  // What the accept/sample kernel behind this one will gather (null: nothing): draft tokens, uniforms and the entries
+  // q_j(x_j), and all of q when it is small.  An idle warp asks for it early on, so that the chain of dependent reads there
+  // finds it in the L2 instead of in DRAM.
+  const int* next_tok;
+  const float* next_u;
+  const char* next_q;
+  int next_n, next_q_elem;      // B * k; bytes per draft probability
+  unsigned next_q_bytes;        // bytes of q to ask for whole (0: only the entries)
   int prefetch_blocks;  // K blocks of its first tile a CTA asks into the L2 before it waits for the kernel before
   unsigned* pace;     // n_pass > 1: one counter per group of pairs (zero at launch), by which the group keeps in step
 };
@@ -155,6 +164,8 @@ struct K3Params {
   int inputs_settled;           // 1: launched right behind this call's own GEMM kernel, whose CTAs have waited for the
                                 // kernel before the call: tokens, uniforms and draft probabilities may be read
                                 // before this grid's dependency wait.  0: wait first.
+  int staged;                   // 1: this CTA's slice of ALL k + 1 rows is brought into shared memory while the statistics are
+                                // merged and the accept test is made, instead of row n afterwards
   int phase;                    // 0: the whole step; 1: stop after the accept test (accept_len, statistics written);
                                 // vocabulary-parallel form: 3: stop after the masses of row n inside this shard,
                                 // 4: the draw, by the shard that holds the point u * R
@@ -333,6 +344,10 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
   asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile.L2::cache_hint [%0, {%1, %2}], %3;"
                ::"l"(map), "r"(x), "r"(y), "l"(policy)
                : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, unsigned bytes) {      // both multiples of 16
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 // A table entry that the kernel before may still be writing, past the L1 (which must not keep what is read ahead of the
 // dependency wait).
@@ -902,6 +917,19 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
+    if (rank == 1 && p.next_tok) {
+      grid_dependency_wait();
+      const int w = pair_of_grid, nw = gridDim.x >> 1;
+      for (int i = w * 32 + lane; i < p.next_n; i += nw * 32) {
+        const int x = p.next_tok[i];
+        prefetch_l2(p.next_u + i);
+        if (x >= 0 && x < p.V) prefetch_l2(p.next_q + (static_cast<size_t>(i) * p.V + x) * p.next_q_elem);
+      }
+      if (p.next_q_bytes && lane == 0) {
+        const unsigned piece = ((p.next_q_bytes + nw - 1) / nw + 15u) & ~15u, at = piece * w;
+        if (at < p.next_q_bytes) bulk_prefetch_l2(p.next_q + at, min(piece, p.next_q_bytes - at));
+      }
+    }
     if (rank == 0 && elect_one()) {
       const uint32_t idesc = kI8 ? make_idesc_s8_m256(static_cast<uint32_t>(p.N))
                                  : make_idesc_bf16_m256(static_cast<uint32_t>(p.N));
@@ -1518,10 +1546,14 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_selftest_kernel(long long 
 }
 
 // ------------------------------------------------------------------------------------------------ K2
+// The statistics of one row over all CTAs, by a warp, the same bits in every lane.  Six loads per lane in flight (192
+// partials per round: one round on a 148-SM part); `while_loading` runs behind their issue.  The maximum first, so that the
+// exponentials of the partials are independent of one another and only additions remain to be passed round: five
+// shuffles for the maximum and five for the sums instead of eleven merges of a hundred cycles each.
+template <typename F>
 __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int part_stride, int row,
-                                                     int lane) {
+                                                     int lane, F while_loading) {
   Stats st = stats_empty();
-  // six loads per lane in flight (192 partials per round: one round on a 148-SM part), then the merges in index order
   for (int base = 0; base < nparts; base += 192) {
     float4 x[6];
 #pragma unroll
@@ -1530,18 +1562,28 @@ __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int
       x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride + row]
                         : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
     }
+    if (base == 0) while_loading();
+    float m = fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x));
 #pragma unroll
-    for (int u = 0; u < 6; ++u) st = stats_merge(st, Stats{x[u].x, x[u].y, x[u].z, __float_as_int(x[u].w)});
-  }
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    float s = 0.f, t = 0.f;
+    int arg = 0x7fffffff;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    Stats o;
-    o.m = __shfl_xor_sync(0xffffffffu, st.m, off);
-    o.s = __shfl_xor_sync(0xffffffffu, st.s, off);
-    o.t = __shfl_xor_sync(0xffffffffu, st.t, off);
-    o.arg = __shfl_xor_sync(0xffffffffu, st.arg, off);
-    // merge in a fixed (lower lane first) order so that every lane holds bit-identical results
-    st = ((lane & off) == 0) ? stats_merge(st, o) : stats_merge(o, st);
+    for (int u = 0; u < 6; ++u) {
+      if (x[u].x == m) arg = min(arg, __float_as_int(x[u].w));
+      if (x[u].x != -CUDART_INF_F) {
+        const float d = x[u].x - m, e = __expf(d);
+        s = fmaf(e, x[u].y, s);
+        t = fmaf(e, fmaf(d, x[u].y, x[u].z), t);
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, off);
+      t += __shfl_xor_sync(0xffffffffu, t, off);
+    }
+    arg = __reduce_min_sync(0xffffffffu, arg);
+    st = stats_merge(st, Stats{m, s, t, arg});
   }
   return st;
 }
@@ -1560,7 +1602,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, i
   const int lane = threadIdx.x & 31;
   grid_dependency_wait();
   if (row >= M) return;
-  Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
+  Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane, [] {});
   if (lane == 0) stats_to_outputs(st, &logZ[row], &entropy[row]);
 }
 
@@ -1576,7 +1618,7 @@ __global__ void __launch_bounds__(256) shard_record_kernel(const float4* partial
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
-    Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
+    Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane, [] {});
     if (lane == 0) {
       const int arg = st.arg == 0x7fffffff ? st.arg : st.arg + v_offset;
       stats_out[row] = make_float4(st.m, st.s, st.t, __int_as_float(arg));
@@ -1662,6 +1704,13 @@ __device__ __forceinline__ void load_r4(const float* lrow, const void* qrow, int
   resid4(l, q, logZ, r);
 }
 
+// Copies into shared memory that nobody waits for yet (cp_async_wait_all: this thread's have landed).
+template <int kBytes>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(kBytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
   if (!(u >= 0.f)) { flags |= HOLA_FLAG_BAD_UNIFORM; return 0.f; }
   if (u >= 1.f) { flags |= HOLA_FLAG_BAD_UNIFORM; return 1.f - 5.9604645e-8f; }   // 1 - 2^-24
@@ -1674,12 +1723,10 @@ __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
 // the total mass R and which slice holds the point u*R; that CTA alone finishes the inverse-CDF search.
 template <bool kVec>
 __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
-  extern __shared__ double csum[];                       // per-chunk residual mass of this CTA's slice
+  extern __shared__ __align__(16) double csum[];                       // per-chunk residual mass of this CTA's slice
   __shared__ double sh_tot[2][8];                        // slice totals of the whole cluster, per attempt
   __shared__ float sh_logZ[kMaxK1], sh_H[kMaxK1], sh_lx[kMaxK1], sh_qx[kMaxK1], sh_u[kMaxK1], sh_Hq[kMaxK1];
   __shared__ int sh_x[kMaxK1], sh_amax[kMaxK1];
-  __shared__ int sh_n;
-  __shared__ unsigned sh_flags;
 
   // The next kernel in the stream (normally the next call's GEMM kernel, which waits for this grid before it touches
   // memory) may be scheduled from now on: its launch and prologue then hide behind this kernel.
@@ -1692,57 +1739,83 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const int k = p.k, V = p.V;
   const int row_first = b * (k + 1);
 
-  // ---- gather the k draft-token logits, draft probabilities and the uniforms (independent of the statistics).
-  // These come from the caller, not from the GEMM kernel.  Behind this call's own GEMM kernel they are known to be in
-  // place (its CTAs waited for whatever ran before the call) and are fetched before this grid's dependency wait; in
-  // every other launch the wait comes first.
+  // ---- the draft tokens and uniforms, a position per thread (k <= 63 < kK3Threads).  These come from the caller, not from
+  // the GEMM kernel.  Behind this call's own GEMM kernel they are known to be in place (its CTAs waited for whatever ran
+  // before the call) and are asked for before this grid's dependency wait; in every other launch the wait comes first.
+  // Nothing looks at a loaded value before everything that does not depend on it has been asked for: each look costs a
+  // round trip to the L2 (or, where the GEMM kernel's idle warps have not asked ahead, to DRAM).
   if (!p.inputs_settled) grid_dependency_wait();
-  for (int j = threadIdx.x; j <= k; j += kK3Threads) sh_u[j] = p.u[b * (k + 1) + j];
-  int x_mine = -1;                                       // (k <= 63 < kK3Threads: one draft position per thread)
-  float qx_mine = 0.f;
   const bool shard = p.shard_world > 0;
   const int Vtok = shard ? p.V_global : V;               // range of valid token ids
-  if (threadIdx.x < k) {
-    const int j = threadIdx.x;
-    x_mine = p.tok[b * k + j];
-    if (x_mine >= 0 && x_mine < Vtok) {
-      const size_t qi = (static_cast<size_t>(b) * k + j) * V + x_mine;
-      if (p.q_tok) qx_mine = p.q_tok[b * k + j];
-      else qx_mine = (p.q_dtype == HOLA_Q_BF16) ? __bfloat162float(static_cast<const __nv_bfloat16*>(p.q)[qi])
-                                                : static_cast<const float*>(p.q)[qi];
-    }
-  }
+  const int j_mine = threadIdx.x;
+  int x_mine = -1;
+  float u_mine = 0.f;
+  if (j_mine < k) x_mine = p.tok[b * k + j_mine];
+  if (j_mine <= k) u_mine = p.u[b * (k + 1) + j_mine];
   // From here on the GEMM kernel's results are read.
   if (p.inputs_settled) grid_dependency_wait();
-  for (int j = threadIdx.x; j < k; j += kK3Threads) {
-    const int x = x_mine;
-    sh_x[j] = x;
-    float lx = 0.f;
-    const float qx = qx_mine;
-    if (x >= 0 && x < Vtok) {
+  const int nchunks = (V + kChunk - 1) / kChunk;
+  const int cpc = (nchunks + S - 1) / S;                 // chunks per CTA
+  const int c_first = rank * cpc;
+  const int mine = max(0, min(nchunks, c_first + cpc) - c_first);
+  const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
+  // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities.  A lane copies
+  // what it will read in the pass: chunk c of every row goes through warp c % kK3Warps.
+  const bool staged = kVec && p.staged;
+  const int slice = cpc * kChunk;
+  float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
+  char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
+  auto stage_rows = [&]() {
+    for (int c = warp; c < mine; c += kK3Warps) {
+      const int at = c * kChunk + lane * 4, v = c_first * kChunk + at;        // (V % 4 == 0: all four or none)
+      if (v >= V) continue;
+      float* dl = sl + at;
+      const float* l = p.logits + static_cast<size_t>(row_first) * p.ldl + v;
+      for (int j = 0; j <= k; ++j, dl += slice, l += p.ldl) cp_async<16>(dl, l);
+      if (p.q_dtype == HOLA_Q_BF16) {
+        char* dq = sq + at * 2;
+        const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + v) * 2;
+        for (int j = 0; j < k; ++j, dq += slice * 2, q += static_cast<size_t>(V) * 2) cp_async<8>(dq, q);
+      } else {
+        char* dq = sq + at * 4;
+        const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + v) * 4;
+        for (int j = 0; j < k; ++j, dq += slice * 4, q += static_cast<size_t>(V) * 4) cp_async<16>(dq, q);
+      }
+    }
+  };
+  // the draft token's logit and probability
+  float lx = 0.f, hq = 0.f;
+  uint32_t q_bits = 0;                                   // (as loaded: converted when it is stored)
+  if (j_mine < k) {
+    const int j = j_mine;
+    if (x_mine >= 0 && x_mine < Vtok) {
+      const size_t qi = (static_cast<size_t>(b) * k + j) * V + x_mine;
+      if (p.q_tok) q_bits = __float_as_uint(p.q_tok[b * k + j]);
+      else if (p.q_dtype == HOLA_Q_BF16) q_bits = static_cast<const uint16_t*>(p.q)[qi];
+      else q_bits = static_cast<const uint32_t*>(p.q)[qi];
       if (shard) {                                       // exactly one shard owns x and left its logit there
         lx = -CUDART_INF_F;
         for (int r = 0; r < p.shard_world; ++r) lx = fmaxf(lx, p.lx_all[static_cast<size_t>(r) * p.rec_stride + b * k + j]);
       } else {
-        lx = p.logits[static_cast<size_t>(row_first + j) * p.ldl + x];
+        lx = p.logits[static_cast<size_t>(row_first + j) * p.ldl + x_mine];
       }
     }
-    sh_lx[j] = lx; sh_qx[j] = qx;
-    float hq = 0.f;
     if (p.gate_source == HOLA_GATE_DRAFT_ENTROPY) {
       double tot = 0.0;
       for (int sl = 0; sl < kHqSlices; ++sl) tot += p.hq_part[(static_cast<size_t>(b) * k + j) * kHqSlices + sl];
       hq = fmaxf(0.f, static_cast<float>(-tot));
       if (rank == 0 && p.draft_entropy) p.draft_entropy[b * k + j] = hq;
     }
-    sh_Hq[j] = hq;
   }
   // ---- softmax statistics of this sequence's k+1 positions
+  bool rows_pending = staged;                            // this warp has not asked for its part of the staged rows yet
   if (p.combine) {
     // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
     // above, gets a row only when there are more than seven)
     for (int j = kK3Warps - 1 - warp; j <= k; j += kK3Warps) {
-      Stats st = warp_merge_partials(p.partials, p.nparts, p.part_stride, row_first + j, lane);
+      Stats st = warp_merge_partials(p.partials, p.nparts, p.part_stride, row_first + j, lane, [&] {
+        if (rows_pending) { stage_rows(); rows_pending = false; }
+      });
       if (lane == 0) {
         float lz, h;
         stats_to_outputs(st, &lz, &h);
@@ -1756,53 +1829,63 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       sh_H[j] = p.entropy[row_first + j];
     }
   }
-  __syncthreads();
-
-  // ---- gate and ratio test in draft order; stop at the first position that is not accepted
-  if (threadIdx.x == 0) {
-    unsigned flags = 0;
-    int n = k;
-    for (int j = 0; j < k; ++j) {
-      const int x = sh_x[j];
-      if (x < 0 || x >= Vtok) { flags |= HOLA_FLAG_BAD_TOKEN; n = j; break; }
-      const float gate_value = p.gate_source == HOLA_GATE_DRAFT_ENTROPY ? sh_Hq[j] : sh_H[j];
-      if (gate_value < p.tau) continue;                  // entropy gate: fast path keeps the draft token
-      if (p.fallback == HOLA_FALLBACK_GREEDY) {          // the verifier's own token, or the run ends here
-        if (x != sh_amax[j]) { n = j; break; }
-        continue;
-      }
-      const float u = clamp_uniform(sh_u[j], flags);
-      const float px = expf(sh_lx[j] - sh_logZ[j]);
-      const float qx = sh_qx[j];
-      const bool accept = (qx > 0.f) ? (u * qx < px) : (px > 0.f);
-      if (!accept) { n = j; break; }
-    }
-    sh_n = n;
-    sh_flags = flags;
-    if (rank == 0) {
-      p.accept_len[b] = n;
-      if (p.fallback == HOLA_FALLBACK_GREEDY) {          // greedy: argmax p_n follows the accepted run; no draw
-        p.next_tok[b] = min(max(sh_amax[n], 0), Vtok - 1);
-        if (flags && p.status) atomicOr(p.status, flags);
-      } else if (p.phase == 1 && flags && p.status) {
-        atomicOr(p.status, flags);
-      }
-    }
+  if (rows_pending) stage_rows();
+  if (j_mine <= k) sh_u[j_mine] = u_mine;
+  if (j_mine < k) {
+    sh_x[j_mine] = x_mine; sh_lx[j_mine] = lx; sh_Hq[j_mine] = hq;
+    sh_qx[j_mine] = __uint_as_float(!p.q_tok && p.q_dtype == HOLA_Q_BF16 ? q_bits << 16 : q_bits);
   }
   __syncthreads();
+
+  // ---- gate and ratio test in draft order; the first position that is not accepted ends the run.  A lane per position,
+  // in every warp (same inputs, same result: no second barrier); what a position past the end would flag does not count.
+  unsigned flags = 0;
+  int n = k;
+  for (int j0 = 0; j0 < k && n == k; j0 += 32) {
+    const int j = j0 + lane;
+    unsigned fl = 0;
+    bool stop = false;
+    if (j < k) {
+      const int x = sh_x[j];
+      const float gate_value = p.gate_source == HOLA_GATE_DRAFT_ENTROPY ? sh_Hq[j] : sh_H[j];
+      if (x < 0 || x >= Vtok) {
+        fl = HOLA_FLAG_BAD_TOKEN;
+        stop = true;
+      } else if (gate_value < p.tau) {                   // entropy gate: fast path keeps the draft token
+      } else if (p.fallback == HOLA_FALLBACK_GREEDY) {   // the verifier's own token, or the run ends here
+        stop = x != sh_amax[j];
+      } else {
+        const float u = clamp_uniform(sh_u[j], fl);
+        const float px = expf(sh_lx[j] - sh_logZ[j]);
+        const float qx = sh_qx[j];
+        stop = !((qx > 0.f) ? (u * qx < px) : (px > 0.f));
+      }
+    }
+    const unsigned stops = __ballot_sync(0xffffffffu, stop);
+    if (stops) n = j0 + __ffs(stops) - 1;
+    flags |= __reduce_or_sync(0xffffffffu, j <= n ? fl : 0u);
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    p.accept_len[b] = n;
+    if (p.fallback == HOLA_FALLBACK_GREEDY) {            // greedy: argmax p_n follows the accepted run; no draw
+      p.next_tok[b] = min(max(sh_amax[n], 0), Vtok - 1);
+      if (flags && p.status) atomicOr(p.status, flags);
+    } else if (p.phase == 1 && flags && p.status) {
+      atomicOr(p.status, flags);
+    }
+  }
   if (p.fallback == HOLA_FALLBACK_GREEDY || p.phase == 1) return;   // same decision in every CTA of the cluster
 
   // ---- this CTA's slice of row n: per-chunk residual mass
-  const int n = sh_n;
   const float logZ = sh_logZ[n];
-  const float* lrow = p.logits + static_cast<size_t>(row_first + n) * p.ldl;
-  const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
   const char* qbase = static_cast<const char*>((p.q_far && n >= p.q_far_from) ? p.q_far : p.q);
-  const void* qrow = (n < k) ? static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem) : nullptr;
-  const int nchunks = (V + kChunk - 1) / kChunk;
-  const int cpc = (nchunks + S - 1) / S;                 // chunks per CTA
-  const int c_first = rank * cpc;
-  const int mine = max(0, min(nchunks, c_first + cpc) - c_first);
+  // (staged: the row as if the slice were the whole of it, entry v at row + v)
+  const float* lrow = staged ? sl + static_cast<size_t>(n) * slice - c_first * kChunk
+                             : p.logits + static_cast<size_t>(row_first + n) * p.ldl;
+  const void* qrow = n >= k ? nullptr
+                   : staged ? static_cast<const void*>(sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem)
+                            : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
+  if (staged) cp_async_wait_all();
   const int per_lane = (mine + 31) / 32;
   bool residual = n < k;
 
@@ -1817,7 +1900,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
     const bool use_p = !residual || !(tot_res > 0.0);
     if (use_p && residual) {
       residual = false;
-      if (threadIdx.x == 0) sh_flags |= HOLA_FLAG_R_ZERO;
+      flags |= HOLA_FLAG_R_ZERO;
     }
     const int idx = use_p ? 1 : 0;
     double total = 0.0;
@@ -1882,16 +1965,21 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       if (lane < S) *cluster.map_shared_rank(&sh_tot[attempt][rank], lane) = slice_total;
     }
     cluster.sync();
-    // every CTA: total mass and the slice that holds u * R (identical arithmetic everywhere)
-    double R = 0.0;
-    for (int r2 = 0; r2 < S; ++r2) R += sh_tot[attempt][r2];
+    // every warp of every CTA: total mass and the slice that holds u * R (identical arithmetic everywhere); lane r has slice r
+    const double slice_mass = lane < S ? sh_tot[attempt][lane] : 0.0;
+    double slice_incl = slice_mass;
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) {
+      const double o = __shfl_up_sync(0xffffffffu, slice_incl, off);
+      if (lane >= off) slice_incl += o;
+    }
+    const double R = __shfl_sync(0xffffffffu, slice_incl, 7);
     if (shard && p.phase == 3) {
       // the shard's masses of row n: of the residual, then (second pass, q taken as 0) of p itself
       if (rank == 0 && threadIdx.x == 0) {
         p.mass_out[b * 2 + attempt] = R;
         if (!residual && attempt == 0) p.mass_out[b * 2 + 1] = R;          // bonus position: both are the mass of p
-        const unsigned fl = sh_flags;
-        if (fl && p.status && (attempt == 1 || !residual)) atomicOr(p.status, fl);
+        if (flags && p.status && (attempt == 1 || !residual)) atomicOr(p.status, flags);
       }
       if (residual) {
         residual = false;
@@ -1902,29 +1990,18 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
     }
     if (!(R > 0.0) && residual && !shard) {              // p <= q everywhere: draw from p instead
       residual = false;
-      if (threadIdx.x == 0) sh_flags |= HOLA_FLAG_R_ZERO;
+      flags |= HOLA_FLAG_R_ZERO;
       __syncthreads();
       continue;
     }
-    unsigned uflags = 0;
-    const float uk = clamp_uniform(sh_u[k], uflags);
+    const float uk = clamp_uniform(sh_u[k], flags);
     const double target = shard ? shard_target : static_cast<double>(uk) * R;
-    int rstar = -1, last_mass = 0;
-    double before_slice = 0.0;
-    {
-      double cum = 0.0;
-      for (int r2 = 0; r2 < S; ++r2) {
-        const double t = sh_tot[attempt][r2];
-        if (t > 0.0) last_mass = r2;
-        if (rstar < 0 && cum + t > target) { rstar = r2; before_slice = cum; }
-        cum += t;
-      }
-    }
-    bool take_last = false;
-    if (rstar < 0) {                                     // rounding left the running sum a hair below u*R
-      rstar = last_mass;
-      take_last = true;
-    }
+    const unsigned slice_over = __ballot_sync(0xffffffffu, lane < S && slice_incl > target);
+    const unsigned slice_has = __ballot_sync(0xffffffffu, slice_mass > 0.0);
+    const bool take_last_slice = slice_over == 0u;       // rounding left the running sum a hair below u*R
+    const int rstar = slice_over ? __ffs(slice_over) - 1 : (slice_has ? 31 - __clz(slice_has) : 0);
+    const double before_slice = __shfl_sync(0xffffffffu, slice_incl - slice_mass, rstar);
+    bool take_last = take_last_slice;
     if (rank == rstar && warp == 0) {
       const unsigned over = __ballot_sync(0xffffffffu, before_slice + incl > target);
       const unsigned has_mass = __ballot_sync(0xffffffffu, tot > 0.0);
@@ -1974,8 +2051,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
         int tokn = (c_first + cstar) * kChunk + src * 4 + idx;
         if (tokn >= V) tokn = V - 1;
         p.next_tok[b] = tokn + (shard ? p.v_offset : 0);
-        const unsigned fl = sh_flags | uflags;
-        if (fl && p.status) atomicOr(p.status, fl);
+        if (flags && p.status) atomicOr(p.status, flags);
       }
     }
     break;
@@ -2645,8 +2721,9 @@ int sample_cluster(const hola_ctx* ctx, int B, int V) {
 
 // Steps 1-2: the LM-head GEMM with fused statistics, one launch (clusters of two CTAs) per pass over W_lm.
 // `few_before`: the kernel in front is expected to be this context's accept/sample kernel on a few SMs.
+// `next_reads_inputs`: the accept/sample kernel of the same arguments is launched right behind this.
 hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits, int ldl, const Plan& pl,
-                        cudaStream_t stream, bool few_before = false) {
+                        cudaStream_t stream, bool few_before = false, bool next_reads_inputs = false) {
   const int M = a->B * (a->k + 1);
   const bool mixed = a->w_dtype == HOLA_W_MIXED;
   const bool w8 = a->w_dtype == HOLA_W_INT8 || mixed, two = a->w_dtype == HOLA_W8A16,
@@ -2778,6 +2855,15 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   // that kernel leaves nearly all SMs to this one's CTAs.  V = 32000, H = 4096, one sequence, none / 16 / 32 / 48 MB: bf16
   // 52.2 / 50.9 / 50.0 / 49.7 us, mixed widths 43.9 / 42.2 / 42.6 / 43.2, 8-bit 37.2 / 36.3 / 36.5 / 36.8; with 16
   // sequences (128 CTAs of the accept/sample kernel in the way) 61.6 / 61.5 / 62.5 / 63.3, hence the limit.
+  kp.next_tok = nullptr; kp.next_u = nullptr; kp.next_q = nullptr;
+  kp.next_n = kp.next_q_elem = 0; kp.next_q_bytes = 0;
+  if (next_reads_inputs && a->k > 0 && a->draft_tok && a->draft_q && a->uniforms) {
+    kp.next_tok = a->draft_tok; kp.next_u = a->uniforms; kp.next_q = static_cast<const char*>(a->draft_q);
+    kp.next_n = a->B * a->k; kp.next_q_elem = a->q_dtype == HOLA_Q_BF16 ? 2 : 4;
+    const double q_bytes = static_cast<double>(kp.next_n) * a->V * kp.next_q_elem;
+    if (q_bytes <= 2e6 && aligned16(a->draft_q) && a->fallback != HOLA_FALLBACK_GREEDY)
+      kp.next_q_bytes = static_cast<unsigned>(q_bytes) & ~15u;
+  }
   kp.prefetch_blocks = 0;
   if (few_before) {
     const int per_tile = w8 ? (pl.n_kblocks + 1) / 2 : pl.n_kblocks - pl.k_tail;
@@ -2868,6 +2954,17 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   cfg.gridDim = dim3(static_cast<unsigned>(a->B * S));
   cfg.blockDim = dim3(kK3Threads);
   cfg.dynamicSmemBytes = static_cast<size_t>(cpc) * sizeof(double);
+  // Small batches (a CTA per SM at most, and no more than 4 MB of rows in all): row n would be asked for only after the
+  // statistics and the accept test, so the slices of all rows are asked for before them.
+  kp.staged = 0;
+  if (vec && (phase == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && a->B * S <= ctx->num_sms) {
+    const size_t row_bytes = static_cast<size_t>(a->k + 1) * 4 + static_cast<size_t>(a->k) * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
+    const size_t bytes = row_bytes * cpc * kChunk + sizeof(double);     // (and the rows start on a 16-byte boundary)
+    if (bytes + cfg.dynamicSmemBytes <= kK3MaxDynSmem && row_bytes * a->V * a->B <= 4u << 20) {
+      kp.staged = 1;
+      cfg.dynamicSmemBytes += bytes;
+    }
+  }
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2930,6 +3027,8 @@ cudaError_t configure_kernels() {
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<3, false>)};
   for (const void* k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(accept_sample_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kK3MaxDynSmem);
   return e;
 }
 
@@ -3194,7 +3293,7 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   const bool side = draft_gate && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
   const bool few_before = a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
-  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before);
+  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, true);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
   if (side) {
