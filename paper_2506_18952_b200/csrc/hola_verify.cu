@@ -705,8 +705,7 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
 //   on-chip expansion only: rawfull[12] @272 per CTA: the codes of the slot have landed (full[] then counts the hidden
 //   bytes and, for 16-bit rows, their bytes); operand[8] @368 leader's copy: the eight converter warps of the pair that
 //   own a K block have put it into tensor memory.
-// After the barrier area: one 2 KB transposition buffer per epilogue warp (reused for the final merge of the
-// statistics of the four tensor-memory lane quarters).
+// After the barrier area: one 2 KB transposition buffer per epilogue warp.
 // kMode 3 is kMode 2 with every verify row present twice in the hidden operand (coarse 8-bit plane and the plane of
 // its remainder, in alternating blocks of 32 rows): the epilogue adds the two int32 sums with their scales.
 // kMode: 0 bf16 x bf16; 1 int8 W_lm expanded to bf16 on chip (exact); 2 int8 W_lm x int8 hidden on the 8-bit MMA
@@ -1348,30 +1347,24 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         }
       }
     }
-    // ---- the CTA's statistics of every row: first the two halves of a quarter (lanes L and L ^ 16), then, after
-    // all epilogue warps are done with their buffers, the quarters side by side in shared memory
-    asm volatile("bar.sync 1, %0;" ::"n"(kNumEpi * 32) : "memory");
-    float4* merge = reinterpret_cast<float4*>(trans_base);          // [4 quarters][rows of the pass]
+    // ---- the CTA's statistics of every row: the eight contributions (lane quarter, half) side by side where the ring was
+    // (this warp has seen the last tile's MMAs complete, so every slot has been filled and read for the last time)
+    float4* merge = reinterpret_cast<float4*>(smem);                // [8][rows of the pass]
 #pragma unroll
     for (int slot = 0; slot < kSlots; ++slot) {
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        Stats a = st[slot][half], o;
-        o.m = __shfl_xor_sync(0xffffffffu, a.m, 16);
-        o.s = __shfl_xor_sync(0xffffffffu, a.s, 16);
-        o.t = __shfl_xor_sync(0xffffffffu, a.t, 16);
-        o.arg = __shfl_xor_sync(0xffffffffu, a.arg, 16);
-        a = stats_merge(a, o);
+        const Stats a = st[slot][half];
+        const float4 x = make_float4(a.m, a.s, a.t, __int_as_float(a.arg));
         if (kTwoPlane) {
           const int r = 32 * (group + slot * kGroups) + half * kTransRows + trow;   // row inside the pass
-          if (slot < 2 && thalf == 0 && r < rows)
-            merge[quarter * rows + r] = make_float4(a.m, a.s, a.t, __int_as_float(a.arg));
-        } else if (slot < my_chunks && thalf == 0) {
+          if (slot < 2 && r < rows) merge[(quarter * 2 + thalf) * rows + r] = x;
+        } else if (slot < my_chunks) {
           const int ch = rot ? slot * sub_chunks + group : group + slot * kGroups;
           const int sub = ch / sub_chunks, j = ch - sub * sub_chunks;
           const int c = j * 32 + half * kTransRows + trow;           // column inside its MMA
           const int r = sub * p.N + c;                               // row inside the pass
-          if (c < p.N && r < rows) merge[quarter * rows + r] = make_float4(a.m, a.s, a.t, __int_as_float(a.arg));
+          if (c < p.N && r < rows) merge[(quarter * 2 + thalf) * rows + r] = x;
         }
       }
     }
@@ -1478,17 +1471,28 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   __syncthreads();
   grid_dependency_wait();                                // (every thread that writes below; long since satisfied)
   if (!*abort_flag) {
-    // one partial per CTA and row: the four quarters merged
-    const float4* merge = reinterpret_cast<const float4*>(trans_base);
+    // one partial per CTA and row: the eight contributions merged around their maximum
+    const float4* merge = reinterpret_cast<const float4*>(smem);
     for (int r = threadIdx.x; r < rows; r += kK1Threads) {
-      Stats a = stats_empty();
+      float4 x[8];
+      float m = -CUDART_INF_F, sum = 0.f, sum_t = 0.f;
+      int arg = 0x7fffffff;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 x = merge[q * rows + r];
-        a = stats_merge(a, Stats{x.x, x.y, x.z, __float_as_int(x.w)});
+      for (int q = 0; q < 8; ++q) {
+        x[q] = merge[q * rows + r];
+        m = fmaxf(m, x[q].x);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (x[q].x == m) arg = min(arg, __float_as_int(x[q].w));
+        if (x[q].x != -CUDART_INF_F) {
+          const float d = x[q].x - m, e = __expf(d);
+          sum = fmaf(e, x[q].y, sum);
+          sum_t = fmaf(e, fmaf(d, x[q].y, x[q].z), sum_t);
+        }
       }
       p.partials[static_cast<size_t>(blockIdx.x) * p.part_stride + row0 + r] =
-          make_float4(a.m, a.s, a.t, __int_as_float(a.arg));
+          make_float4(m, sum, sum_t, __int_as_float(arg));
     }
     if (p.n_pass > 1) {
       // the accept/sample kernel merges the partials of every CTA for every row: this CTA has seen only its pass
