@@ -263,30 +263,50 @@ class _FreshOutputs(VerifyOutputs):
     much as a fifth of a call), the others when somebody asks for them.  The status word is cleared by the call
     (HOLA_ARG_CLEAR_STATUS); an empty batch launches nothing."""
 
-    def __init__(self, ctx: "HolaVerify", B: int, k: int, want_logits: bool, draws: bool, draft_gate: bool):
+    def __init__(self, ctx: "HolaVerify", B: int, k1: int, want_logits: bool, draws: bool, draft_gate: bool):
         dev = self._dev = ctx._dev
-        self._B, self._k = B, k
-        self.entropy = torch.empty((B, k + 1), dtype=torch.float32, device=dev)
-        self.logZ = torch.empty((B, k + 1), dtype=torch.float32, device=dev)
-        self.logits = torch.empty((B, k + 1, ctx.V), dtype=torch.float32, device=dev) if want_logits else None
+        self._B, self._k = B, k1 - 1
+        # (sizes one by one and empty_like: the cheapest forms, 1.7 and 1.3 us against 2.4 with a tuple)
+        self.entropy = e = torch.empty(B, k1, dtype=torch.float32, device=dev)
+        self.logZ = torch.empty_like(e)
+        self.logits = torch.empty(B, k1, ctx.V, dtype=torch.float32, device=dev) if want_logits else None
         self.status = (torch.empty if B else torch.zeros)(1, dtype=torch.int32, device=dev)
-        self._lazy = {"draft_entropy": torch.empty((B, k), dtype=torch.float32, device=dev)} if draft_gate else {}
+        self._accept_len = self._next_tok = self._draft_entropy = None
         if draws:
-            self._lazy["accept_len"] = torch.empty(B, dtype=torch.int32, device=dev)
-            self._lazy["next_tok"] = torch.empty(B, dtype=torch.int32, device=dev)
+            self._accept_len = a = torch.empty(B, dtype=torch.int32, device=dev)
+            self._next_tok = torch.empty_like(a)
+        if draft_gate:
+            self._draft_entropy = torch.empty(B, k1 - 1, dtype=torch.float32, device=dev)
 
-    def _get(self, name, make):
-        t = self._lazy.get(name)
-        if t is None:
-            t = self._lazy[name] = make()
-        return t
+    @property
+    def accept_len(self):
+        if self._accept_len is None:
+            self._accept_len = torch.empty(self._B, dtype=torch.int32, device=self._dev)
+        return self._accept_len
 
-    accept_len = property(lambda self: self._get("accept_len", lambda: torch.empty(self._B, dtype=torch.int32, device=self._dev)),
-                          lambda self, t: self._lazy.__setitem__("accept_len", t))
-    next_tok = property(lambda self: self._get("next_tok", lambda: torch.empty(self._B, dtype=torch.int32, device=self._dev)),
-                        lambda self, t: self._lazy.__setitem__("next_tok", t))
-    draft_entropy = property(lambda self: self._get("draft_entropy", lambda: torch.zeros((self._B, self._k), device=self._dev)),
-                             lambda self, t: self._lazy.__setitem__("draft_entropy", t))
+    @accept_len.setter
+    def accept_len(self, t):
+        self._accept_len = t
+
+    @property
+    def next_tok(self):
+        if self._next_tok is None:
+            self._next_tok = torch.empty(self._B, dtype=torch.int32, device=self._dev)
+        return self._next_tok
+
+    @next_tok.setter
+    def next_tok(self, t):
+        self._next_tok = t
+
+    @property
+    def draft_entropy(self):
+        if self._draft_entropy is None:
+            self._draft_entropy = torch.zeros(self._B, self._k, dtype=torch.float32, device=self._dev)
+        return self._draft_entropy
+
+    @draft_entropy.setter
+    def draft_entropy(self, t):
+        self._draft_entropy = t
 
 
 class HolaVerify:
@@ -438,7 +458,7 @@ class HolaVerify:
         B, k1 = hidden.shape[:2]
         fresh = not out
         if fresh:
-            out = _FreshOutputs(self, B, k1 - 1, want_logits, True, gate_source == HOLA_GATE_DRAFT_ENTROPY)
+            out = _FreshOutputs(self, B, k1, want_logits, True, gate_source == HOLA_GATE_DRAFT_ENTROPY)
         a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k1 - 1, gate_source, fallback, w_scale, a8)
         if fresh:
             a.flags = HOLA_ARG_CLEAR_STATUS
@@ -452,7 +472,7 @@ class HolaVerify:
         B, k1 = hidden.shape[:2]
         fresh = not out
         if fresh:
-            out = _FreshOutputs(self, B, k1 - 1, want_logits, False, False)
+            out = _FreshOutputs(self, B, k1, want_logits, False, False)
         a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k1 - 1, w_scale=w_scale, a8=a8, draws=False)
         if fresh:
             a.flags = HOLA_ARG_CLEAR_STATUS
