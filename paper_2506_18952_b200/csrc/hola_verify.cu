@@ -1551,12 +1551,11 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_selftest_kernel(long long 
 
 // ------------------------------------------------------------------------------------------------ K2
 // The statistics of one row over all CTAs, by a warp, the same bits in every lane.  Six loads per lane in flight (192
-// partials per round: one round on a 148-SM part); `while_loading` runs behind their issue.  The maximum first, so that the
+// partials per round: one round on a 148-SM part).  The maximum first, so that the
 // exponentials of the partials are independent of one another and only additions remain to be passed round: five
 // shuffles for the maximum and five for the sums instead of eleven merges of a hundred cycles each.
-template <typename F>
 __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int part_stride, int row,
-                                                     int lane, F while_loading) {
+                                                     int lane) {
   Stats st = stats_empty();
   for (int base = 0; base < nparts; base += 192) {
     float4 x[6];
@@ -1566,7 +1565,6 @@ __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int
       x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride + row]
                         : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
     }
-    if (base == 0) while_loading();
     float m = fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -1606,7 +1604,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, i
   const int lane = threadIdx.x & 31;
   grid_dependency_wait();
   if (row >= M) return;
-  Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane, [] {});
+  Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
   if (lane == 0) stats_to_outputs(st, &logZ[row], &entropy[row]);
 }
 
@@ -1622,7 +1620,7 @@ __global__ void __launch_bounds__(256) shard_record_kernel(const float4* partial
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
-    Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane, [] {});
+    Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
     if (lane == 0) {
       const int arg = st.arg == 0x7fffffff ? st.arg : st.arg + v_offset;
       stats_out[row] = make_float4(st.m, st.s, st.t, __int_as_float(arg));
@@ -1708,12 +1706,15 @@ __device__ __forceinline__ void load_r4(const float* lrow, const void* qrow, int
   resid4(l, q, logZ, r);
 }
 
-// Copies into shared memory that nobody waits for yet (cp_async_wait_all: this thread's have landed).
-template <int kBytes>
-__device__ __forceinline__ void cp_async(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(kBytes) : "memory");
+// Untiled bulk copy into this CTA's shared memory (addresses and size multiples of 16 bytes), counted on an mbarrier.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 
 __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
   if (!(u >= 0.f)) { flags |= HOLA_FLAG_BAD_UNIFORM; return 0.f; }
@@ -1731,6 +1732,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   __shared__ double sh_tot[2][8];                        // slice totals of the whole cluster, per attempt
   __shared__ float sh_logZ[kMaxK1], sh_H[kMaxK1], sh_lx[kMaxK1], sh_qx[kMaxK1], sh_u[kMaxK1], sh_Hq[kMaxK1];
   __shared__ int sh_x[kMaxK1], sh_amax[kMaxK1];
+  __shared__ __align__(8) uint64_t sh_bar;               // staged rows have landed
 
   // The next kernel in the stream (normally the next call's GEMM kernel, which waits for this grid before it touches
   // memory) may be scheduled from now on: its launch and prologue then hide behind this kernel.
@@ -1763,30 +1765,24 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const int c_first = rank * cpc;
   const int mine = max(0, min(nchunks, c_first + cpc) - c_first);
   const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
-  // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities.  A lane copies
-  // what it will read in the pass: chunk c of every row goes through warp c % kK3Warps.
+  // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities, each row's
+  // slice by one bulk copy that a thread of the last warp (the first to have nothing else to wait for) starts.
   const bool staged = kVec && p.staged;
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
   char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
-  auto stage_rows = [&]() {
-    for (int c = warp; c < mine; c += kK3Warps) {
-      const int at = c * kChunk + lane * 4, v = c_first * kChunk + at;        // (V % 4 == 0: all four or none)
-      if (v >= V) continue;
-      float* dl = sl + at;
-      const float* l = p.logits + static_cast<size_t>(row_first) * p.ldl + v;
-      for (int j = 0; j <= k; ++j, dl += slice, l += p.ldl) cp_async<16>(dl, l);
-      if (p.q_dtype == HOLA_Q_BF16) {
-        char* dq = sq + at * 2;
-        const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + v) * 2;
-        for (int j = 0; j < k; ++j, dq += slice * 2, q += static_cast<size_t>(V) * 2) cp_async<8>(dq, q);
-      } else {
-        char* dq = sq + at * 4;
-        const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + v) * 4;
-        for (int j = 0; j < k; ++j, dq += slice * 4, q += static_cast<size_t>(V) * 4) cp_async<16>(dq, q);
-      }
-    }
-  };
+  const int here = min(V - c_first * kChunk, mine * kChunk);           // entries of this slice (0 or less: none)
+  if (staged && warp == kK3Warps - 1 && elect_one() && here > 0) {
+    const uint32_t bar = smem_u32(&sh_bar), lbytes = here * 4u, qbytes = static_cast<uint32_t>(here * q_elem);
+    mbar_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    mbar_expect_tx(bar, (k + 1) * lbytes + k * qbytes);
+    const float* l = p.logits + static_cast<size_t>(row_first) * p.ldl + c_first * kChunk;
+    for (int j = 0; j <= k; ++j, l += p.ldl) bulk_load(smem_u32(sl + static_cast<size_t>(j) * slice), l, lbytes, bar);
+    const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + c_first * kChunk) * q_elem;
+    for (int j = 0; j < k; ++j, q += V * q_elem) bulk_load(smem_u32(sq + static_cast<size_t>(j) * slice * q_elem), q, qbytes, bar);
+  }
+  __syncwarp();
   // the draft token's logit and probability
   float lx = 0.f, hq = 0.f;
   uint32_t q_bits = 0;                                   // (as loaded: converted when it is stored)
@@ -1812,14 +1808,11 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
     }
   }
   // ---- softmax statistics of this sequence's k+1 positions
-  bool rows_pending = staged;                            // this warp has not asked for its part of the staged rows yet
   if (p.combine) {
     // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
     // above, gets a row only when there are more than seven)
     for (int j = kK3Warps - 1 - warp; j <= k; j += kK3Warps) {
-      Stats st = warp_merge_partials(p.partials, p.nparts, p.part_stride, row_first + j, lane, [&] {
-        if (rows_pending) { stage_rows(); rows_pending = false; }
-      });
+      Stats st = warp_merge_partials(p.partials, p.nparts, p.part_stride, row_first + j, lane);
       if (lane == 0) {
         float lz, h;
         stats_to_outputs(st, &lz, &h);
@@ -1833,7 +1826,6 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       sh_H[j] = p.entropy[row_first + j];
     }
   }
-  if (rows_pending) stage_rows();
   if (j_mine <= k) sh_u[j_mine] = u_mine;
   if (j_mine < k) {
     sh_x[j_mine] = x_mine; sh_lx[j_mine] = lx; sh_Hq[j_mine] = hq;
@@ -1889,7 +1881,15 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const void* qrow = n >= k ? nullptr
                    : staged ? static_cast<const void*>(sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem)
                             : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
-  if (staged) cp_async_wait_all();
+  if (staged && here > 0) {                              // (bounded, and only this CTA's own copies to wait for)
+    const long long t0 = clock64();
+    while (!mbar_try_wait(smem_u32(&sh_bar), 0u)) {
+      if (clock64() - t0 > kWaitLimitCycles) {
+        flags |= HOLA_FLAG_TIMEOUT;
+        break;
+      }
+    }
+  }
   const int per_lane = (mine + 31) / 32;
   bool residual = n < k;
 
@@ -2959,9 +2959,10 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   cfg.blockDim = dim3(kK3Threads);
   cfg.dynamicSmemBytes = static_cast<size_t>(cpc) * sizeof(double);
   // Small batches (a CTA per SM at most, and no more than 4 MB of rows in all): row n would be asked for only after the
-  // statistics and the accept test, so the slices of all rows are asked for before them.
+  // statistics and the accept test, so the slices of all rows are asked for before them (bulk copies: rows of whole
+  // 16-byte pieces).
   kp.staged = 0;
-  if (vec && (phase == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && a->B * S <= ctx->num_sms) {
+  if (vec && phase == 0 && (a->q_dtype == HOLA_Q_F32 || a->V % 8 == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && a->B * S <= ctx->num_sms) {
     const size_t row_bytes = static_cast<size_t>(a->k + 1) * 4 + static_cast<size_t>(a->k) * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
     const size_t bytes = row_bytes * cpc * kChunk + sizeof(double);     // (and the rows start on a 16-byte boundary)
     if (bytes + cfg.dynamicSmemBytes <= kK3MaxDynSmem && row_bytes * a->V * a->B <= 4u << 20) {
