@@ -3354,6 +3354,9 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
     if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, stream);
     down += bytes;
   };
+  // The hidden rows first and with the bus to themselves: the GEMM waits for them, while the draft rows have until its end.
+  // The host gathers the k probabilities per sequence (a cache miss each) while they travel.
+  h2d(ctx->st_hidden, a->hidden, rows * a->H * 2, stream);
   for (int b = 0; b < B; ++b)
     for (int j = 0; j < k; ++j) {
       const int x = a->draft_tok[b * k + j];
@@ -3369,7 +3372,6 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
       }
       ctx->h_qtok[b * k + j] = qx;
     }
-  h2d(ctx->st_hidden, a->hidden, rows * a->H * 2, stream);
   // tokens, uniforms and the gathered probabilities: into the pinned mirror, then one copy of the span in use
   memcpy(ctx->h_small, a->draft_tok, static_cast<size_t>(B) * k * 4);
   memcpy(ctx->h_small + ctx->small_u_off, a->uniforms, rows * 4);
@@ -3379,6 +3381,8 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
   ahead = ahead < 1 ? 1 : (ahead > k ? k : ahead);
   const size_t ahead_bytes = static_cast<size_t>(ahead) * row_bytes;     // rows 0 .. ahead-1 of a sequence are adjacent
   if (sample) {
+    if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_point, stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
     if (seq_pitch < (1ull << 31)) {
       if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(ctx->st_q, seq_pitch, a->draft_q, seq_pitch, ahead_bytes, static_cast<size_t>(B),
@@ -3547,6 +3551,12 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   const size_t q_bytes = static_cast<size_t>(a->B) * a->k * a->V * q_elem;
   const bool overlap = q_bytes && ctx->host_overlap;
   if (overlap) {
+    // Behind the inputs that the GEMM waits for, unless the draft entropy gates: its pass over the whole tensor then takes
+    // longer than the GEMM (16 sequences, V = 32000: 153 us with the tensor on the bus from the start, 166 behind).
+    if (a->gate_source == HOLA_GATE_TARGET_ENTROPY) {
+      if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_point, stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->st_q, a->draft_q, q_bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_done, ctx->copy_stream);
     up += q_bytes;
