@@ -187,6 +187,8 @@ struct K3Params {
   float* entropy;
   float* logZ;
   unsigned* status;
+  unsigned* flags_out;      // optional [B], in host memory: every sequence's flags, with what is in the status word, by plain
+                            // stores instead of OR-ing them into the status word
 };
 
 // ------------------------------------------------------------------------------------------------ PTX wrappers
@@ -1716,6 +1718,11 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 
+__device__ __forceinline__ void report_flags(const K3Params& p, int b, unsigned flags) {
+  if (p.flags_out) p.flags_out[b] = flags | (p.status ? *reinterpret_cast<volatile unsigned*>(p.status) : 0u);
+  else if (flags && p.status) atomicOr(p.status, flags);
+}
+
 __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
   if (!(u >= 0.f)) { flags |= HOLA_FLAG_BAD_UNIFORM; return 0.f; }
   if (u >= 1.f) { flags |= HOLA_FLAG_BAD_UNIFORM; return 1.f - 5.9604645e-8f; }   // 1 - 2^-24
@@ -1865,9 +1872,9 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
     p.accept_len[b] = n;
     if (p.fallback == HOLA_FALLBACK_GREEDY) {            // greedy: argmax p_n follows the accepted run; no draw
       p.next_tok[b] = min(max(sh_amax[n], 0), Vtok - 1);
-      if (flags && p.status) atomicOr(p.status, flags);
-    } else if (p.phase == 1 && flags && p.status) {
-      atomicOr(p.status, flags);
+      report_flags(p, b, flags);
+    } else if (p.phase == 1) {
+      report_flags(p, b, flags);
     }
   }
   if (p.fallback == HOLA_FALLBACK_GREEDY || p.phase == 1) return;   // same decision in every CTA of the cluster
@@ -1983,7 +1990,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       if (rank == 0 && threadIdx.x == 0) {
         p.mass_out[b * 2 + attempt] = R;
         if (!residual && attempt == 0) p.mass_out[b * 2 + 1] = R;          // bonus position: both are the mass of p
-        if (flags && p.status && (attempt == 1 || !residual)) atomicOr(p.status, flags);
+        if (attempt == 1 || !residual) report_flags(p, b, flags);
       }
       if (residual) {
         residual = false;
@@ -2055,7 +2062,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
         int tokn = (c_first + cstar) * kChunk + src * 4 + idx;
         if (tokn >= V) tokn = V - 1;
         p.next_tok[b] = tokn + (shard ? p.v_offset : 0);
-        if (flags && p.status) atomicOr(p.status, flags);
+        report_flags(p, b, flags);
       }
     }
     break;
@@ -2493,7 +2500,9 @@ struct hola_ctx {
   // staging for hola_verify_host
   void* st_hidden; int* st_tok; void* st_q; float* st_u;
   unsigned char* st_out;      // device block of one call's outputs (status, accept_len, next_tok, entropy, logZ, ...)
-  unsigned char* h_out;       // pinned host mirror: the outputs come back in ONE copy
+  unsigned char* h_out;       // pinned host block of the same layout, and where the device sees it: the accept/sample
+  unsigned char* h_out_dev;   // kernel writes the outputs there itself, or they come back in ONE copy
+  unsigned* flags_out;        // K3Params::flags_out of the launch being prepared
   int force_stages;
   int no_rot;                 // tuning override: never use the rotating accumulator units
   int force_passes;           // tuning override: passes over W_lm (0: chosen by cost)
@@ -2528,7 +2537,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // Where one call's outputs sit inside the output block of hola_verify_host (16-byte aligned pieces, packed for the
 // call's own B and k so that one copy brings them all back).
 struct OutBlock {
-  size_t status, accept, next, entropy, logZ, dent, total;
+  size_t status, accept, next, entropy, logZ, dent, flags, total;
 };
 OutBlock out_block(int B, int k) {
   const size_t rows = static_cast<size_t>(B) * (k + 1);
@@ -2539,7 +2548,8 @@ OutBlock out_block(int B, int k) {
   o.entropy = o.next + align_up(static_cast<size_t>(B) * 4, 16);
   o.logZ = o.entropy + align_up(rows * 4, 16);
   o.dent = o.logZ + align_up(rows * 4, 16);
-  o.total = o.dent + align_up(static_cast<size_t>(B) * (k > 0 ? k : 1) * 4, 16);
+  o.flags = o.dent + align_up(static_cast<size_t>(B) * (k > 0 ? k : 1) * 4, 16);
+  o.total = o.flags + align_up(static_cast<size_t>(B) * 4, 16);
   return o;
 }
 
@@ -2943,6 +2953,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   }
   kp.accept_len = a->accept_len; kp.next_tok = a->next_tok; kp.entropy = a->entropy; kp.logZ = a->logZ;
   kp.status = a->status_word ? a->status_word : ctx->status;
+  kp.flags_out = ctx->flags_out;
   if (sh) {
     kp.shard_world = sh->world; kp.shard_rank = sh->rank; kp.v_offset = sh->v_offset; kp.V_global = sh->V_global;
     kp.lx_all = reinterpret_cast<const float*>(sh->stats_all) + 4 * static_cast<size_t>(a->B) * (a->k + 1);
@@ -3145,6 +3156,11 @@ hola_status hola_create(hola_ctx** out, int device, int maxB, int maxK, int H, i
   ctx->h_accept = reinterpret_cast<int*>(ctx->h_small + ctx->small_span);
   (void)n_qtok;
   ctx->h_out = reinterpret_cast<unsigned char*>(align_up(reinterpret_cast<size_t>(ctx->h_accept + maxB), 16));
+  void* pinned_dev = nullptr;
+  if (cudaHostGetDevicePointer(&pinned_dev, pinned, 0) == cudaSuccess)
+    ctx->h_out_dev = static_cast<unsigned char*>(pinned_dev) + (ctx->h_out - ctx->h_small);
+  else
+    cudaGetLastError();                                  // (outputs are copied then)
   *out = ctx;
   return HOLA_OK;
 }
@@ -3298,7 +3314,7 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   const bool side = draft_gate && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
   const bool few_before = a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
-  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, true);
+  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
   if (side) {
@@ -3338,6 +3354,26 @@ int rows_under_gemm(hola_ctx* ctx, const hola_verify_args* a) {
   return n > 1e6 ? 1000000 : static_cast<int>(n);
 }
 
+// Points a call's outputs into the pinned host block, where the accept/sample kernel can write them (a few KB, posted
+// writes: some 8 us less than a copy back behind the kernel).  The status word stays on the device, where kernels OR into
+// it; its bits and each sequence's flags come back as plain words (collect_flags).
+bool outputs_to_host(hola_ctx* ctx, hola_verify_args* d, const OutBlock& ob) {
+  if (!ctx->h_out_dev) return false;
+  d->accept_len = reinterpret_cast<int*>(ctx->h_out_dev + ob.accept);
+  d->next_tok = reinterpret_cast<int*>(ctx->h_out_dev + ob.next);
+  d->entropy = reinterpret_cast<float*>(ctx->h_out_dev + ob.entropy);
+  d->logZ = reinterpret_cast<float*>(ctx->h_out_dev + ob.logZ);
+  if (d->draft_entropy) d->draft_entropy = reinterpret_cast<float*>(ctx->h_out_dev + ob.dent);
+  ctx->flags_out = reinterpret_cast<unsigned*>(ctx->h_out_dev + ob.flags);
+  return true;
+}
+void collect_flags(hola_ctx* ctx, const OutBlock& ob, int B) {
+  const unsigned* f = reinterpret_cast<const unsigned*>(ctx->h_out + ob.flags);
+  unsigned all = 0;
+  for (int b = 0; b < B; ++b) all |= f[b];
+  memcpy(ctx->h_out + ob.status, &all, 4);
+}
+
 hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t stream, int ahead) {
   const int B = a->B, k = a->k, V = a->V;
   const size_t rows = static_cast<size_t>(B) * (k + 1);
@@ -3372,17 +3408,18 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
       }
       ctx->h_qtok[b * k + j] = qx;
     }
-  // tokens, uniforms and the gathered probabilities: into the pinned mirror, then one copy of the span in use
+  // tokens, uniforms and the gathered probabilities: into the pinned mirror, then one copy of the span in use.  Only the
+  // accept/sample part reads them: they travel with the draft rows, out of the GEMM's way.
   memcpy(ctx->h_small, a->draft_tok, static_cast<size_t>(B) * k * 4);
   memcpy(ctx->h_small + ctx->small_u_off, a->uniforms, rows * 4);
-  h2d(ctx->st_tok, ctx->h_small, ctx->small_qtok_off + static_cast<size_t>(B) * k * 4, stream);
+  if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_point, stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
+  h2d(ctx->st_tok, ctx->h_small, ctx->small_qtok_off + static_cast<size_t>(B) * k * 4, ctx->copy_stream);
   const OutBlock ob = out_block(B, k);
   const size_t seq_pitch = static_cast<size_t>(k) * row_bytes;   // from row (b, 0) to row (b + 1, 0)
   ahead = ahead < 1 ? 1 : (ahead > k ? k : ahead);
   const size_t ahead_bytes = static_cast<size_t>(ahead) * row_bytes;     // rows 0 .. ahead-1 of a sequence are adjacent
   if (sample) {
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_point, stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
     if (seq_pitch < (1ull << 31)) {
       if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(ctx->st_q, seq_pitch, a->draft_q, seq_pitch, ahead_bytes, static_cast<size_t>(B),
@@ -3393,8 +3430,8 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
         h2d(static_cast<char*>(ctx->st_q) + b * seq_pitch, static_cast<const char*>(a->draft_q) + b * seq_pitch,
             ahead_bytes, ctx->copy_stream);
     }
-    if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_done, ctx->copy_stream);
   }
+  if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_done, ctx->copy_stream);
   if (e != cudaSuccess) { set_error(ctx, "host-to-device copy", e); return HOLA_ERR_CUDA; }
   hola_verify_args d = *a;
   d.hidden = ctx->st_hidden; d.draft_tok = ctx->st_tok; d.draft_q = ctx->st_q; d.uniforms = ctx->st_u;
@@ -3419,15 +3456,18 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
     else
       cudaGetLastError();                                // (an unregistered pointer is not an error of this call)
   }
-  if (!sample) {
-    if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 0)) != HOLA_OK) return s;
-  } else if (q_far) {
+  bool direct = false;
+  if (!sample || q_far) {
+    // one accept/sample launch: it writes the outputs into the pinned block itself
     if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
-    if (e != cudaSuccess) { set_error(ctx, "wait for the draft rows sent ahead", e); return HOLA_ERR_CUDA; }
-    if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 0, nullptr, false, q_far,
-                               ahead)) != HOLA_OK)
-      return s;
+    if (e != cudaSuccess) { set_error(ctx, "wait for the inputs sent ahead", e); return HOLA_ERR_CUDA; }
+    direct = outputs_to_host(ctx, &d, ob);
+    s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 0, nullptr, false, q_far, ahead);
+    ctx->flags_out = nullptr;
+    if (s != HOLA_OK) return s;
   } else {
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
+    if (e != cudaSuccess) { set_error(ctx, "host-to-device copy of draft rows", e); return HOLA_ERR_CUDA; }
     if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 1)) != HOLA_OK) return s;
     d2h(ctx->h_accept, d.accept_len, static_cast<size_t>(B) * 4);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -3439,14 +3479,15 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
         h2d(static_cast<char*>(ctx->st_q) + off, static_cast<const char*>(a->draft_q) + off, row_bytes, stream);
       }
     }
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
     if (e != cudaSuccess) { set_error(ctx, "host-to-device copy of draft rows", e); return HOLA_ERR_CUDA; }
     // statistics and accept lengths are in place: this launch repeats the (cheap) accept test and draws the token
     if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 0, 0, stream, ctx->st_qtok, 0)) != HOLA_OK) return s;
   }
-  d2h(ctx->h_out, ctx->st_out, ob.dent);                 // every output in one copy
+  if (direct) down += ob.dent;
+  else d2h(ctx->h_out, ctx->st_out, ob.dent);            // every output in one copy
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-  if (e != cudaSuccess) { set_error(ctx, "device-to-host copy", e); return HOLA_ERR_CUDA; }
+  if (e != cudaSuccess) { set_error(ctx, "outputs to host", e); return HOLA_ERR_CUDA; }
+  if (direct) collect_flags(ctx, ob, B);
   memcpy(a->accept_len, ctx->h_out + ob.accept, static_cast<size_t>(B) * 4);
   memcpy(a->next_tok, ctx->h_out + ob.next, static_cast<size_t>(B) * 4);
   memcpy(a->entropy, ctx->h_out + ob.entropy, rows * 4);
@@ -3547,9 +3588,9 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   h2d(ctx->st_hidden, a->hidden, rows * a->H * 2);
   memcpy(ctx->h_small, a->draft_tok, static_cast<size_t>(a->B) * a->k * 4);
   memcpy(ctx->h_small + ctx->small_u_off, a->uniforms, rows * 4);
-  h2d(ctx->st_tok, ctx->h_small, ctx->small_u_off + rows * 4);
   const size_t q_bytes = static_cast<size_t>(a->B) * a->k * a->V * q_elem;
   const bool overlap = q_bytes && ctx->host_overlap;
+  const size_t small_bytes = ctx->small_u_off + rows * 4;
   if (overlap) {
     // Behind the inputs that the GEMM waits for, unless the draft entropy gates: its pass over the whole tensor then takes
     // longer than the GEMM (16 sequences, V = 32000: 153 us with the tensor on the bus from the start, 166 behind).
@@ -3557,10 +3598,13 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
       if (e == cudaSuccess) e = cudaEventRecord(ctx->fork_point, stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
     }
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(ctx->st_tok, ctx->h_small, small_bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->st_q, a->draft_q, q_bytes, cudaMemcpyHostToDevice, ctx->copy_stream);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->copy_done, ctx->copy_stream);
-    up += q_bytes;
+    up += small_bytes + q_bytes;
   } else {
+    h2d(ctx->st_tok, ctx->h_small, small_bytes);
     h2d(ctx->st_q, a->draft_q, q_bytes);
   }
   const OutBlock ob = out_block(a->B, a->k);
@@ -3576,9 +3620,14 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   const bool want_dent = a->draft_entropy && a->gate_source == HOLA_GATE_DRAFT_ENTROPY;
   d.draft_entropy = a->draft_entropy ? reinterpret_cast<float*>(ctx->st_out + ob.dent) : nullptr;
   if ((s = check_lm_head_args(ctx, &d)) != HOLA_OK) return s;
-  if ((s = verify_device(ctx, &d, stream, overlap ? ctx->copy_done : nullptr)) != HOLA_OK) return s;
-  d2h(ctx->h_out, ctx->st_out, want_dent ? ob.total : ob.dent);      // every output in one copy
+  const bool direct = outputs_to_host(ctx, &d, ob);
+  s = verify_device(ctx, &d, stream, overlap ? ctx->copy_done : nullptr);
+  ctx->flags_out = nullptr;
+  if (s != HOLA_OK) return s;
+  if (direct) down += want_dent ? ob.flags : ob.dent;
+  else d2h(ctx->h_out, ctx->st_out, want_dent ? ob.flags : ob.dent); // every output in one copy
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess && direct) collect_flags(ctx, ob, a->B);
   if (e != cudaSuccess) { set_error(ctx, "device-to-host copy", e); return HOLA_ERR_CUDA; }
   memcpy(a->accept_len, ctx->h_out + ob.accept, static_cast<size_t>(a->B) * 4);
   memcpy(a->next_tok, ctx->h_out + ob.next, static_cast<size_t>(a->B) * 4);
