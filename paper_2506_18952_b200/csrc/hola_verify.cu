@@ -70,15 +70,17 @@ constexpr int kTransBytes = kTransRows * 32 * 4; // its staging buffer: [16 rows
 // 8-bit and 4-bit W_lm, expanded on chip (mode 1): the codes of a K block land in the ring slot and converter warps
 // expand them, through registers, into the bf16 operand in TENSOR MEMORY that the MMA reads (64 columns hold the 128
 // channels of a K block, one lane per vocabulary row).  Warps 2..9 are epilogue warps, warps 10..17 convert: two groups
-// of four warps (one per quarter of the tensor-memory lanes) take the K blocks in turn.
+// of four warps (one per quarter of the tensor-memory lanes) take the K blocks in turn.  With at most 32 verify rows (one
+// chunk per lane quarter) four epilogue warps do, and there are three groups of converters: the chain of one block, some
+// 1600 cycles, then no longer bounds (whole step of one sequence, V = 32000, H = 4096: widths 20 / 70 / 10 % 39.3 -> 37.4 us).
 constexpr int kExpandK = 128;                     // channels per K block of 4- and 8-bit rows (16-bit rows: kBlockK)
 constexpr int kExpandMaxN = 192;                  // two accumulators of 192 columns leave 128 columns for the operand
 constexpr int kOperandCols = kExpandK / 2;        // tensor-memory columns of one K block of the expanded operand
 constexpr int kGroupRows = 256;                   // vocabulary rows per group of one width
 constexpr int kSubBlock = 128;                    // hidden channels per 4-bit sub-block (one shared exponent each)
-constexpr int kW8EpiWarps = 8;
+constexpr int kW8EpiWarps = 8, kW8FewEpiWarps = 4;
 constexpr int kConvGroup = 4;                     // converter warps per K block: one per tensor-memory lane quarter
-constexpr int kConvGroups = (kK1Warps - 2 - kW8EpiWarps) / kConvGroup;   // 2
+constexpr int kConvGroups = (kK1Warps - 2 - kW8EpiWarps) / kConvGroup, kConvGroupsFew = (kK1Warps - 2 - kW8FewEpiWarps) / kConvGroup;
 // What the expansion leaves in the operand is the code times a power of two (see expand_*); the epilogue takes it out
 // of the accumulators together with the row's scale.  Both are exact.
 constexpr float kExpandUnscale8 = 64.f, kExpandUnscale4 = 1024.f;
@@ -245,6 +247,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n .reg .pred P1;\n mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n selp.u32 %0, 1, 0, P1;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// One look, no waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred P1;\n mbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n selp.u32 %0, 1, 0, P1;\n}"
       : "=r"(ok)
       : "r"(bar), "r"(parity)
       : "memory");
@@ -704,9 +717,9 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
 //   tempty[4]  @208  leader's copy: all epilogue warps of the pair have read their accumulators (per buffer; per
 //                    128-column unit when the accumulators rotate)
 //   tensor-memory base @256, abort flag @260
-//   on-chip expansion only: rawfull[12] @272 per CTA: the codes of the slot have landed (full[] then counts the hidden
-//   bytes and, for 16-bit rows, their bytes); operand[8] @368 leader's copy: the eight converter warps of the pair that
-//   own a K block have put it into tensor memory.
+//   on-chip expansion only: rawfull[12] @272 per CTA: the codes of the slot have landed.  full[] then counts the hidden
+//   bytes (and, for 16-bit rows, their bytes) and one arrival per converter warp of the pair that owns the K block: the
+//   operand is in tensor memory.
 // After the barrier area: one 2 KB transposition buffer per epilogue warp.
 // kMode 3 is kMode 2 with every verify row present twice in the hidden operand (coarse 8-bit plane and the plane of
 // its remainder, in alternating blocks of 32 rows): the epilogue adds the two int32 sums with their scales.
@@ -714,7 +727,8 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
 // kind (K blocks of 128 elements, so that a block is 128 bytes per row exactly as in mode 0; int32 accumulators).
 // kRot: 257..384 rows per pass, three MMAs of N <= 128 per K step on rotating 128-column accumulator units (a
 // specialisation of its own because its epilogue holds a different set of values in registers).
-template <int kMode, bool kRot>
+// kFew (mode 1): at most 32 verify rows, four epilogue warps and three groups of converters.
+template <int kMode, bool kRot, bool kFew = false>
 __global__ void __launch_bounds__(kK1Threads, 1)
 lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __grid_constant__ CUtensorMap tmap_w,
                        const __grid_constant__ CUtensorMap tmap_w4, const __grid_constant__ CUtensorMap tmap_w16,
@@ -753,8 +767,8 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   const int pair_rows = 2 * p.tile_rows;                 // vocabulary rows of a pair's tile
   const uint32_t bar_base = base + p.stages * stage_bytes;
   const uint32_t full_bar = bar_base, empty_bar = bar_base + 96, tfull_bar = bar_base + 192,
-                 tempty_bar = bar_base + 208, rawfull_bar = bar_base + 272, operand_bar = bar_base + 368;
-  constexpr int kNumEpi = kW8 ? kW8EpiWarps : kEpiWarps;      // epilogue warps 2 .. 2 + kNumEpi - 1
+                 tempty_bar = bar_base + 208, rawfull_bar = bar_base + 272;
+  constexpr int kNumEpi = kFew ? kW8FewEpiWarps : kW8 ? kW8EpiWarps : kEpiWarps;      // epilogue warps 2 .. 2 + kNumEpi - 1
   constexpr int kGroups = kNumEpi / 4;                        // warps per tensor-memory lane quarter
   constexpr int kWarpTransBytes = kRot ? 2 * kTransBytes : kTransBytes;   // rotating units: a whole 32-row chunk at once
   float* trans_base = reinterpret_cast<float*>(smem + p.stages * stage_bytes + kBarrierBytes);
@@ -763,12 +777,10 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.stages; ++i) {
-      mbar_init(full_bar + 8 * i, 2);
+      mbar_init(full_bar + 8 * i, kW8 ? 2 + 2 * kConvGroup : 2);     // (+ the converter warps of a K block, both CTAs)
       mbar_init(empty_bar + 8 * i, 1);
       if (kW8) mbar_init(rawfull_bar + 8 * i, 1);
     }
-    if (kW8)
-      for (int i = 0; i < p.a_slots; ++i) mbar_init(operand_bar + 8 * i, 2 * kConvGroup);
     for (int i = 0; i < 2; ++i) mbar_init(tfull_bar + 8 * i, 1);
     for (int i = 0; i < 4; ++i) mbar_init(tempty_bar + 8 * i, 2 * kNumEpi);
     *abort_flag = 0u;
@@ -1001,7 +1013,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         // either case the converters report for it, so that all barriers move on block by block.
         const uint32_t operand0 = tmem_base + 2 * p.acc_cols;
         int aslot = 0;
-        uint32_t aphase = 0;
+        bool ready = false;                                // the next block has been seen complete
         if (p.group_width) grid_dependency_wait();         // the width table may come from the kernel before
         int width_next = p.group_width && my_tiles > 0 ? p.group_width[pair] : 8;
         for (int t = 0; t < my_tiles && ok; ++t) {
@@ -1014,8 +1026,10 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           const uint32_t d0 = tmem_base + buf * p.acc_cols;
           const int n_blocks = in_smem ? p.n_kblocks : code_blocks;
           for (int kb = 0; kb < n_blocks; ++kb) {
-            if (!mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status)) { ok = false; break; }
-            if (!mbar_wait(operand_bar + 8 * aslot, aphase, abort_flag, p.status)) { ok = false; break; }
+            if (!ready && !mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status)) { ok = false; break; }
+            // a look at the next block's barrier, whose answer (some 90 cycles) arrives while this block's MMAs are issued
+            const int next = stage + 1 == p.stages ? 0 : stage + 1;
+            ready = mbar_test(full_bar + 8 * next, next ? phase : phase ^ 1u);
             tc_fence_after();
             const uint64_t adesc = desc0 + ((stage * stage_bytes) >> 4);
             const uint64_t bdesc = adesc + (kWBlockBytes >> 4);
@@ -1036,7 +1050,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
             }
             umma_commit_pair(empty_bar + 8 * stage);
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
-            if (++aslot == p.a_slots) { aslot = 0; aphase ^= 1u; }
+            if (++aslot == p.a_slots) aslot = 0;
           }
           if (ok) umma_commit_pair(tfull_bar + 8 * buf);
         }
@@ -1098,7 +1112,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                               : (group < n_chunks ? (n_chunks - 1 - group) / kGroups + 1 : 0);
     float* tbuf = trans_base + (warp - 2) * (kWarpTransBytes / 4);
     const int trow = lane & 15, thalf = lane >> 4;       // row of a transposition step; which 16 of the 32 entries
-    constexpr int kSlots = (kRot || kW8) ? 3 : kEpiSlots;   // chunks per tile this warp keeps statistics for
+    constexpr int kSlots = kFew ? 1 : (kRot || kW8) ? 3 : kEpiSlots;   // chunks per tile this warp keeps statistics for
     Stats st[kSlots][2];
 #pragma unroll
     for (int i = 0; i < kSlots; ++i) { st[i][0] = stats_empty(); st[i][1] = stats_empty(); }
@@ -1377,18 +1391,19 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     // eight neighbouring rows over all banks), are expanded in registers and go out 32 columns per tcgen05.st.  The
     // expanded operand never touches shared memory.  Two groups of four warps (a warp reaches only its own quarter of the
     // lanes) take the blocks in turn.
-    // What bounds it: with few verify rows the chain of one block, ~1600 cycles per group (expansion 570, waits and loop
-    // the rest), against ~690 cycles per block and two groups that HBM allows at 8 bits; with 129..192 rows the MMAs (768
-    // cycles per block), of whose operand tensor memory then holds only two blocks.  Measured against the form before
-    // (bf16 tile written to shared memory by groups of two warps, K blocks of 64; three byte permutes or more per two
-    // codes): whole step of one sequence, H = 4096, V = 32000, widths 20/70/10 % 68.3 -> 44.0 us, all 8-bit 58.1 -> 39.2;
-    // 192 rows, V = 128256 331 -> 236 us, 120 rows 277 -> 184.  K blocks of 64 with the same warps: 81 us (the waits
-    // cost as much per block as the expansion does).
+    // What bounds it: with few verify rows the thread that issues the MMAs (some 650 cycles per block: its look at the
+    // barrier, eight MMAs, two commits), close to the 700 cycles that HBM needs for a block at 8 bits; with 129..192 rows
+    // the MMAs (768 cycles per block) and, in long loops, the power cap.  Measured (whole step, widths 20/70/10 %): one
+    // sequence, H = 4096, V = 32000 68.3 us with the operand expanded into shared memory by groups of two warps, K blocks of
+    // 64 and a byte permute or more per code; 44.0 in this form, 41.0 with the tail and the accept/sample kernel
+    // shortened, 37.4 with three groups, 35.3 with one barrier per block for hidden rows and operand and an early look at
+    // the next one (all 8-bit: 58.1 -> 31.6).  192 rows, V = 128256: 331 -> 220.  Operand slots of half a block (four of
+    // 32 columns next to two accumulators of 192): no gain at 192 rows, 39.4 -> 47.6 with one sequence.
     const int quarter = warp & 3;
-    const int grp = (warp - (2 + kW8EpiWarps)) / kConvGroup;
+    const int grp = (warp - (2 + kNumEpi)) / kConvGroup;
     const int row = quarter * 32 + lane;
     const int G = p.conv_groups;
-    const uint32_t leader_operand = map_to_cta(operand_bar, 0);
+    const uint32_t leader_full = map_to_cta(full_bar, 0);
     const uint32_t operand_lane = tmem_base + 2 * p.acc_cols + (static_cast<uint32_t>(quarter * 32) << 16);
     grid_dependency_wait();                              // the width table and the exponents may come from the kernel before
     // Where this lane's row starts in the slot, and what the swizzle does to the index of its 16-byte pieces.
@@ -1398,7 +1413,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     // i - a_slots, whose MMAs must be done before the operand slot is overwritten.  a_slots <= stages, so having waited
     // for that block implies that the slot's previous codes have been used up, and no wait is more than a phase behind.
     int stage = grp, aslot = grp;                        // (grp < conv_groups <= a_slots <= stages)
-    int old_stage = (grp - p.a_slots) & (G - 1);         // first block >= a_slots of this group, less a_slots
+    int old_stage = (grp + G * kMaxStages - p.a_slots) % G;       // first block >= a_slots of this group, less a_slots
     uint32_t phase = 0, old_phase = 0;
     int i = grp, kb = grp;                               // block i is block kb of tile t
     bool ok = grp < G;
@@ -1456,7 +1471,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           tc_fence_before();
         }
         __syncwarp();
-        if (elect_one()) mbar_arrive_cluster(leader_operand + 8 * aslot);
+        if (elect_one()) mbar_arrive_cluster(leader_full + 8 * stage);
         sh0 = sh1; sh1 = sh2;
         stage += G;
         if (stage >= p.stages) { stage -= p.stages; phase ^= 1u; }
@@ -2833,10 +2848,12 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   kp.M = M; kp.V = a->V; kp.n_ptiles = pl.n_ptiles; kp.n_kblocks = pl.n_kblocks;
   kp.pair256 = (pl.rot && pl.N == 128 && !ctx->no_pair256) ? 1 : 0;
   kp.kpb = pl.kpb; kp.k_tail = pl.k_tail;
-  kp.acc_cols = !w8 ? 256 : (pl.N <= 128 ? 128 : kExpandMaxN);
-  kp.conv_groups = ctx->conv_group > kConvGroup ? 1 : kConvGroups;
+  kp.acc_cols = w8 ? round_up(pl.N, 32) : 256;
+  const bool few = w8 && pl.N <= 32;                     // (four epilogue warps, one chunk each)
+  kp.conv_groups = ctx->conv_group > kConvGroup ? 1 : few ? kConvGroupsFew : kConvGroups;
   const int a_slots = (kTmemCols - 2 * kp.acc_cols) / kOperandCols;
   kp.a_slots = a_slots < pl.stages ? a_slots : pl.stages;
+  if (kp.conv_groups > kp.a_slots) kp.conv_groups = kp.a_slots;
   kp.stages = pl.stages; kp.nbuf = pl.nbuf; kp.rot = pl.rot; kp.n_sub = pl.n_sub; kp.N = pl.N; kp.tile_rows = pl.tile_rows; kp.ldl = ldl;
   kp.logits = logits; kp.partials = ctx->partials; kp.part_stride = ctx->max_rows;
   kp.status = a->status_word ? a->status_word : ctx->status;
@@ -2900,6 +2917,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     e = two ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<3, false>, th, tw, tw4, tw16, kp)
       : i8 ? (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, true>, th, tw, tw4, tw16, kp)
                      : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, false>, th, tw, tw4, tw16, kp))
+      : few ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<1, false, true>, th, tw, tw4, tw16, kp)
       : w8 ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<1, false>, th, tw, tw4, tw16, kp)
            : (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, true>, th, tw, tw4, tw16, kp)
                      : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, false>, th, tw, tw4, tw16, kp));
@@ -3038,6 +3056,7 @@ cudaError_t configure_kernels() {
   const void* kernels[] = {reinterpret_cast<const void*>(lm_head_entropy_kernel<0, false>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<0, true>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<1, false>),
+                           reinterpret_cast<const void*>(lm_head_entropy_kernel<1, false, true>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<2, false>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<2, true>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<3, false>)};

@@ -191,6 +191,9 @@ def test_converter_group_size_changes_speed_not_results(binding):
     (43, 2, 384, 2100, [16, 4, 8]),            # 129 rows: wider accumulators, two operand slots
     (64, 2, 640, 2500, [8, 16, 4, 4]),         # 192 rows, the most one pass holds; an odd number of K blocks
     (193, 0, 256, 900, [4, 16]),               # 193 rows: two passes
+    (8, 3, 1408, 5000, [8, 4, 16]),            # 32 rows, the most that four epilogue warps serve: three converter groups
+    (11, 2, 384, 40000, [4, 8, 8, 16]),        # 33 rows: two groups again; three tiles per pair
+    (1, 4, 2176, 60000, [8, 16, 4]),           # one sequence, several tiles of every width per pair
     (3, 4, 176, 1100, None), (64, 2, 112, 37000, None),   # all 8-bit (no width table): ragged last K block, many tiles
 ])
 def test_expansion_at_the_edges_of_its_tiles(binding, B, k, H, V, pattern):
