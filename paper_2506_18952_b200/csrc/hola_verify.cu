@@ -137,7 +137,7 @@ struct K1Params {
                           // wait runs out, or in a later kernel)
   int stream_logits;      // 1: store the logits with the streaming hint (they exceed what the L2 keeps until they are read)
   float* logits;
-  float4* partials;   // [grid][part_stride] (m, s, t, arg-max index)
+  float4* partials;   // [M][part_stride] (m, s, t, arg-max index): a row's partials side by side, one per CTA of its pass
   int part_stride;
   unsigned* status;
   // What the accept/sample kernel behind this one will gather (null: nothing): draft tokens, uniforms and the entries
@@ -155,8 +155,8 @@ struct K1Params {
 struct K3Params {
   int B, k, V, ldl;
   const float* logits;
-  const float4* partials;
-  int nparts, part_stride, combine;
+  const float4* partials;       // partial i of row r at [r * row_stride + i * part_stride]
+  int nparts, row_stride, part_stride, combine;
   const int* tok;
   const void* q;
   int q_dtype;
@@ -1508,15 +1508,8 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           sum_t = fmaf(e, fmaf(d, x[q].y, x[q].z), sum_t);
         }
       }
-      p.partials[static_cast<size_t>(blockIdx.x) * p.part_stride + row0 + r] =
+      p.partials[static_cast<size_t>(row0 + r) * p.part_stride + 2 * pair + rank] =
           make_float4(m, sum, sum_t, __int_as_float(arg));
-    }
-    if (p.n_pass > 1) {
-      // the accept/sample kernel merges the partials of every CTA for every row: this CTA has seen only its pass
-      const Stats none = stats_empty();
-      const float4 blank = make_float4(none.m, none.s, none.t, __int_as_float(none.arg));
-      for (int r = threadIdx.x; r < p.M; r += kK1Threads)
-        if (r < row0 || r >= row0 + rows) p.partials[static_cast<size_t>(blockIdx.x) * p.part_stride + r] = blank;
     }
   }
   cluster_sync_execution_only();                         // the peer no longer signals this CTA's barriers or tensor memory
@@ -1568,18 +1561,20 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_selftest_kernel(long long 
 
 // ------------------------------------------------------------------------------------------------ K2
 // The statistics of one row over all CTAs, by a warp, the same bits in every lane.  Six loads per lane in flight (192
-// partials per round: one round on a 148-SM part).  The maximum first, so that the
+// partials per round: one round on a 148-SM part; a GEMM launch leaves a row's partials side by side, part_stride 1).  The
+// maximum first, so that the
 // exponentials of the partials are independent of one another and only additions remain to be passed round: five
 // shuffles for the maximum and five for the sums instead of eleven merges of a hundred cycles each.
-__device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int part_stride, int row,
-                                                     int lane) {
+__device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int row_stride, int part_stride,
+                                                     int row, int lane) {
+  partials += static_cast<size_t>(row) * row_stride;
   Stats st = stats_empty();
   for (int base = 0; base < nparts; base += 192) {
     float4 x[6];
 #pragma unroll
     for (int u = 0; u < 6; ++u) {
       const int i = base + lane + 32 * u;
-      x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride + row]
+      x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride]
                         : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
     }
     float m = fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x));
@@ -1613,7 +1608,7 @@ __device__ __forceinline__ void stats_to_outputs(Stats st, float* logZ, float* H
   *H = fmaxf(0.f, ls - st.t / st.s);
 }
 
-__global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, int nparts, int part_stride, int M,
+__global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, int nparts, int row_stride, int M,
                                                        float* logZ, float* entropy) {
   // (launched like the accept/sample kernel: the next kernel in the stream may be put in place behind this one)
   grid_dependency_release();
@@ -1621,14 +1616,14 @@ __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, i
   const int lane = threadIdx.x & 31;
   grid_dependency_wait();
   if (row >= M) return;
-  Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
+  Stats st = warp_merge_partials(partials, nparts, row_stride, 1, row, lane);
   if (lane == 0) stats_to_outputs(st, &logZ[row], &entropy[row]);
 }
 
 // Vocabulary-parallel form, first exchange record of a rank: per verify row the statistics of this shard's logits
 // (m, s, t, arg-max as a GLOBAL vocabulary index), then per draft position the logit of the draft token if this shard
 // owns it (-inf otherwise).  Blocks 0 .. ceil(M/8)-1 merge the per-CTA partials, the others gather the logits.
-__global__ void __launch_bounds__(256) shard_record_kernel(const float4* partials, int nparts, int part_stride, int M,
+__global__ void __launch_bounds__(256) shard_record_kernel(const float4* partials, int nparts, int row_stride, int M,
                                                            int v_offset, int V, const float* logits, int ldl,
                                                            const int* tok, int B, int k, float4* stats_out,
                                                            float* lx_out) {
@@ -1637,7 +1632,7 @@ __global__ void __launch_bounds__(256) shard_record_kernel(const float4* partial
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
-    Stats st = warp_merge_partials(partials, nparts, part_stride, row, lane);
+    Stats st = warp_merge_partials(partials, nparts, row_stride, 1, row, lane);
     if (lane == 0) {
       const int arg = st.arg == 0x7fffffff ? st.arg : st.arg + v_offset;
       stats_out[row] = make_float4(st.m, st.s, st.t, __int_as_float(arg));
@@ -1834,7 +1829,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
     // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
     // above, gets a row only when there are more than seven)
     for (int j = kK3Warps - 1 - warp; j <= k; j += kK3Warps) {
-      Stats st = warp_merge_partials(p.partials, p.nparts, p.part_stride, row_first + j, lane);
+      Stats st = warp_merge_partials(p.partials, p.nparts, p.row_stride, p.part_stride, row_first + j, lane);
       if (lane == 0) {
         float lz, h;
         stats_to_outputs(st, &lz, &h);
@@ -2506,7 +2501,8 @@ struct hola_ctx {
   char* ws;                 // one device allocation, carved below
   size_t ws_bytes;
   float* logits;            // [max_rows][ldl]
-  float4* partials;         // [num_sms][max_rows]
+  float4* partials;         // [max_rows][part_stride]
+  int part_stride;          // CTAs a row may have partials of (the SM count)
   unsigned* status;         // [1]
   unsigned* pace;           // [kMaxPaceGroups] counters of the groups of pairs when all passes share a launch
   double* hq;               // [max_rows][kHqSlices] slice sums of q ln q over the draft rows
@@ -2855,7 +2851,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   kp.a_slots = a_slots < pl.stages ? a_slots : pl.stages;
   if (kp.conv_groups > kp.a_slots) kp.conv_groups = kp.a_slots;
   kp.stages = pl.stages; kp.nbuf = pl.nbuf; kp.rot = pl.rot; kp.n_sub = pl.n_sub; kp.N = pl.N; kp.tile_rows = pl.tile_rows; kp.ldl = ldl;
-  kp.logits = logits; kp.partials = ctx->partials; kp.part_stride = ctx->max_rows;
+  kp.logits = logits; kp.partials = ctx->partials; kp.part_stride = ctx->part_stride;
   kp.status = a->status_word ? a->status_word : ctx->status;
   kp.w_scale = a->w_scale;
   kp.h_scale = ctx->hid_scale;
@@ -2926,6 +2922,9 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   return HOLA_OK;
 }
 
+// Partials per row that a GEMM launch (or one per pass) leaves: one per CTA that works on the row's pass.
+int row_partials(const Plan& pl) { return pl.fused ? pl.grid / pl.passes : pl.grid; }
+
 cudaError_t launch_finalize(const hola_ctx* ctx, const hola_verify_args* a, int M, int nparts, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>((M + 7) / 8)); cfg.blockDim = dim3(256); cfg.stream = stream;
@@ -2933,7 +2932,7 @@ cudaError_t launch_finalize(const hola_ctx* ctx, const hola_verify_args* a, int 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, finalize_kernel, static_cast<const float4*>(ctx->partials), nparts, ctx->max_rows, M,
+  return cudaLaunchKernelEx(&cfg, finalize_kernel, static_cast<const float4*>(ctx->partials), nparts, ctx->part_stride, M,
                             a->logZ, a->entropy);
 }
 
@@ -2955,7 +2954,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   kp.q_far = q_far; kp.q_far_from = q_far_from;
   kp.q_tok = q_tok; kp.phase = phase; kp.inputs_settled = settled ? 1 : 0;
   kp.B = a->B; kp.k = a->k; kp.V = a->V; kp.ldl = ldl; kp.logits = logits;
-  kp.partials = ctx->partials; kp.nparts = nparts; kp.part_stride = ctx->max_rows; kp.combine = combine;
+  kp.partials = ctx->partials; kp.nparts = nparts; kp.row_stride = ctx->part_stride; kp.part_stride = 1; kp.combine = combine;
   kp.tok = a->draft_tok; kp.q = a->draft_q; kp.q_dtype = a->q_dtype; kp.u = a->uniforms; kp.tau = a->tau;
   kp.gate_source = a->gate_source; kp.fallback = a->fallback; kp.hq_part = nullptr; kp.draft_entropy = a->draft_entropy;
   if (a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0) {
@@ -2977,7 +2976,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     kp.lx_all = reinterpret_cast<const float*>(sh->stats_all) + 4 * static_cast<size_t>(a->B) * (a->k + 1);
     kp.rec_stride = sh->rec_floats;
     kp.mass_out = sh->mass_out; kp.mass_all = sh->mass_all;
-    if (combine) { kp.partials = sh->stats_all; kp.nparts = sh->world; kp.part_stride = sh->rec_floats / 4; }
+    if (combine) { kp.partials = sh->stats_all; kp.nparts = sh->world; kp.row_stride = 1; kp.part_stride = sh->rec_floats / 4; }
   }
   const bool vec = (a->V % 4 == 0) && (ldl % 4 == 0) && aligned16(logits) && (a->k == 0 || aligned16(a->draft_q));
   const int nchunks = (a->V + kChunk - 1) / kChunk;
@@ -3143,6 +3142,7 @@ hola_status hola_create(hola_ctx** out, int device, int maxB, int maxK, int H, i
   ctx->ws_bytes = w.total;
   ctx->logits = reinterpret_cast<float*>(ctx->ws + w.logits);
   ctx->partials = reinterpret_cast<float4*>(ctx->ws + w.partials);
+  ctx->part_stride = ctx->num_sms;
   ctx->status = reinterpret_cast<unsigned*>(ctx->ws + w.status);
   ctx->pace = reinterpret_cast<unsigned*>(ctx->ws + w.pace);
   ctx->hq = reinterpret_cast<double*>(ctx->ws + w.hq);
@@ -3293,7 +3293,7 @@ hola_status hola_lm_head_entropy(hola_ctx* ctx, const hola_verify_args* a, void*
   float* logits = a->logits_out ? a->logits_out : ctx->logits;
   const int ldl = a->logits_out ? a->V : ctx->ldl;
   if ((s = run_lm_head(ctx, a, logits, ldl, pl, stream, M <= 256)) != HOLA_OK) return s;
-  const cudaError_t e = launch_finalize(ctx, a, M, pl.grid, stream);
+  const cudaError_t e = launch_finalize(ctx, a, M, row_partials(pl), stream);
   if (e != cudaSuccess) { set_error(ctx, "launch finalize_kernel", e); return HOLA_ERR_CUDA; }
   return HOLA_OK;
 }
@@ -3351,7 +3351,7 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   if (before_sample && cudaStreamWaitEvent(stream, before_sample, 0) != cudaSuccess) return HOLA_ERR_CUDA;
   ctx->hq_ready = side ? 1 : 0;
   // (behind the GEMM kernel: the caller's inputs are settled; an event wait in between makes it an ordinary launch)
-  s = run_accept_sample(ctx, a, logits, ldl, 1, pl.grid, stream, nullptr, 0, nullptr, true);
+  s = run_accept_sample(ctx, a, logits, ldl, 1, row_partials(pl), stream, nullptr, 0, nullptr, true);
   ctx->hq_ready = 0;
   if (prof) { cudaEventRecord(ev[2], stream); ctx->prof_n++; }
   return s;
@@ -3481,13 +3481,13 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
     if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
     if (e != cudaSuccess) { set_error(ctx, "wait for the inputs sent ahead", e); return HOLA_ERR_CUDA; }
     direct = outputs_to_host(ctx, &d, ob);
-    s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 0, nullptr, false, q_far, ahead);
+    s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, row_partials(pl), stream, ctx->st_qtok, 0, nullptr, false, q_far, ahead);
     ctx->flags_out = nullptr;
     if (s != HOLA_OK) return s;
   } else {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
     if (e != cudaSuccess) { set_error(ctx, "host-to-device copy of draft rows", e); return HOLA_ERR_CUDA; }
-    if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, pl.grid, stream, ctx->st_qtok, 1)) != HOLA_OK) return s;
+    if ((s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, row_partials(pl), stream, ctx->st_qtok, 1)) != HOLA_OK) return s;
     d2h(ctx->h_accept, d.accept_len, static_cast<size_t>(B) * 4);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) { set_error(ctx, "accept lengths to host", e); return HOLA_ERR_CUDA; }
@@ -3699,7 +3699,7 @@ hola_status hola_shard_lm_head(hola_ctx* ctx, const hola_verify_args* a, const h
   float4* stats_out = static_cast<float4*>(sh->record_out);
   float* lx_out = reinterpret_cast<float*>(stats_out + M);
   const int blocks = (M + 7) / 8 + (a->B * a->k + 255) / 256;
-  shard_record_kernel<<<blocks, 256, 0, stream>>>(ctx->partials, pl.grid, ctx->max_rows, M, sh->v_offset, a->V, logits,
+  shard_record_kernel<<<blocks, 256, 0, stream>>>(ctx->partials, row_partials(pl), ctx->part_stride, M, sh->v_offset, a->V, logits,
                                                   ldl, a->draft_tok, a->B, a->k, stats_out, lx_out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { set_error(ctx, "launch shard_record_kernel", e); return HOLA_ERR_CUDA; }
@@ -3833,6 +3833,7 @@ hola_status static_setup(int dev, hola_ctx* out) {
     c->encode = reinterpret_cast<EncodeTiledFn>(fn);
     c->status = reinterpret_cast<unsigned*>(base);
     c->partials = reinterpret_cast<float4*>(static_cast<unsigned char*>(base) + kStaticStatusBytes);
+    c->part_stride = kStaticMaxCtas;
     c->max_rows = kStaticMaxRows;
     g_static_ready[dev] = true;
   }
@@ -3868,5 +3869,5 @@ extern "C" hola_status hola_lm_head_entropy_static(const hola_verify_args* a, vo
   // call before they are read; the internal status word is the one thing that must start at zero.
   if (cudaMemsetAsync(local.status, 0, sizeof(unsigned), stream) != cudaSuccess) return HOLA_ERR_CUDA;
   if ((s = run_lm_head(&local, a, a->logits_out, a->V, pl, stream)) != HOLA_OK) return s;
-  return launch_finalize(&local, a, M, pl.grid, stream) == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
+  return launch_finalize(&local, a, M, row_partials(pl), stream) == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
 }
