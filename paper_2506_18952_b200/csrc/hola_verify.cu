@@ -2479,6 +2479,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 struct Plan {
   int n_sub, N, rows_per_pass, passes, grid, stages, nbuf, rot, n_ptiles, n_kblocks, smem_bytes, tile_rows;
   int fused;            // all passes in one launch, groups of `passes` CTA pairs sharing the vocabulary tiles
+  double mma_share;     // estimated tensor time over HBM time of a pass
   int kpb, k_tail;      // K blocks per ring slot; a partial last K block in a slot of its own
   double est_seconds;   // rough duration of all passes (the cost the split was chosen by)
 };
@@ -2635,6 +2636,7 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
       best_cost = cost;
       best.n_sub = n_sub; best.N = N; best.rows_per_pass = two ? n_sub * N / 2 : n_sub * N; best.passes = passes;
       best.est_seconds = cost;
+      best.mma_share = t_mma / t_hbm;
     }
   }
   // a pass may end up empty when rows_per_pass * (passes - 1) already covers M
@@ -2654,6 +2656,11 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   if (tile_rows < 104) tile_rows = round_up(tile_rows, 8);         // whole swizzle patterns: several K blocks per slot
   if (tile_rows < 8) tile_rows = 8;
   if (tile_rows > kLanes) tile_rows = kLanes;
+  // Near and beyond the point where the tensor cores bound, a tile costs the same whatever its rows: as few tiles as
+  // possible (the busiest pair has as many either way), because these loops run at the power cap and every MMA counts.
+  // us: V = 32000, 384 rows (143 tiles of 224 rows -> 125 of 256) 117 -> 113, 8-bit 74.7 -> 72.9; V = 128256 (517 -> 501),
+  // 384 rows 434 -> 430, 192 rows at 8 bits (0.87 of the HBM time) 144 -> 140, two planes 221 -> 212.
+  if (rounds >= 2 && best.mma_share > 0.8) tile_rows = kLanes;
   if (mixed) tile_rows = kLanes;                 // a pair's tile is one group of 256 rows of one width
   best.tile_rows = tile_rows;
   best.n_ptiles = (ctx->V + 2 * tile_rows - 1) / (2 * tile_rows);
