@@ -2420,6 +2420,9 @@ __device__ __forceinline__ float qlnq4(const float4 x) { return (qlnq(x.x) + qln
 // before the GEMM kernel had finished and made the step 45 us longer).
 __global__ void __launch_bounds__(256) draft_entropy_kernel(const void* q, int q_dtype, int V, double* part) {
   __shared__ double sh_part[8];
+  // (no-ops unless launched with programmatic serialization: the GEMM kernel behind it may be put in place at once)
+  grid_dependency_release();
+  grid_dependency_wait();
   const size_t row = blockIdx.x;
   const int slice = blockIdx.y;
   double acc = 0.0;
@@ -2929,6 +2932,16 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   return HOLA_OK;
 }
 
+cudaError_t launch_draft_entropy(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a->B * a->k), kHqSlices); cfg.blockDim = dim3(256); cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, draft_entropy_kernel, a->draft_q, a->q_dtype, a->V, ctx->hq);
+}
+
 // Partials per row that a GEMM launch (or one per pass) leaves: one per CTA that works on the row's pass.
 int row_partials(const Plan& pl) { return pl.fused ? pl.grid / pl.passes : pl.grid; }
 
@@ -2968,9 +2981,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     // one more pass over the draft rows: H(q_j) for every (sequence, draft position) - unless the caller has put it
     // on the side stream already, next to the GEMM
     if (!ctx->hq_ready) {
-      draft_entropy_kernel<<<dim3(static_cast<unsigned>(a->B * a->k), kHqSlices), 256, 0, stream>>>(
-          a->draft_q, a->q_dtype, a->V, ctx->hq);
-      const cudaError_t e0 = cudaGetLastError();
+      const cudaError_t e0 = launch_draft_entropy(ctx, a, stream);
       if (e0 != cudaSuccess) { set_error(ctx, "launch draft_entropy_kernel", e0); return HOLA_ERR_CUDA; }
     }
     kp.hq_part = ctx->hq;
@@ -3121,9 +3132,11 @@ hola_status hola_create(hola_ctx** out, int device, int maxB, int maxK, int H, i
   if (H % 8 != 0 || maxK + 1 > kMaxK1 || V > kMaxChunks * kChunk) return HOLA_ERR_UNSUPPORTED_SHAPE;
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return HOLA_ERR_NO_DEVICE;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return HOLA_ERR_NO_DEVICE;
-  if (prop.major != 10) return HOLA_ERR_NO_DEVICE;       // the kernels are sm_100a only; there is no fallback
+  int major = 0, sms = 0;                                // (cudaGetDeviceProperties would take a millisecond or more)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return HOLA_ERR_NO_DEVICE;
+  if (major != 10) return HOLA_ERR_NO_DEVICE;            // the kernels are sm_100a only; there is no fallback
   DeviceGuard guard(device);
   if (!guard.ok) return HOLA_ERR_NO_DEVICE;
 
@@ -3135,7 +3148,7 @@ hola_status hola_create(hola_ctx** out, int device, int maxB, int maxK, int H, i
 
   hola_ctx* ctx = static_cast<hola_ctx*>(calloc(1, sizeof(hola_ctx)));
   if (!ctx) return HOLA_ERR_WORKSPACE;
-  ctx->device = device; ctx->num_sms = prop.multiProcessorCount; ctx->maxB = maxB; ctx->maxK = maxK;
+  ctx->device = device; ctx->num_sms = sms; ctx->maxB = maxB; ctx->maxK = maxK;
   ctx->H = H; ctx->V = V; ctx->ldl = static_cast<int>(align_up(static_cast<size_t>(V), 4));
   ctx->max_rows = maxB * (maxK + 1);
   ctx->encode = reinterpret_cast<EncodeTiledFn>(fn);
@@ -3330,16 +3343,26 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   cudaEvent_t* ev = prof ? ctx->prof_ev + 3 * ctx->prof_n : nullptr;
   if (prof) cudaEventRecord(ev[0], stream);
   const bool draft_gate = a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0;
+  // A small draft tensor: the pass over it goes in front of the GEMM, whose CTAs take their places (and ask for their first
+  // blocks) while it runs; no events, and the accept/sample kernel keeps its place in the chain of dependent launches.
+  // us, side stream against in front: V = 1000 14.9 / 13.8; 4 sequences, V = 9000 (360 KB) 17.6 / 17.1; one, V = 32000 (256 KB)
+  // 49.9 / 50.2, called alone 68.2 / 66.8; 16, V = 32000 (5 MB) 62.3 / 64.9: there the GEMM hides the pass.
+  const double q_bytes = static_cast<double>(a->B) * a->k * a->V * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
+  const bool ahead = draft_gate && !before_sample && q_bytes <= 512e3;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (draft_gate && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
+  if (draft_gate && !ahead && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
   // The pass over the draft rows (draft-entropy gate) depends on nothing the GEMM makes, and its small CTAs fit on the
   // SMs beside the GEMM's: it runs on the context's side stream (behind the copy of the draft tensor, when the host
   // entry put one there), branching off the caller's stream before the GEMM and joining it again before the
   // accept/sample kernel.  It is launched AFTER the GEMM so that the GEMM's CTAs get their SMs first.
   // (While the caller records a graph everything stays on the caller's stream.)
-  const bool side = draft_gate && (before_sample || capturing == cudaStreamCaptureStatusNone);
+  const bool side = draft_gate && !ahead && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
-  const bool few_before = a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
+  if (ahead) {
+    const cudaError_t e = launch_draft_entropy(ctx, a, stream);
+    if (e != cudaSuccess) { set_error(ctx, "launch draft_entropy_kernel", e); return HOLA_ERR_CUDA; }
+  }
+  const bool few_before = ahead || a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
@@ -3356,7 +3379,7 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
     before_sample = ctx->copy_done;
   }
   if (before_sample && cudaStreamWaitEvent(stream, before_sample, 0) != cudaSuccess) return HOLA_ERR_CUDA;
-  ctx->hq_ready = side ? 1 : 0;
+  ctx->hq_ready = side || ahead ? 1 : 0;
   // (behind the GEMM kernel: the caller's inputs are settled; an event wait in between makes it an ordinary launch)
   s = run_accept_sample(ctx, a, logits, ldl, 1, row_partials(pl), stream, nullptr, 0, nullptr, true);
   ctx->hq_ready = 0;
