@@ -148,6 +148,9 @@ struct K1Params {
   const char* next_q;
   int next_n, next_q_elem;      // B * k; bytes per draft probability
   unsigned next_q_bytes;        // bytes of q to ask for whole (0: only the entries)
+  const void* draft_q;          // draft-entropy gate (else null; not with rotating units): the epilogue warps make the pass over the draft rows while
+  int draft_q_dtype, draft_units;   // the first tile's MMAs run; a unit is one slice of one row (draft_rows * kHqSlices)
+  double* draft_part;
   int prefetch_blocks;  // K blocks of its first tile a CTA asks into the L2 before it waits for the kernel before
   unsigned* pace;     // n_pass > 1: one counter per group of pairs (zero at launch), by which the group keeps in step
 };
@@ -708,6 +711,60 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
   return acc;
 }
 
+__device__ __forceinline__ double warp_sum_f64(double x) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
+}
+
+// ------------------------------------------------------------------------------------------------ draft entropy, a slice
+// H(q) = -sum_v q ln q of a draft row: the gate value when the gate looks at the draft distribution, as the HSD section words
+// it.  q is used as stored; entries with q <= 0 contribute nothing.
+// q ln q for q > 0, else 0.  The fast logarithm (absolute error about 2^-21 near 1, a few ulp elsewhere) is
+// ample here: every term is weighted by q <= 1 and the sum is compared at 1e-4.
+__device__ __forceinline__ float qlnq(float a) { return a > 0.f ? a * __logf(a) : 0.f; }
+__device__ __forceinline__ float qlnq8(const uint4 raw) {     // sum over eight bf16 values
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  float part = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) part += qlnq(__uint_as_float(w[j] << 16)) + qlnq(__uint_as_float(w[j] & 0xFFFF0000u));
+  return part;
+}
+__device__ __forceinline__ float qlnq4(const uint4 x) {        // sum over four fp32 values
+  return (qlnq(__uint_as_float(x.x)) + qlnq(__uint_as_float(x.y))) + (qlnq(__uint_as_float(x.z)) + qlnq(__uint_as_float(x.w)));
+}
+
+// This thread's share (of `nthr`) of sum q ln q over slice `slice` of a row: the 16-byte pieces of the row are cut into
+// kHqSlices runs; what lies before the first piece and behind the last goes to slice 0.
+__device__ __noinline__ double draft_slice_sum(const void* q, int q_dtype, int V, size_t row, int slice, int tid, int nthr) {
+  const bool half = q_dtype == HOLA_Q_BF16;
+  const int elem = half ? 2 : 4, per16 = 16 / elem;
+  const char* qr = static_cast<const char*>(q) + row * V * elem;
+  const int head = min(V, static_cast<int>((16u - (reinterpret_cast<uintptr_t>(qr) & 15u)) & 15u) / elem);
+  const int nvec = (V - head) / per16;
+  const uint4* q16 = reinterpret_cast<const uint4*>(qr + head * elem);
+  const int per = (nvec + kHqSlices - 1) / kHqSlices, end = min(nvec, (slice + 1) * per);
+  constexpr int kInFlight = 4;                           // independent 16-byte loads per thread and step
+  double acc = 0.0;
+  int i = slice * per + tid;
+  for (; i + (kInFlight - 1) * nthr < end; i += kInFlight * nthr) {
+    uint4 raw[kInFlight];
+#pragma unroll
+    for (int u = 0; u < kInFlight; ++u) raw[u] = q16[i + u * nthr];
+#pragma unroll
+    for (int u = 0; u < kInFlight; ++u) acc += half ? qlnq8(raw[u]) : qlnq4(raw[u]);
+  }
+  for (; i < end; i += nthr) acc += half ? qlnq8(q16[i]) : qlnq4(q16[i]);
+  if (slice == 0) {
+    const int tail = head + nvec * per16;
+    for (int n = tid; n < head + V - tail; n += nthr) {
+      const int v = n < head ? n : tail + n - head;
+      acc += qlnq(half ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(qr)[v]) : reinterpret_cast<const float*>(qr)[v]);
+    }
+  }
+  return acc;
+}
+
 // ------------------------------------------------------------------------------------------------ K1
 // Shared memory: `stages` ring slots of [W_lm block 128 x 64 | hidden block(s) n_sub x (N/2) x 64], then the
 // barrier area.  Barriers (8 bytes each, offsets in the barrier area):
@@ -1118,6 +1175,13 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     for (int i = 0; i < kSlots; ++i) { st[i][0] = stats_empty(); st[i][1] = stats_empty(); }
     bool ok = true;
     grid_dependency_wait();                              // the logits buffer may still be read by the kernel before
+    if (!kRot && p.draft_q) {
+      // Nothing else for these warps to do until the first tile is complete.
+      for (int u = blockIdx.x + static_cast<int>(gridDim.x) * (warp - 2); u < p.draft_units; u += gridDim.x * kNumEpi) {
+        const double sum = warp_sum_f64(draft_slice_sum(p.draft_q, p.draft_q_dtype, p.V, u / kHqSlices, u % kHqSlices, lane, 32));
+        if (lane == 0) p.draft_part[u] = sum;
+      }
+    }
     for (int t = 0; t < my_tiles && ok; ++t) {
       const int buf = t % p.nbuf;
       const uint32_t acc_phase = static_cast<uint32_t>(t / p.nbuf) & 1u;
@@ -1647,12 +1711,6 @@ __global__ void __launch_bounds__(256) shard_record_kernel(const float4* partial
 }
 
 // ------------------------------------------------------------------------------------------------ K3
-__device__ __forceinline__ double warp_sum_f64(double x) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-  return x;
-}
-
 // Four sums over the warp at once (lanes 8 i .. 8 i + 7 return the sum of v[i]): the first two rounds halve the
 // number of values a lane carries instead of adding all of them everywhere, six shuffles in all.
 __device__ __forceinline__ float warp_sum4_f32(const float v[4], int lane) {
@@ -2399,78 +2457,19 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
 }
 
 // ------------------------------------------------------------------------------------------------ draft entropy
-// H(q) = -sum_v q ln q of each draft row (one CTA per row): the gate value when the gate looks at the draft
-// distribution, as the HSD section words it.  q is used as stored; entries with q <= 0 contribute nothing.
-// q ln q for q > 0, else 0.  The fast logarithm (absolute error about 2^-21 near 1, a few ulp elsewhere) is
-// ample here: every term is weighted by q <= 1 and the sum is compared at 1e-4.
-__device__ __forceinline__ float qlnq(float a) { return a > 0.f ? a * __logf(a) : 0.f; }
-__device__ __forceinline__ float qlnq8(const uint4 raw) {     // sum over eight bf16 values
-  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-  float part = 0.f;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) part += qlnq(__uint_as_float(w[j] << 16)) + qlnq(__uint_as_float(w[j] & 0xFFFF0000u));
-  return part;
-}
-__device__ __forceinline__ float qlnq4(const float4 x) { return (qlnq(x.x) + qlnq(x.y)) + (qlnq(x.z) + qlnq(x.w)); }
-
-// Grid (rows, kHqSlices): CTA (r, s) sums slice s of row r and leaves the partial sum in part[r][s]; the
-// accept/sample kernel adds the slices in index order.  Small CTAs of 32 registers per thread on purpose: the pass
-// runs on a side stream while the GEMM kernel holds every SM, and only a CTA of this size fits into the registers
-// that kernel leaves free (a persistent form with eight loads in flight per thread, 100 registers, could not start
-// before the GEMM kernel had finished and made the step 45 us longer).
+// Grid (rows, kHqSlices): CTA (r, s) leaves slice s of row r in part[r][s]; the accept/sample kernel adds the slices in
+// index order.  Where the GEMM kernel does not make the pass itself: on a side stream under it, hence CTAs of 32 registers
+// per thread, which fit beside that kernel's (a persistent form with eight loads in flight per thread, 100 registers, could
+// not start before it had finished and made the step 45 us longer).
 __global__ void __launch_bounds__(256) draft_entropy_kernel(const void* q, int q_dtype, int V, double* part) {
   __shared__ double sh_part[8];
-  // (no-ops unless launched with programmatic serialization: the GEMM kernel behind it may be put in place at once)
-  grid_dependency_release();
-  grid_dependency_wait();
-  const size_t row = blockIdx.x;
-  const int slice = blockIdx.y;
-  double acc = 0.0;
-  constexpr int kInFlight = 4;                           // independent 16-byte loads per thread and step
-  if (q_dtype == HOLA_Q_BF16) {
-    const __nv_bfloat16* qr = static_cast<const __nv_bfloat16*>(q) + row * V;
-    const bool vec = (reinterpret_cast<uintptr_t>(qr) & 15u) == 0;
-    const int nvec = vec ? V / 8 : 0;
-    const uint4* q16 = reinterpret_cast<const uint4*>(qr);
-    const int per = (nvec + kHqSlices - 1) / kHqSlices, end = min(nvec, (slice + 1) * per);
-    int i = slice * per + threadIdx.x;
-    for (; i + (kInFlight - 1) * 256 < end; i += kInFlight * 256) {
-      uint4 raw[kInFlight];
-#pragma unroll
-      for (int u = 0; u < kInFlight; ++u) raw[u] = q16[i + u * 256];
-#pragma unroll
-      for (int u = 0; u < kInFlight; ++u) acc += qlnq8(raw[u]);
-    }
-    for (; i < end; i += 256) acc += qlnq8(q16[i]);
-    for (int v = nvec * 8 + threadIdx.x; slice == 0 && v < V; v += 256) {    // scalar tail (or whole row): slice 0
-      acc += qlnq(__bfloat162float(qr[v]));
-    }
-  } else {
-    const float* qr = static_cast<const float*>(q) + row * V;
-    const bool vec = (reinterpret_cast<uintptr_t>(qr) & 15u) == 0;
-    const int nvec = vec ? V / 4 : 0;
-    const float4* q16 = reinterpret_cast<const float4*>(qr);
-    const int per = (nvec + kHqSlices - 1) / kHqSlices, end = min(nvec, (slice + 1) * per);
-    int i = slice * per + threadIdx.x;
-    for (; i + (kInFlight - 1) * 256 < end; i += kInFlight * 256) {
-      float4 raw[kInFlight];
-#pragma unroll
-      for (int u = 0; u < kInFlight; ++u) raw[u] = q16[i + u * 256];
-#pragma unroll
-      for (int u = 0; u < kInFlight; ++u) acc += qlnq4(raw[u]);
-    }
-    for (; i < end; i += 256) acc += qlnq4(q16[i]);
-    for (int v = nvec * 4 + threadIdx.x; slice == 0 && v < V; v += 256) {
-      acc += qlnq(qr[v]);
-    }
-  }
-  acc = warp_sum_f64(acc);
+  const double acc = warp_sum_f64(draft_slice_sum(q, q_dtype, V, blockIdx.x, blockIdx.y, threadIdx.x, 256));
   if ((threadIdx.x & 31) == 0) sh_part[threadIdx.x >> 5] = acc;
   __syncthreads();
   if (threadIdx.x == 0) {
     double tot = 0.0;
     for (int i = 0; i < 8; ++i) tot += sh_part[i];
-    part[row * kHqSlices + slice] = tot;
+    part[blockIdx.x * kHqSlices + blockIdx.y] = tot;
   }
 }
 
@@ -2756,9 +2755,11 @@ int sample_cluster(const hola_ctx* ctx, int B, int V) {
 
 // Steps 1-2: the LM-head GEMM with fused statistics, one launch (clusters of two CTAs) per pass over W_lm.
 // `few_before`: the kernel in front is expected to be this context's accept/sample kernel on a few SMs.
+// `draft_pass`: the pass over the draft rows (draft-entropy gate) is made on the way.
 // `next_reads_inputs`: the accept/sample kernel of the same arguments is launched right behind this.
 hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits, int ldl, const Plan& pl,
-                        cudaStream_t stream, bool few_before = false, bool next_reads_inputs = false) {
+                        cudaStream_t stream, bool few_before = false, bool next_reads_inputs = false,
+                        bool draft_pass = false) {
   const int M = a->B * (a->k + 1);
   const bool mixed = a->w_dtype == HOLA_W_MIXED;
   const bool w8 = a->w_dtype == HOLA_W_INT8 || mixed, two = a->w_dtype == HOLA_W8A16,
@@ -2919,6 +2920,9 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     kp.row0 = pass * pl.rows_per_pass;
     kp.rows = M - kp.row0 < pl.rows_per_pass ? M - kp.row0 : pl.rows_per_pass;
     if (kp.rows <= 0) break;
+    const bool draft = pass == 0 && draft_pass;
+    kp.draft_q = draft ? a->draft_q : nullptr;
+    kp.draft_q_dtype = a->q_dtype; kp.draft_units = a->B * a->k * kHqSlices; kp.draft_part = ctx->hq;
     kp.clear_status = pass == 0 && (a->flags & HOLA_ARG_CLEAR_STATUS) && a->status_word;
     e = two ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<3, false>, th, tw, tw4, tw16, kp)
       : i8 ? (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, true>, th, tw, tw4, tw16, kp)
@@ -2930,16 +2934,6 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     if (e != cudaSuccess) { set_error(ctx, "launch lm_head_entropy_kernel", e); return HOLA_ERR_CUDA; }
   }
   return HOLA_OK;
-}
-
-cudaError_t launch_draft_entropy(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(a->B * a->k), kHqSlices); cfg.blockDim = dim3(256); cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, draft_entropy_kernel, a->draft_q, a->q_dtype, a->V, ctx->hq);
 }
 
 // Partials per row that a GEMM launch (or one per pass) leaves: one per CTA that works on the row's pass.
@@ -2981,7 +2975,9 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     // one more pass over the draft rows: H(q_j) for every (sequence, draft position) - unless the caller has put it
     // on the side stream already, next to the GEMM
     if (!ctx->hq_ready) {
-      const cudaError_t e0 = launch_draft_entropy(ctx, a, stream);
+      draft_entropy_kernel<<<dim3(static_cast<unsigned>(a->B * a->k), kHqSlices), 256, 0, stream>>>(
+          a->draft_q, a->q_dtype, a->V, ctx->hq);
+      const cudaError_t e0 = cudaGetLastError();
       if (e0 != cudaSuccess) { set_error(ctx, "launch draft_entropy_kernel", e0); return HOLA_ERR_CUDA; }
     }
     kp.hq_part = ctx->hq;
@@ -3342,28 +3338,23 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   const bool prof = ctx->prof_on && ctx->prof_n < ctx->prof_cap;
   cudaEvent_t* ev = prof ? ctx->prof_ev + 3 * ctx->prof_n : nullptr;
   if (prof) cudaEventRecord(ev[0], stream);
+  // The pass over the draft rows (draft-entropy gate) depends on nothing the GEMM makes.  Up to 32 MB of them, that kernel's
+  // epilogue warps make the pass while they wait for the first tile (us, against a kernel on a side stream: 16 sequences,
+  // V = 32000 62.6 -> 59.4, one 49.6 -> 47.4, V = 1000 12.8 -> 10.9, 4 sequences, V = 9000 17.5 -> 14.5).  Beyond that, and with
+  // rotating units (whose epilogue has no register to spare: 384 rows, V = 32000 0.9 % slower with the code in it, V = 128256
+  // 441 -> 448 with the gate), a kernel of its own does, on the context's side stream, behind the copy of the draft tensor
+  // where the host entry put one there; else it branches off the caller's stream before the GEMM and joins it again before
+  // the accept/sample kernel.  It is launched AFTER the GEMM so that the GEMM's CTAs get their SMs first; its small CTAs fit
+  // beside them.  (While the caller records a graph everything stays on the caller's stream.)
   const bool draft_gate = a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0;
-  // A small draft tensor: the pass over it goes in front of the GEMM, whose CTAs take their places (and ask for their first
-  // blocks) while it runs; no events, and the accept/sample kernel keeps its place in the chain of dependent launches.
-  // us, side stream against in front: V = 1000 14.9 / 13.8; 4 sequences, V = 9000 (360 KB) 17.6 / 17.1; one, V = 32000 (256 KB)
-  // 49.9 / 50.2, called alone 68.2 / 66.8; 16, V = 32000 (5 MB) 62.3 / 64.9: there the GEMM hides the pass.
   const double q_bytes = static_cast<double>(a->B) * a->k * a->V * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
-  const bool ahead = draft_gate && !before_sample && q_bytes <= 512e3;
+  const bool inside = draft_gate && !before_sample && !pl.rot && q_bytes <= 32e6;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (draft_gate && !ahead && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
-  // The pass over the draft rows (draft-entropy gate) depends on nothing the GEMM makes, and its small CTAs fit on the
-  // SMs beside the GEMM's: it runs on the context's side stream (behind the copy of the draft tensor, when the host
-  // entry put one there), branching off the caller's stream before the GEMM and joining it again before the
-  // accept/sample kernel.  It is launched AFTER the GEMM so that the GEMM's CTAs get their SMs first.
-  // (While the caller records a graph everything stays on the caller's stream.)
-  const bool side = draft_gate && !ahead && (before_sample || capturing == cudaStreamCaptureStatusNone);
+  if (draft_gate && !inside && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
+  const bool side = draft_gate && !inside && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
-  if (ahead) {
-    const cudaError_t e = launch_draft_entropy(ctx, a, stream);
-    if (e != cudaSuccess) { set_error(ctx, "launch draft_entropy_kernel", e); return HOLA_ERR_CUDA; }
-  }
-  const bool few_before = ahead || a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
-  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample);
+  const bool few_before = a->B * sample_cluster(ctx, a->B, a->V) * 4 <= ctx->num_sms;
+  hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample, inside);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
   if (side) {
@@ -3379,7 +3370,7 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
     before_sample = ctx->copy_done;
   }
   if (before_sample && cudaStreamWaitEvent(stream, before_sample, 0) != cudaSuccess) return HOLA_ERR_CUDA;
-  ctx->hq_ready = side || ahead ? 1 : 0;
+  ctx->hq_ready = side || inside ? 1 : 0;
   // (behind the GEMM kernel: the caller's inputs are settled; an event wait in between makes it an ordinary launch)
   s = run_accept_sample(ctx, a, logits, ldl, 1, row_partials(pl), stream, nullptr, 0, nullptr, true);
   ctx->hq_ready = 0;

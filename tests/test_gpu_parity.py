@@ -1040,3 +1040,25 @@ def test_several_k_blocks_per_slot(binding, B, k, H, V, weights):
             assert torch.all((out.logits.double().reshape(-1, V) - want).abs() <= limit)
             full = ctx.hola_verify(w.hidden, head, w.draft_tok, w.draft_q, w.uniforms, w.tau, w_scale=scale, a8=a8)
             assert torch.allclose(full.logZ.double().reshape(-1), torch.logsumexp(want, -1), atol=2e-3)
+
+
+@pytest.mark.parametrize("B,k,H,V,qd", [
+    (2, 3, 64, 7, torch.bfloat16),            # rows shorter than one 16-byte piece, at every alignment
+    (5, 4, 128, 1001, torch.bfloat16), (5, 4, 128, 1003, torch.float32),     # odd rows: a head and a tail beside the pieces
+    (30, 5, 256, 9000, torch.bfloat16),       # more slices than epilogue warps in use
+    (43, 5, 64, 4100, torch.float32),         # 258 rows: rotating units, the pass on the side stream
+])
+def test_draft_entropy_of_rows_at_every_alignment(binding, B, k, H, V, qd):
+    """H(q_j) against fp64 (every term's logarithm is good to 2^-21 and weighted by q: 1e-5 of a sum of at most ln V), and
+    the same value whether the GEMM kernel made the pass or a kernel of its own did (host entry)."""
+    w = workloads.gaussian_head("draft-rows", B, k, H, V, seed=V, device=DEV, w_std=0.3, q_dtype=qd)
+    q = w.draft_q.double()
+    want = -(q * q.clamp_min(1e-300).log()).sum(-1)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        out = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, float(want.median()), gate_source=1)
+        torch.cuda.synchronize()
+        pin = [t.cpu().pin_memory() for t in (w.hidden, w.draft_tok, w.draft_q, w.uniforms)]
+        host = ctx.hola_verify_host(pin[0], w.W_lm, pin[1], pin[2], pin[3], float(want.median()), gate_source=1)
+    assert torch.all((out.draft_entropy.double() - want).abs() <= 1e-5 * math.log(V) + 1e-6)
+    assert torch.allclose(host.draft_entropy.to(DEV), out.draft_entropy, atol=2e-6)
+    assert int(out.status.item()) == 0
