@@ -135,6 +135,8 @@ struct K1Params {
   int rows4;
   int clear_status;       // 1: the status word holds anything; CTA 0 clears it (what sets bits comes seconds later, when a
                           // wait runs out, or in a later kernel)
+  int bulk_logits;        // (rotating units) 1: the logits buffer has a tensor map (rows of whole 16-byte pieces), full blocks
+                          // leave by bulk stores
   int stream_logits;      // 1: store the logits with the streaming hint (they exceed what the L2 keeps until they are read)
   float* logits;
   float4* partials;   // [M][part_stride] (m, s, t, arg-max index): a row's partials side by side, one per CTA of its pass
@@ -325,6 +327,11 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
+__device__ __forceinline__ uint64_t l2_policy_evict_normal() {
+  uint64_t pol;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
@@ -341,6 +348,18 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(x), "r"(y), "l"(policy)
       : "memory");
 }
+
+// A block of 16 rows x 32 logits from its (128-byte-swizzled) staging buffer to the logits buffer.  The rows past the last
+// one and the entries past the vocabulary fall outside the map and are dropped.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y, uint64_t policy) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3}], [%1], %4;"
+               ::"l"(map), "r"(src), "r"(x), "r"(y), "l"(policy)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // Three-dimensional form: (element of a K block, row, K block).
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int row, int kb,
@@ -777,7 +796,7 @@ __device__ __noinline__ double draft_slice_sum(const void* q, int q_dtype, int V
 //   on-chip expansion only: rawfull[12] @272 per CTA: the codes of the slot have landed.  full[] then counts the hidden
 //   bytes (and, for 16-bit rows, their bytes) and one arrival per converter warp of the pair that owns the K block: the
 //   operand is in tensor memory.
-// After the barrier area: one 2 KB transposition buffer per epilogue warp.
+// After the barrier area (with rotating units before it): one transposition buffer of 2 KB (4 KB) per epilogue warp.
 // kMode 3 is kMode 2 with every verify row present twice in the hidden operand (coarse 8-bit plane and the plane of
 // its remainder, in alternating blocks of 32 rows): the epilogue adds the two int32 sums with their scales.
 // kMode: 0 bf16 x bf16; 1 int8 W_lm expanded to bf16 on chip (exact); 2 int8 W_lm x int8 hidden on the 8-bit MMA
@@ -785,6 +804,7 @@ __device__ __noinline__ double draft_slice_sum(const void* q, int q_dtype, int V
 // kRot: 257..384 rows per pass, three MMAs of N <= 128 per K step on rotating 128-column accumulator units (a
 // specialisation of its own because its epilogue holds a different set of values in registers).
 // kFew (mode 1): at most 32 verify rows, four epilogue warps and three groups of converters.
+// (tmap_w4 is the map of the logits buffer with kRot.)
 template <int kMode, bool kRot, bool kFew = false>
 __global__ void __launch_bounds__(kK1Threads, 1)
 lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __grid_constant__ CUtensorMap tmap_w,
@@ -822,15 +842,19 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   const uint32_t tx_bytes = static_cast<uint32_t>(p.tile_rows) * 128u + hid_tx_bytes;   // bf16 W_lm: per CTA and slot
   const int code_blocks = (p.n_kblocks + 1) >> 1;        // (on-chip expansion) K blocks of a tile of 4- or 8-bit rows
   const int pair_rows = 2 * p.tile_rows;                 // vocabulary rows of a pair's tile
-  const uint32_t bar_base = base + p.stages * stage_bytes;
+  constexpr int kWarpTransBytes = kRot ? 2 * kTransBytes : kTransBytes;   // rotating units: a whole 32-row chunk at once
+  // Staging buffers: behind the barrier area; with rotating units before it, on 1024-byte boundaries, as the swizzle of the
+  // bulk stores wants them.
+  constexpr int kTransFirst = kRot ? kEpiWarps * kWarpTransBytes : 0;
+  const uint32_t bar_off = p.stages * stage_bytes + kTransFirst;
+  const uint32_t bar_base = base + bar_off;
   const uint32_t full_bar = bar_base, empty_bar = bar_base + 96, tfull_bar = bar_base + 192,
                  tempty_bar = bar_base + 208, rawfull_bar = bar_base + 272;
   constexpr int kNumEpi = kFew ? kW8FewEpiWarps : kW8 ? kW8EpiWarps : kEpiWarps;      // epilogue warps 2 .. 2 + kNumEpi - 1
   constexpr int kGroups = kNumEpi / 4;                        // warps per tensor-memory lane quarter
-  constexpr int kWarpTransBytes = kRot ? 2 * kTransBytes : kTransBytes;   // rotating units: a whole 32-row chunk at once
-  float* trans_base = reinterpret_cast<float*>(smem + p.stages * stage_bytes + kBarrierBytes);
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + p.stages * stage_bytes + 256);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + p.stages * stage_bytes + 260);
+  float* trans_base = reinterpret_cast<float*>(smem + (kRot ? bar_off - kTransFirst : bar_off + kBarrierBytes));
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + bar_off + 256);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem + bar_off + 260);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < p.stages; ++i) {
@@ -1169,6 +1193,15 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                               : (group < n_chunks ? (n_chunks - 1 - group) / kGroups + 1 : 0);
     float* tbuf = trans_base + (warp - 2) * (kWarpTransBytes / 4);
     const int trow = lane & 15, thalf = lane >> 4;       // row of a transposition step; which 16 of the 32 entries
+    // Rotating units: logits leave by bulk stores out of the staging buffer, 16 rows each, where the lane quarter is all this
+    // CTA's (rows past the last one fall outside the map; a pass ends on a multiple of 16); otherwise lane by lane.  The 32
+    // store instructions of a chunk, their addresses and their way through the L1 bound the read-out of a tile, which a
+    // small H does not hide: us, 384 rows, V = 32000, H = 128 29.9 -> 25.7, 512 34.8 -> 32.9 (8-bit 40.7 -> 37.1),
+    // 4096 110.4 -> 108.5; 2304 rows, V = 128256, H = 8192 3715 -> 3685.  (With at most 256 rows the read-out hides under the
+    // next tile; the same stores there: one sequence 46.6 -> 49.5, 192 rows at 8 bits 141 -> 153.)
+    const bool bulk = kRot && p.bulk_logits && quarter * 32 + 32 <= p.tile_rows;
+    const uint32_t tbuf_addr = smem_u32(tbuf);
+    const uint64_t pol_l = p.stream_logits ? l2_policy_evict_first() : l2_policy_evict_normal();
     constexpr int kSlots = kFew ? 1 : (kRot || kW8) ? 3 : kEpiSlots;   // chunks per tile this warp keeps statistics for
     Stats st[kSlots][2];
 #pragma unroll
@@ -1308,21 +1341,15 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                   if (i < n_ok) v[i] = scaled<kMode>(v[i], w_scale, p.h_scale, r0 + i);
                 if (kMode >= 2) asm volatile("" ::: "memory");   // the row scales eight at a time, not all 32 ahead
               }
-              if (vocab_ok) {
+              if (vocab_ok && !bulk) {
                 float* dst = p.logits + static_cast<size_t>(r0) * p.ldl + vocab;
-                if (n_ok == 32 && p.stream_logits) {
 #pragma unroll
-                  for (int i = 0; i < 32; ++i) __stcs(dst + static_cast<size_t>(i) * p.ldl, v[i]);
-                } else if (n_ok == 32) {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i) dst[static_cast<size_t>(i) * p.ldl] = v[i];
-                } else {
-#pragma unroll
-                  for (int i = 0; i < 32; ++i)
-                    if (i < n_ok) store_logit(dst + static_cast<size_t>(i) * p.ldl, v[i], p.stream_logits);
-                }
+                for (int i = 0; i < 32; ++i)
+                  if (i < n_ok) store_logit(dst + static_cast<size_t>(i) * p.ldl, v[i], p.stream_logits);
               }
             }
+            const bool out = bulk && n_ok > 0 && nv > 0;
+            if (bulk && lane == 0) bulk_wait_read();     // (the stores of the chunk before have left the buffer)
             const bool fold = n_ok > 0 && nv > 0;
             __syncwarp();                                // every lane has folded the chunk before out of the buffer
             if (fold) {
@@ -1331,8 +1358,15 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
 #pragma unroll
               for (int i = 0; i < 32; ++i)
                 tbuf[i * 32 + ((((lane >> 2) ^ (i & 7))) << 2) + (lane & 3)] = v[i];
+              if (out) fence_async_shared();
             }
             __syncwarp();
+            if (out && lane == 0) {
+              tma_store_2d(&tmap_w4, tbuf_addr, vbase + quarter * 32, r0, pol_l);
+              if (n_ok > kTransRows)
+                tma_store_2d(&tmap_w4, tbuf_addr + kTransBytes, vbase + quarter * 32, r0 + kTransRows, pol_l);
+              bulk_commit();
+            }
             if (slot < 2) {                              // the registers are free: take the next unit's chunk, free the unit
               const int unit = (3 * t + slot + 1) & 3;
               tmem_ld32(lane_addr + unit * 128 + group * 32, v);
@@ -1427,6 +1461,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         }
       }
     }
+    if (bulk && lane == 0) bulk_wait_all();
     // ---- the CTA's statistics of every row: the eight contributions (lane quarter, half) side by side where the ring was
     // (this warp has seen the last tile's MMAs complete, so every slot has been filled and read for the last time)
     float4* merge = reinterpret_cast<float4*>(smem);                // [8][rows of the pass]
@@ -2492,7 +2527,8 @@ struct Plan {
 // mode) pair and the two tensor maps of a (hidden pointer, W_lm pointer, rows, weight mode) quadruple.
 struct PlanEntry { int valid, M, w_dtype; Plan pl; };
 struct MapEntry { int valid, M, w_dtype; const void* hidden; const void* W; const void* W4; const void* W16;
-                  CUtensorMap th, tw, tw4, tw16; };
+                  CUtensorMap th, tw, tw4, tw16;
+                  const float* logits; int ldl; };       // rotating units: the logits buffer that tw4 maps (null: none)
 constexpr int kPlanCache = 8, kMapCache = 8;
 
 struct hola_ctx {
@@ -2796,6 +2832,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     me = &ctx->maps[ctx->map_next];
     ctx->map_next = (ctx->map_next + 1) % kMapCache;
     me->valid = 0;
+    me->logits = nullptr;
     if (two)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(2 * round_up(M, 32)), static_cast<uint64_t>(a->H),
                      static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb);
@@ -2847,6 +2884,24 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     }
     me->hidden = hid_src; me->W = w_main; me->M = M; me->w_dtype = a->w_dtype; me->valid = 1;
   }
+  // Rotating units: the logits buffer, where its rows are whole 16-byte pieces; boxes of 16 rows x 32 entries, swizzled like
+  // the staging buffers.
+  const bool bulk_logits = pl.rot && ldl % 4 == 0 && aligned16(logits);
+  if (bulk_logits && (me->logits != logits || me->ldl != ldl)) {
+    me->logits = nullptr;
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(a->V), static_cast<cuuint64_t>(M)};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ldl) * 4};
+    const cuuint32_t box[2] = {32, kTransRows}, estr[2] = {1, 1};
+    const CUresult r = ctx->encode(&me->tw4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, logits, dims, strides, box, estr,
+                                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+      me->valid = 0;
+      snprintf(ctx->last_error, sizeof ctx->last_error, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
+      return HOLA_ERR_CUDA;
+    }
+    me->logits = logits; me->ldl = ldl;
+  }
   const CUtensorMap& th = me->th;
   const CUtensorMap& tw = me->tw;
   const CUtensorMap& tw4 = me->tw4;
@@ -2867,6 +2922,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   kp.w_scale = a->w_scale;
   kp.h_scale = ctx->hid_scale;
   kp.h_scale2 = ctx->hid_scale ? ctx->hid_scale + ctx->max_rows : nullptr;
+  kp.bulk_logits = bulk_logits ? 1 : 0;
   kp.stream_logits = static_cast<double>(M) * a->V * 4.0 > 96e6 ? 1 : 0;     // beyond ~3/4 of the L2
   kp.group_width = mixed ? mx->group_width : nullptr;
   kp.group_row = mixed ? mx->group_row : nullptr;

@@ -1062,3 +1062,32 @@ def test_draft_entropy_of_rows_at_every_alignment(binding, B, k, H, V, qd):
     assert torch.all((out.draft_entropy.double() - want).abs() <= 1e-5 * math.log(V) + 1e-6)
     assert torch.allclose(host.draft_entropy.to(DEV), out.draft_entropy, atol=2e-6)
     assert int(out.status.item()) == 0
+
+
+@pytest.mark.parametrize("B,k,H,V,pad", [
+    (43, 5, 128, 3000, 0),       # 258 rows: N = 96, the last block of 16 rows is mostly past the end; ragged last quarter
+    (50, 5, 64, 40004, 0),       # 300 rows: N = 112, half a chunk per MMA; two tiles per pair, vocabulary ends inside a quarter
+    (64, 5, 128, 37888, 0),      # 384 rows, whole quarters only
+    (64, 5, 64, 2999, 0),        # rows that 16-byte pieces do not tile: lane by lane
+    (150, 4, 64, 5000, 0),       # 750 rows: two passes of 384 in one launch, the second ends inside a block
+    (64, 5, 64, 2996, 4),        # a caller's logits that do not start on a 16-byte boundary
+])
+def test_logits_of_rotating_units_land_where_they_belong(binding, B, k, H, V, pad):
+    """257..384 rows per pass: every logit against an fp64 product ((H / 16 + 16) 2^-23 of sum |terms|, fp32 accumulation), and
+    nothing around the buffer is touched."""
+    w = workloads.gaussian_head("bulk", B, k, H, V, seed=B + V, device=DEV, w_std=0.3)
+    guard = 64
+    flat = torch.full((B * (k + 1) * V + 2 * guard,), 777.0, device=DEV)
+    lo = guard + (1 if pad else 0)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        out = ctx.alloc_outputs(B, k)
+        out.logits = flat[lo:lo + B * (k + 1) * V].view(B, k + 1, V)
+        ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau, out=out)
+        inner = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)       # the context's own scratch
+        torch.cuda.synchronize()
+    assert int(out.status.item()) == 0
+    h, Wd = w.hidden.double().reshape(-1, H), w.W_lm.double()
+    want = h @ Wd.T
+    assert torch.all((out.logits.double().reshape(-1, V) - want).abs() <= (H / 16 + 16) * 2.0 ** -23 * (h.abs() @ Wd.abs().T))
+    assert torch.all(flat[:lo] == 777.0) and torch.all(flat[lo + B * (k + 1) * V:] == 777.0)
+    assert torch.equal(inner.next_tok, out.next_tok) and torch.equal(inner.accept_len, out.accept_len)
