@@ -1198,7 +1198,8 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     // store instructions of a chunk, their addresses and their way through the L1 bound the read-out of a tile, which a
     // small H does not hide: us, 384 rows, V = 32000, H = 128 29.9 -> 25.7, 512 34.8 -> 32.9 (8-bit 40.7 -> 37.1),
     // 4096 110.4 -> 108.5; 2304 rows, V = 128256, H = 8192 3715 -> 3685.  (With at most 256 rows the read-out hides under the
-    // next tile; the same stores there: one sequence 46.6 -> 49.5, 192 rows at 8 bits 141 -> 153.)
+    // next tile, and its bulk stores stand in the way of the next tile's loads: one sequence 47.3 -> 49.0, 240 rows 79 -> 86, 192 rows
+    // at 8 bits 136 -> 147.)
     const bool bulk = kRot && p.bulk_logits && quarter * 32 + 32 <= p.tile_rows;
     const uint32_t tbuf_addr = smem_u32(tbuf);
     const uint64_t pol_l = p.stream_logits ? l2_policy_evict_first() : l2_policy_evict_normal();
@@ -1586,16 +1587,28 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
   tc_fence_before();
   __syncthreads();
   grid_dependency_wait();                                // (every thread that writes below; long since satisfied)
+  // 8-bit modes: what the tail needs is worked out anew.  Values that lived through the epilogue's loops on its account were
+  // spilled (72 and 108 bytes of reloads, some of them per K block, by the threads that feed the tensor cores).  us: 192 rows,
+  // V = 128256 137.8 -> 135.6, two planes, V = 32000 118.9 -> 117.8.  (The other modes do not spill on its account and gain nothing.)
+  constexpr bool kAnew = kMode >= 2 && !kRot;
+  int bid = blockIdx.x, tid = threadIdx.x, pair_end = pair, row0_end = row0, rows_end = rows;
+  if (kAnew) {
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(bid));
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    pair_end = p.n_pass > 1 ? (bid >> 1) / p.n_pass : bid >> 1;
+    row0_end = p.n_pass > 1 ? ((bid >> 1) - pair_end * p.n_pass) * p.rows_per_pass : p.row0;
+    rows_end = p.n_pass > 1 ? min(p.rows_per_pass, p.M - row0_end) : p.rows;
+  }
   if (!*abort_flag) {
     // one partial per CTA and row: the eight contributions merged around their maximum
     const float4* merge = reinterpret_cast<const float4*>(smem);
-    for (int r = threadIdx.x; r < rows; r += kK1Threads) {
+    for (int r = tid; r < rows_end; r += kK1Threads) {
       float4 x[8];
       float m = -CUDART_INF_F, sum = 0.f, sum_t = 0.f;
       int arg = 0x7fffffff;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        x[q] = merge[q * rows + r];
+        x[q] = merge[q * rows_end + r];
         m = fmaxf(m, x[q].x);
       }
 #pragma unroll
@@ -1607,14 +1620,14 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           sum_t = fmaf(e, fmaf(d, x[q].y, x[q].z), sum_t);
         }
       }
-      p.partials[static_cast<size_t>(row0 + r) * p.part_stride + 2 * pair + rank] =
+      p.partials[static_cast<size_t>(row0_end + r) * p.part_stride + 2 * pair_end + (kAnew ? bid & 1 : static_cast<int>(rank))] =
           make_float4(m, sum, sum_t, __int_as_float(arg));
     }
   }
   cluster_sync_execution_only();                         // the peer no longer signals this CTA's barriers or tensor memory
-  if (warp == 1) {
+  if ((kAnew ? tid >> 5 : warp) == 1) {
     if (*abort_flag) __nanosleep(200000);                // let copies already in flight land before leaving
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc(kAnew ? *reinterpret_cast<volatile uint32_t*>(tmem_holder) : tmem_base, kTmemCols);
   }
 }
 
