@@ -805,7 +805,8 @@ __device__ __noinline__ double draft_slice_sum(const void* q, int q_dtype, int V
 // specialisation of its own because its epilogue holds a different set of values in registers).
 // kFew (mode 1): at most 32 verify rows, four epilogue warps and three groups of converters.
 // (tmap_w4 is the map of the logits buffer with kRot.)
-template <int kMode, bool kRot, bool kFew = false>
+// kWide: logits leave the staging buffer 16 bytes per lane (see the epilogue).
+template <int kMode, bool kRot, bool kFew = false, bool kWide = false>
 __global__ void __launch_bounds__(kK1Threads, 1)
 lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __grid_constant__ CUtensorMap tmap_w,
                        const __grid_constant__ CUtensorMap tmap_w4, const __grid_constant__ CUtensorMap tmap_w16,
@@ -1200,6 +1201,10 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
     // 4096 110.4 -> 108.5; 2304 rows, V = 128256, H = 8192 3715 -> 3685.  (With at most 256 rows the read-out hides under the
     // next tile, and its bulk stores stand in the way of the next tile's loads: one sequence 47.3 -> 49.0, 240 rows 79 -> 86, 192 rows
     // at 8 bits 136 -> 147.)
+    // kWide: they leave out of the staging buffer too, 16 bytes per lane, and half of the warps fold their statistics first and
+    // store then: in step, all sixteen wait for the store path (1400 cycles per chunk) and then for the exponentials (1400).
+    // From 128 rows on; fewer leave too little to store for the longer code (us, V = 32000: 240 rows, H = 512 25.8 -> 25.3, 1024
+    // 33.5 -> 32.7, 4096 80.8 -> 79.8; 96 rows 18.7 -> 18.9, one sequence 47.4 -> 47.8).
     const bool bulk = kRot && p.bulk_logits && quarter * 32 + 32 <= p.tile_rows;
     const uint32_t tbuf_addr = smem_u32(tbuf);
     const uint64_t pol_l = p.stream_logits ? l2_policy_evict_first() : l2_policy_evict_normal();
@@ -1420,7 +1425,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                 if (i < n_ok) v[i] = scaled<kMode>(v[i], w_scale, p.h_scale, r0 + i);
               if (kMode >= 2) asm volatile("" ::: "memory");     // the row scales eight at a time, not all 32 ahead
             }
-            if (vocab_ok) {
+            if (vocab_ok && !kWide) {
               float* dst = p.logits + static_cast<size_t>(r0) * p.ldl + vocab;
               if (n_ok == 32 && p.stream_logits) {       // (the common cases without a test per store)
 #pragma unroll
@@ -1445,6 +1450,21 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                   for (int i = 0; i < kTransRows; ++i)
                     tbuf[i * 32 + ((((lane >> 2) ^ (i & 7))) << 2) + (lane & 3)] = v[half * kTransRows + i];
                   __syncwarp();
+                  auto put = [&]() {                     // the 16 rows out of the staging buffer, 16 bytes per lane and row group
+                    float* dst = p.logits + static_cast<size_t>(r0 + half * kTransRows + (lane >> 3)) * p.ldl + vbase +
+                                 quarter * 32 + (lane & 7) * 4;
+#pragma unroll
+                    for (int it = 0; it < 4; ++it) {
+                      const int row = it * 4 + (lane >> 3);
+                      if (half * kTransRows + row < n_ok && (lane & 7) * 4 < nv) {
+                        const float4 x = *reinterpret_cast<const float4*>(tbuf + row * 32 + (((lane & 7) ^ (row & 7)) << 2));
+                        float4* d4 = reinterpret_cast<float4*>(dst + static_cast<size_t>(it * 4) * p.ldl);
+                        if (p.stream_logits) __stcs(d4, x);
+                        else *d4 = x;
+                      }
+                    }
+                  };
+                  if (kWide && !(group & 1)) put();
                   float e[16];
 #pragma unroll
                   for (int jj = 0; jj < 4; ++jj) {
@@ -1455,6 +1475,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                   // (rows at or beyond n_ok fold whatever the unused columns held; they are never written out)
                   if (n16 == 16) stats_fold16_packed(e, vocab16, st[slot][half]);
                   else if (n16 > 0) stats_fold16<false>(e, n16, vocab16, st[slot][half]);
+                  if (kWide && (group & 1)) put();
                 }
               }
             }
@@ -2899,6 +2920,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   }
   // Rotating units: the logits buffer, where its rows are whole 16-byte pieces; boxes of 16 rows x 32 entries, swizzled like
   // the staging buffers.
+  const bool wide_logits = !pl.rot && pl.N >= 128 && ldl % 4 == 0 && aligned16(logits) && a->V % 4 == 0;
   const bool bulk_logits = pl.rot && ldl % 4 == 0 && aligned16(logits);
   if (bulk_logits && (me->logits != logits || me->ldl != ldl)) {
     me->logits = nullptr;
@@ -2995,11 +3017,13 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     kp.clear_status = pass == 0 && (a->flags & HOLA_ARG_CLEAR_STATUS) && a->status_word;
     e = two ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<3, false>, th, tw, tw4, tw16, kp)
       : i8 ? (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, true>, th, tw, tw4, tw16, kp)
-                     : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, false>, th, tw, tw4, tw16, kp))
+             : wide_logits ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, false, false, true>, th, tw, tw4, tw16, kp)
+                           : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<2, false>, th, tw, tw4, tw16, kp))
       : few ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<1, false, true>, th, tw, tw4, tw16, kp)
       : w8 ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<1, false>, th, tw, tw4, tw16, kp)
            : (pl.rot ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, true>, th, tw, tw4, tw16, kp)
-                     : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, false>, th, tw, tw4, tw16, kp));
+             : wide_logits ? cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, false, false, true>, th, tw, tw4, tw16, kp)
+                           : cudaLaunchKernelEx(&cfg, lm_head_entropy_kernel<0, false>, th, tw, tw4, tw16, kp));
     if (e != cudaSuccess) { set_error(ctx, "launch lm_head_entropy_kernel", e); return HOLA_ERR_CUDA; }
   }
   return HOLA_OK;
@@ -3136,6 +3160,8 @@ hola_status check_sample_args(const hola_verify_args* a) {
 cudaError_t configure_kernels() {
   cudaError_t e = cudaSuccess;
   const void* kernels[] = {reinterpret_cast<const void*>(lm_head_entropy_kernel<0, false>),
+                           reinterpret_cast<const void*>(lm_head_entropy_kernel<0, false, false, true>),
+                           reinterpret_cast<const void*>(lm_head_entropy_kernel<2, false, false, true>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<0, true>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<1, false>),
                            reinterpret_cast<const void*>(lm_head_entropy_kernel<1, false, true>),
