@@ -2737,7 +2737,14 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int pairs = best.fused ? all_pairs / best.passes : all_pairs;     // pairs that divide the tiles among them
   const int rounds = (ctx->V + pairs * kPairTile - 1) / (pairs * kPairTile);
   int tile_rows = round_up((ctx->V + 2 * pairs * rounds - 1) / (2 * pairs * rounds), 4);
-  if (tile_rows < 104) tile_rows = round_up(tile_rows, 8);         // whole swizzle patterns: several K blocks per slot
+  // Whole swizzle patterns, so that a slot can take several K blocks: always where tiles are narrow; a tall tile pays for
+  // the rows added (up to 4 % of the busiest pair's work), which 32 K blocks per tile and more are worth, and rows that do
+  // not start on a 128-byte line (the next K block then finds its share of the line in the L2).  us: one sequence,
+  // V = 128256 172 -> 168, V = 50000, H = 2048 40.4 -> 39.2; 96 rows, V = 128256 210 -> 207; 92 rows, V = 50000, H = 4096
+  // 81.7 -> 79.8, V = 90004, H = 1032 53 -> 52; but 32 rows, V = 50003, H = 1024 20.9 -> 21.5 (8-bit, one sequence: within
+  // 1.5 % either way).
+  const int row_bytes = ctx->H * (i8 ? 1 : 2);
+  if (tile_rows < 104 || (!i8 && ctx->H >= 32 * kBlockK) || row_bytes % 128 != 0) tile_rows = round_up(tile_rows, 8);
   if (tile_rows < 8) tile_rows = 8;
   if (tile_rows > kLanes) tile_rows = kLanes;
   // Near and beyond the point where the tensor cores bound, a tile costs the same whatever its rows: as few tiles as
