@@ -192,8 +192,9 @@ size_t hola_workspace_bytes(int maxB, int maxK, int H, int V);
  * before their first read of any input.)
  * Only a kernel that the CALLER launches right behind this call with programmatic stream serialization must execute
  * griddepcontrol.wait (cudaGridDependencySynchronize) before it reads this call's outputs.  (2) With the
- * draft-entropy gate one kernel runs on a stream owned by the context, forked from and joined back to `cuda_stream`
- * by events (it stays on `cuda_stream` while that stream is being captured into a graph). */
+ * draft-entropy gate and more than 32 MB of draft rows (or 257..384 verify rows per pass) one kernel runs on a stream
+ * owned by the context, forked from and joined back to `cuda_stream` by events (it stays on `cuda_stream` while that
+ * stream is being captured into a graph). */
 hola_status hola_verify(hola_ctx* ctx, const hola_verify_args* args, void* cuda_stream);
 
 /* End-to-end form for callers whose per-step data lives in host memory.  Same computation as hola_verify, but
@@ -204,8 +205,9 @@ hola_status hola_verify(hola_ctx* ctx, const hola_verify_args* args, void* cuda_
  * crosses the bus: the k probabilities q_j(x_j) of each sequence, gathered on the host, and the one row q_n that the
  * residual draw of a sequence needs (none when all k drafts were kept or the fallback is greedy).  The first rows
  * of every sequence (as many as fit under the LM-head GEMM, at least row 0) are copied ahead on a stream owned by
- * the context while the GEMM runs; the accept lengths are read back once in the middle of the call and the rows
- * still missing follow.  Results are identical to hola_verify on the same data.  With the draft-entropy gate every
+ * the context behind the hidden rows, while the GEMM runs; a row still missing after the accept test is read in place
+ * over the bus by the accept/sample kernel where draft_q is pinned memory, and copied after a read-back of the accept
+ * lengths otherwise.  Results are identical to hola_verify on the same data.  With the draft-entropy gate every
  * draft row is read, and for small draft tensors the whole copy hides under the GEMM anyway: then the whole tensor
  * is copied (on the context's stream, under the GEMM).  HOLA_OPT_HOST_ROWS_ON_DEMAND forces one or the
  * other.  The host buffers must stay valid until the call returns. */

@@ -1010,6 +1010,8 @@ def test_fresh_outputs_start_with_a_clear_status_word_and_hold_every_field(bindi
     (44, 4, 320, 23680, "bf16"),      # 220 rows: two K blocks per slot
     (1, 4, 1040, 30000, "w8a8"), (9, 3, 1168, 9001, "w8a8"),      # K blocks of 128: a part of 16 channels; one of 16 beyond nine
     (5, 2, 528, 6000, "w8a16"), (30, 2, 256, 3000, "w8a16"),
+    (1, 4, 2048, 50003, "bf16"), (4, 3, 1032, 33000, "bf16"),     # tall tiles rounded up to 120 and 112 rows
+    (23, 3, 2056, 37880, "bf16"),     # 128 rows, a K block that H fills in part
 ])
 def test_several_k_blocks_per_slot(binding, B, k, H, V, weights):
     """Narrow tiles take two or four K blocks per ring slot.  Logits against fp64 products of the operands as the mode
