@@ -2736,7 +2736,17 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   best.fused = (best.passes > 1 && !ctx->no_fuse && all_pairs / best.passes >= 1) ? 1 : 0;
   const int pairs = best.fused ? all_pairs / best.passes : all_pairs;     // pairs that divide the tiles among them
   const int rounds = (ctx->V + pairs * kPairTile - 1) / (pairs * kPairTile);
-  int tile_rows = round_up((ctx->V + 2 * pairs * rounds - 1) / (2 * pairs * rounds), 4);
+  // One tile per pair: a tile costs the tensor cores and the traffic of the hidden rows the same whatever its height, and
+  // the statistics of all CTAs have to be merged, so as many pairs as there are is not the best split of a small vocabulary.
+  // At least 64 rows per CTA; with more than 96 operand rows no more than 42 pairs (still enough to stream W_lm through),
+  // with more than 256 as few pairs as there are tiles of 256.  us, H = 4096: V = 4000, 5 rows 16.6 -> 16.1, 96 rows 20.6 ->
+  // 20.0 (V = 12000 27.6 as it is, 28.4 on 47 pairs); V = 8000, 192 rows 34.6 -> 28.6 (29.6 on 32 pairs), 384 rows 57.4 ->
+  // 45.0, two planes of 192 rows 38.2 -> 35.4; V = 12000, 192 rows 37.4 -> 33.6, 384 rows 61.0 -> 51.4.
+  const int op_rows = best.n_sub * best.N;
+  int spread = pairs;
+  if (rounds == 1 && op_rows > 96) spread = op_rows > 256 ? 1 : (pairs < 42 ? pairs : 42);
+  int tile_rows = round_up((ctx->V + 2 * spread * rounds - 1) / (2 * spread * rounds), 4);
+  if (tile_rows < kLanes / 2) tile_rows = kLanes / 2;
   // Whole swizzle patterns, so that a slot can take several K blocks: always where tiles are narrow; a tall tile pays for
   // the rows added (up to 4 % of the busiest pair's work), which 32 K blocks per tile and more are worth, and rows that do
   // not start on a 128-byte line (the next K block then finds its share of the line in the L2).  us: one sequence,
@@ -2745,7 +2755,6 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   // 1.5 % either way).
   const int row_bytes = ctx->H * (i8 ? 1 : 2);
   if (tile_rows < 104 || (!i8 && ctx->H >= 32 * kBlockK) || row_bytes % 128 != 0) tile_rows = round_up(tile_rows, 8);
-  if (tile_rows < 8) tile_rows = 8;
   if (tile_rows > kLanes) tile_rows = kLanes;
   // Near and beyond the point where the tensor cores bound, a tile costs the same whatever its rows: as few tiles as
   // possible (the busiest pair has as many either way), because these loops run at the power cap and every MMA counts.
