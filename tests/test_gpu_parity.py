@@ -1012,6 +1012,9 @@ def test_fresh_outputs_start_with_a_clear_status_word_and_hold_every_field(bindi
     (5, 2, 528, 6000, "w8a16"), (30, 2, 256, 3000, "w8a16"),
     (1, 4, 2048, 50003, "bf16"), (4, 3, 1032, 33000, "bf16"),     # tall tiles rounded up to 120 and 112 rows
     (23, 3, 2056, 37880, "bf16"),     # 128 rows, a K block that H fills in part
+    (1, 4, 256, 100, "bf16"), (1, 4, 264, 129, "bf16"),           # one pair, its second CTA partly or almost empty
+    (32, 5, 320, 8005, "bf16"),       # 42 pairs at most
+    (64, 5, 320, 6001, "bf16"), (33, 5, 256, 6001, "w8a16"),      # one round of tiles of 256 rows
 ])
 def test_several_k_blocks_per_slot(binding, B, k, H, V, weights):
     """Narrow tiles take two or four K blocks per ring slot.  Logits against fp64 products of the operands as the mode
