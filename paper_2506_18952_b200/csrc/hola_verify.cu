@@ -3472,23 +3472,23 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   // V = 32000 62.6 -> 59.4, one 49.6 -> 47.4, V = 1000 12.8 -> 10.9, 4 sequences, V = 9000 17.5 -> 14.5).  Beyond that, and with
   // rotating units (whose epilogue has no register to spare: 384 rows, V = 32000 0.9 % slower with the code in it, V = 128256
   // 441 -> 448 with the gate), a kernel of its own does, on the context's side stream, behind the copy of the draft tensor
-  // where the host entry put one there; else it branches off the caller's stream before the GEMM and joins it again before
-  // the accept/sample kernel.  It is launched AFTER the GEMM so that the GEMM's CTAs get their SMs first; its small CTAs fit
-  // beside them.  (While the caller records a graph everything stays on the caller's stream.)
+  // where the host entry put one there.  It branches off the caller's stream before the GEMM and joins it again before the
+  // accept/sample kernel: earlier calls that are still queued on that stream write and read ctx->hq too.  It is launched
+  // AFTER the GEMM so that the GEMM's CTAs get their SMs first; its small CTAs fit beside them.  (While the caller records a
+  // graph everything stays on the caller's stream.)
   const bool draft_gate = a->gate_source == HOLA_GATE_DRAFT_ENTROPY && a->k > 0;
   const double q_bytes = static_cast<double>(a->B) * a->k * a->V * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
   const bool inside = draft_gate && !before_sample && !pl.rot && q_bytes <= 32e6;
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   if (draft_gate && !inside && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
   const bool side = draft_gate && !inside && (before_sample || capturing == cudaStreamCaptureStatusNone);
-  if (side && !before_sample && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
+  if (side && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
   const bool few_before = a->B * sample_cluster(ctx, a) * 4 <= ctx->num_sms;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample, inside);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
   if (side) {
-    cudaError_t e = cudaSuccess;
-    if (!before_sample) e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
+    cudaError_t e = cudaStreamWaitEvent(ctx->copy_stream, ctx->fork_point, 0);
     if (e == cudaSuccess) {
       draft_entropy_kernel<<<dim3(static_cast<unsigned>(a->B * a->k), kHqSlices), 256, 0, ctx->copy_stream>>>(
           a->draft_q, a->q_dtype, a->V, ctx->hq);

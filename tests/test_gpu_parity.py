@@ -1096,3 +1096,33 @@ def test_logits_of_rotating_units_land_where_they_belong(binding, B, k, H, V, pa
     assert torch.all((out.logits.double().reshape(-1, V) - want).abs() <= (H / 16 + 16) * 2.0 ** -23 * (h.abs() @ Wd.abs().T))
     assert torch.all(flat[:lo] == 777.0) and torch.all(flat[lo + B * (k + 1) * V:] == 777.0)
     assert torch.equal(inner.next_tok, out.next_tok) and torch.equal(inner.accept_len, out.accept_len)
+
+
+@pytest.mark.parametrize("B,k,H,V", [
+    (3, 4, 128, 4100),                        # the device entry's GEMM kernel makes the pass over the draft rows
+    (43, 5, 64, 4100),                        # a kernel of its own does, on the side stream
+])
+def test_host_entry_behind_queued_device_calls_keeps_their_draft_entropies_apart(binding, B, k, H, V):
+    """With the draft gate every call leaves H(q_j) in the context's scratch.  Device calls that are still queued when a host
+    call comes in gate on their own values, and the host call on its own."""
+    w = workloads.gaussian_head("queued", B, k, H, V, seed=91, device=DEV, w_std=0.3, tau=0.0)
+    flat = torch.full_like(w.draft_q, 1.0 / V)                # ln V everywhere: the gate never fires
+    peaked = torch.zeros_like(w.draft_q)                      # 0 everywhere: it always does
+    peaked[..., 0] = 1.0
+    tau = 1.0
+    host = [t.cpu().pin_memory() for t in (w.hidden, w.draft_tok, w.uniforms)]
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        for first, second in ((flat, peaked), (peaked, flat)):
+            q_host = second.cpu().pin_memory()
+            alone = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, first, w.uniforms, tau, gate_source=1)
+            torch.cuda.synchronize()
+            host_alone = ctx.hola_verify_host(host[0], w.W_lm, host[1], q_host, host[2], tau, gate_source=1)
+            torch.cuda._sleep(20_000_000)                     # some 10 ms of the stream: the host call's copies are long done
+            queued = [ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, first, w.uniforms, tau, gate_source=1) for _ in range(3)]
+            h = ctx.hola_verify_host(host[0], w.W_lm, host[1], q_host, host[2], tau, gate_source=1)
+            torch.cuda.synchronize()
+            for got, want in [(d, alone) for d in queued] + [(h, host_alone)]:
+                for f in ("draft_entropy", "accept_len", "next_tok"):
+                    assert torch.equal(getattr(got, f), getattr(want, f)), f
+        assert alone.draft_entropy.max() == 0.0 and torch.all(alone.accept_len == k)
+        assert h.draft_entropy.min() > 8.0
