@@ -2570,9 +2570,12 @@ struct Plan {
 }  // namespace
 
 // What a call needs besides its arguments, kept from one call to the next: the launch geometry of a (rows, weight
-// mode) pair and the two tensor maps of a (hidden pointer, W_lm pointer, rows, weight mode) quadruple.
+// mode) pair and the tensor maps of a (hidden pointer, W_lm pointer, rows, weight mode) quadruple.  The key holds all that
+// goes into a map: with mixed widths the three buffers and their row counts, because a head may be quantised anew, at other
+// widths, into the same memory.
 struct PlanEntry { int valid, M, w_dtype; Plan pl; };
 struct MapEntry { int valid, M, w_dtype; const void* hidden; const void* W; const void* W4; const void* W16;
+                  int rows8, rows4, rows16;
                   CUtensorMap th, tw, tw4, tw16;
                   const float* logits; int ldl; };       // rotating units: the logits buffer that tw4 maps (null: none)
 constexpr int kPlanCache = 8, kMapCache = 8;
@@ -2891,7 +2894,8 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   for (int i = 0; i < kMapCache; ++i) {
     MapEntry& c = ctx->maps[i];
     if (c.valid && c.hidden == hid_src && c.W == w_main && c.M == M && c.w_dtype == a->w_dtype &&
-        (!mixed || (c.W4 == mx->W4 && c.W16 == mx->W16))) { me = &c; break; }
+        (!mixed || (c.W4 == mx->W4 && c.W16 == mx->W16 && c.rows8 == mx->rows8 && c.rows4 == mx->rows4 &&
+                    c.rows16 == mx->rows16))) { me = &c; break; }
   }
   if (!me) {
     me = &ctx->maps[ctx->map_next];
@@ -2946,6 +2950,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
       if (mx->rows4 <= 0) me->tw4 = me->tw;
       if (mx->rows16 <= 0) me->tw16 = me->tw;
       me->W4 = mx->W4; me->W16 = mx->W16;
+      me->rows8 = mx->rows8; me->rows4 = mx->rows4; me->rows16 = mx->rows16;
     }
     me->hidden = hid_src; me->W = w_main; me->M = M; me->w_dtype = a->w_dtype; me->valid = 1;
   }

@@ -308,3 +308,33 @@ def test_quantisers_round_every_quotient_of_two_bf16_mantissas_like_the_division
     want = p1.double() * sa.double()[:, None] + p2.double() * sb.double()[:, None]
     assert torch.all((two.double() - want).abs() <= 2.0 ** -22 * want.abs() + 1e-30)       # one fused multiply-add
     assert torch.equal(((two - p1.float() * sa[:, None]) / sb[:, None]).round(), p2.float())
+
+
+def test_a_head_quantised_anew_into_the_same_buffers_is_the_one_that_is_used(binding):
+    """Other widths into the same (large enough) buffers, on one context: the same logits as a head in buffers of its own."""
+    import ctypes
+    B, k, H, V = 3, 2, 256, 1000
+    w = workloads.gaussian_head("anew", B, k, H, V, seed=8, device=DEV, w_std=0.3)
+    lib = binding.load_library()
+    buf = dict(W16=torch.empty((V, H), dtype=torch.bfloat16, device=DEV), W8=torch.empty((V, H), dtype=torch.int8, device=DEV),
+               W4=torch.empty((V, H // 2), dtype=torch.uint8, device=DEV),
+               shift4=torch.empty((H // 128 * V,), dtype=torch.uint8, device=DEV))
+    scale = torch.empty((V,), dtype=torch.float32, device=DEV)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        for widths in ([8, 16, 4, 8], [4, 8, 8, 16], [8, 8, 8, 4], [16, 4, 8, 4]):
+            own = binding.hola_quantize_mixed(w.W_lm, widths)
+            st = binding.hola_wmix()
+            for name, t in buf.items():
+                setattr(st, name, t.data_ptr())
+            st.group_width, st.group_row = own.group_width.data_ptr(), own.group_row.data_ptr()
+            st.rows16, st.rows8, st.rows4 = own.struct.rows16, own.struct.rows8, own.struct.rows4
+            assert lib.hola_quantize_mixed(ctypes.c_void_p(w.W_lm.data_ptr()), V, H, ctypes.byref(st),
+                                           ctypes.c_void_p(scale.data_ptr()), None) == 0
+            head = binding.MixedHead(V, H, widths, buf["W16"], buf["W8"], buf["W4"], buf["shift4"], scale, own.group_width,
+                                     own.group_row, st)
+            got = ctx.hola_lm_head_entropy(w.hidden, head)
+            with binding.HolaVerify(B, k, H, V) as other:
+                want = other.hola_lm_head_entropy(w.hidden, own)
+                torch.cuda.synchronize()
+            assert int(got.status.item()) == 0
+            assert torch.equal(got.logits, want.logits), widths
