@@ -333,6 +333,14 @@ hola_status hola_profile_end(hola_ctx* ctx, void* cuda_stream, double* lm_head_m
 hola_status hola_selftest_bounded_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word,
                                        uint32_t* counters, void* cuda_stream);
 
+/* The same for the wait of the accept/sample kernel on the rows it brings into shared memory: a cluster of two CTAs of 64
+ * threads, of which the second waits in vain, for `limit_cycles` SM cycles (1e3 .. 1e8) until it says so and for as long
+ * again until it goes on, and the first reports.  Afterwards *status_word has HOLA_FLAG_TIMEOUT set (OR-ed in),
+ * counters[0] = 128 (every thread reached the end), counters[1] = 64 (the waits that gave up) and counters[2] =
+ * HOLA_FLAG_TIMEOUT (what the first CTA reported).  counters is uint32 [3], zeroed by the call. */
+hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                      void* cuda_stream);
+
 const char* hola_strerror(hola_status s);
 /* Text of the last CUDA error seen by this context (empty string if none). */
 const char* hola_last_cuda_error(const hola_ctx* ctx);

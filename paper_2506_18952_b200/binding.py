@@ -26,7 +26,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -103,9 +103,10 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_profile_begin.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.hola_set_option.restype = ctypes.c_int
     lib.hola_set_option.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
-    lib.hola_selftest_bounded_wait.restype = ctypes.c_int
-    lib.hola_selftest_bounded_wait.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p,
-                                               ctypes.c_void_p]
+    for name in ("hola_selftest_bounded_wait", "hola_selftest_staged_wait"):
+        fn = getattr(lib, name)
+        fn.restype = ctypes.c_int
+        fn.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     lib.hola_shard_record_bytes.restype = ctypes.c_size_t
     lib.hola_shard_record_bytes.argtypes = [ctypes.c_int, ctypes.c_int]
     for name in ("hola_shard_lm_head", "hola_shard_accept", "hola_shard_sample"):
@@ -360,6 +361,17 @@ class HolaVerify:
         _check(self.lib, self._ctx, st, "hola_selftest_bounded_wait")
         (torch.cuda.current_stream() if stream is None else stream).synchronize()
         return int(status.item()), int(counters[0].item()), int(counters[1].item())
+
+    def hola_selftest_staged_wait(self, limit_cycles: int = 100000, stream=None) -> tuple[int, int, int, int]:
+        """Runs the self-test of the wait on staged rows; returns (status word, threads that reached the end, waits that gave
+        up, flags that the other CTA reported) after synchronising the stream."""
+        status = torch.zeros(1, dtype=torch.int32, device=self._dev)
+        counters = torch.zeros(3, dtype=torch.int32, device=self._dev)
+        st = self.lib.hola_selftest_staged_wait(self._ctx, int(limit_cycles), _dptr(status), _dptr(counters),
+                                                _stream_ptr(stream))
+        _check(self.lib, self._ctx, st, "hola_selftest_staged_wait")
+        (torch.cuda.current_stream() if stream is None else stream).synchronize()
+        return (int(status.item()), *counters.tolist())
 
     def hola_profile_begin(self, max_calls: int):
         _check(self.lib, self._ctx, self.lib.hola_profile_begin(self._ctx, max_calls), "hola_profile_begin")

@@ -22,7 +22,8 @@
 //   quantize_rows_kernel        the Lo-Bi quantiser on W_lm ahead of time: rows at 8 bits, at 4 bits (codes in [-7, 7], one
 //       shared exponent per sub-block of 128 channels) or in groups of mixed width, one launch for the whole head.
 //   quantize_hidden_kernel      the hidden rows of a call as one or two 8-bit planes.
-//   bounded_wait_selftest_kernel  a wait that is made to run out, to exercise the give-up path without breaking anything.
+//   bounded_wait_selftest_kernel, staged_wait_selftest_kernel  waits that are made to run out, to exercise the give-up paths
+//       without breaking anything.
 //   draft_entropy_kernel        H(q_j) of the draft rows, for the gate on the draft distribution.
 //   shard_record_kernel         vocabulary-parallel form: a rank's statistics record for the first all-gather.
 //   finalize_kernel             merges the per-CTA statistics:  logZ = m + ln s,  H = ln s - t/s  (entropy
@@ -1866,6 +1867,47 @@ __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
   return u;
 }
 
+// Waits for the staged rows of this CTA, whose own copies they are.  When the time is up the status word is told at once:
+// the CTA that draws the token, and reports, may be another one of the cluster, whose rows did land (it looks at the status
+// word behind the cluster barrier).  The copies then have as long again before the CTA goes on (and sooner or later leaves
+// the memory they write to).  False: gave up.
+__device__ __forceinline__ bool wait_staged_rows(uint32_t bar, unsigned* status, long long limit_cycles) {
+  const long long t0 = clock64();
+  bool late = false;
+  while (!mbar_try_wait(bar, 0u)) {
+    const long long waited = clock64() - t0;
+    if (waited > limit_cycles && !late) {
+      late = true;
+      if (status) atomicOr(status, HOLA_FLAG_TIMEOUT);
+    }
+    if (waited > 2 * limit_cycles) break;
+  }
+  return !late;
+}
+
+// The way that wait gives up, in miniature: a cluster of two CTAs, of which the second waits on a barrier that nothing ever
+// arrives on.  The first, whose barrier is complete, must find the time-out in the status word when it reports.
+// out[0] counts the threads that reached the end, out[1] the waits that gave up, out[2] is the word of flags that the first
+// CTA leaves.
+__global__ void __launch_bounds__(64, 1) staged_wait_selftest_kernel(long long limit_cycles, unsigned* status, unsigned* out) {
+  __shared__ __align__(8) uint64_t bar;
+  const uint32_t rank = cluster_cta_rank();
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&bar), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (rank == 0) mbar_arrive(smem_u32(&bar));
+  }
+  __syncthreads();
+  if (!wait_staged_rows(smem_u32(&bar), status, limit_cycles)) atomicAdd(out + 1, 1u);
+  cluster_sync_all();
+  if (rank == 0 && threadIdx.x == 0) {
+    K3Params p;
+    p.status = status; p.flags_out = out + 2;
+    report_flags(p, 0, 0u);
+  }
+  atomicAdd(out, 1u);
+}
+
 // One cluster of S CTAs per sequence.  Every CTA derives accept_len on its own (same inputs, same arithmetic,
 // same result), sums the residual mass of its slice of the vocabulary chunk by chunk, and publishes its slice
 // total to all CTAs of the cluster through distributed shared memory.  After one cluster barrier each CTA knows
@@ -2026,15 +2068,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const void* qrow = n >= k ? nullptr
                    : staged ? static_cast<const void*>(sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem)
                             : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
-  if (staged && here > 0) {                              // (bounded, and only this CTA's own copies to wait for)
-    const long long t0 = clock64();
-    while (!mbar_try_wait(smem_u32(&sh_bar), 0u)) {
-      if (clock64() - t0 > kWaitLimitCycles) {
-        flags |= HOLA_FLAG_TIMEOUT;
-        break;
-      }
-    }
-  }
+  if (staged && here > 0) wait_staged_rows(smem_u32(&sh_bar), p.status, kWaitLimitCycles);
   // Several CTAs per SM and short slices (up to 8192 entries): a slice into the L2 by two bulk requests instead of by the loads
   // alone.  us, V = 32000, H = 512, 384 rows 33.2 -> 32.5, 240 rows 25.3 -> 24.7; V = 128256 (16032 entries) no gain.  With a CTA
   // per SM the loads are all out at once, and the code alone costs 0.2 us, hence a kernel without it.
@@ -3427,6 +3461,25 @@ hola_status hola_selftest_bounded_wait(hola_ctx* ctx, long long limit_cycles, ui
   const cudaError_t e = cudaLaunchKernelEx(&cfg, bounded_wait_selftest_kernel, limit_cycles,
                                            static_cast<unsigned*>(status_word), static_cast<unsigned*>(counters));
   if (e != cudaSuccess) { set_error(ctx, "launch bounded_wait_selftest_kernel", e); return HOLA_ERR_CUDA; }
+  return HOLA_OK;
+}
+
+hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                      void* cuda_stream) {
+  if (!ctx || !status_word || !counters) return HOLA_ERR_INVALID_ARG;
+  if (limit_cycles < 1000 || limit_cycles > 100000000ll) return HOLA_ERR_INVALID_ARG;   // (twice that is waited at most)
+  DeviceGuard guard(ctx->device);
+  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  if (cudaMemsetAsync(counters, 0, 3 * sizeof(uint32_t), stream) != cudaSuccess) return HOLA_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2); cfg.blockDim = dim3(64); cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, staged_wait_selftest_kernel, limit_cycles,
+                                           static_cast<unsigned*>(status_word), static_cast<unsigned*>(counters));
+  if (e != cudaSuccess) { set_error(ctx, "launch staged_wait_selftest_kernel", e); return HOLA_ERR_CUDA; }
   return HOLA_OK;
 }
 

@@ -1126,3 +1126,19 @@ def test_host_entry_behind_queued_device_calls_keeps_their_draft_entropies_apart
                     assert torch.equal(getattr(got, f), getattr(want, f)), f
         assert alone.draft_entropy.max() == 0.0 and torch.all(alone.accept_len == k)
         assert h.draft_entropy.min() > 8.0
+
+
+def test_a_staged_wait_that_runs_out_is_reported_by_the_cta_that_draws(binding):
+    """The wait of the accept/sample kernel on the rows it brings into shared memory, in miniature: it runs out in one CTA of
+    a cluster, and another one, whose own wait was satisfied, is the one that reports."""
+    w = workloads.gaussian_head("after-staged", 2, 3, 128, 3000, seed=6, device=DEV, w_std=0.3)
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        for limit in (20000, 100000):
+            assert ctx.hola_selftest_staged_wait(limit) == (binding.FLAG_TIMEOUT, 128, 64, binding.FLAG_TIMEOUT)
+        for bad in (10, 10 ** 12):
+            with pytest.raises(binding.HolaError):
+                ctx.hola_selftest_staged_wait(bad)
+        got = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)      # (rows staged, small batch)
+        torch.cuda.synchronize()
+        assert int(got.status.item()) == 0
+    check_against_oracle(binding, w, out=got, want_logits=False)
