@@ -1142,3 +1142,27 @@ def test_a_staged_wait_that_runs_out_is_reported_by_the_cta_that_draws(binding):
         torch.cuda.synchronize()
         assert int(got.status.item()) == 0
     check_against_oracle(binding, w, out=got, want_logits=False)
+
+
+def test_fresh_outputs_are_an_ordinary_dataclass(binding):
+    """Outputs that a call allocates itself can be copied, replaced and taken apart like those of alloc_outputs, the fields
+    that the call did not fill included."""
+    import copy
+    import dataclasses
+    import pickle
+    w = workloads.gaussian_head("plain", 3, 2, 64, 300, seed=2, device=DEV, w_std=0.3)
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        full = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)
+        stats = ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
+        torch.cuda.synchronize()
+    want = {"accept_len": (torch.int32, (3,)), "next_tok": (torch.int32, (3,)), "draft_entropy": (torch.float32, (3, 2))}
+    for out in (full, stats):
+        assert type(out) is binding.VerifyOutputs
+        for twin in (dataclasses.replace(out, status=None), copy.copy(out), copy.deepcopy(out), pickle.loads(pickle.dumps(out))):
+            assert type(twin) is binding.VerifyOutputs and torch.equal(twin.entropy, out.entropy)
+            for name, (dtype, shape) in want.items():
+                assert getattr(twin, name).dtype == dtype and tuple(getattr(twin, name).shape) == shape, name
+        assert dataclasses.replace(out, accept_len=None).accept_len is None
+        assert set(dataclasses.asdict(out)) == {f.name for f in dataclasses.fields(binding.VerifyOutputs)}
+        assert not hasattr(out, "no_such_field")
+    assert binding.VerifyOutputs(1, 2, 3, 4, 5, 6).draft_entropy is None
