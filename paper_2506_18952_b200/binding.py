@@ -409,9 +409,16 @@ class HolaVerify:
         if uniforms is not None:
             a.uniforms = uniforms.data_ptr()
         a.tau = float(tau)
+        # (an output that is missing stays a null pointer, which the library refuses where it needs it)
         if draws:
-            a.accept_len, a.next_tok = out.accept_len.data_ptr(), out.next_tok.data_ptr()
-        a.entropy, a.logZ = out.entropy.data_ptr(), out.logZ.data_ptr()
+            if (t := out.accept_len) is not None:
+                a.accept_len = t.data_ptr()
+            if (t := out.next_tok) is not None:
+                a.next_tok = t.data_ptr()
+        if out.entropy is not None:
+            a.entropy = out.entropy.data_ptr()
+        if out.logZ is not None:
+            a.logZ = out.logZ.data_ptr()
         if out.logits is not None:
             a.logits_out = out.logits.data_ptr()
         if out.status is not None:

@@ -1166,3 +1166,19 @@ def test_fresh_outputs_are_an_ordinary_dataclass(binding):
         assert set(dataclasses.asdict(out)) == {f.name for f in dataclasses.fields(binding.VerifyOutputs)}
         assert not hasattr(out, "no_such_field")
     assert binding.VerifyOutputs(1, 2, 3, 4, 5, 6).draft_entropy is None
+
+
+def test_missing_output_tensors_are_refused_by_the_library(binding):
+    w = workloads.gaussian_head("missing", 2, 2, 64, 300, seed=2, device=DEV, w_std=0.3)
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        for name in ("accept_len", "next_tok", "entropy", "logZ"):
+            out = ctx.alloc_outputs(w.B, w.k)
+            setattr(out, name, None)
+            with pytest.raises(binding.HolaError, match="invalid argument"):
+                ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau, out=out)
+            if name in ("entropy", "logZ"):
+                with pytest.raises(binding.HolaError, match="invalid argument"):
+                    ctx.hola_lm_head_entropy(w.hidden, w.W_lm, out=out)
+            else:                                             # statistics only: not needed
+                ctx.hola_lm_head_entropy(w.hidden, w.W_lm, out=out)
+        torch.cuda.synchronize()
