@@ -204,9 +204,14 @@ def hola_quantize_mixed(W_lm: torch.Tensor, widths, stream=None) -> MixedHead:
     for wd in widths:
         group_row.append(rows[wd])
         rows[wd] += GROUP_ROWS
-    rows[widths[-1]] -= ng * GROUP_ROWS - V                      # the last group may be ragged
-    tables = torch.frombuffer(bytearray(group_row.tobytes() + bytes(widths)), dtype=torch.uint8)
+    if ng:
+        rows[widths[-1]] -= ng * GROUP_ROWS - V                  # the last group may be ragged
+        tables = torch.frombuffer(bytearray(group_row.tobytes() + bytes(widths)), dtype=torch.uint8)
+    else:
+        tables = torch.empty(0, dtype=torch.uint8)
     s = torch.cuda.current_stream(dev) if stream is None else stream
+    if not isinstance(s, torch.cuda.Stream):                     # (as elsewhere, whatever has a cuda_stream)
+        s = torch.cuda.ExternalStream(s.cuda_stream, device=dev)
     with torch.cuda.device(dev), torch.cuda.stream(s):
         W16 = torch.empty((rows[16], H), dtype=torch.bfloat16, device=dev) if rows[16] else None
         W8 = torch.empty((rows[8], H), dtype=torch.int8, device=dev) if rows[8] else None
@@ -221,8 +226,9 @@ def hola_quantize_mixed(W_lm: torch.Tensor, widths, stream=None) -> MixedHead:
         st.group_width, st.group_row = head.group_width.data_ptr(), head.group_row.data_ptr()
         st.rows16, st.rows8, st.rows4 = rows[16], rows[8], rows[4]
         head.struct = st
-        _check(lib, None, lib.hola_quantize_mixed(_dptr(W_lm), V, H, ctypes.byref(st), _dptr(w_scale), _stream_ptr(s)),
-               "hola_quantize_mixed")
+        if V:
+            _check(lib, None, lib.hola_quantize_mixed(_dptr(W_lm), V, H, ctypes.byref(st), _dptr(w_scale), _stream_ptr(s)),
+                   "hola_quantize_mixed")
     return head
 
 

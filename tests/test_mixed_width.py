@@ -338,3 +338,19 @@ def test_a_head_quantised_anew_into_the_same_buffers_is_the_one_that_is_used(bin
                 torch.cuda.synchronize()
             assert int(got.status.item()) == 0
             assert torch.equal(got.logits, want.logits), widths
+
+
+def test_quantiser_takes_an_empty_head_and_any_object_with_a_cuda_stream(binding):
+    import types
+    empty = binding.hola_quantize_mixed(torch.empty((0, 128), dtype=torch.bfloat16, device=DEV), [])
+    assert empty.V == 0 and empty.weight_bytes() == 0 and empty.group_width.numel() == 0 and empty.group_row.numel() == 0
+    g = torch.Generator(device=DEV).manual_seed(1)
+    W = torch.randn((700, 256), generator=g, device=DEV).bfloat16()
+    want = binding.hola_quantize_mixed(W, [4, 8, 16])
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for stream in (side, types.SimpleNamespace(cuda_stream=side.cuda_stream)):
+        got = binding.hola_quantize_mixed(W, [4, 8, 16], stream=stream)
+        side.synchronize()
+        for name in ("W16", "W8", "W4", "shift4", "w_scale", "group_width", "group_row"):
+            assert torch.equal(getattr(got, name), getattr(want, name)), name
