@@ -3668,8 +3668,7 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
   d.logZ = reinterpret_cast<float*>(ctx->st_out + ob.logZ);
   d.logits_out = nullptr; d.status_word = reinterpret_cast<uint32_t*>(ctx->st_out); d.draft_entropy = nullptr;
   d.flags = HOLA_ARG_CLEAR_STATUS;
-  hola_status s = check_lm_head_args(ctx, &d);
-  if (s != HOLA_OK) return s;
+  hola_status s;
   const Plan& pl = plan_for(ctx, B * (k + 1), a->w_dtype);
   if ((s = run_lm_head(ctx, &d, ctx->logits, ctx->ldl, pl, stream)) != HOLA_OK) return s;
   // Where the caller's draft tensor is pinned host memory that the device can address, the rows still missing after the
@@ -3787,7 +3786,11 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   hola_status s = check_common(ctx, a);
   if (s != HOLA_OK) return s;
   if (a->B == 0) return HOLA_OK;
-  if (!a->hidden || (!a->W_lm && a->w_dtype != HOLA_W_MIXED)) return HOLA_ERR_INVALID_ARG;
+  if (!a->hidden) return HOLA_ERR_INVALID_ARG;
+  // (what is refused is refused before any copy is queued: the caller's buffers need not outlive the call)
+  hola_verify_args staged = *a;
+  staged.hidden = ctx->st_hidden;
+  if ((s = check_lm_head_args(ctx, &staged)) != HOLA_OK) return s;
   if ((s = check_sample_args(a)) != HOLA_OK) return s;
   DeviceGuard guard(ctx->device);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
@@ -3846,7 +3849,6 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
   d.flags = HOLA_ARG_CLEAR_STATUS;
   const bool want_dent = a->draft_entropy && a->gate_source == HOLA_GATE_DRAFT_ENTROPY;
   d.draft_entropy = a->draft_entropy ? reinterpret_cast<float*>(ctx->st_out + ob.dent) : nullptr;
-  if ((s = check_lm_head_args(ctx, &d)) != HOLA_OK) return s;
   const bool direct = outputs_to_host(ctx, &d, ob);
   s = verify_device(ctx, &d, stream, overlap ? ctx->copy_done : nullptr);
   ctx->flags_out = nullptr;

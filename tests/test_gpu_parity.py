@@ -1182,3 +1182,23 @@ def test_missing_output_tensors_are_refused_by_the_library(binding):
             else:                                             # statistics only: not needed
                 ctx.hola_lm_head_entropy(w.hidden, w.W_lm, out=out)
         torch.cuda.synchronize()
+
+
+def test_host_entry_refuses_before_it_queues_anything(binding):
+    """Buffers of a refused call are the caller's again at once: nothing may still be copying from them."""
+    B, k, H, V = 256, 8, 8200, 64                             # H is no multiple of 16: refused with an 8-bit head
+    hidden = torch.zeros((B, k + 1, H), dtype=torch.bfloat16).pin_memory()      # 38 MB, most of a millisecond on the bus
+    tok = torch.zeros((B, k), dtype=torch.int32).pin_memory()
+    q = torch.full((B, k, V), 1.0 / V).pin_memory()
+    u = torch.full((B, k + 1), 0.5).pin_memory()
+    W = torch.zeros((V, H), dtype=torch.int8, device=DEV)
+    scale = torch.ones((V,), device=DEV)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        torch.cuda.synchronize()
+        for lazy in (0, 1):
+            ctx.hola_set_option(binding.HOLA_OPT_HOST_ROWS_ON_DEMAND, lazy)
+            with pytest.raises(binding.HolaError, match="unsupported shape"):
+                ctx.hola_verify_host(hidden, W, tok, q, u, 1.0, w_scale=scale)
+            idle = torch.cuda.current_stream().query()
+            torch.cuda.synchronize()
+            assert idle
