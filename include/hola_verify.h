@@ -110,7 +110,8 @@ typedef struct hola_wmix {
 
 /* Bits of hola_verify_args::flags. */
 #define HOLA_ARG_CLEAR_STATUS 1 /* the call stores 0 to status_word before it OR-s anything in, so the caller need not  */
-                                /* (calls that run the LM head; one stream operation less per call)                   */
+                                /* (calls that run the LM head, an empty batch included; one stream operation less per  */
+                                /* call).  Other bits are not looked at; leave them 0.                                 */
 
 typedef struct {
   int32_t B; /* sequences, >= 0 */

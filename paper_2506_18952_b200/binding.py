@@ -281,7 +281,7 @@ class VerifyOutputs:
 def _fresh_outputs(ctx: "HolaVerify", B: int, k1: int, want_logits: bool, draws: bool, draft_gate: bool) -> VerifyOutputs:
     """Outputs a call makes for itself: only the tensors that it fills are allocated (one allocation costs the host as
     much as a fifth of a call), the others when somebody asks for them.  The status word is cleared by the call
-    (HOLA_ARG_CLEAR_STATUS); an empty batch launches nothing."""
+    (HOLA_ARG_CLEAR_STATUS)."""
     out = VerifyOutputs.__new__(VerifyOutputs)
     dev = ctx._dev
     out._lazy = (B, k1 - 1, dev)
@@ -289,7 +289,7 @@ def _fresh_outputs(ctx: "HolaVerify", B: int, k1: int, want_logits: bool, draws:
     out.entropy = e = torch.empty(B, k1, dtype=torch.float32, device=dev)
     out.logZ = torch.empty_like(e)
     out.logits = torch.empty(B, k1, ctx.V, dtype=torch.float32, device=dev) if want_logits else None
-    out.status = (torch.empty if B else torch.zeros)(1, dtype=torch.int32, device=dev)
+    out.status = torch.empty(1, dtype=torch.int32, device=dev)
     if draws:
         out.accept_len = a = torch.empty(B, dtype=torch.int32, device=dev)
         out.next_tok = torch.empty_like(a)

@@ -3261,6 +3261,17 @@ struct DeviceGuard {
   ~DeviceGuard() { if (changed) cudaSetDevice(prev); }
 };
 
+// An empty batch launches nothing; all there is to do is what HOLA_ARG_CLEAR_STATUS promises.
+hola_status empty_batch(const hola_verify_args* a, void* cuda_stream) {
+  if (!(a->flags & HOLA_ARG_CLEAR_STATUS) || !a->status_word) return HOLA_OK;
+  return cudaMemsetAsync(a->status_word, 0, sizeof(uint32_t), static_cast<cudaStream_t>(cuda_stream)) == cudaSuccess ? HOLA_OK
+                                                                                                                  : HOLA_ERR_CUDA;
+}
+hola_status empty_batch(const hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {
+  DeviceGuard guard(ctx->device);
+  return empty_batch(a, cuda_stream);
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------------------------------------ C ABI
@@ -3486,7 +3497,7 @@ hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uin
 hola_status hola_lm_head_entropy(hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {
   hola_status s = check_common(ctx, a);
   if (s != HOLA_OK) return s;
-  if (a->B == 0) return HOLA_OK;
+  if (a->B == 0) return empty_batch(ctx, a, cuda_stream);
   if ((s = check_lm_head_args(ctx, a)) != HOLA_OK) return s;
   if (!a->entropy || !a->logZ) return HOLA_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
@@ -3736,7 +3747,7 @@ extern "C" {
 hola_status hola_verify(hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {
   hola_status s = check_common(ctx, a);
   if (s != HOLA_OK) return s;
-  if (a->B == 0) return HOLA_OK;
+  if (a->B == 0) return empty_batch(ctx, a, cuda_stream);
   if ((s = check_lm_head_args(ctx, a)) != HOLA_OK) return s;
   if ((s = check_sample_args(a)) != HOLA_OK) return s;
   DeviceGuard guard(ctx->device);
@@ -3785,7 +3796,10 @@ hola_status hola_profile_end(hola_ctx* ctx, void* cuda_stream, double* lm_head_m
 hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {
   hola_status s = check_common(ctx, a);
   if (s != HOLA_OK) return s;
-  if (a->B == 0) return HOLA_OK;
+  if (a->B == 0) {                                       // (the status word is the caller's host memory here)
+    if ((a->flags & HOLA_ARG_CLEAR_STATUS) && a->status_word) *a->status_word = 0u;
+    return HOLA_OK;
+  }
   if (!a->hidden) return HOLA_ERR_INVALID_ARG;
   // (what is refused is refused before any copy is queued: the caller's buffers need not outlive the call)
   hola_verify_args staged = *a;
@@ -3895,7 +3909,7 @@ static ShardLaunch shard_launch(const hola_verify_args* a, const hola_shard_args
 hola_status hola_shard_lm_head(hola_ctx* ctx, const hola_verify_args* a, const hola_shard_args* sh, void* cuda_stream) {
   hola_status s = check_common(ctx, a);
   if (s != HOLA_OK) return s;
-  if (a->B == 0) return HOLA_OK;
+  if (a->B == 0) return empty_batch(ctx, a, cuda_stream);
   if ((s = check_lm_head_args(ctx, a)) != HOLA_OK) return s;
   if ((s = check_shard(ctx, a, sh)) != HOLA_OK) return s;
   if (!sh->record_out || !aligned16(sh->record_out) || (a->k > 0 && !a->draft_tok)) return HOLA_ERR_INVALID_ARG;
@@ -4056,7 +4070,7 @@ hola_status static_setup(int dev, hola_ctx* out) {
 extern "C" hola_status hola_lm_head_entropy_static(const hola_verify_args* a, void* cuda_stream) {
   if (!a) return HOLA_ERR_INVALID_ARG;
   if (a->B < 0 || a->k < 0 || a->H <= 0 || a->V <= 0) return HOLA_ERR_INVALID_ARG;
-  if (a->B == 0) return HOLA_OK;
+  if (a->B == 0) return empty_batch(a, cuda_stream);
   if (!a->hidden || !a->W_lm || !a->logits_out || !a->entropy || !a->logZ) return HOLA_ERR_INVALID_ARG;
   if (!aligned16(a->hidden) || !aligned16(a->W_lm)) return HOLA_ERR_INVALID_ARG;
   if (a->H % 8 != 0) return HOLA_ERR_UNSUPPORTED_SHAPE;

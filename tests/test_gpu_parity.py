@@ -1202,3 +1202,26 @@ def test_host_entry_refuses_before_it_queues_anything(binding):
             idle = torch.cuda.current_stream().query()
             torch.cuda.synchronize()
             assert idle
+
+
+def test_an_empty_batch_clears_the_status_word_when_asked_to(binding):
+    import ctypes
+    w = workloads.gaussian_head("empty", 2, 2, 64, 300, seed=2, device=DEV, w_std=0.3)
+    e = w.slice([])
+    lib = binding.load_library()
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        def status_after(fn, device, flags, *more, own_ctx=True):
+            out = ctx.alloc_outputs(0, w.k, True, device=device)
+            out.status.fill_(64)
+            a = ctx._args(e.hidden, w.W_lm, e.draft_tok, e.draft_q, e.uniforms, 1.0, out, 0, w.k)
+            a.flags = flags
+            assert fn(*([ctx._ctx] if own_ctx else []), ctypes.byref(a), *more, None) == 0
+            torch.cuda.synchronize()
+            return int(out.status.item())
+        for flags, want in ((binding.HOLA_ARG_CLEAR_STATUS, 0), (0, 64)):
+            assert status_after(lib.hola_verify, DEV, flags) == want
+            assert status_after(lib.hola_lm_head_entropy, DEV, flags) == want
+            assert status_after(lib.hola_shard_lm_head, DEV, flags, ctypes.byref(binding.hola_shard_args())) == want
+            assert status_after(lib.hola_lm_head_entropy_static, DEV, flags, own_ctx=False) == want
+            assert status_after(lib.hola_verify_host, "cpu", flags) == want
+        assert int(ctx.hola_verify(e.hidden, w.W_lm, e.draft_tok, e.draft_q, e.uniforms, 1.0).status.item()) == 0
