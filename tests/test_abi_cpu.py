@@ -90,7 +90,7 @@ def test_launch_geometry_for_shapes_without_a_device():
                     continue
                 p = b.hola_plan_for_shape(sms, H, V, rows, wd)
                 what = (H, V, rows, wd, p)
-                cap = 256 if wd in expansion or wd == b.HOLA_W8A16 else 512
+                cap = 192 if wd in expansion else 256 if wd == b.HOLA_W8A16 else 512
                 assert 1 <= p["rows_per_pass"] <= cap, what
                 assert p["passes"] == -(-rows // p["rows_per_pass"]), what            # no empty pass, every row covered
                 assert p["grid"] % 2 == 0 and 2 <= p["grid"] <= sms, what

@@ -904,7 +904,7 @@ def test_wide_head_config(binding):
     (150, 5, 256, 9000, "bf16"),       # 900 rows: several passes, the last one ragged; more tiles than groups of pairs
     (150, 5, 256, 700, "bf16"),        # three tiles only: fewer tiles than groups of pairs
     (100, 7, 128, 5000, "w8a8"),       # 800 rows on the 8-bit kind
-    (130, 3, 256, 4000, "mixed"),      # 520 rows, at most 256 per pass in the on-chip expansion
+    (130, 3, 256, 4000, "mixed"),      # 520 rows, at most 192 per pass in the on-chip expansion
 ])
 def test_all_passes_in_one_launch_match_the_oracle_and_the_launch_per_pass(binding, B, k, H, V, weights):
     """More verify rows than one pass over W_lm holds: by default every pass runs in the same launch (groups of CTA
@@ -1225,3 +1225,40 @@ def test_an_empty_batch_clears_the_status_word_when_asked_to(binding):
             assert status_after(lib.hola_lm_head_entropy_static, DEV, flags, own_ctx=False) == want
             assert status_after(lib.hola_verify_host, "cpu", flags) == want
         assert int(ctx.hola_verify(e.hidden, w.W_lm, e.draft_tok, e.draft_q, e.uniforms, 1.0).status.item()) == 0
+
+
+@pytest.mark.parametrize("lazy,in_place", [(0, 1), (1, 1), (1, 0)])
+@pytest.mark.parametrize("gate,fallback", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_host_entry_reports_the_flags_of_every_sequence(binding, lazy, in_place, gate, fallback):
+    """A bad token, a bad uniform and a vanishing residual, each in a sequence of its own and alone or together: the host
+    entry's status word (whose bits come back as a word per sequence) against the oracle's flags and the device entry's."""
+    B, k, H, V = 6, 3, 64, 3000
+    w = workloads.gaussian_head("host-flags", B, k, H, V, seed=3, device=DEV, w_std=0.3, q_dtype=torch.float32, tau=0.0)
+    base = [t.clone() for t in (w.draft_tok, w.draft_q, w.uniforms)]
+    double = 2.0 * torch.softmax(workloads._target_logits(w.hidden, w.W_lm)[4, :k], -1)        # q = 2 p: R = 0
+    seen = set()
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        ctx.hola_set_option(binding.HOLA_OPT_HOST_ROWS_ON_DEMAND, lazy)
+        ctx.hola_set_option(binding.HOLA_OPT_HOST_IN_PLACE, in_place)
+        for faults in ((), ("token",), ("uniform",), ("mass",), ("token", "uniform", "mass"), ()):
+            w.draft_tok, w.draft_q, w.uniforms = (t.clone() for t in base)
+            if "token" in faults:
+                w.draft_tok[0, 0] = V
+            if "uniform" in faults:
+                w.uniforms[2, k] = 1.0
+            if "mass" in faults:
+                w.draft_q[4], w.uniforms[4, 0] = double, 0.75
+            orc = compare.run_oracle(w, keep_logits=True, gate_source=gate, fallback=fallback)
+            want = int(np.bitwise_or.reduce(orc.flags))
+            d = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau, gate_source=gate, fallback=fallback)
+            torch.cuda.synchronize()
+            pin = [t.cpu().pin_memory() for t in (w.hidden, w.draft_tok, w.draft_q, w.uniforms)]
+            out = ctx.alloc_outputs(B, k, device=torch.device("cpu"))
+            out.status.fill_(64)                              # (overwritten, not added to)
+            h = ctx.hola_verify_host(pin[0], w.W_lm, pin[1], pin[2], pin[3], w.tau, out=out, gate_source=gate, fallback=fallback)
+            assert int(d.status.item()) == want and int(h.status.item()) == want, (faults, want)
+            assert torch.equal(h.accept_len, d.accept_len.cpu()) and torch.equal(h.next_tok, d.next_tok.cpu())
+            seen.add(want)
+    if fallback == 0:
+        every = binding.FLAG_BAD_TOKEN | binding.FLAG_BAD_UNIFORM | binding.FLAG_R_ZERO
+        assert {0, binding.FLAG_BAD_TOKEN, binding.FLAG_BAD_UNIFORM, binding.FLAG_R_ZERO, every} <= seen
