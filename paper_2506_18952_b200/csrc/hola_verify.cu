@@ -1404,16 +1404,15 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
 #pragma unroll
       for (int slot = 0; slot < kSlots; ++slot) {
         if (slot < my_chunks) {
-          const int ch = rot ? slot * sub_chunks + group : group + slot * kGroups;
+          const int ch = group + slot * kGroups;
           const int sub = ch / sub_chunks, j = ch - sub * sub_chunks;
-          const int unit = (3 * t + slot) & 3;           // (rotating accumulators only)
           float v[32];
           __syncwarp();                                  // tcgen05.ld is warp-collective: reconverge first
-          tmem_ld32(lane_addr + (rot ? unit * 128 : kW8 ? buf * p.acc_cols : buf * 256 + sub * 256) + j * 32, v);
-          if (rot || slot == my_chunks - 1) {            // this warp's accumulators (of this unit) may be overwritten
+          tmem_ld32(lane_addr + (kW8 ? buf * p.acc_cols : buf * 256 + sub * 256) + j * 32, v);
+          if (slot == my_chunks - 1) {                   // this warp's accumulators may be overwritten
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * (rot ? unit : buf));
+            if (lane == 0) mbar_arrive_cluster(leader_tempty + 8 * buf);
           }
           const int c0 = j * 32;                         // first column of the chunk inside its MMA
           const int r0 = row0 + sub * p.N + c0;        // verify row of column c0
