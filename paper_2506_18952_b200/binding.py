@@ -8,7 +8,7 @@ from __future__ import annotations
 import ctypes
 import os
 from array import array
-from dataclasses import dataclass, field
+from dataclasses import dataclass
 
 import torch
 
@@ -262,20 +262,32 @@ class VerifyOutputs:
     logZ: torch.Tensor         # fp32 [B, k+1]
     logits: torch.Tensor | None
     status: torch.Tensor       # uint32 as int32 [1]
-    # fp32 [B, k], filled when the gate looks at the draft rows.  (A factory, so that the class itself has no attribute of
-    # this name and __getattr__ below is asked for it.)
-    draft_entropy: torch.Tensor | None = field(default_factory=lambda: None)
+    draft_entropy: torch.Tensor | None = None   # fp32 [B, k], filled when the gate looks at the draft rows
 
-    def __getattr__(self, name):
-        """Only reached for what an instance lacks: the fields that _fresh_outputs left out, made when somebody asks."""
-        lazy = self.__dict__.get("_lazy")
-        if lazy is None or name not in ("accept_len", "next_tok", "draft_entropy"):
-            raise AttributeError(f"{type(self).__name__!r} object has no attribute {name!r}")
+
+class _FieldOnDemand:
+    """What VerifyOutputs has of a field that an instance lacks: _fresh_outputs leaves out what the call does not fill, and it
+    is made when somebody asks.  (Without __set__, so that an instance's own tensor comes first; a __getattr__ would make
+    every attribute of every outputs object dearer.)"""
+
+    def __init__(self, name: str):
+        self.name = name
+
+    def __get__(self, out, cls=None):
+        lazy = None if out is None else out.__dict__.get("_lazy")
+        if lazy is None:
+            if out is None and self.name == "draft_entropy":
+                return None                                      # (the field's default)
+            raise AttributeError(f"{cls.__name__!r} object has no attribute {self.name!r}")
         B, k, dev = lazy
-        t = (torch.zeros((B, k), dtype=torch.float32, device=dev) if name == "draft_entropy"
+        t = (torch.zeros((B, k), dtype=torch.float32, device=dev) if self.name == "draft_entropy"
              else torch.empty(B, dtype=torch.int32, device=dev))
-        setattr(self, name, t)
+        setattr(out, self.name, t)
         return t
+
+
+for _name in ("accept_len", "next_tok", "draft_entropy"):
+    setattr(VerifyOutputs, _name, _FieldOnDemand(_name))
 
 
 def _fresh_outputs(ctx: "HolaVerify", B: int, k1: int, want_logits: bool, draws: bool, draft_gate: bool) -> VerifyOutputs:
@@ -421,10 +433,10 @@ class HolaVerify:
                 a.accept_len = t.data_ptr()
             if (t := out.next_tok) is not None:
                 a.next_tok = t.data_ptr()
-        if out.entropy is not None:
-            a.entropy = out.entropy.data_ptr()
-        if out.logZ is not None:
-            a.logZ = out.logZ.data_ptr()
+        if (t := out.entropy) is not None:
+            a.entropy = t.data_ptr()
+        if (t := out.logZ) is not None:
+            a.logZ = t.data_ptr()
         if out.logits is not None:
             a.logits_out = out.logits.data_ptr()
         if out.status is not None:
