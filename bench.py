@@ -48,8 +48,8 @@ NOMINAL_PEAKS = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}
 # time counters on the full-size launch; their logits are stored with the streaming hint, so most of them reach DRAM
 # inside the kernel; "wide" is the one launch that holds all six passes).  Other workloads, and the other weight modes,
 # report null.
-NCU_TRAFFIC = {"batched": 265923328 + 8595200, "large_vocab": 1055559936 + 172039680,
-               "wide": 2809281024 + 1177498112}
+NCU_TRAFFIC = {"batched": 265911680 + 8094490, "large_vocab": 1055523742 + 165214129,
+               "wide": 2598598827 + 1165225941}
 
 
 def ncu_traffic_bytes(w):

@@ -166,8 +166,9 @@ typedef enum {
                                      * device can address, the accept/sample kernel reads the rows not sent ahead in
                                      * place over the bus (default), 0 = they are copied after a read-back of accept_len */
   HOLA_OPT_CONVERTER_GROUP = 8,     /* on-chip expansion (HOLA_W_INT8, HOLA_W_MIXED): a K block takes four converter
-                                     * warps, one per quarter of the tensor-memory lanes; 1..4 or 0 (default) = both
-                                     * groups of four take blocks in turn, 5..8 = one group takes them all            */
+                                     * warps, one per quarter of the tensor-memory lanes.  0 (default) = all groups of
+                                     * four (two, or three with at most 32 verify rows) take blocks in turn; 1..4 are the
+                                     * same as 0; 5..8 = one group takes them all                                     */
   HOLA_OPT_FUSED_PASSES = 9,        /* more verify rows than one pass over W_lm holds: 1 = all passes in one launch, in
                                      * which as many neighbouring CTA pairs as there are passes walk the same vocabulary
                                      * tiles together and keep in step (default), 2 = the same without keeping in

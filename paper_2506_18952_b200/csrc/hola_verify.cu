@@ -2374,9 +2374,9 @@ struct QuantOut {
 
 // A head (or rows of it) to 4, 8 or 16 bits in ONE launch, a warp per row: one pass for the row's maximum, one that
 // rounds (the row, 8 KB at 4096 channels, then comes out of the L1 or the L2).  Bound: HBM (2 bytes in, half to two out
-// per weight).  32000 x 4096 at 4 / 8 / 16 bits in the proportions 20 / 70 / 10 %: 75 us = 4.9 TB/s (61 us at the measured
-// copy rate), of which the instructions (eleven per weight) take half; one launch per run of groups with a CTA per row, two
-// bytes per load and a division per weight needed 540 us.  Rows kept in registers between the passes: 102 registers,
+// per weight).  32000 x 4096 at 4 / 8 / 16 bits in the proportions 20 / 70 / 10 %: a call of 81 us for 393 MB = 4.9 TB/s (61 us at
+// the measured copy rate), of which the instructions (eleven per weight) take half; one launch per run of groups with a CTA per
+// row, two bytes per load and a division per weight needed 540 us.  Rows kept in registers between the passes: 102 registers,
 // 217 us with a slow path that divides next to half integers.
 // kVec: rows and buffers that 16-byte pieces tile and that are aligned for it; otherwise the same element by element.
 template <bool kVec>
@@ -2763,9 +2763,9 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   best.passes = (rows + best.rows_per_pass - 1) / best.rows_per_pass;
   best.nbuf = best.n_sub == 1 ? 2 : 1;
   best.rot = best.n_sub == 3 ? 1 : 0;
-  // Vocabulary rows per CTA per tile: the smallest multiple of 4 that covers V in the fewest whole rounds over
+  // Vocabulary rows per CTA per tile.  To begin with the smallest multiple of 4 that covers V in the fewest whole rounds over
   // all pairs, so that every pair streams the same number of bytes (V = 32000 on 74 pairs: 2 rounds of 112 + 112
-  // rows instead of 1.69 rounds of 128 + 128).
+  // rows instead of 1.69 rounds of 128 + 128); the rules below make tiles taller where something else counts for more.
   const int all_pairs = ctx->num_sms / 2 > 0 ? ctx->num_sms / 2 : 1;
   // Several passes: one launch in which `passes` neighbouring pairs walk the same tiles together, one pass each (W_lm
   // then leaves HBM once, not once per pass), as long as every pass gets a pair.
@@ -2774,8 +2774,9 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int rounds = (ctx->V + pairs * kPairTile - 1) / (pairs * kPairTile);
   // One tile per pair: a tile costs the tensor cores and the traffic of the hidden rows the same whatever its height, and
   // the statistics of all CTAs have to be merged, so as many pairs as there are is not the best split of a small vocabulary.
-  // At least 64 rows per CTA; with more than 96 operand rows no more than 42 pairs (still enough to stream W_lm through),
-  // with more than 256 as few pairs as there are tiles of 256.  us, H = 4096: V = 4000, 5 rows 16.6 -> 16.1, 96 rows 20.6 ->
+  // At least 64 rows per CTA; with more than 96 operand rows a 42nd of the vocabulary per pair, or tiles of 256 rows where that
+  // would be more (V > 10752: 43 pairs and up); with more than 256 operand rows tiles of 256 throughout.  42 pairs still stream
+  // W_lm fast enough; the number is the best of those tried at the three sizes below on 74 pairs, not derived.  us, H = 4096: V = 4000, 5 rows 16.6 -> 16.1, 96 rows 20.6 ->
   // 20.0 (V = 12000 27.6 as it is, 28.4 on 47 pairs); V = 8000, 192 rows 34.6 -> 28.6 (29.6 on 32 pairs), 384 rows 57.4 ->
   // 45.0, two planes of 192 rows 38.2 -> 35.4; V = 12000, 192 rows 37.4 -> 33.6, 384 rows 61.0 -> 51.4.
   const int op_rows = best.n_sub * best.N;
@@ -3825,9 +3826,9 @@ hola_status hola_verify_host(hola_ctx* ctx, const hola_verify_args* a, void* cud
     if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, stream);
     down += bytes;
   };
-  // The small inputs go first (copies queue on the DMA engine in issue order).  The draft tensor is by far the
-  // largest input and only the accept/sample part reads it: it travels on the context's own stream while the
-  // GEMM runs on the caller's.  (The previous call synchronised before returning, so the staging is free.)
+  // The hidden rows go first, on the caller's stream: the GEMM waits for them.  The draft tensor, by far the largest input,
+  // and the small ones are read by the accept/sample part only: they travel on the context's own stream while the GEMM runs.
+  // (Only calls of this entry point use the staging, and they synchronise before they return: it is free.)
   h2d(ctx->st_hidden, a->hidden, rows * a->H * 2);
   memcpy(ctx->h_small, a->draft_tok, static_cast<size_t>(a->B) * a->k * 4);
   memcpy(ctx->h_small + ctx->small_u_off, a->uniforms, rows * 4);
