@@ -103,7 +103,7 @@ constexpr int kK3Unroll = 4;                     // vocabulary chunks a warp has
 
 constexpr int kHqSlices = 8;                     // CTAs that share one draft row in draft_entropy_kernel
 
-constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 
 struct K1Params {
   int M;          // total verify rows B(k+1)
@@ -629,10 +629,11 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-// stats_fold16<true> with half the issue slots: the maximum by three-input comparisons, the exponents' arguments, the
-// sum of the exponentials and the sum of e * l two at a time.  The centred sum of the sixteen entries,
-// sum e (l - m), is taken as  sum e l - m sum e : both terms are of size |m| * (sum e), so the rounding of the
-// difference is about 1e-7 |m| relative to s, far inside the tolerance on H = ln s - t / s.
+// stats_fold16<true> with half the issue slots: the maximum by three-input comparisons, the exponents' arguments
+// x = (l - m) log2 e, the sum of the exponentials and the sum of e * x two at a time.  The centred sum is ln 2 times the
+// last one.  What the rounding of m log2 e puts on every x (up to 2^-24 |m|) then counts as a shift of the reference in s and
+// t alike and leaves H = ln s - t / s alone.  (Taken as  sum e l - m sum e  the centred sum has a rounding error of that size
+// relative to s: entropies of rows with logits of +-40 were 1.3e-6 off in the 2-norm at V = 1000 instead of 3e-7.)
 __device__ __forceinline__ void stats_fold16_packed(const float* v, int vocab0, Stats& st) {
   const float c0 = max3(v[0], v[1], v[2]), c1 = max3(v[3], v[4], v[5]), c2 = max3(v[6], v[7], v[8]),
               c3 = max3(v[9], v[10], v[11]), c4 = max3(v[12], v[13], v[14]);
@@ -658,19 +659,18 @@ __device__ __forceinline__ void stats_fold16_packed(const float* v, int vocab0, 
   uint64_t s2 = pack2(0.f, 0.f), a2 = pack2(0.f, 0.f);
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const uint64_t vp = pack2(v[2 * j], v[2 * j + 1]);
+    const uint64_t xp = fma2(pack2(v[2 * j], v[2 * j + 1]), l2e, mn);
     float x0, x1;
-    unpack2(fma2(vp, l2e, mn), x0, x1);
+    unpack2(xp, x0, x1);
     const uint64_t ep = pack2(ex2_approx(x0), ex2_approx(x1));
     s2 = add2(s2, ep);
-    a2 = fma2(ep, vp, a2);
+    a2 = fma2(ep, xp, a2);
   }
   float sa, sb, aa, ab;
   unpack2(s2, sa, sb);
   unpack2(a2, aa, ab);
-  const float sc = sa + sb;
-  st.s += sc;
-  st.t += fmaf(-m, sc, aa + ab);
+  st.s += sa + sb;
+  st.t = fmaf(kLn2, aa + ab, st.t);
 }
 
 // Integer codes to bf16 without conversion instructions.  A byte u in the low half of a 16-bit lane, high half zero, IS

@@ -1262,3 +1262,22 @@ def test_host_entry_reports_the_flags_of_every_sequence(binding, lazy, in_place,
     if fallback == 0:
         every = binding.FLAG_BAD_TOKEN | binding.FLAG_BAD_UNIFORM | binding.FLAG_R_ZERO
         assert {0, binding.FLAG_BAD_TOKEN, binding.FLAG_BAD_UNIFORM, binding.FLAG_R_ZERO, every} <= seen
+
+
+@pytest.mark.parametrize("V", [64, 300, 1000, 1700, 2300, 40000])
+def test_entropy_of_rows_with_large_logits_keeps_its_accuracy(binding, V):
+    """Logits of +-40: the statistics against 64-bit ones of the call's own logits.  Every e^(l - m) is good to 2^-22 (the
+    hardware's 2^x), which moves H by about as much relative to itself, and the other roundings (arguments, sums, merges, the
+    logarithm) together by no more: 2 * 2^-22 in the 2-norm.  (A centred sum made of two sums of size |m| s is off by 1.3e-6.)"""
+    B, k, H = 12, 4, 64
+    err = norm = 0.0
+    for seed in range(4):
+        w = workloads.gaussian_head("large-logits", B, k, H, V, seed=seed, device=DEV, w_std=9.0 / math.sqrt(H))
+        with binding.HolaVerify(B, k, H, V) as ctx:
+            out = ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
+            torch.cuda.synchronize()
+        l = out.logits.double()
+        want = torch.logsumexp(l, -1) - (torch.softmax(l, -1) * l).sum(-1)
+        err += float(((out.entropy - want) ** 2).sum())
+        norm += float((want ** 2).sum())
+    assert math.sqrt(err / norm) <= 2.0 ** -21
