@@ -129,7 +129,8 @@ typedef struct {
   int32_t* next_tok;       /* out int32 [B], 0..V-1: the token that follows them                              */
   float* entropy;          /* out fp32 [B][k+1], nats, >= 0                                                    */
   float* logZ;             /* out fp32 [B][k+1], log-sum-exp of the logits                                     */
-  float* logits_out;       /* out fp32 [B][k+1][V], optional (NULL: the context's own scratch is used)         */
+  float* logits_out;       /* out fp32 [B][k+1][V], optional (NULL: the context's own scratch is used, or none by
+                            * hola_verify and hola_verify_host with the greedy fallback, which reads no logits)   */
   uint32_t* status_word;   /* in/out uint32 [1], optional: HOLA_FLAG_* bits are OR-ed in                       */
   int32_t gate_source;     /* hola_gate_source; 0 (zero-initialised struct) = target entropy                   */
   int32_t fallback;        /* hola_fallback; 0 = speculative sampling.  With GREEDY the uniforms are not read  */

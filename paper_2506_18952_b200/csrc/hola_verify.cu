@@ -139,7 +139,7 @@ struct K1Params {
   int bulk_logits;        // (rotating units) 1: the logits buffer has a tensor map (rows of whole 16-byte pieces), full blocks
                           // leave by bulk stores
   int stream_logits;      // 1: store the logits with the streaming hint (they exceed what the L2 keeps until they are read)
-  float* logits;
+  float* logits;      // null: nobody reads them, none are stored
   float4* partials;   // [M][part_stride] (m, s, t, arg-max index): a row's partials side by side, one per CTA of its pass
   int part_stride;
   unsigned* status;
@@ -1284,7 +1284,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                                 static_cast<float>(static_cast<int>(a[i])) * (w_scale * p.h_scale[r]));
                   }
                 }
-                if (vocab_ok) {
+                if (vocab_ok && p.logits) {
                   float* dst = p.logits + static_cast<size_t>(vr0 + 16 * half) * p.ldl + vocab;
 #pragma unroll
                   for (int i = 0; i < 16; ++i)
@@ -1348,7 +1348,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                   if (i < n_ok) v[i] = scaled<kMode>(v[i], w_scale, p.h_scale, r0 + i);
                 if (kMode >= 2) asm volatile("" ::: "memory");   // the row scales eight at a time, not all 32 ahead
               }
-              if (vocab_ok && !bulk) {
+              if (vocab_ok && !bulk && p.logits) {
                 float* dst = p.logits + static_cast<size_t>(r0) * p.ldl + vocab;
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
@@ -1425,7 +1425,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                 if (i < n_ok) v[i] = scaled<kMode>(v[i], w_scale, p.h_scale, r0 + i);
               if (kMode >= 2) asm volatile("" ::: "memory");     // the row scales eight at a time, not all 32 ahead
             }
-            if (vocab_ok && !kWide) {
+            if (vocab_ok && !kWide && p.logits) {
               float* dst = p.logits + static_cast<size_t>(r0) * p.ldl + vocab;
               if (n_ok == 32 && p.stream_logits) {       // (the common cases without a test per store)
 #pragma unroll
@@ -1464,7 +1464,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                       }
                     }
                   };
-                  if (kWide && !(group & 1)) put();
+                  if (kWide && p.logits && !(group & 1)) put();
                   float e[16];
 #pragma unroll
                   for (int jj = 0; jj < 4; ++jj) {
@@ -1475,7 +1475,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
                   // (rows at or beyond n_ok fold whatever the unused columns held; they are never written out)
                   if (n16 == 16) stats_fold16_packed(e, vocab16, st[slot][half]);
                   else if (n16 > 0) stats_fold16<false>(e, n16, vocab16, st[slot][half]);
-                  if (kWide && (group & 1)) put();
+                  if (kWide && p.logits && (group & 1)) put();
                 }
               }
             }
@@ -1974,7 +1974,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   uint32_t q_bits = 0;                                   // (as loaded: converted when it is stored)
   if (j_mine < k) {
     const int j = j_mine;
-    if (x_mine >= 0 && x_mine < Vtok) {
+    if (x_mine >= 0 && x_mine < Vtok && p.fallback != HOLA_FALLBACK_GREEDY) {     // (greedy: compared by its index alone)
       const size_t qi = (static_cast<size_t>(b) * k + j) * V + x_mine;
       if (p.q_tok) q_bits = __float_as_uint(p.q_tok[b * k + j]);
       else if (p.q_dtype == HOLA_Q_BF16) q_bits = static_cast<const uint16_t*>(p.q)[qi];
@@ -2891,7 +2891,15 @@ int sample_cluster(const hola_ctx* ctx, const hola_verify_args* a) {
   return S;
 }
 
+// Where the logits of a verify step that does not hand them out go.  The greedy rule reads none (the arg-max travels with the
+// statistics), so none are stored then.  8-bit head and hidden rows, 192 rows, V = 128256 (98 MB of logits beside 525 MB of
+// codes): 137 -> 121 us.
+float* logits_buffer(const hola_ctx* ctx, const hola_verify_args* a) {
+  return a->fallback == HOLA_FALLBACK_GREEDY ? nullptr : ctx->logits;
+}
+
 // Steps 1-2: the LM-head GEMM with fused statistics, one launch (clusters of two CTAs) per pass over W_lm.
+// `logits` null: statistics only.
 // `few_before`: the kernel in front is expected to be this context's accept/sample kernel on a few SMs.
 // `draft_pass`: the pass over the draft rows (draft-entropy gate) is made on the way.
 // `next_reads_inputs`: the accept/sample kernel of the same arguments is launched right behind this.
@@ -2991,7 +2999,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   // Rotating units: the logits buffer, where its rows are whole 16-byte pieces; boxes of 16 rows x 32 entries, swizzled like
   // the staging buffers.
   const bool wide_logits = !pl.rot && pl.N >= 128 && ldl % 4 == 0 && aligned16(logits) && a->V % 4 == 0;
-  const bool bulk_logits = pl.rot && ldl % 4 == 0 && aligned16(logits);
+  const bool bulk_logits = pl.rot && logits && ldl % 4 == 0 && aligned16(logits);
   if (bulk_logits && (me->logits != logits || me->ldl != ldl)) {
     me->logits = nullptr;
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(a->V), static_cast<cuuint64_t>(M)};
@@ -3531,7 +3539,7 @@ namespace {
 // (the draft tensor still being copied in by hola_verify_host).
 hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t stream, cudaEvent_t before_sample) {
   const Plan& pl = plan_for(ctx, a->B * (a->k + 1), a->w_dtype);
-  float* logits = a->logits_out ? a->logits_out : ctx->logits;
+  float* logits = a->logits_out ? a->logits_out : logits_buffer(ctx, a);
   const int ldl = a->logits_out ? a->V : ctx->ldl;
   const bool prof = ctx->prof_on && ctx->prof_n < ctx->prof_cap;
   cudaEvent_t* ev = prof ? ctx->prof_ev + 3 * ctx->prof_n : nullptr;
@@ -3681,7 +3689,8 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
   d.flags = HOLA_ARG_CLEAR_STATUS;
   hola_status s;
   const Plan& pl = plan_for(ctx, B * (k + 1), a->w_dtype);
-  if ((s = run_lm_head(ctx, &d, ctx->logits, ctx->ldl, pl, stream)) != HOLA_OK) return s;
+  float* logits = logits_buffer(ctx, a);
+  if ((s = run_lm_head(ctx, &d, logits, ctx->ldl, pl, stream)) != HOLA_OK) return s;
   // Where the caller's draft tensor is pinned host memory that the device can address, the rows still missing after the
   // accept test are not copied at all: the accept/sample kernel reads row accept_len of a sequence in place, over the
   // bus, when that row is not among the ones sent ahead.  One launch, no read-back in the middle of the call.
@@ -3699,7 +3708,7 @@ hola_status verify_host_lazy(hola_ctx* ctx, const hola_verify_args* a, cudaStrea
     if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copy_done, 0);
     if (e != cudaSuccess) { set_error(ctx, "wait for the inputs sent ahead", e); return HOLA_ERR_CUDA; }
     direct = outputs_to_host(ctx, &d, ob);
-    s = run_accept_sample(ctx, &d, ctx->logits, ctx->ldl, 1, row_partials(pl), stream, ctx->st_qtok, 0, nullptr, false, q_far, ahead);
+    s = run_accept_sample(ctx, &d, logits, ctx->ldl, 1, row_partials(pl), stream, ctx->st_qtok, 0, nullptr, false, q_far, ahead);
     ctx->flags_out = nullptr;
     if (s != HOLA_OK) return s;
   } else {

@@ -242,6 +242,33 @@ def test_draft_entropy_gate_and_greedy_verifier(binding, gate_source, fallback, 
         assert np.array_equal(nxt, lg[np.arange(B), acc].argmax(-1))
 
 
+@pytest.mark.parametrize("B,k,H,V,weights", [
+    (1, 4, 64, 1000, "bf16"),        # one chunk of rows
+    (23, 3, 136, 5003, "bf16"),      # 92 rows, unaligned pitch
+    (32, 5, 128, 20000, "bf16"),     # 192 rows: logits would leave 16 bytes per lane
+    (60, 4, 128, 5000, "bf16"),      # 300 rows: rotating units
+    (60, 7, 128, 5000, "bf16"),      # 480 rows: two MMAs
+    (130, 4, 64, 3001, "bf16"),      # two passes
+    (40, 5, 128, 3000, "int8"), (4, 2, 128, 3000, "int8"),
+    (32, 5, 128, 20000, "w8a8"), (60, 4, 128, 3000, "w8a8"), (9, 4, 128, 3001, "w8a8"),
+    (30, 5, 128, 3001, "w8a16"),
+])
+def test_logits_that_nobody_reads_change_nothing_by_their_absence(binding, B, k, H, V, weights):
+    """The greedy step without logits_out stores no logits; everything else is the same, bit for bit, as with logits_out."""
+    w = workloads.gaussian_head("greedy", B, k, H, V, seed=B + V, device=DEV, w_std=0.3, sigma=0.5, tau=2.0)
+    W, kw = w.W_lm, {}
+    if weights != "bf16":
+        W, kw["w_scale"] = binding.hola_quantize_w8(w.W_lm)
+        kw["a8"] = {"int8": False, "w8a8": True, "w8a16": "a16"}[weights]
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        got = [ctx.hola_verify(w.hidden, W, w.draft_tok, w.draft_q, w.uniforms, w.tau, want_logits=x, fallback=1, **kw)
+               for x in (False, True)]
+        torch.cuda.synchronize()
+    for name in ("accept_len", "next_tok", "entropy", "logZ", "status"):
+        assert torch.equal(getattr(got[0], name), getattr(got[1], name)), name
+    assert torch.equal(got[1].logits.argmax(-1).gather(1, got[0].accept_len.long()[:, None])[:, 0].int(), got[0].next_tok)
+
+
 def test_greedy_verifier_on_the_large_vocabulary_shape(binding):
     w = workloads.make_config("large_vocab", DEV)
     out, _, _ = check_against_oracle(binding, w, seqs=[3, 30, 59], gate_source=1, fallback=1, want_logits=False)
