@@ -740,6 +740,11 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
   return acc;
 }
 
+__device__ __forceinline__ float warp_max_f32(float x) {       // (of numbers; -inf among them)
+  float r;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ double warp_sum_f64(double x) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
@@ -1704,9 +1709,8 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_selftest_kernel(long long 
 // ------------------------------------------------------------------------------------------------ K2
 // The statistics of one row over all CTAs, by a warp, the same bits in every lane.  Six loads per lane in flight (192
 // partials per round: one round on a 148-SM part; a GEMM launch leaves a row's partials side by side, part_stride 1).  The
-// maximum first, so that the
-// exponentials of the partials are independent of one another and only additions remain to be passed round: five
-// shuffles for the maximum and five for the sums instead of eleven merges of a hundred cycles each.
+// maximum first (one instruction), so that the exponentials of the partials are independent of one another and only additions
+// remain to be passed round: five shuffles instead of eleven merges of a hundred cycles each.
 __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int row_stride, int part_stride,
                                                      int row, int lane) {
   partials += static_cast<size_t>(row) * row_stride;
@@ -1719,9 +1723,7 @@ __device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int
       x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride]
                         : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
     }
-    float m = fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    const float m = warp_max_f32(fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x)));
     float s = 0.f, t = 0.f;
     int arg = 0x7fffffff;
 #pragma unroll
@@ -1805,34 +1807,33 @@ __device__ __forceinline__ float warp_sum4_f32(const float v[4], int lane) {
 // Logits and draft probabilities of vocabulary entries base..base+3 of one row (q = 0 when the row is drawn
 // from p itself; entries at or beyond V get l = -inf, q = 0 and so no mass).  Loads only: a caller can issue
 // several of these before using any, which keeps more requests in flight.
-template <bool kVec>
-__device__ __forceinline__ void fetch4(const float* lrow, const void* qrow, int q_dtype, bool residual, int base,
-                                       int V, float l[4], float q[4]) {
+template <bool kVec, bool kHalf>
+__device__ __forceinline__ void fetch4(const float* lrow, const void* qrow, bool residual, int base, int V, float l[4], float q[4]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) q[i] = 0.f;
-  if (kVec && base + 3 < V) {
-    const float4 l4 = *reinterpret_cast<const float4*>(lrow + base);
-    l[0] = l4.x; l[1] = l4.y; l[2] = l4.z; l[3] = l4.w;
-    if (residual) {
-      if (q_dtype == HOLA_Q_BF16) {
-        const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(qrow) + base);
-        q[0] = __uint_as_float(raw.x << 16); q[1] = __uint_as_float(raw.x & 0xFFFF0000u);
-        q[2] = __uint_as_float(raw.y << 16); q[3] = __uint_as_float(raw.y & 0xFFFF0000u);
-      } else {
-        const float4 q4 = *reinterpret_cast<const float4*>(static_cast<const float*>(qrow) + base);
-        q[0] = q4.x; q[1] = q4.y; q[2] = q4.z; q[3] = q4.w;
+  for (int i = 0; i < 4; ++i) { l[i] = -CUDART_INF_F; q[i] = 0.f; }
+  if (kVec) {                                            // (V is a multiple of 4)
+    if (base < V) {
+      const float4 l4 = *reinterpret_cast<const float4*>(lrow + base);
+      l[0] = l4.x; l[1] = l4.y; l[2] = l4.z; l[3] = l4.w;
+      if (residual) {
+        if (kHalf) {
+          const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(qrow) + base);
+          q[0] = __uint_as_float(raw.x << 16); q[1] = __uint_as_float(raw.x & 0xFFFF0000u);
+          q[2] = __uint_as_float(raw.y << 16); q[3] = __uint_as_float(raw.y & 0xFFFF0000u);
+        } else {
+          const float4 q4 = *reinterpret_cast<const float4*>(static_cast<const float*>(qrow) + base);
+          q[0] = q4.x; q[1] = q4.y; q[2] = q4.z; q[3] = q4.w;
+        }
       }
     }
   } else {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int v = base + i;
-      l[i] = -CUDART_INF_F;
       if (v < V) {
         l[i] = lrow[v];
         if (residual)
-          q[i] = (q_dtype == HOLA_Q_BF16) ? __bfloat162float(static_cast<const __nv_bfloat16*>(qrow)[v])
-                                          : static_cast<const float*>(qrow)[v];
+          q[i] = kHalf ? __bfloat162float(static_cast<const __nv_bfloat16*>(qrow)[v]) : static_cast<const float*>(qrow)[v];
       }
     }
   }
@@ -1846,12 +1847,36 @@ __device__ __forceinline__ void resid4(const float l[4], const float q[4], float
   for (int i = 0; i < 4; ++i) r[i] = fmaxf(0.f, ex2_approx((l[i] - logZ) * kLog2e) - q[i]);
 }
 
-template <bool kVec>
-__device__ __forceinline__ void load_r4(const float* lrow, const void* qrow, int q_dtype, bool residual, int base,
-                                        int V, float logZ, float r[4]) {
-  float l[4], q[4];
-  fetch4<kVec>(lrow, qrow, q_dtype, residual, base, V, l, q);
-  resid4(l, q, logZ, r);
+// The residual mass of every chunk of a slice (chunks c_first .. c_first + mine - 1), by the whole CTA of kWarps warps.  In
+// fp32 (128 non-negative terms added pairwise: relative error a few 1e-7), kept as fp64 for the scans that follow.  lrow,
+// qrow: entry 0 of the row, which a staged slice does not hold.  (Inlined once for rows in shared memory and once for rows in
+// global memory, so that each gets loads of its own kind, and once per type of q: us, 50 rows, V = 60000 53.2 -> 52.4, 32 rows,
+// V = 128256 61.0 -> 59.7, 5 rows, V = 32000 46.67 -> 46.46.)
+template <bool kVec, bool kHalf, int kWarps>
+__device__ __forceinline__ void sum_chunks(const float* lrow, const void* qrow, bool residual, int c_first, int mine, int V,
+                                           float logZ, double* csum, int warp, int lane) {
+  for (int c0 = warp; c0 < mine; c0 += kK3Unroll * kWarps) {
+    float l[kK3Unroll][4], q[kK3Unroll][4];
+#pragma unroll
+    for (int i = 0; i < kK3Unroll; ++i) {                // all loads of this step first
+      const int c = c0 + i * kWarps;
+      fetch4<kVec, kHalf>(lrow, qrow, residual, c < mine ? (c_first + c) * kChunk + lane * 4 : V, V, l[i], q[i]);
+    }
+    float part[kK3Unroll];
+#pragma unroll
+    for (int i = 0; i < kK3Unroll; ++i) {
+      part[i] = 0.f;
+      if (c0 + i * kWarps < mine) {
+        float r[4];
+        resid4(l[i], q[i], logZ, r);
+        part[i] = (r[0] + r[1]) + (r[2] + r[3]);
+      }
+    }
+    // lanes 0, 8, 16, 24 end up with chunks 0, 1, 2, 3 of this step
+    const float sum = warp_sum4_f32(part, lane);
+    const int c = c0 + (lane >> 3) * kWarps;
+    if ((lane & 7) == 0 && c < mine) csum[c] = static_cast<double>(sum);
+  }
 }
 
 // Untiled bulk copy into this CTA's shared memory (addresses and size multiples of 16 bytes), counted on an mbarrier.
@@ -1961,23 +1986,31 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const int mine = max(0, min(nchunks, c_first + cpc) - c_first);
   const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
   // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities, each row's
-  // slice by one bulk copy that a thread of the last warp (the first to have nothing else to wait for) starts.
+  // slice by one bulk copy, a lane of the first warp per copy, while the other warps merge statistics (with eight rows and more
+  // that one does so too, after its gathers: then the last warp).  (One thread after the
+  // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows: V = 32000 46.67 -> 46.31, mixed widths
+  // 34.84 -> 34.47, V = 3000 11.0 -> 10.7.)
   const bool staged = kVec && p.staged;
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
   char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
   const int here = min(V - c_first * kChunk, mine * kChunk);           // entries of this slice (0 or less: none)
-  if (staged && warp == kK3Warps - 1 && elect_one() && here > 0) {
+  if (staged && warp == (k + 1 < kK3Warps ? 0 : kK3Warps - 1) && here > 0) {
     const uint32_t bar = smem_u32(&sh_bar), lbytes = here * 4u, qbytes = static_cast<uint32_t>(here * q_elem);
-    mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(bar, (k + 1) * lbytes + k * qbytes);
+    if (lane == 0) {
+      mbar_init(bar, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_expect_tx(bar, (k + 1) * lbytes + k * qbytes);
+    }
+    __syncwarp();
     const float* l = p.logits + static_cast<size_t>(row_first) * p.ldl + c_first * kChunk;
-    for (int j = 0; j <= k; ++j, l += p.ldl) bulk_load(smem_u32(sl + static_cast<size_t>(j) * slice), l, lbytes, bar);
     const char* q = static_cast<const char*>(p.q) + (static_cast<size_t>(b) * k * V + c_first * kChunk) * q_elem;
-    for (int j = 0; j < k; ++j, q += V * q_elem) bulk_load(smem_u32(sq + static_cast<size_t>(j) * slice * q_elem), q, qbytes, bar);
+    for (int i = lane; i <= 2 * k; i += 32) {
+      if (i <= k) bulk_load(smem_u32(sl + static_cast<size_t>(i) * slice), l + static_cast<size_t>(i) * p.ldl, lbytes, bar);
+      else bulk_load(smem_u32(sq + static_cast<size_t>(i - k - 1) * slice * q_elem), q + static_cast<size_t>(i - k - 1) * V * q_elem, qbytes, bar);
+    }
+    __syncwarp();
   }
-  __syncwarp();
   // the draft token's logit and probability
   float lx = 0.f, hq = 0.f;
   uint32_t q_bits = 0;                                   // (as loaded: converted when it is stored)
@@ -2071,11 +2104,11 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   const float logZ = sh_logZ[n];
   const char* qbase = static_cast<const char*>((p.q_far && n >= p.q_far_from) ? p.q_far : p.q);
   // (staged: the row as if the slice were the whole of it, entry v at row + v)
-  const float* lrow = staged ? sl + static_cast<size_t>(n) * slice - c_first * kChunk
-                             : p.logits + static_cast<size_t>(row_first + n) * p.ldl;
-  const void* qrow = n >= k ? nullptr
-                   : staged ? static_cast<const void*>(sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem)
-                            : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
+  const float* lstaged = sl + static_cast<size_t>(n) * slice - c_first * kChunk;
+  const char* qstaged = n >= k ? sq : sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem;
+  const float* lrow = p.logits + static_cast<size_t>(row_first + n) * p.ldl;
+  const void* qrow = n >= k ? nullptr : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
+  const bool half = p.q_dtype == HOLA_Q_BF16;
   if (staged && here > 0) wait_staged_rows(smem_u32(&sh_bar), p.status, kWaitLimitCycles);
   // Several CTAs per SM and short slices (up to 8192 entries): a slice into the L2 by two bulk requests instead of by the loads
   // alone.  us, V = 32000, H = 512, 384 rows 33.2 -> 32.5, 240 rows 25.3 -> 24.7; V = 128256 (16032 entries) no gain.  With a CTA
@@ -2127,29 +2160,12 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   }
 
   for (int attempt = 0; attempt < 2; ++attempt) {
-    for (int c0 = warp; c0 < mine; c0 += kK3Unroll * kK3Warps) {
-      float l[kK3Unroll][4], q[kK3Unroll][4];
-#pragma unroll
-      for (int i = 0; i < kK3Unroll; ++i) {              // all loads of this step first
-        const int c = c0 + i * kK3Warps;
-        if (c < mine) fetch4<kVec>(lrow, qrow, p.q_dtype, residual, (c_first + c) * kChunk + lane * 4, V, l[i], q[i]);
-      }
-      // the mass of each chunk in fp32 (128 non-negative terms added pairwise: relative error a few 1e-7), kept as
-      // fp64 for the scans that follow; lanes 0, 8, 16, 24 end up with chunks 0, 1, 2, 3 of this step
-      float part[kK3Unroll];
-#pragma unroll
-      for (int i = 0; i < kK3Unroll; ++i) {
-        const int c = c0 + i * kK3Warps;
-        part[i] = 0.f;
-        if (c < mine) {
-          float r[4];
-          resid4(l[i], q[i], logZ, r);
-          part[i] = (r[0] + r[1]) + (r[2] + r[3]);
-        }
-      }
-      const float sum = warp_sum4_f32(part, lane);
-      const int c = c0 + (lane >> 3) * kK3Warps;
-      if ((lane & 7) == 0 && c < mine) csum[c] = static_cast<double>(sum);
+    if (staged) {
+      if (half) sum_chunks<kVec, true, kK3Warps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
+      else sum_chunks<kVec, false, kK3Warps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
+    } else {
+      if (half) sum_chunks<kVec, true, kK3Warps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
+      else sum_chunks<kVec, false, kK3Warps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
     }
     __syncthreads();
     // warp 0: scan of the slice; lane L owns chunks [lo, hi)
@@ -2226,8 +2242,16 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       before = __shfl_sync(0xffffffffu, before, L);
       take_last = __shfl_sync(0xffffffffu, take_last ? 1 : 0, L) != 0;
       // inside the chunk: lane prefix, then the lane's four entries in ascending order
-      float r4[4];
-      load_r4<kVec>(lrow, qrow, p.q_dtype, residual, (c_first + cstar) * kChunk + lane * 4, V, logZ, r4);
+      const int base = (c_first + cstar) * kChunk + lane * 4;
+      float l4[4], q4[4], r4[4];
+      if (staged) {
+        if (half) fetch4<kVec, true>(lstaged, qstaged, residual, base, V, l4, q4);
+        else fetch4<kVec, false>(lstaged, qstaged, residual, base, V, l4, q4);
+      } else {
+        if (half) fetch4<kVec, true>(lrow, qrow, residual, base, V, l4, q4);
+        else fetch4<kVec, false>(lrow, qrow, residual, base, V, l4, q4);
+      }
+      resid4(l4, q4, logZ, r4);
       const double mine4 = ((static_cast<double>(r4[0]) + r4[1]) + r4[2]) + r4[3];
       double lincl = mine4;
 #pragma unroll

@@ -305,6 +305,28 @@ def test_degenerate_inputs_are_flagged_not_fatal(binding):
     assert orc.flags[3] & ref.FLAG_R_ZERO
 
 
+@pytest.mark.parametrize("B,k,V,qd", [
+    (1, 4, 1920, torch.float32),       # fewer chunks than a cluster of two wants: a single small CTA
+    (1, 4, 2048, torch.float32),       # the smallest vocabulary with a CTA of 1024 threads per sequence
+    (3, 2, 4001, torch.bfloat16),      # the same, rows of no whole 16-byte pieces
+    (2, 8, 8192, torch.bfloat16), (2, 8, 8196, torch.bfloat16),        # its end for small batches: rows staged beyond
+    (5, 1, 8196, torch.float32), (9, 3, 8193, torch.bfloat16),
+    (20, 2, 16384, torch.float32), (20, 2, 16388, torch.bfloat16),     # its end: clusters beyond
+    (160, 1, 3000, torch.bfloat16),    # more sequences than SMs
+    (5, 40, 4100, torch.bfloat16),     # more rows than warps
+])
+def test_forms_of_the_accept_kernel_at_the_edges_of_their_ranges(binding, B, k, V, qd):
+    w = workloads.gaussian_head("forms", B, k, 64, V, seed=B + V, device=DEV, w_std=0.3, q_dtype=qd, sigma=1.0, sigma_far=0.1,
+                                tau=2.5)
+    w.draft_q[B // 2] = 2.0            # above p everywhere: no residual mass, the draw is from p
+    w.uniforms[B // 2, 0] = 0.99
+    w.tau = 0.0
+    out, orc, _ = check_against_oracle(binding, w)
+    check_ranges(w, out)
+    assert orc.flags[B // 2] & ref.FLAG_R_ZERO and int(out.status.item()) & binding.FLAG_R_ZERO
+    check_against_oracle(binding, w, tau=2.5)
+
+
 def test_empty_batch_and_argument_errors(binding):
     import ctypes
     lib = binding.load_library()
