@@ -93,7 +93,7 @@ constexpr int kBarrierBytes = 512;
 constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s of SM clock per wait, far above any legitimate wait
 
 constexpr int kK3Threads = 256;
-constexpr int kK3Warps = kK3Threads / 32;
+constexpr int kSoloThreads = 1024;               // its form with one CTA per sequence
 constexpr int kK3MaxPerSm = 4;                   // CTAs of the accept/sample kernel an SM holds (register budget: 64 per thread)
 constexpr int kChunk = 128;                      // vocabulary entries per warp step (32 lanes x 4)
 constexpr int kMaxChunks = 4096;                 // => V <= 524288
@@ -1946,8 +1946,10 @@ __global__ void __launch_bounds__(64, 1) staged_wait_selftest_kernel(long long l
 // total to all CTAs of the cluster through distributed shared memory.  After one cluster barrier each CTA knows
 // the total mass R and which slice holds the point u*R; that CTA alone finishes the inverse-CDF search.
 // kAsk: the slice of row n is asked into the L2 as soon as n is known.
-template <bool kVec, bool kAsk>
-__global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
+// kSolo: one CTA of 1024 threads instead of the cluster (see sample_solo).
+template <bool kVec, bool kAsk, bool kSolo = false>
+__global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 : kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
+  constexpr int kThreads = kSolo ? kSoloThreads : kK3Threads, kWarps = kThreads / 32;
   extern __shared__ __align__(16) double csum[];                       // per-chunk residual mass of this CTA's slice
   __shared__ double sh_tot[2][8];                        // slice totals of the whole cluster, per attempt
   __shared__ float sh_logZ[kMaxK1], sh_H[kMaxK1], sh_lx[kMaxK1], sh_qx[kMaxK1], sh_u[kMaxK1], sh_Hq[kMaxK1];
@@ -1958,8 +1960,8 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   // memory) may be scheduled from now on: its launch and prologue then hide behind this kernel.
   grid_dependency_release();
   cg::cluster_group cluster = cg::this_cluster();
-  const int S = static_cast<int>(cluster.num_blocks());
-  const int rank = static_cast<int>(cluster.block_rank());
+  const int S = kSolo ? 1 : static_cast<int>(cluster.num_blocks());
+  const int rank = kSolo ? 0 : static_cast<int>(cluster.block_rank());
   const int b = blockIdx.x / S;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k = p.k, V = p.V;
@@ -1990,12 +1992,12 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   // that one does so too, after its gathers: then the last warp).  (One thread after the
   // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows: V = 32000 46.67 -> 46.31, mixed widths
   // 34.84 -> 34.47, V = 3000 11.0 -> 10.7.)
-  const bool staged = kVec && p.staged;
+  const bool staged = kVec && !kSolo && p.staged;
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
   char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
   const int here = min(V - c_first * kChunk, mine * kChunk);           // entries of this slice (0 or less: none)
-  if (staged && warp == (k + 1 < kK3Warps ? 0 : kK3Warps - 1) && here > 0) {
+  if (staged && warp == (k + 1 < kWarps ? 0 : kWarps - 1) && here > 0) {
     const uint32_t bar = smem_u32(&sh_bar), lbytes = here * 4u, qbytes = static_cast<uint32_t>(here * q_elem);
     if (lane == 0) {
       mbar_init(bar, 1);
@@ -2039,7 +2041,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   if (p.combine) {
     // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
     // above, gets a row only when there are more than seven)
-    for (int j = kK3Warps - 1 - warp; j <= k; j += kK3Warps) {
+    for (int j = kWarps - 1 - warp; j <= k; j += kWarps) {
       Stats st = warp_merge_partials(p.partials, p.nparts, p.row_stride, p.part_stride, row_first + j, lane);
       if (lane == 0) {
         float lz, h;
@@ -2049,7 +2051,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
       }
     }
   } else {
-    for (int j = threadIdx.x; j <= k; j += kK3Threads) {
+    for (int j = threadIdx.x; j <= k; j += kThreads) {
       sh_logZ[j] = p.logZ[row_first + j];
       sh_H[j] = p.entropy[row_first + j];
     }
@@ -2113,7 +2115,7 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
   // Several CTAs per SM and short slices (up to 8192 entries): a slice into the L2 by two bulk requests instead of by the loads
   // alone.  us, V = 32000, H = 512, 384 rows 33.2 -> 32.5, 240 rows 25.3 -> 24.7; V = 128256 (16032 entries) no gain.  With a CTA
   // per SM the loads are all out at once, and the code alone costs 0.2 us, hence a kernel without it.
-  if (kAsk && threadIdx.x == (kK3Warps - 1) * 32 && here > 0) {
+  if (kAsk && threadIdx.x == (kWarps - 1) * 32 && here > 0) {
     bulk_prefetch_l2(lrow + c_first * kChunk, static_cast<unsigned>(here) * 4u);
     if (n < k && qbase == static_cast<const char*>(p.q)) {
       const uintptr_t q0 = reinterpret_cast<uintptr_t>(qrow) + c_first * kChunk * q_elem;
@@ -2161,11 +2163,11 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
 
   for (int attempt = 0; attempt < 2; ++attempt) {
     if (staged) {
-      if (half) sum_chunks<kVec, true, kK3Warps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
-      else sum_chunks<kVec, false, kK3Warps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
+      if (half) sum_chunks<kVec, true, kWarps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
+      else sum_chunks<kVec, false, kWarps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
     } else {
-      if (half) sum_chunks<kVec, true, kK3Warps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
-      else sum_chunks<kVec, false, kK3Warps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
+      if (half) sum_chunks<kVec, true, kWarps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
+      else sum_chunks<kVec, false, kWarps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
     }
     __syncthreads();
     // warp 0: scan of the slice; lane L owns chunks [lo, hi)
@@ -2180,18 +2182,25 @@ __global__ void __launch_bounds__(kK3Threads, kK3MaxPerSm) accept_sample_kernel(
         if (lane >= off) incl += o;
       }
       const double slice_total = __shfl_sync(0xffffffffu, incl, 31);
-      if (lane < S) *cluster.map_shared_rank(&sh_tot[attempt][rank], lane) = slice_total;
+      if (kSolo) {
+        if (lane == 0) sh_tot[attempt][0] = slice_total;
+      } else if (lane < S) {
+        *cluster.map_shared_rank(&sh_tot[attempt][rank], lane) = slice_total;
+      }
     }
-    cluster.sync();
+    if (kSolo) __syncthreads();
+    else cluster.sync();
     // every warp of every CTA: total mass and the slice that holds u * R (identical arithmetic everywhere); lane r has slice r
     const double slice_mass = lane < S ? sh_tot[attempt][lane] : 0.0;
     double slice_incl = slice_mass;
+    if (!kSolo) {
 #pragma unroll
-    for (int off = 1; off < 8; off <<= 1) {
-      const double o = __shfl_up_sync(0xffffffffu, slice_incl, off);
-      if (lane >= off) slice_incl += o;
+      for (int off = 1; off < 8; off <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, slice_incl, off);
+        if (lane >= off) slice_incl += o;
+      }
     }
-    const double R = __shfl_sync(0xffffffffu, slice_incl, 7);
+    const double R = __shfl_sync(0xffffffffu, slice_incl, kSolo ? 0 : 7);
     if (shard && p.phase == 3) {
       // the shard's masses of row n: of the residual, then (second pass, q taken as 0) of p itself
       if (rank == 0 && threadIdx.x == 0) {
@@ -2924,6 +2933,19 @@ int sample_cluster(const hola_ctx* ctx, const hola_verify_args* a) {
   return S;
 }
 
+// One CTA of 1024 threads per sequence instead of a cluster: no cluster barrier, the statistics of a row merged once, and with
+// one sequence per SM most SMs stay free for the next call's GEMM kernel, which then asks for its W_lm while this one runs.
+// Up to 16384 entries (more take one SM too long); beyond 8192 only where clusters would take more than a quarter of the
+// SMs (small batches have their rows staged), and only for rows of whole 16-byte pieces.
+// us, cluster -> one CTA, k = 4, H = 1024: V = 3000, 2 / 32 / 100 sequences 11.1 -> 10.6, 15.1 -> 14.5, 26.3 -> 25.1;
+// V = 8000, 4 / 16 / 64 13.3 -> 13.1, 14.9 -> 13.6, 19.5 -> 17.8; V = 16000, 1 / 8 / 24 14.3 -> 14.9, 16.6 -> 15.4,
+// 18.1 -> 17.4; V = 24000, 32 26.8 -> 28.2; V = 11001, 16 16.7 -> 17.0, V = 4001, 60 15.2 -> 15.1.  (V < 2048: a cluster
+// would be a single CTA, of 256 threads, which is enough.)
+bool sample_solo(const hola_ctx* ctx, const hola_verify_args* a) {
+  const int S = sample_cluster(ctx, a);
+  return S > 1 && a->B <= ctx->num_sms && a->V <= 16384 && (a->V <= 8192 || (a->V % 4 == 0 && 4 * a->B * S > ctx->num_sms));
+}
+
 // Where the logits of a verify step that does not hand them out go.  The greedy rule reads none (the arg-max travels with the
 // statistics), so none are stored then.  8-bit head and hidden rows, 192 rows, V = 128256 (98 MB of logits beside 525 MB of
 // codes): 137 -> 121 us.
@@ -3200,7 +3222,8 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   }
   const bool vec = (a->V % 4 == 0) && (ldl % 4 == 0) && aligned16(logits) && (a->k == 0 || aligned16(a->draft_q));
   const int nchunks = (a->V + kChunk - 1) / kChunk;
-  const int S = phase == 1 ? 1 : sample_cluster(ctx, a);             // (phase 1: no vocabulary pass)
+  const bool solo = phase == 0 && !sh && !q_far && sample_solo(ctx, a);
+  const int S = phase == 1 || solo ? 1 : sample_cluster(ctx, a);     // (phase 1: no vocabulary pass)
   const int cpc = (nchunks + S - 1) / S;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(a->B * S));
@@ -3211,7 +3234,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   // statistics and the accept test, so the slices of all rows are asked for before them (bulk copies: rows of whole
   // 16-byte pieces).
   kp.staged = 0;
-  if (vec && phase == 0 && (a->q_dtype == HOLA_Q_F32 || a->V % 8 == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && a->B * S <= ctx->num_sms) {
+  if (vec && phase == 0 && (a->q_dtype == HOLA_Q_F32 || a->V % 8 == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && !solo && a->B * S <= ctx->num_sms) {
     const size_t row_bytes = static_cast<size_t>(a->k + 1) * 4 + static_cast<size_t>(a->k) * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
     const size_t bytes = row_bytes * cpc * kChunk + sizeof(double);     // (and the rows start on a 16-byte boundary)
     if (bytes + cfg.dynamicSmemBytes <= kK3MaxDynSmem && row_bytes * a->V * a->B <= 4u << 20) {
@@ -3233,7 +3256,14 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   const bool ask = vec && !kp.staged && cpc <= 64 && a->B * S > ctx->num_sms;
-  const cudaError_t e = ask   ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, true>, kp)
+  if (solo) {
+    cfg.blockDim = dim3(kSoloThreads);
+    attr[0] = attr[1];                                   // (no cluster)
+    cfg.numAttrs = 1;
+  }
+  const cudaError_t e = solo  ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, true>, kp)
+                                     : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, true>, kp))
+                        : ask ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, true>, kp)
                         : vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false>, kp)
                               : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false>, kp);
   if (e != cudaSuccess) { set_error(ctx, "launch accept_sample_kernel", e); return HOLA_ERR_CUDA; }
@@ -3595,7 +3625,8 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   if (draft_gate && !inside && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
   const bool side = draft_gate && !inside && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
-  const bool few_before = a->B * sample_cluster(ctx, a) * 4 <= ctx->num_sms;
+  // (one CTA per sequence: half of the SMs free are enough; us, V = 8000, 64 sequences without / with 18.3 / 17.8)
+  const bool few_before = sample_solo(ctx, a) ? a->B * 2 <= ctx->num_sms : a->B * sample_cluster(ctx, a) * 4 <= ctx->num_sms;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample, inside);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);
