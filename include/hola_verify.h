@@ -306,6 +306,13 @@ hola_status hola_quantize_w4(const void* W_bf16, int rows, int H, void* packed_o
  * here).  Current device, asynchronous on the stream, allocates nothing. */
 hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream);
 
+/* The same with the widths on the host, widths[g] in {4, 8, 16} for group g: they travel as launch parameters, and the
+ * kernel fills the two tables too (out->group_width, out->group_row: device buffers for one entry per group, written here;
+ * out->rows4 / rows8 / rows16 must be the row counts that follow from the widths).  At most 2048 groups, else
+ * HOLA_ERR_UNSUPPORTED_SHAPE; nothing is read from `widths` after the call. */
+hola_status hola_quantize_mixed_widths(const void* W_bf16, int V, int H, const uint8_t* widths, const hola_wmix* out,
+                                       float* scale_out, void* cuda_stream);
+
 /* Launch geometry chosen for a shape (for reports): vocabulary rows per tile of a CTA pair, grid size (CTAs),
  * shared-memory ring slots, verify rows per pass, passes over W_lm, kernel launches per hola_verify call. */
 typedef struct {

@@ -7,6 +7,8 @@ from __future__ import annotations
 
 import ctypes
 import os
+import subprocess
+import warnings
 from array import array
 from dataclasses import dataclass
 
@@ -26,7 +28,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -62,6 +64,25 @@ class hola_plan_info(ctypes.Structure):
 
 
 _lib = None
+_host = None            # the native helper (csrc/host_call.cpp), or None: arguments are then filled from Python
+_entry = {}             # addresses of the entry points that it calls
+
+
+def _load_host(lib: ctypes.CDLL):
+    """The helper reads tensors through torch's C++ classes, so it must have been built against the torch that runs."""
+    global _host
+    try:
+        _build.build_host()
+        from . import _host_call
+        if _host_call.torch_version != torch.__version__:
+            _build.build_host(force=True)                        # (for the next process)
+            return
+    except (ImportError, OSError, subprocess.CalledProcessError) as e:
+        warnings.warn(f"host-side helper not available, calls cost a few microseconds more: {e}")
+        return
+    for name in ("hola_verify", "hola_verify_host", "hola_lm_head_entropy", "hola_quantize_mixed_widths"):
+        _entry[name] = ctypes.cast(getattr(lib, name), ctypes.c_void_p).value
+    _host = _host_call
 
 
 def load_library(path: str | None = None) -> ctypes.CDLL:
@@ -93,6 +114,9 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_quantize_mixed.restype = ctypes.c_int
     lib.hola_quantize_mixed.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_wmix),
                                         ctypes.c_void_p, ctypes.c_void_p]
+    lib.hola_quantize_mixed_widths.restype = ctypes.c_int
+    lib.hola_quantize_mixed_widths.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
+                                               ctypes.POINTER(hola_wmix), ctypes.c_void_p, ctypes.c_void_p]
     lib.hola_plan.restype = ctypes.c_int
     lib.hola_plan.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_plan_info)]
     lib.hola_plan_for_shape.restype = ctypes.c_int
@@ -127,6 +151,7 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_version.restype = ctypes.c_char_p
     if path is None:
         _lib = lib
+        _load_host(lib)
     return lib
 
 
@@ -188,11 +213,18 @@ class MixedHead:
 
 def hola_quantize_mixed(W_lm: torch.Tensor, widths, stream=None) -> MixedHead:
     """bf16 W_lm [V, H] -> the mixed-width form: widths[g] in {4, 8, 16} for group g of 256 vocabulary rows.  Codes,
-    scales and exponents are made by one launch of the library's quantiser; torch provides the buffers (and carries the
-    two tables of groups to the device in one copy)."""
+    scales and exponents are made by one launch of the library's quantiser, to which the widths go as launch parameters (on
+    another stream, for widths that are no plain list of integers and beyond 2048 groups: as two tables, in one copy);
+    torch provides the buffers."""
     if W_lm.dtype != torch.bfloat16 or not W_lm.is_cuda or not W_lm.is_contiguous():
         raise HolaError("hola_quantize_mixed takes a contiguous bfloat16 device tensor")
     lib = load_library()
+    if _host is not None and stream is None:
+        st = hola_wmix()
+        got = _host.quantize(_entry["hola_quantize_mixed_widths"], W_lm, widths, st, torch._C._cuda_getDevice(), _stream_ptr(None))
+        if got is not None:
+            _check(lib, None, got[0], "hola_quantize_mixed")
+            return MixedHead(*got[1:], st)
     V, H = W_lm.shape
     ng = -(-V // GROUP_ROWS)
     widths = [int(x) for x in widths]
@@ -297,6 +329,9 @@ def _fresh_outputs(ctx: "HolaVerify", B: int, k1: int, want_logits: bool, draws:
     out = VerifyOutputs.__new__(VerifyOutputs)
     dev = ctx._dev
     out._lazy = (B, k1 - 1, dev)
+    if _host is not None:
+        _host.outputs(out, ctx.device, B, k1, ctx.V, want_logits, draws, draft_gate)
+        return out
     # (sizes one by one and empty_like: the cheapest forms, 1.7 and 1.3 us against 2.4 with a tuple)
     out.entropy = e = torch.empty(B, k1, dtype=torch.float32, device=dev)
     out.logZ = torch.empty_like(e)
@@ -474,28 +509,41 @@ class HolaVerify:
         """The whole verify step on device tensors, asynchronous on the stream.  With w_scale, W_lm is the int8 form
         made by hola_quantize_w8; with a8 as well, the hidden rows are quantised on the fly and the products run on
         the 8-bit tensor-core kind."""
-        B, k1 = hidden.shape[:2]
         fresh = not out
         if fresh:
+            B, k1 = hidden.shape[:2]
             out = _fresh_outputs(self, B, k1, want_logits, True, gate_source == HOLA_GATE_DRAFT_ENTROPY)
-        a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k1 - 1, gate_source, fallback, w_scale, a8)
-        if fresh:
-            a.flags = HOLA_ARG_CLEAR_STATUS
-        st = self.lib.hola_verify(self._ctx, ctypes.byref(a), _stream_ptr(stream))
+        st = None
+        if _host is not None and self.lib is _lib:
+            st = _host.call(_entry["hola_verify"], self._ctx.value, self.H, self.V, hidden, W_lm, draft_tok, draft_q, uniforms,
+                            tau, out, 1, HOLA_ARG_CLEAR_STATUS if fresh else 0, gate_source, fallback, w_scale, a8,
+                            _stream_ptr(stream))
+        if st is None:
+            B, k1 = hidden.shape[:2]
+            a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k1 - 1, gate_source, fallback, w_scale, a8)
+            if fresh:
+                a.flags = HOLA_ARG_CLEAR_STATUS
+            st = self.lib.hola_verify(self._ctx, ctypes.byref(a), _stream_ptr(stream))
         if st:
             _check(self.lib, self._ctx, st, "hola_verify")
         return out
 
     def hola_lm_head_entropy(self, hidden, W_lm, out: VerifyOutputs | None = None, want_logits: bool = True,
                              stream=None, w_scale=None, a8: bool = False) -> VerifyOutputs:
-        B, k1 = hidden.shape[:2]
         fresh = not out
         if fresh:
+            B, k1 = hidden.shape[:2]
             out = _fresh_outputs(self, B, k1, want_logits, False, False)
-        a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k1 - 1, w_scale=w_scale, a8=a8, draws=False)
-        if fresh:
-            a.flags = HOLA_ARG_CLEAR_STATUS
-        st = self.lib.hola_lm_head_entropy(self._ctx, ctypes.byref(a), _stream_ptr(stream))
+        st = None
+        if _host is not None and self.lib is _lib:
+            st = _host.call(_entry["hola_lm_head_entropy"], self._ctx.value, self.H, self.V, hidden, W_lm, None, None, None, 0.0,
+                            out, 0, HOLA_ARG_CLEAR_STATUS if fresh else 0, 0, 0, w_scale, a8, _stream_ptr(stream))
+        if st is None:
+            B, k1 = hidden.shape[:2]
+            a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k1 - 1, w_scale=w_scale, a8=a8, draws=False)
+            if fresh:
+                a.flags = HOLA_ARG_CLEAR_STATUS
+            st = self.lib.hola_lm_head_entropy(self._ctx, ctypes.byref(a), _stream_ptr(stream))
         if st:
             _check(self.lib, self._ctx, st, "hola_lm_head_entropy")
         return out
@@ -525,16 +573,21 @@ class HolaVerify:
         """End-to-end form: per-step inputs and all outputs are HOST tensors (pinned for async copies);
         W_lm is the resident device weight.  Returns after the stream has been synchronised."""
         B, k = hidden.shape[0], hidden.shape[1] - 1
-        if not isinstance(W_lm, MixedHead) and W_lm.device.type != "cuda":
+        if not isinstance(W_lm, MixedHead) and not W_lm.is_cuda:
             raise HolaError("W_lm must be resident on the device")
         for t in (hidden, draft_tok, draft_q, uniforms):
-            if t is not None and t.device.type != "cpu":
+            if t is not None and not t.is_cpu:
                 raise HolaError("hola_verify_host takes host tensors for the per-step inputs")
         out = out or self.alloc_outputs(B, k, False, device=torch.device("cpu"))
-        a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k, gate_source, fallback, w_scale, a8)
-        a.logits_out = None
-        _check(self.lib, self._ctx, self.lib.hola_verify_host(self._ctx, ctypes.byref(a), _stream_ptr(stream)),
-               "hola_verify_host")
+        st = None
+        if _host is not None and self.lib is _lib and out.logits is None:
+            st = _host.call(_entry["hola_verify_host"], self._ctx.value, self.H, self.V, hidden, W_lm, draft_tok, draft_q,
+                            uniforms, tau, out, 1, 0, gate_source, fallback, w_scale, a8, _stream_ptr(stream))
+        if st is None:
+            a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k, gate_source, fallback, w_scale, a8)
+            a.logits_out = None
+            st = self.lib.hola_verify_host(self._ctx, ctypes.byref(a), _stream_ptr(stream))
+        _check(self.lib, self._ctx, st, "hola_verify_host")
         return out
 
 

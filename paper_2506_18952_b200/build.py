@@ -1,24 +1,32 @@
-"""Builds libhola_verify.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libhola_verify.so (nvcc, sm_100a; cross-compiles without a GPU) and the host-side helper _host_call.so (g++, against
+the installed torch) in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(_PKG, "csrc", "hola_verify.cu")
 HEADER = os.path.join(os.path.dirname(_PKG), "include", "hola_verify.h")
 LIB = os.path.join(_PKG, "libhola_verify.so")
+HOST_SRC = os.path.join(_PKG, "csrc", "host_call.cpp")
+HOST_LIB = os.path.join(_PKG, "_host_call.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-shared", "-Xcompiler", "-fPIC"]
 
 
-def needs_build() -> bool:
-    if not os.path.exists(LIB):
+def _older(out: str, *sources: str) -> bool:
+    if not os.path.exists(out):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in (SRC, HEADER))
+    t = os.path.getmtime(out)
+    return any(os.path.getmtime(f) > t for f in sources)
+
+
+def needs_build() -> bool:
+    return _older(LIB, SRC, HEADER)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -29,5 +37,19 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def build_host(force: bool = False) -> str:
+    if force or _older(HOST_LIB, HOST_SRC, HEADER):
+        import torch
+        root = os.path.dirname(os.path.abspath(torch.__file__))
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               f'-DHOLA_TORCH_VERSION="{torch.__version__}"',
+               f"-I{os.path.join(root, 'include')}", f"-I{sysconfig.get_paths()['include']}", "-o", HOST_LIB, HOST_SRC,
+               f"-L{os.path.join(root, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
+        subprocess.run(cmd, check=True)
+    return HOST_LIB
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    print(build_host(force="--force" in sys.argv))

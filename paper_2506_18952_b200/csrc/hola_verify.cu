@@ -2403,6 +2403,8 @@ __device__ __forceinline__ void scatter(T* dst, const uint4 x, int n) {
 
 // Where the quantised rows go: rows of one width sit compactly in that width's buffer.
 struct QuantOut {
+  uint8_t* tables_width;        // where the tables of the groups go, when their widths come as launch parameters (else null)
+  int* tables_row;
   const uint8_t* group_width;   // null: every row is `width` bits wide and row v of W is row v of its buffer
   const int* group_row;
   int width;
@@ -2414,6 +2416,20 @@ struct QuantOut {
   float* scale;
 };
 
+// Widths of a head's groups as launch parameters, two bits each (0: 4 bits, 1: 8, 2: 16; 3 past the last one), and how many
+// groups of 4 and of 8 bits come before each word: the kernel then makes the two tables as well, and no copy to the device
+// precedes it.
+constexpr int kMaxCodedGroups = 2048;                    // V <= 524288
+struct GroupCodes {
+  uint32_t w[kMaxCodedGroups / 16];
+  uint32_t before[kMaxCodedGroups / 16];                 // 4 bits in the low half, 8 bits in the high half
+};
+struct NoCodes {};
+__device__ __forceinline__ int same_codes(uint32_t word, uint32_t code) {        // fields of `word` that hold `code`
+  const uint32_t x = word ^ (code * 0x55555555u);
+  return __popc(~(x | (x >> 1)) & 0x55555555u);
+}
+
 // A head (or rows of it) to 4, 8 or 16 bits in ONE launch, a warp per row: one pass for the row's maximum, one that
 // rounds (the row, 8 KB at 4096 channels, then comes out of the L1 or the L2).  Bound: HBM (2 bytes in, half to two out
 // per weight).  32000 x 4096 at 4 / 8 / 16 bits in the proportions 20 / 70 / 10 %: a call of 81 us for 393 MB = 4.9 TB/s (61 us at
@@ -2421,8 +2437,9 @@ struct QuantOut {
 // row, two bytes per load and a division per weight needed 540 us.  Rows kept in registers between the passes: 102 registers,
 // 217 us with a slow path that divides next to half integers.
 // kVec: rows and buffers that 16-byte pieces tile and that are aligned for it; otherwise the same element by element.
-template <bool kVec>
-__global__ void __launch_bounds__(256, 3) quantize_rows_kernel(const uint16_t* W, int V, int H, const QuantOut out) {
+template <bool kVec, typename Codes = NoCodes>
+__global__ void __launch_bounds__(256, 3) quantize_rows_kernel(const uint16_t* W, int V, int H, const QuantOut out,
+                                                               const __grid_constant__ Codes codes) {
   const int v = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (v >= V) return;
@@ -2430,7 +2447,21 @@ __global__ void __launch_bounds__(256, 3) quantize_rows_kernel(const uint16_t* W
   const uint16_t* src = W + static_cast<size_t>(v) * H;
   int width = out.width;
   size_t row = v;
-  if (out.group_width) {
+  if constexpr (sizeof(Codes) == sizeof(GroupCodes)) {
+    // the groups before this one that have its width come first in that width's buffer (every one of them is whole)
+    const int g = v / kGroupRows;
+    const uint32_t mine = codes.w[g >> 4], code = (mine >> (2 * (g & 15))) & 3u;
+    const uint32_t n = codes.before[g >> 4], n4 = n & 0xFFFFu, n8 = n >> 16;
+    const int before = static_cast<int>(code == 0u ? n4 : code == 1u ? n8 : static_cast<uint32_t>(g & ~15) - n4 - n8) +
+                       same_codes(mine | (0xFFFFFFFFu << (2 * (g & 15))), code);
+    width = 4 << code;
+    const int first = before * kGroupRows;
+    row = static_cast<size_t>(first) + (v - g * kGroupRows);
+    if (lane == 0 && v == g * kGroupRows) {
+      out.tables_width[g] = static_cast<uint8_t>(width);
+      out.tables_row[g] = first;
+    }
+  } else if (out.group_width) {
     const int g = v / kGroupRows;
     width = out.group_width[g];
     row = static_cast<size_t>(out.group_row[g]) + (v - g * kGroupRows);
@@ -4037,13 +4068,16 @@ hola_status hola_host_traffic(const hola_ctx* ctx, unsigned long long* h2d_bytes
   return HOLA_OK;
 }
 
-static hola_status launch_quantiser(const void* W, int V, int H, const QuantOut& o, void* cuda_stream) {
+static hola_status launch_quantiser(const void* W, int V, int H, const QuantOut& o, void* cuda_stream,
+                                    const GroupCodes* codes = nullptr) {
   const bool vec = H % 8 == 0 && aligned16(W) && aligned16(o.w16) && aligned16(o.w8) && aligned16(o.w4);
   const unsigned grid = static_cast<unsigned>((V + 7) / 8);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   const uint16_t* src = static_cast<const uint16_t*>(W);
-  if (vec) quantize_rows_kernel<true><<<grid, 256, 0, stream>>>(src, V, H, o);
-  else quantize_rows_kernel<false><<<grid, 256, 0, stream>>>(src, V, H, o);
+  if (codes && vec) quantize_rows_kernel<true, GroupCodes><<<grid, 256, 0, stream>>>(src, V, H, o, *codes);
+  else if (codes) quantize_rows_kernel<false, GroupCodes><<<grid, 256, 0, stream>>>(src, V, H, o, *codes);
+  else if (vec) quantize_rows_kernel<true><<<grid, 256, 0, stream>>>(src, V, H, o, NoCodes{});
+  else quantize_rows_kernel<false><<<grid, 256, 0, stream>>>(src, V, H, o, NoCodes{});
   return cudaGetLastError() == cudaSuccess ? HOLA_OK : HOLA_ERR_CUDA;
 }
 
@@ -4064,7 +4098,8 @@ hola_status hola_quantize_w8(const void* W_bf16, int V, int H, void* q_out, floa
   return launch_quantiser(W_bf16, V, H, o, cuda_stream);
 }
 
-hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream) {
+static hola_status quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream,
+                                  const GroupCodes* codes) {
   if (!W_bf16 || !out || !scale_out || V <= 0 || H <= 0 || !out->group_width || !out->group_row) return HOLA_ERR_INVALID_ARG;
   if (H % kSubBlock != 0) return HOLA_ERR_UNSUPPORTED_SHAPE;
   if (out->rows4 < 0 || out->rows8 < 0 || out->rows16 < 0 ||
@@ -4074,11 +4109,36 @@ hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmi
     return HOLA_ERR_INVALID_ARG;
   QuantOut o = {};
   o.group_width = out->group_width; o.group_row = out->group_row;
+  o.tables_width = const_cast<uint8_t*>(out->group_width); o.tables_row = const_cast<int*>(out->group_row);
   o.w16 = static_cast<uint16_t*>(const_cast<void*>(out->W16));
   o.w8 = static_cast<signed char*>(const_cast<void*>(out->W8));
   o.w4 = static_cast<uint8_t*>(const_cast<void*>(out->W4));
   o.shift4 = const_cast<uint8_t*>(out->shift4); o.shift_stride = out->rows4; o.scale = scale_out;
-  return launch_quantiser(W_bf16, V, H, o, cuda_stream);
+  return launch_quantiser(W_bf16, V, H, o, cuda_stream, codes);
+}
+
+hola_status hola_quantize_mixed(const void* W_bf16, int V, int H, const hola_wmix* out, float* scale_out, void* cuda_stream) {
+  return quantize_mixed(W_bf16, V, H, out, scale_out, cuda_stream, nullptr);
+}
+
+hola_status hola_quantize_mixed_widths(const void* W_bf16, int V, int H, const uint8_t* widths, const hola_wmix* out,
+                                       float* scale_out, void* cuda_stream) {
+  if (!widths || !out || V <= 0) return HOLA_ERR_INVALID_ARG;
+  const int groups = (V + kGroupRows - 1) / kGroupRows;
+  if (groups > kMaxCodedGroups) return HOLA_ERR_UNSUPPORTED_SHAPE;
+  GroupCodes codes;
+  memset(&codes, 0xFF, sizeof codes);
+  int rows[3] = {0, 0, 0}, count[3] = {0, 0, 0};
+  for (int g = 0; g < groups; ++g) {
+    if (widths[g] != 4 && widths[g] != 8 && widths[g] != 16) return HOLA_ERR_INVALID_ARG;
+    const uint32_t code = widths[g] >> 3;                // 0, 1, 2
+    if ((g & 15) == 0) codes.before[g >> 4] = static_cast<uint32_t>(count[0]) | static_cast<uint32_t>(count[1]) << 16;
+    codes.w[g >> 4] ^= (3u ^ code) << (2 * (g & 15));
+    ++count[code];
+    rows[code] += g + 1 < groups ? kGroupRows : V - g * kGroupRows;
+  }
+  if (rows[0] != out->rows4 || rows[1] != out->rows8 || rows[2] != out->rows16) return HOLA_ERR_INVALID_ARG;
+  return quantize_mixed(W_bf16, V, H, out, scale_out, cuda_stream, &codes);
 }
 
 }  // extern "C"

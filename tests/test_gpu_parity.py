@@ -1330,3 +1330,25 @@ def test_entropy_of_rows_with_large_logits_keeps_its_accuracy(binding, V):
         err += float(((out.entropy - want) ** 2).sum())
         norm += float((want ** 2).sum())
     assert math.sqrt(err / norm) <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(want_logits=True), dict(gate_source=1), dict(fallback=1)])
+def test_native_marshalling_gives_what_python_gives(binding, monkeypatch, kw):
+    w = workloads.gaussian_head("native", 5, 3, 64, 1000, seed=5, device=DEV, w_std=0.3, tau=2.0)
+    assert binding._host is not None
+    with binding.HolaVerify(5, 3, 64, 1000) as ctx:
+        args = (w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)
+        got = [ctx.hola_verify(*args, **kw), ctx.hola_verify(*args, out=ctx.alloc_outputs(5, 3, "want_logits" in kw), **{
+            n: v for n, v in kw.items() if n != "want_logits"})]
+        stats = ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
+        monkeypatch.setattr(binding, "_host", None)
+        want, want_stats = ctx.hola_verify(*args, **kw), ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
+        torch.cuda.synchronize()
+    for out in got:
+        for name in ("accept_len", "next_tok", "entropy", "logZ", "status"):
+            a, b = getattr(out, name), getattr(want, name)
+            assert a.dtype == b.dtype and torch.equal(a, b), name
+        assert (out.logits is None) == (want.logits is None) and (want.logits is None or torch.equal(out.logits, want.logits))
+        assert torch.equal(out.draft_entropy, want.draft_entropy)
+    for name in ("entropy", "logZ", "logits", "status"):
+        assert torch.equal(getattr(stats, name), getattr(want_stats, name)), name

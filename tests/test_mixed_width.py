@@ -354,3 +354,43 @@ def test_quantiser_takes_an_empty_head_and_any_object_with_a_cuda_stream(binding
         side.synchronize()
         for name in ("W16", "W8", "W4", "shift4", "w_scale", "group_width", "group_row"):
             assert torch.equal(getattr(got, name), getattr(want, name)), name
+
+
+@pytest.mark.parametrize("groups,rest,H,pattern", [
+    (1, 256, 128, [4]), (2, 44, 128, [16, 4]), (16, 256, 128, [8, 4, 16]), (17, 1, 256, [4, 8, 8, 16, 4]),
+    (33, 255, 384, [16]), (100, 100, 1152, [8, 16, 8, 4, 4]), (2048, 256, 128, [8, 4, 16, 8]),
+    (2049, 3, 128, [4, 16, 8]),                          # more groups than launch parameters hold: through the tables
+])
+def test_widths_as_launch_parameters_give_the_head_that_tables_give(binding, monkeypatch, groups, rest, H, pattern):
+    V = 256 * (groups - 1) + rest
+    g = torch.Generator(device=DEV).manual_seed(groups)
+    W = (torch.randn((V, H), generator=g, device=DEV) * 0.02).bfloat16()
+    widths = _widths(V, pattern)
+    assert binding._host is not None
+    got = [binding.hola_quantize_mixed(W, x) for x in (widths, tuple(widths))]
+    monkeypatch.setattr(binding, "_host", None)
+    want = binding.hola_quantize_mixed(W, widths)
+    torch.cuda.synchronize()
+    for head in got:
+        assert (head.V, head.H, head.widths) == (V, H, widths)
+        for name in ("W16", "W8", "W4", "shift4", "w_scale", "group_width", "group_row"):
+            a, b = getattr(head, name), getattr(want, name)
+            assert (a is None and b is None) or (a.dtype == b.dtype and torch.equal(a, b)), name
+        for name in ("rows16", "rows8", "rows4"):
+            assert getattr(head.struct, name) == getattr(want.struct, name)
+
+
+def test_widths_on_the_host_are_checked(binding):
+    import ctypes
+    lib = binding.load_library()
+    W = torch.zeros((600, 128), dtype=torch.bfloat16, device=DEV)
+    head = binding.hola_quantize_mixed(W, [4, 8, 16])
+
+    def status(widths, V=600, H=128):
+        return lib.hola_quantize_mixed_widths(ctypes.c_void_p(W.data_ptr()), V, H, bytes(widths), ctypes.byref(head.struct),
+                                              ctypes.c_void_p(head.w_scale.data_ptr()), None)
+    assert status([4, 8, 16]) == 0
+    assert status([4, 8, 5]) == 1 and status([4, 16, 8]) == 1 and status([8, 4, 16], V=599) == 1     # row counts that do not fit
+    assert status([4, 8, 16], H=100) == 2 and lib.hola_quantize_mixed_widths(None, 600, 128, None, None, None, None) == 1
+    assert status([4] * 2049, V=2049 * 256) == 2
+    torch.cuda.synchronize()
