@@ -2572,6 +2572,12 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
                                                                       float* s1, float* s2) {
   __shared__ float sh_max[kHidThreads / 32];
   grid_dependency_wait();                                // (no-op unless launched with programmatic serialization)
+  // The GEMM kernel may be put in place beside this one (its CTA and several of these fit an SM): its launch and set-up and,
+  // on small batches, its first requests for W_lm hide behind the quantisation.  It waits for this grid's end before it reads
+  // anything.  us, 8-bit planes, no release / at entry / here / behind the loads: one sequence, V = 32000 33.0 / 30.7 / 30.6 /
+  // 31.9, two planes 33.4 / 30.8 / 31.3 / 31.2; 80 rows, V = 11000 17.5 / 16.5 / 16.2 / 16.3; 300 rows, V = 16000 28.1 / 26.9 /
+  // 26.7 / 28.4.
+  grid_dependency_release();
   const int row = blockIdx.x;
   const int pieces = H >> 3;
   const size_t row1 = kTwoPlane ? static_cast<size_t>(64) * (row >> 5) + (row & 31) : static_cast<size_t>(row);
