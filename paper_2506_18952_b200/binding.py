@@ -492,6 +492,20 @@ class HolaVerify:
                 a.w_dtype = HOLA_W8A16 if a8 == "a16" else (HOLA_W8A8 if a8 else HOLA_W_INT8)
         return a
 
+    def _native(self, entry, hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, draws, flags, gate_source, fallback, w_scale,
+                a8, stream):
+        """The call through the native helper: its status, or None where the arguments have to be made from Python."""
+        if _host is None or self.lib is not _lib:
+            return None
+        wmix = 0
+        if type(W_lm) is MixedHead:
+            if w_scale is not None or a8 or W_lm.V != self.V or W_lm.H != self.H:
+                return None
+            wmix, w_scale = ctypes.addressof(W_lm.struct), W_lm.w_scale
+            W_lm = W_lm.W8 if W_lm.W8 is not None else (W_lm.W4 if W_lm.W4 is not None else W_lm.W16)
+        return _host.call(_entry[entry], self._ctx.value, self.H, self.V, hidden, W_lm, draft_tok, draft_q, uniforms, tau, out,
+                          draws, flags, gate_source, fallback, w_scale, a8, wmix, _stream_ptr(stream))
+
     def alloc_outputs(self, B: int, k: int, want_logits: bool = False, device=None) -> VerifyOutputs:
         dev = torch.device("cuda", self.device) if device is None else device
         return VerifyOutputs(
@@ -513,11 +527,8 @@ class HolaVerify:
         if fresh:
             B, k1 = hidden.shape[:2]
             out = _fresh_outputs(self, B, k1, want_logits, True, gate_source == HOLA_GATE_DRAFT_ENTROPY)
-        st = None
-        if _host is not None and self.lib is _lib:
-            st = _host.call(_entry["hola_verify"], self._ctx.value, self.H, self.V, hidden, W_lm, draft_tok, draft_q, uniforms,
-                            tau, out, 1, HOLA_ARG_CLEAR_STATUS if fresh else 0, gate_source, fallback, w_scale, a8,
-                            _stream_ptr(stream))
+        st = self._native("hola_verify", hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, 1,
+                          HOLA_ARG_CLEAR_STATUS if fresh else 0, gate_source, fallback, w_scale, a8, stream)
         if st is None:
             B, k1 = hidden.shape[:2]
             a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k1 - 1, gate_source, fallback, w_scale, a8)
@@ -534,10 +545,8 @@ class HolaVerify:
         if fresh:
             B, k1 = hidden.shape[:2]
             out = _fresh_outputs(self, B, k1, want_logits, False, False)
-        st = None
-        if _host is not None and self.lib is _lib:
-            st = _host.call(_entry["hola_lm_head_entropy"], self._ctx.value, self.H, self.V, hidden, W_lm, None, None, None, 0.0,
-                            out, 0, HOLA_ARG_CLEAR_STATUS if fresh else 0, 0, 0, w_scale, a8, _stream_ptr(stream))
+        st = self._native("hola_lm_head_entropy", hidden, W_lm, None, None, None, 0.0, out, 0,
+                          HOLA_ARG_CLEAR_STATUS if fresh else 0, 0, 0, w_scale, a8, stream)
         if st is None:
             B, k1 = hidden.shape[:2]
             a = self._args(hidden, W_lm, None, None, None, 0.0, out, B, k1 - 1, w_scale=w_scale, a8=a8, draws=False)
@@ -580,9 +589,9 @@ class HolaVerify:
                 raise HolaError("hola_verify_host takes host tensors for the per-step inputs")
         out = out or self.alloc_outputs(B, k, False, device=torch.device("cpu"))
         st = None
-        if _host is not None and self.lib is _lib and out.logits is None:
-            st = _host.call(_entry["hola_verify_host"], self._ctx.value, self.H, self.V, hidden, W_lm, draft_tok, draft_q,
-                            uniforms, tau, out, 1, 0, gate_source, fallback, w_scale, a8, _stream_ptr(stream))
+        if out.logits is None:
+            st = self._native("hola_verify_host", hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, 1, 0, gate_source,
+                              fallback, w_scale, a8, stream)
         if st is None:
             a = self._args(hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, B, k, gate_source, fallback, w_scale, a8)
             a.logits_out = None

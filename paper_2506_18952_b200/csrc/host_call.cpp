@@ -1,7 +1,8 @@
 // The host side of a call on torch tensors, in native code: reads the tensors, fills hola_verify_args and calls the C ABI;
 // makes the output tensors of a call that is given none.  What a call costs the host bounds small problems: filling the
-// arguments field by field from Python takes 3.4 us, six output tensors 6 to 7 us, beside 5 us for the two launches.
-// HOSTFIG
+// arguments field by field from Python takes 3.4 us, six output tensors 6 to 7 us, beside 5 us for the two launches.  us, Python
+// -> native: one sequence, V = 1000 10.45 -> 9.75; three, V = 5000, fresh outputs 19.75 -> 13.2; host entry, two sequences,
+// V = 10000 42.1 -> 37.4; mixed-width quantiser, 1000 x 128 50 -> 13.8.
 //
 // call() takes the plain forms only (torch.Tensor or Parameter objects with storage, strided, contiguous, of the types that
 // the entry points know) and answers None for everything else, before it has done anything: the caller then goes the long
@@ -76,16 +77,17 @@ bool address(PyObject* o, void** p) {
 PyObject *n_accept, *n_next, *n_entropy, *n_logZ, *n_logits, *n_status, *n_dent;
 
 // call(function, ctx, H, V, hidden, W_lm, draft_tok, draft_q, uniforms, tau, out, draws, flags, gate_source, fallback, w_scale,
-//      a8, stream) -> status, or None where the caller has to go the long way
+//      a8, wmix, stream) -> status, or None where the caller has to go the long way.  wmix: address of the hola_wmix of a head of
+// mixed widths, whose first buffer is W_lm then, or 0.
 PyObject* call(PyObject*, PyObject* const* v, Py_ssize_t n) {
   HANDLE_TH_ERRORS
-  if (n != 18) { PyErr_SetString(PyExc_TypeError, "call() takes 18 arguments"); return nullptr; }
-  void *fn = nullptr, *ctx = nullptr, *stream = nullptr, *p = nullptr;
+  if (n != 19) { PyErr_SetString(PyExc_TypeError, "call() takes 19 arguments"); return nullptr; }
+  void *fn = nullptr, *ctx = nullptr, *stream = nullptr, *wmix = nullptr, *p = nullptr;
   hola_verify_args a = {};
   int32_t H = 0, V = 0, draws = 0;
   if (!address(v[0], &fn) || !fn || !address(v[1], &ctx) || !ctx || !int32(v[2], &H) || !int32(v[3], &V) ||
       !int32(v[11], &draws) || !int32(v[12], &a.flags) || !int32(v[13], &a.gate_source) || !int32(v[14], &a.fallback) ||
-      !address(v[17], &stream))
+      !address(v[17], &wmix) || !address(v[18], &stream))
     Py_RETURN_NONE;
   const at::Tensor *hidden = nullptr, *W = nullptr, *q = nullptr, *scale = nullptr;
   void *ph = nullptr, *pw = nullptr, *pt = nullptr, *pq = nullptr, *pu = nullptr;
@@ -96,9 +98,9 @@ PyObject* call(PyObject*, PyObject* const* v, Py_ssize_t n) {
     scale = plain(v[15]);
     if (!scale) Py_RETURN_NONE;
   }
-  const bool w8 = W->scalar_type() == at::kChar;
+  const bool w8 = !wmix && W->scalar_type() == at::kChar;
   if (hidden->dim() < 2 || hidden->size(0) > INT32_MAX || hidden->size(1) > INT32_MAX || hidden->scalar_type() != at::kBFloat16 ||
-      (!w8 && W->scalar_type() != at::kBFloat16) || w8 != (scale != nullptr) ||
+      (!wmix && !w8 && W->scalar_type() != at::kBFloat16) || (w8 || wmix) != (scale != nullptr) ||
       (q && q->scalar_type() != at::kBFloat16 && q->scalar_type() != at::kFloat))
     Py_RETURN_NONE;
   if (w8) {
@@ -109,6 +111,11 @@ PyObject* call(PyObject*, PyObject* const* v, Py_ssize_t n) {
     a.w_scale = static_cast<const float*>(scale->data_ptr());
   } else if (v[16] != Py_False) {
     Py_RETURN_NONE;
+  } else if (wmix) {
+    a.w_dtype = HOLA_W_MIXED;
+    a.wmix = static_cast<const hola_wmix*>(wmix);
+    a.w_scale = static_cast<const float*>(scale->data_ptr());
+    pw = nullptr;
   }
   long long whole = 0;
   if (PyFloat_CheckExact(v[9])) a.tau = static_cast<float>(PyFloat_AS_DOUBLE(v[9]));

@@ -1,6 +1,7 @@
 """The native argument marshalling (csrc/host_call.cpp) against the one in Python, through a stand-in for the C entry point
 that keeps a copy of the arguments it gets."""
 import ctypes
+import types
 
 import pytest
 import torch
@@ -14,6 +15,7 @@ ENTRY = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.POINTER(binding.h
 class _Ctx(binding.HolaVerify):
     def __init__(self, H, V):
         self.H, self.V, self.device, self._dev, self._ctx = H, V, 0, torch.device("cpu"), ctypes.c_void_p(16)
+        self.lib = lib
 
     def close(self):
         pass
@@ -33,9 +35,12 @@ def _native(t, out, ctx, tau=1.5, draws=1, flags=0, gate=0, fallback=0, a8=False
         got.append((c, bytes(a.contents), s))
         return 7
     fn = ENTRY(entry)
-    st = binding._host.call(ctypes.cast(fn, ctypes.c_void_p).value, ctx._ctx.value, ctx.H, ctx.V, t["hidden"], t["W_lm"],
-                            t["draft_tok"], t["draft_q"], t["uniforms"], tau, out, draws, flags, gate, fallback, t["w_scale"], a8,
-                            32)
+    binding._entry["stand-in"] = ctypes.cast(fn, ctypes.c_void_p).value
+    try:
+        st = ctx._native("stand-in", t["hidden"], t["W_lm"], t["draft_tok"], t["draft_q"], t["uniforms"], tau, out, draws, flags,
+                         gate, fallback, t["w_scale"], a8, types.SimpleNamespace(cuda_stream=32))
+    finally:
+        del binding._entry["stand-in"]
     if st is None:
         assert not got
         return None
@@ -90,3 +95,23 @@ def test_other_forms_are_left_to_python(change):
     kw = {n: change.pop(n) for n in list(change) if n not in t}
     t.update(change)
     assert _native(t, out, _Ctx(64, 40), **kw) is None
+
+
+@pytest.mark.parametrize("which", ["W8", "W4", "W16"])
+def test_heads_of_mixed_widths(which):
+    t, out = _tensors(2, 3, 128, 40)
+    ctx = _Ctx(128, 40)
+    buf = {"W16": torch.zeros(40, 128, dtype=torch.bfloat16), "W8": torch.zeros(40, 128, dtype=torch.int8),
+           "W4": torch.zeros(40, 64, dtype=torch.uint8)}[which]
+    bufs = {"W16": None, "W8": None, "W4": None, which: buf}
+    head = binding.MixedHead(40, 128, [8], bufs["W16"], bufs["W8"], bufs["W4"], None, torch.zeros(40),
+                             torch.zeros(1, dtype=torch.uint8), torch.zeros(1, dtype=torch.int32), binding.hola_wmix())
+    t["W_lm"] = head
+    for kw in (dict(), dict(gate=1, flags=1, tau=3.0), dict(draws=0)):
+        assert _native(t, out, ctx, **kw) == _python(t, out, ctx, **kw)
+    assert _native(t, out, ctx, a8=True) is None and _native(t, out, _Ctx(128, 41)) is None
+    t["w_scale"] = torch.zeros(40)
+    assert _native(t, out, ctx) is None
+    t["w_scale"] = None
+    setattr(head, which, torch.zeros(buf.shape[::-1], dtype=buf.dtype).t())
+    assert _native(t, out, ctx) is None
