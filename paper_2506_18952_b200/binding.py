@@ -1,4 +1,5 @@
-"""ctypes binding of libhola_verify.so: argument marshalling only, every step runs in the CUDA kernels.
+"""Binding of libhola_verify.so (ctypes, and native code for the calls of a serving loop, csrc/host_call.cpp): argument
+marshalling only, every step runs in the CUDA kernels.
 
 Function names mirror the C ABI (include/hola_verify.h).  Tensors are torch CUDA tensors; torch is used for
 device memory and streams, nothing else.

@@ -28,7 +28,7 @@
 //   shard_record_kernel         vocabulary-parallel form: a rank's statistics record for the first all-gather.
 //   finalize_kernel             merges the per-CTA statistics:  logZ = m + ln s,  H = ln s - t/s  (entropy
 //       definition of the HSD section, rearranged around the running maximum).
-//   accept_sample_kernel        one cluster of CTAs per sequence: merges the statistics for its k+1 positions (warp
+//   accept_sample_kernel        one cluster of CTAs, or one large CTA, per sequence: merges the statistics for its k+1 positions (warp
 //       shuffles), applies the entropy gate and the ratio test in draft order, then makes one vectorised pass
 //       over the logits row and the draft row of the first rejected position: residual max(0, p - q), per-chunk
 //       sums, a scan, and the inverse-CDF pick with the supplied uniform.
