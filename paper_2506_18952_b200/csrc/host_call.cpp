@@ -160,8 +160,8 @@ PyObject* outputs(PyObject*, PyObject* const* v, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   long long x[7];
   if (n != 8) { PyErr_SetString(PyExc_TypeError, "outputs() takes 8 arguments"); return nullptr; }
-  for (int i = 0; i < 7; ++i) {
-    x[i] = PyLong_AsLongLong(v[1 + i]);
+  for (int i = 0; i < 7; ++i) {                          // (what is wanted: any object, by its truth value)
+    x[i] = i < 4 ? PyLong_AsLongLong(v[1 + i]) : PyObject_IsTrue(v[1 + i]);
     if (x[i] == -1 && PyErr_Occurred()) return nullptr;
   }
   const long long B = x[1], k1 = x[2], V = x[3];

@@ -1332,13 +1332,16 @@ def test_entropy_of_rows_with_large_logits_keeps_its_accuracy(binding, V):
     assert math.sqrt(err / norm) <= 2.0 ** -21
 
 
-@pytest.mark.parametrize("kw", [dict(), dict(want_logits=True), dict(gate_source=1), dict(fallback=1)])
+@pytest.mark.parametrize("kw", [
+    dict(), dict(want_logits=True), dict(gate_source=1), dict(fallback=1),
+    dict(want_logits=None), dict(want_logits=np.True_), dict(gate_source=np.int64(1)), dict(fallback=np.int32(1), want_logits=1.0),
+])
 def test_native_marshalling_gives_what_python_gives(binding, monkeypatch, kw):
     w = workloads.gaussian_head("native", 5, 3, 64, 1000, seed=5, device=DEV, w_std=0.3, tau=2.0)
     assert binding._host is not None
     with binding.HolaVerify(5, 3, 64, 1000) as ctx:
         args = (w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)
-        got = [ctx.hola_verify(*args, **kw), ctx.hola_verify(*args, out=ctx.alloc_outputs(5, 3, "want_logits" in kw), **{
+        got = [ctx.hola_verify(*args, **kw), ctx.hola_verify(*args, out=ctx.alloc_outputs(5, 3, bool(kw.get("want_logits"))), **{
             n: v for n, v in kw.items() if n != "want_logits"})]
         stats = ctx.hola_lm_head_entropy(w.hidden, w.W_lm)
         monkeypatch.setattr(binding, "_host", None)

@@ -3,6 +3,7 @@ that keeps a copy of the arguments it gets."""
 import ctypes
 import types
 
+import numpy as np
 import pytest
 import torch
 
@@ -115,3 +116,35 @@ def test_heads_of_mixed_widths(which):
     t["w_scale"] = None
     setattr(head, which, torch.zeros(buf.shape[::-1], dtype=buf.dtype).t())
     assert _native(t, out, ctx) is None
+
+
+class _Truth:
+    """An object that has a truth value and nothing else."""
+
+    def __init__(self, value):
+        self.value = value
+
+    def __bool__(self):
+        return self.value
+
+
+@pytest.mark.parametrize("wanted", [None, np.True_, np.bool_(False), torch.tensor(True), [], "yes", 2.5, _Truth(True)])
+def test_outputs_take_the_truth_value_of_what_is_wanted(wanted):
+    """Without a device the call ends where the first tensor is allocated: past the arguments."""
+    def made(*flags):
+        out = types.SimpleNamespace()
+        try:
+            binding._host.outputs(out, 0, 2, 4, 40, *flags)
+        except RuntimeError:
+            assert not torch.cuda.is_available()
+            return None
+        return out
+    for out in (made(wanted, True, False), made(True, wanted, False), made(False, True, wanted)):
+        assert out is None or out.entropy.shape == (2, 4)
+    if torch.cuda.is_available():
+        assert (made(wanted, False, False).logits is not None) == bool(wanted)
+        assert hasattr(made(False, wanted, False), "next_tok") == hasattr(made(False, False, wanted), "draft_entropy") == bool(wanted)
+    with pytest.raises(TypeError):
+        binding._host.outputs(types.SimpleNamespace(), 0, "2", 4, 40, True, True, True)
+    with pytest.raises(ValueError, match="ambiguous"):
+        made(np.zeros(2), True, True)
