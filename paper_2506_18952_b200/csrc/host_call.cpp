@@ -254,9 +254,16 @@ PyObject* quantize(PyObject*, PyObject* const* v, Py_ssize_t n) {
   }
   Py_END_ALLOW_THREADS
   PyBuffer_Release(&buf);
+  PyObject* used = PyList_New(static_cast<Py_ssize_t>(groups));          // (what was used: the caller's list may be another by now)
+  if (!used) return nullptr;
+  for (int64_t g = 0; g < groups; ++g) {
+    PyObject* w = PyLong_FromLong(widths[g]);
+    if (!w) { Py_DECREF(used); return nullptr; }
+    PyList_SET_ITEM(used, g, w);
+  }
   auto wrap = [](const at::Tensor& t) { return t.defined() ? THPVariable_Wrap(t) : Py_NewRef(Py_None); };
   return Py_BuildValue("iLLNNNNNNNN", static_cast<int>(s), static_cast<long long>(V), static_cast<long long>(H),
-                       PySequence_List(v[2]), wrap(W16), wrap(W8), wrap(W4), wrap(shift4), wrap(scale), wrap(group_width),
+                       used, wrap(W16), wrap(W8), wrap(W4), wrap(shift4), wrap(scale), wrap(group_width),
                        wrap(group_row));
   END_HANDLE_TH_ERRORS
 }

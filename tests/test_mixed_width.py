@@ -394,3 +394,21 @@ def test_widths_on_the_host_are_checked(binding):
     assert status([4, 8, 16], H=100) == 2 and lib.hola_quantize_mixed_widths(None, 600, 128, None, None, None, None) == 1
     assert status([4] * 2049, V=2049 * 256) == 2
     torch.cuda.synchronize()
+
+
+def test_a_list_of_widths_that_changes_during_the_call_leaves_the_head_as_it_was_made(binding, monkeypatch):
+    """The native quantiser call lets other threads run; one of them may reuse the list."""
+    import ctypes
+    lib = binding.load_library()
+    W = torch.zeros((600, 128), dtype=torch.bfloat16, device=DEV)
+    widths = [4, 8, 16]
+
+    def entry(*args):
+        widths[:] = [16, 16]
+        return lib.hola_quantize_mixed_widths(*args)
+    p = ctypes.c_void_p
+    fn = ctypes.CFUNCTYPE(ctypes.c_int, p, ctypes.c_int, ctypes.c_int, p, ctypes.POINTER(binding.hola_wmix), p, p)(entry)
+    monkeypatch.setitem(binding._entry, "hola_quantize_mixed_widths", ctypes.cast(fn, p).value)
+    head = binding.hola_quantize_mixed(W, widths)
+    torch.cuda.synchronize()
+    assert widths == [16, 16] and head.widths == [4, 8, 16] and head.group_width.tolist() == [4, 8, 16]
