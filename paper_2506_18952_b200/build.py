@@ -2,6 +2,8 @@
 the installed torch) in-tree."""
 from __future__ import annotations
 
+import contextlib
+import fcntl
 import os
 import subprocess
 import sys
@@ -25,28 +27,59 @@ def _older(out: str, *sources: str) -> bool:
     return any(os.path.getmtime(f) > t for f in sources)
 
 
+@contextlib.contextmanager
+def _build_lock():
+    """One build at a time in this tree: a lock on the package's folder.  (Where the file system has none, processes that
+    start together build more often than needed, nothing else.)"""
+    fd = os.open(_PKG, os.O_RDONLY)
+    try:
+        with contextlib.suppress(OSError):
+            fcntl.flock(fd, fcntl.LOCK_EX)
+        yield
+    finally:
+        os.close(fd)
+
+
+def _link(cmd: list, out: str, wanted) -> None:
+    """Runs the compiler on a file of its own beside `out` and moves it there whole, so that nobody meets the half of a
+    library, now or after an interrupted build.  `wanted` is asked again once the lock is held: another process may have
+    built meanwhile."""
+    with _build_lock():
+        if not wanted():
+            return
+        tmp = f"{out.removesuffix('.so')}.{os.getpid()}.tmp.so"
+        try:
+            subprocess.run([*cmd, "-o", tmp], check=True)
+            os.replace(tmp, out)
+        finally:
+            with contextlib.suppress(FileNotFoundError):
+                os.unlink(tmp)
+
+
 def needs_build() -> bool:
     return _older(LIB, SRC, HEADER)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if force or needs_build():
+    def wanted():
+        return force or needs_build()
+    if wanted():
         nvcc = os.environ.get("NVCC", "nvcc")
-        cmd = [nvcc, *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), "-o", LIB, SRC]
-        subprocess.run(cmd, check=True)
+        _link([nvcc, *NVCC_FLAGS, *(["-Xptxas", "-v"] if verbose else []), SRC], LIB, wanted)
     return LIB
 
 
 def build_host(force: bool = False) -> str:
-    if force or _older(HOST_LIB, HOST_SRC, HEADER):
+    def wanted():
+        return force or _older(HOST_LIB, HOST_SRC, HEADER)
+    if wanted():
         import torch
         root = os.path.dirname(os.path.abspath(torch.__file__))
-        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+        _link([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
                f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
                f'-DHOLA_TORCH_VERSION="{torch.__version__}"',
-               f"-I{os.path.join(root, 'include')}", f"-I{sysconfig.get_paths()['include']}", "-o", HOST_LIB, HOST_SRC,
-               f"-L{os.path.join(root, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
-        subprocess.run(cmd, check=True)
+               f"-I{os.path.join(root, 'include')}", f"-I{sysconfig.get_paths()['include']}", HOST_SRC,
+               f"-L{os.path.join(root, 'lib')}", "-ltorch_python", "-ltorch_cpu", "-lc10"], HOST_LIB, wanted)
     return HOST_LIB
 
 
