@@ -70,20 +70,16 @@ _entry = {}             # addresses of the entry points that it calls
 
 
 def _load_host(lib: ctypes.CDLL):
-    """The helper reads tensors through torch's C++ classes, so it must have been built against the torch that runs."""
+    """The helper reads tensors through torch's C++ classes: it is built against the torch that runs."""
     global _host
     try:
-        _build.build_host()
-        from . import _host_call
-        if _host_call.torch_version != torch.__version__:
-            _build.build_host(force=True)                        # (for the next process)
-            return
+        helper = _build.load_host()
     except (ImportError, OSError, subprocess.CalledProcessError) as e:
         warnings.warn(f"host-side helper not available, calls cost a few microseconds more: {e}")
         return
     for name in ("hola_verify", "hola_verify_host", "hola_lm_head_entropy", "hola_quantize_mixed_widths"):
         _entry[name] = ctypes.cast(getattr(lib, name), ctypes.c_void_p).value
-    _host = _host_call
+    _host = helper
 
 
 def load_library(path: str | None = None) -> ctypes.CDLL:

@@ -284,6 +284,5 @@ PyMODINIT_FUNC PyInit__host_call(void) {
   n_entropy = PyUnicode_InternFromString("entropy"); n_logZ = PyUnicode_InternFromString("logZ");
   n_logits = PyUnicode_InternFromString("logits"); n_status = PyUnicode_InternFromString("status");
   n_dent = PyUnicode_InternFromString("draft_entropy");
-  if (PyModule_AddStringConstant(m, "torch_version", HOLA_TORCH_VERSION) < 0) return nullptr;
   return m;
 }
