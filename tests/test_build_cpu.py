@@ -105,3 +105,18 @@ def test_a_helper_of_another_torch_or_python_is_not_looked_at(helpers, compiler,
         m.setattr(b.sysconfig, "get_config_var", lambda name: "cpython-399" if name == "SOABI" else None)
         assert callable(b.load_host().call) and compiler.runs() == 2
     assert len(os.listdir(b._PKG)) == 3
+
+
+def test_the_build_succeeds_without_the_helper(monkeypatch):
+    """As on a box without Python headers: calls are then filled from Python."""
+    import __graft_entry__
+    from paper_2506_18952_b200 import binding
+
+    def no_headers(*args, **kw):
+        raise subprocess.CalledProcessError(1, "g++")
+    monkeypatch.setattr(b, "build_host", no_headers)
+    for name, empty in (("_lib", None), ("_host", None), ("_entry", {})):
+        monkeypatch.setattr(binding, name, empty)
+    with pytest.warns(UserWarning, match="host-side helper not available"):
+        __graft_entry__.build()
+    assert binding._lib is not None and binding._host is None
