@@ -46,8 +46,8 @@ NOMINAL_PEAKS = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of lm_head_entropy_kernel<0>, from the ncu captures
 # summarised under profiles/: "batched" (--set full capture), "large_vocab" and "wide" (captures of the three DRAM /
 # time counters on the full-size launch; their logits are stored with the streaming hint, so most of them reach DRAM
-# inside the kernel; "wide" is the one launch that holds all six passes).  Other workloads, and the other weight modes,
-# report null.
+# inside the kernel; "wide" is the one launch that holds all six passes).  Other workloads, weight modes, gates and
+# fallbacks report null.
 NCU_TRAFFIC = {"batched": 265911680 + 8094490, "large_vocab": 1055523742 + 165214129,
                "wide": 2598598827 + 1165225941}
 
@@ -462,7 +462,9 @@ def main():
         # (w8a16 runs two 8-bit rows per verify row: per algorithmic flop its peak is the bf16 one again)
         roof = fractions(work, peaks, k1_ms * 1e-3 * k1_launches, ms_max / args.steps * 1e-3,
                          2.0 if a8 is True else 1.0)
-        traffic = ncu_traffic_bytes(w) if args.weights == "bf16" else None
+        # (the captures are of the default step: a greedy one stores no logits, the draft gate's pass adds reads)
+        default_step = args.weights == "bf16" and args.fallback == "sample" and args.gate == "target"
+        traffic = ncu_traffic_bytes(w) if default_step else None
         roof["traffic"] = traffic
         roof["traffic_source"] = ("ncu capture summarised under profiles/ (a constant of this file, not measured by this "
                                   "run)") if traffic is not None else None
