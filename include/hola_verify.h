@@ -323,6 +323,12 @@ hola_status hola_plan_ex(const hola_ctx* ctx, int B, int k, int w_dtype, hola_pl
 /* The same for a shape alone: no context and no device (host arithmetic only), default tuning options.  num_sms is
  * the SM count the grid is cut for (148 on a B200), rows = B (k + 1) verify rows. */
 hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype, hola_plan_info* out);
+/* And for the accept/sample kernel of hola_verify: CTAs per sequence, threads per CTA, and whether the rows go through shared
+ * memory (1) or are read where they are (0).  For tensors that start on a 16-byte boundary. */
+typedef struct {
+  int32_t ctas, threads, staged;
+} hola_sample_info;
+hola_status hola_sample_plan_for_shape(int num_sms, int B, int k, int V, int q_dtype, int fallback, hola_sample_info* out);
 
 /* Per-kernel timing for reports.  Between hola_profile_begin and hola_profile_end every hola_verify call (at
  * most max_calls of them, max_calls <= 4096) records CUDA events on its stream around the LM-head GEMM launches

@@ -29,7 +29,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -62,6 +62,10 @@ class hola_shard_args(ctypes.Structure):
 
 class hola_plan_info(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int32) for n in ("tile_v", "grid", "stages", "rows_per_pass", "passes", "kernels_per_call")]
+
+
+class hola_sample_info(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("ctas", "threads", "staged")]
 
 
 _lib = None
@@ -118,6 +122,8 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_plan.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_plan_info)]
     lib.hola_plan_for_shape.restype = ctypes.c_int
     lib.hola_plan_for_shape.argtypes = [ctypes.c_int] * 5 + [ctypes.POINTER(hola_plan_info)]
+    lib.hola_sample_plan_for_shape.restype = ctypes.c_int
+    lib.hola_sample_plan_for_shape.argtypes = [ctypes.c_int] * 6 + [ctypes.POINTER(hola_sample_info)]
     lib.hola_plan_ex.restype = ctypes.c_int
     lib.hola_plan_ex.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_plan_info)]
     lib.hola_profile_begin.restype = ctypes.c_int
@@ -605,3 +611,14 @@ def hola_plan_for_shape(num_sms: int, H: int, V: int, rows: int, w_dtype: int = 
     if st != 0:
         raise HolaError(f"hola_plan_for_shape: status {st}")
     return {n: getattr(info, n) for n, _ in hola_plan_info._fields_}
+
+
+def hola_sample_plan_for_shape(num_sms: int, B: int, k: int, V: int, q_dtype: int = HOLA_Q_BF16,
+                               fallback: int = HOLA_FALLBACK_SAMPLE) -> dict:
+    """Form of the accept/sample kernel for a shape (host arithmetic; needs the library, not a device)."""
+    lib = load_library()
+    info = hola_sample_info()
+    st = lib.hola_sample_plan_for_shape(int(num_sms), int(B), int(k), int(V), int(q_dtype), int(fallback), ctypes.byref(info))
+    if st != 0:
+        raise HolaError(f"hola_sample_plan_for_shape: status {st}")
+    return {n: getattr(info, n) for n, _ in hola_sample_info._fields_}

@@ -2959,28 +2959,74 @@ hola_status check_common(const hola_ctx* ctx, const hola_verify_args* a) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Cluster size of the accept/sample launch (CTAs per sequence): as many as keep the grid within one wave of the SMs; one
+// Logits and draft rows that 16-byte loads tile.
+bool rows_of_pieces(const hola_verify_args* a, const float* logits, int ldl) {
+  return a->V % 4 == 0 && ldl % 4 == 0 && aligned16(logits) && (a->k == 0 || aligned16(a->draft_q));
+}
+
+// How the accept/sample kernel is launched.
+struct SampleForm {
+  int S;            // CTAs per sequence
+  bool solo;        // the one CTA has 1024 threads
+  bool staged;      // the slices of all rows go through shared memory
+  int cpc;          // chunks per CTA
+  size_t smem;      // dynamic shared memory
+};
+
+// Cluster size (CTAs per sequence): as many as keep the grid within one wave of the SMs; one
 // where no pass over the vocabulary follows the accept test (greedy fallback; us, V = 32000, H = 512, clusters of eight ->
 // one: 384 rows 28.7 -> 27.8, 96 rows 15.2 -> 13.7).
-int sample_cluster(const hola_ctx* ctx, const hola_verify_args* a) {
-  if (a->fallback == HOLA_FALLBACK_GREEDY) return 1;
-  const int nchunks = (a->V + kChunk - 1) / kChunk;
+int sample_cluster(int num_sms, int B, int V, int fallback) {
+  if (fallback == HOLA_FALLBACK_GREEDY) return 1;
+  const int nchunks = (V + kChunk - 1) / kChunk;
   int S = 8;
-  while (S > 1 && (a->B * S > kK3MaxPerSm * ctx->num_sms || nchunks / S < 8)) S >>= 1;
+  while (S > 1 && (B * S > kK3MaxPerSm * num_sms || nchunks / S < 8)) S >>= 1;
   return S;
 }
 
-// One CTA of 1024 threads per sequence instead of a cluster: no cluster barrier, the statistics of a row merged once, and with
-// one sequence per SM most SMs stay free for the next call's GEMM kernel, which then asks for its W_lm while this one runs.
-// Up to 16384 entries (more take one SM too long); beyond 8192 only where clusters would take more than a quarter of the
-// SMs (small batches have their rows staged), and only for rows of whole 16-byte pieces.
-// us, cluster -> one CTA, k = 4, H = 1024: V = 3000, 2 / 32 / 100 sequences 11.1 -> 10.6, 15.1 -> 14.5, 26.3 -> 25.1;
-// V = 8000, 4 / 16 / 64 13.3 -> 13.1, 14.9 -> 13.6, 19.5 -> 17.8; V = 16000, 1 / 8 / 24 14.3 -> 14.9, 16.6 -> 15.4,
-// 18.1 -> 17.4; V = 24000, 32 26.8 -> 28.2; V = 11001, 16 16.7 -> 17.0, V = 4001, 60 15.2 -> 15.1.  (V < 2048: a cluster
-// would be a single CTA, of 256 threads, which is enough.)
-bool sample_solo(const hola_ctx* ctx, const hola_verify_args* a) {
-  const int S = sample_cluster(ctx, a);
-  return S > 1 && a->B <= ctx->num_sms && a->V <= 16384 && (a->V <= 8192 || (a->V % 4 == 0 && 4 * a->B * S > ctx->num_sms));
+// One CTA of 1024 threads per sequence instead of a cluster of S: no cluster barrier, the statistics of a row merged once, and
+// with one sequence per SM most SMs stay free for the next call's GEMM kernel, which then asks for its W_lm while this one runs.
+// Up to 16384 entries (more take one SM too long).  Where clusters would take at most a quarter of the SMs they ask ahead as
+// well, and have their rows staged: then only up to 8192 entries.  Rows of no whole 16-byte pieces are loaded element by element,
+// and one SM is slow at that: only up to 8192 entries, and where clusters would take at most a quarter of the SMs only against
+// clusters of two, or of four whose CTAs have more rows to merge than warps (8).
+// us, cluster -> one CTA, k = 4, H = 1024: V = 3000, 2 / 32 / 100 sequences 11.1 -> 10.6, 15.1 -> 14.5, 26.3 -> 25.1; V = 6000, 1
+// 11.5 -> 11.6; V = 8192, 1 / 4 / 16 / 64 12.3 -> 12.2, 13.1 -> 12.6, 14.5 -> 13.2, 22.5 -> 20.3; k = 30, V = 4000, 1 15.0 -> 11.4;
+// V = 16000, 1 / 8 / 24 / 148 14.3 -> 14.9, 16.6 -> 15.4, 18.1 -> 17.4, 47.2 -> 43.0; V = 16384, 5 / 100 16.6 -> 16.1, 32.0 -> 31.5;
+// V = 24000, 32 26.8 -> 28.2.  No whole pieces: V = 3001, 2 / 12 11.9 -> 11.7, 13.2 -> 13.0; V = 4001, 1 / 7 / 30 11.6 -> 11.9,
+// 12.2 -> 12.6, 16.2 -> 16.2; V = 6001, 2 / 9 12.4 -> 12.7, 13.3 -> 13.7; V = 8191, 1 / 4 / 5 / 16 / 64 12.3 -> 13.1, 13.6 -> 14.2,
+// 14.3 -> 13.9, 15.5 -> 14.9, 24.8 -> 23.8; k = 8, V = 4001 / 6001 / 8191, 1 / 3 / 3 12.4 -> 12.0, 13.9 -> 13.6, 14.1 -> 14.4; k = 20,
+// V = 4001, 1 12.7 -> 11.9; V = 11001, 16 16.7 -> 17.0.  (S = 1, up to 1920 entries: one CTA of 256 threads is enough.)
+bool sample_solo(int num_sms, int B, int k, int V, int S, bool vec) {
+  const bool many = 4 * B * S > num_sms;
+  if (S == 1 || B > num_sms) return false;
+  if (vec) return V <= (many ? 16384 : 8192);
+  return V <= 8192 && (many || S <= (k < kK3Threads / 32 ? 2 : 4));
+}
+
+// `vec`: rows_of_pieces.  `phase`, `shard`, `far`: see K3Params (a row read in place over the bus is not staged).
+SampleForm sample_form(int num_sms, int B, int k, int V, int q_dtype, int fallback, bool vec, int phase = 0, bool shard = false,
+                       bool far = false) {
+  SampleForm f = {};
+  const int S = phase == 1 ? 1 : sample_cluster(num_sms, B, V, fallback);            // (phase 1: no vocabulary pass)
+  f.solo = phase == 0 && !shard && !far && sample_solo(num_sms, B, k, V, S, vec);
+  f.S = f.solo ? 1 : S;
+  const int nchunks = (V + kChunk - 1) / kChunk;
+  f.cpc = (nchunks + f.S - 1) / f.S;
+  if (phase == 1 || fallback == HOLA_FALLBACK_GREEDY) return f;
+  f.smem = static_cast<size_t>(f.cpc) * sizeof(double);
+  // Small batches (a CTA per SM at most, and no more than 4 MB of rows in all): row n would be asked for only after the
+  // statistics and the accept test, so the slices of all rows are asked for before them (bulk copies: rows of whole
+  // 16-byte pieces).
+  if (vec && phase == 0 && (q_dtype == HOLA_Q_F32 || V % 8 == 0) && !far && !f.solo && B * S <= num_sms) {
+    const size_t row_bytes = static_cast<size_t>(k + 1) * 4 + static_cast<size_t>(k) * (q_dtype == HOLA_Q_BF16 ? 2 : 4);
+    const size_t bytes = row_bytes * f.cpc * kChunk + sizeof(double);   // (and the rows start on a 16-byte boundary)
+    if (bytes + f.smem <= kK3MaxDynSmem && row_bytes * V * B <= 4u << 20) {
+      f.staged = true;
+      f.smem += bytes;
+    }
+  }
+  return f;
 }
 
 // Where the logits of a verify step that does not hand them out go.  The greedy rule reads none (the arg-max travels with the
@@ -3257,32 +3303,17 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     kp.mass_out = sh->mass_out; kp.mass_all = sh->mass_all;
     if (combine) { kp.partials = sh->stats_all; kp.nparts = sh->world; kp.row_stride = 1; kp.part_stride = sh->rec_floats / 4; }
   }
-  const bool vec = (a->V % 4 == 0) && (ldl % 4 == 0) && aligned16(logits) && (a->k == 0 || aligned16(a->draft_q));
-  const int nchunks = (a->V + kChunk - 1) / kChunk;
-  const bool solo = phase == 0 && !sh && !q_far && sample_solo(ctx, a);
-  const int S = phase == 1 || solo ? 1 : sample_cluster(ctx, a);     // (phase 1: no vocabulary pass)
-  const int cpc = (nchunks + S - 1) / S;
+  const bool vec = rows_of_pieces(a, logits, ldl);
+  const SampleForm f = sample_form(ctx->num_sms, a->B, a->k, a->V, a->q_dtype, a->fallback, vec, phase, sh != nullptr, q_far != nullptr);
+  kp.staged = f.staged;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(a->B * S));
-  cfg.blockDim = dim3(kK3Threads);
-  const bool no_pass = phase == 1 || a->fallback == HOLA_FALLBACK_GREEDY;
-  cfg.dynamicSmemBytes = no_pass ? 0 : static_cast<size_t>(cpc) * sizeof(double);
-  // Small batches (a CTA per SM at most, and no more than 4 MB of rows in all): row n would be asked for only after the
-  // statistics and the accept test, so the slices of all rows are asked for before them (bulk copies: rows of whole
-  // 16-byte pieces).
-  kp.staged = 0;
-  if (vec && phase == 0 && (a->q_dtype == HOLA_Q_F32 || a->V % 8 == 0) && a->fallback != HOLA_FALLBACK_GREEDY && !q_far && !solo && a->B * S <= ctx->num_sms) {
-    const size_t row_bytes = static_cast<size_t>(a->k + 1) * 4 + static_cast<size_t>(a->k) * (a->q_dtype == HOLA_Q_BF16 ? 2 : 4);
-    const size_t bytes = row_bytes * cpc * kChunk + sizeof(double);     // (and the rows start on a 16-byte boundary)
-    if (bytes + cfg.dynamicSmemBytes <= kK3MaxDynSmem && row_bytes * a->V * a->B <= 4u << 20) {
-      kp.staged = 1;
-      cfg.dynamicSmemBytes += bytes;
-    }
-  }
+  cfg.gridDim = dim3(static_cast<unsigned>(a->B * f.S));
+  cfg.blockDim = dim3(f.solo ? kSoloThreads : kK3Threads);
+  cfg.dynamicSmemBytes = f.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(S);
+  attr[0].val.clusterDim.x = static_cast<unsigned>(f.S);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   // May be scheduled as soon as every CTA of the kernel before it in the stream has exited; it waits for that
@@ -3292,13 +3323,12 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const bool ask = vec && !kp.staged && cpc <= 64 && a->B * S > ctx->num_sms;
-  if (solo) {
-    cfg.blockDim = dim3(kSoloThreads);
+  const bool ask = vec && !f.staged && f.cpc <= 64 && a->B * f.S > ctx->num_sms;
+  if (f.solo) {
     attr[0] = attr[1];                                   // (no cluster)
     cfg.numAttrs = 1;
   }
-  const cudaError_t e = solo  ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, true>, kp)
+  const cudaError_t e = f.solo ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, true>, kp)
                                      : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, true>, kp))
                         : ask ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, true>, kp)
                         : vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false>, kp)
@@ -3517,6 +3547,16 @@ hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype
   return HOLA_OK;
 }
 
+hola_status hola_sample_plan_for_shape(int num_sms, int B, int k, int V, int q_dtype, int fallback, hola_sample_info* out) {
+  if (!out || num_sms < 2 || B <= 0 || k < 0 || V <= 0 || (q_dtype != HOLA_Q_BF16 && q_dtype != HOLA_Q_F32) ||
+      (fallback != HOLA_FALLBACK_SAMPLE && fallback != HOLA_FALLBACK_GREEDY))
+    return HOLA_ERR_INVALID_ARG;
+  if (k >= kMaxK1 || V > kMaxChunks * kChunk) return HOLA_ERR_UNSUPPORTED_SHAPE;
+  const SampleForm f = sample_form(num_sms, B, k, V, q_dtype, fallback, V % 4 == 0);
+  out->ctas = f.S; out->threads = f.solo ? kSoloThreads : kK3Threads; out->staged = f.staged;
+  return HOLA_OK;
+}
+
 hola_status hola_plan_ex(const hola_ctx* ctx, int B, int k, int w_dtype, hola_plan_info* out) {
   if (!ctx || !out || B < 0 || k < 0) return HOLA_ERR_INVALID_ARG;
   if (w_dtype < HOLA_W_BF16 || w_dtype > HOLA_W_MIXED) return HOLA_ERR_INVALID_ARG;
@@ -3663,7 +3703,8 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   const bool side = draft_gate && !inside && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
   // (one CTA per sequence: half of the SMs free are enough; us, V = 8000, 64 sequences without / with 18.3 / 17.8)
-  const bool few_before = sample_solo(ctx, a) ? a->B * 2 <= ctx->num_sms : a->B * sample_cluster(ctx, a) * 4 <= ctx->num_sms;
+  const SampleForm f = sample_form(ctx->num_sms, a->B, a->k, a->V, a->q_dtype, a->fallback, rows_of_pieces(a, logits, ldl));
+  const bool few_before = a->B * f.S * (f.solo ? 2 : 4) <= ctx->num_sms;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample, inside);
   if (s != HOLA_OK) return s;
   if (prof) cudaEventRecord(ev[1], stream);

@@ -115,3 +115,26 @@ def test_launch_geometry_for_shapes_without_a_device():
                 (sms, 4096, 32000, 5, 9)):
         with pytest.raises(b.HolaError):
             b.hola_plan_for_shape(*bad)
+
+
+@pytest.mark.parametrize("B,k,V,f32,want", [
+    # one CTA of 1024 threads: up to 8192 entries, or 16384 where clusters would take more than a quarter of the SMs
+    (1, 4, 1924, 0, (1, 1024, 0)), (1, 4, 8192, 0, (1, 1024, 0)), (5, 4, 16384, 0, (1, 1024, 0)), (148, 4, 16384, 1, (1, 1024, 0)),
+    # rows of no whole 16-byte pieces: up to 8192 entries beyond that quarter; before it against clusters of two, or of four
+    # with more than eight rows
+    (5, 4, 8191, 0, (1, 1024, 0)), (10, 4, 4001, 1, (1, 1024, 0)), (1, 4, 1921, 0, (1, 1024, 0)), (1, 4, 3967, 0, (1, 1024, 0)),
+    (1, 8, 4001, 0, (1, 1024, 0)), (1, 8, 8063, 0, (1, 1024, 0)),
+    (4, 4, 8191, 0, (8, 256, 0)), (1, 4, 3969, 0, (4, 256, 0)), (9, 7, 4001, 0, (4, 256, 0)), (1, 8, 8065, 0, (8, 256, 0)),
+    (5, 4, 8193, 0, (8, 256, 0)),
+    # clusters: small batches have their rows staged (16-bit rows of no whole 16-byte pieces excepted)
+    (4, 4, 8196, 1, (8, 256, 1)), (4, 4, 8200, 0, (8, 256, 1)), (4, 4, 8196, 0, (8, 256, 0)), (1, 20, 9000, 1, (8, 256, 1)),
+    (1, 4, 1920, 0, (1, 256, 1)), (1, 40, 128256, 1, (8, 256, 0)), (18, 4, 32000, 0, (8, 256, 0)), (149, 4, 8192, 0, (2, 256, 0)),
+])
+def test_form_of_the_accept_kernel_for_shapes(B, k, V, f32, want):
+    from paper_2506_18952_b200 import binding as b
+    got = b.hola_sample_plan_for_shape(148, B, k, V, b.HOLA_Q_F32 if f32 else b.HOLA_Q_BF16)
+    assert (got["ctas"], got["threads"], got["staged"]) == want
+    assert b.hola_sample_plan_for_shape(148, B, k, V, fallback=1) == {"ctas": 1, "threads": 256, "staged": 0}
+    for bad in ((1, B, k, V), (148, 0, k, V), (148, B, -1, V), (148, B, 64, V), (148, B, k, 0), (148, B, k, V, 7), (148, B, k, V, 0, 2)):
+        with pytest.raises(b.HolaError):
+            b.hola_sample_plan_for_shape(*bad)

@@ -312,6 +312,7 @@ def test_degenerate_inputs_are_flagged_not_fatal(binding):
     (2, 8, 8192, torch.bfloat16), (2, 8, 8196, torch.bfloat16),        # its end for small batches: rows staged beyond
     (5, 1, 8196, torch.float32), (9, 3, 8193, torch.bfloat16),
     (20, 2, 16384, torch.float32), (20, 2, 16388, torch.bfloat16),     # its end: clusters beyond
+    (4, 2, 8191, torch.bfloat16), (5, 2, 8191, torch.float32),         # its beginning for rows of no whole 16-byte pieces
     (160, 1, 3000, torch.bfloat16),    # more sequences than SMs
     (5, 40, 4100, torch.bfloat16),     # more rows than warps
 ])
