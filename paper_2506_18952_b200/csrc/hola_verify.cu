@@ -742,7 +742,7 @@ __device__ __forceinline__ float scaled(float acc, float w_scale, const float* h
 
 __device__ __forceinline__ float warp_max_f32(float x) {       // (of numbers; -inf among them)
   float r;
-  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));       // (volatile: whole warps, stays where it is)
   return r;
 }
 __device__ __forceinline__ double warp_sum_f64(double x) {
