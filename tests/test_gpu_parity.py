@@ -305,18 +305,30 @@ def test_degenerate_inputs_are_flagged_not_fatal(binding):
     assert orc.flags[3] & ref.FLAG_R_ZERO
 
 
-@pytest.mark.parametrize("B,k,V,qd", [
-    (1, 4, 1920, torch.float32),       # fewer chunks than a cluster of two wants: a single small CTA
-    (1, 4, 2048, torch.float32),       # the smallest vocabulary with a CTA of 1024 threads per sequence
-    (3, 2, 4001, torch.bfloat16),      # the same, rows of no whole 16-byte pieces
-    (2, 8, 8192, torch.bfloat16), (2, 8, 8196, torch.bfloat16),        # its end for small batches: rows staged beyond
-    (5, 1, 8196, torch.float32), (9, 3, 8193, torch.bfloat16),
-    (20, 2, 16384, torch.float32), (20, 2, 16388, torch.bfloat16),     # its end: clusters beyond
-    (4, 2, 8191, torch.bfloat16), (5, 2, 8191, torch.float32),         # its beginning for rows of no whole 16-byte pieces
-    (160, 1, 3000, torch.bfloat16),    # more sequences than SMs
-    (5, 40, 4100, torch.bfloat16),     # more rows than warps
+_SOLO = (1, 1024, 0)        # one CTA of 1024 threads per sequence
+
+
+@pytest.mark.parametrize("B,k,V,qd,form", [
+    # fewer chunks than a cluster of two wants: a single small CTA, its rows staged; the smallest vocabularies beyond
+    (1, 4, 1920, torch.float32, (1, 256, 1)), (1, 4, 1921, torch.float32, _SOLO), (1, 4, 1924, torch.float32, _SOLO),
+    (1, 4, 2048, torch.float32, _SOLO),
+    # its end for small batches: rows staged beyond, or not (16-bit rows of no whole 16-byte pieces)
+    (2, 8, 8192, torch.bfloat16, _SOLO), (2, 8, 8200, torch.bfloat16, (8, 256, 1)), (2, 8, 8196, torch.bfloat16, (8, 256, 0)),
+    (4, 1, 8196, torch.float32, (8, 256, 1)), (5, 1, 8196, torch.float32, _SOLO),
+    # its end: clusters beyond
+    (20, 2, 16384, torch.float32, _SOLO), (20, 2, 16388, torch.bfloat16, (8, 256, 0)),
+    # logits rows of no whole 16-byte pieces
+    (3, 2, 4001, torch.bfloat16, (4, 256, 0)), (3, 8, 4001, torch.bfloat16, _SOLO), (4, 2, 8191, torch.bfloat16, (8, 256, 0)),
+    (5, 2, 8191, torch.float32, _SOLO), (9, 3, 8193, torch.bfloat16, (8, 256, 0)),
+    # more sequences than SMs; more rows than warps
+    (160, 1, 3000, torch.bfloat16, (2, 256, 0)), (5, 40, 4100, torch.bfloat16, _SOLO),
+    # staged: rows merged by every warp, the last one copies; more copies than lanes, in one CTA and in a cluster
+    (1, 9, 640, torch.bfloat16, (1, 256, 1)), (1, 20, 640, torch.float32, (1, 256, 1)), (1, 20, 9000, torch.float32, (8, 256, 1)),
 ])
-def test_forms_of_the_accept_kernel_at_the_edges_of_their_ranges(binding, B, k, V, qd):
+def test_forms_of_the_accept_kernel_at_the_edges_of_their_ranges(binding, B, k, V, qd, form):
+    plan = binding.hola_sample_plan_for_shape(torch.cuda.get_device_properties(0).multi_processor_count, B, k, V,
+                                              binding.HOLA_Q_F32 if qd == torch.float32 else binding.HOLA_Q_BF16)
+    assert tuple(plan.values()) == form
     w = workloads.gaussian_head("forms", B, k, 64, V, seed=B + V, device=DEV, w_std=0.3, q_dtype=qd, sigma=1.0, sigma_far=0.1,
                                 tau=2.5)
     w.draft_q[B // 2] = 2.0            # above p everywhere: no residual mass, the draw is from p
@@ -1181,14 +1193,15 @@ def test_host_entry_behind_queued_device_calls_keeps_their_draft_entropies_apart
 def test_a_staged_wait_that_runs_out_is_reported_by_the_cta_that_draws(binding):
     """The wait of the accept/sample kernel on the rows it brings into shared memory, in miniature: it runs out in one CTA of
     a cluster, and another one, whose own wait was satisfied, is the one that reports."""
-    w = workloads.gaussian_head("after-staged", 2, 3, 128, 3000, seed=6, device=DEV, w_std=0.3)
+    w = workloads.gaussian_head("after-staged", 2, 3, 128, 20000, seed=6, device=DEV, w_std=0.3)
+    assert binding.hola_sample_plan_for_shape(148, w.B, w.k, w.V)["staged"]
     with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
         for limit in (20000, 100000):
             assert ctx.hola_selftest_staged_wait(limit) == (binding.FLAG_TIMEOUT, 128, 64, binding.FLAG_TIMEOUT)
         for bad in (10, 10 ** 12):
             with pytest.raises(binding.HolaError):
                 ctx.hola_selftest_staged_wait(bad)
-        got = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)      # (rows staged, small batch)
+        got = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)      # (rows staged)
         torch.cuda.synchronize()
         assert int(got.status.item()) == 0
     check_against_oracle(binding, w, out=got, want_logits=False)
