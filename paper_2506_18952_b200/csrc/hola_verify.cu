@@ -1990,8 +1990,8 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
   // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities, each row's
   // slice by one bulk copy, a lane of the first warp per copy, while the other warps merge statistics (with eight rows and more
   // that one does so too, after its gathers: then the last warp).  (One thread after the
-  // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows: V = 32000 46.67 -> 46.31, mixed widths
-  // 34.84 -> 34.47, V = 3000 11.0 -> 10.7.)
+  // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows, V = 32000: 46.67 -> 46.31, mixed widths
+  // 34.84 -> 34.47.)
   const bool staged = kVec && !kSolo && p.staged;
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
@@ -2040,7 +2040,7 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
   // ---- softmax statistics of this sequence's k+1 positions
   if (p.combine) {
     // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
-    // above, gets a row only when there are more than seven)
+    // above, gets a row only when there are as many rows as warps)
     for (int j = kWarps - 1 - warp; j <= k; j += kWarps) {
       Stats st = warp_merge_partials(p.partials, p.nparts, p.row_stride, p.part_stride, row_first + j, lane);
       if (lane == 0) {
@@ -3702,7 +3702,9 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
   if (draft_gate && !inside && cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) capturing = cudaStreamCaptureStatusActive;
   const bool side = draft_gate && !inside && (before_sample || capturing == cudaStreamCaptureStatusNone);
   if (side && cudaEventRecord(ctx->fork_point, stream) != cudaSuccess) return HOLA_ERR_CUDA;
-  // (one CTA per sequence: half of the SMs free are enough; us, V = 8000, 64 sequences without / with 18.3 / 17.8)
+  // (One CTA per sequence: half of the SMs free are enough; us, V = 8000, 64 sequences without / with 18.3 / 17.8.  Clusters: three
+  // quarters; on up to half of the SMs V = 30000, 9 sequences 18.2 / 17.0, V = 32000, 5 / 8 50.6 / 49.9, 51.7 / 52.0, V = 128256,
+  // 8 59.9 / 61.4: no line there that holds for all.)
   const SampleForm f = sample_form(ctx->num_sms, a->B, a->k, a->V, a->q_dtype, a->fallback, rows_of_pieces(a, logits, ldl));
   const bool few_before = a->B * f.S * (f.solo ? 2 : 4) <= ctx->num_sms;
   hola_status s = run_lm_head(ctx, a, logits, ldl, pl, stream, few_before, !before_sample, inside);
@@ -3732,8 +3734,10 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
 // per sequence (q_j(x_j), gathered here on the host) and at most ONE row per sequence: row accept_len, and none when
 // every draft token was kept or the fallback is greedy.  Rows 0 .. ahead-1 of every sequence (as many as the bus
 // carries while the GEMM runs, at least one) are sent ahead on the context's own stream; after the accept test the
-// accept lengths come back and only the rows still missing follow.  Same kernels, same arithmetic and so the same
-// results as the whole-tensor copy.
+// accept lengths come back and only the rows still missing follow, or the accept/sample kernel reads those in place.  Same
+// arithmetic and so the same results as the whole-tensor copy, with one exception: a launch that reads rows in place keeps
+// clusters where the others take one CTA (sample_solo), so that the chunks' masses are summed in another order, in fp64; a
+// token differs only where u R falls within that rounding (some 1e-16) of a boundary.
 constexpr double kHostBusBytesPerSecond = 50e9;          // what a pinned host-to-device copy reaches here
 
 // Draft rows per sequence that can cross the bus while the GEMM of this call runs.

@@ -1,7 +1,7 @@
 // The host side of a call on torch tensors, in native code: reads the tensors, fills hola_verify_args and calls the C ABI;
-// makes the output tensors of a call that is given none.  What a call costs the host bounds small problems: filling the
-// arguments field by field from Python takes 3.4 us, six output tensors 6 to 7 us, beside 5 us for the two launches.  us, Python
-// -> native: one sequence, V = 1000 10.45 -> 9.75; three, V = 5000, fresh outputs 19.75 -> 13.2; host entry, two sequences,
+// makes the output tensors of a call that is given none.  What a call costs the host bounds small problems.  us, Python -> native:
+// arguments filled and a call that is refused 3.5 -> 0.8, five output tensors 8.2 -> 5.1, seven 11.7 -> 7.0, beside 5 for the two
+// launches; whole calls: one sequence, V = 1000 10.45 -> 9.75; three, V = 5000, fresh outputs 19.75 -> 13.2; host entry, two sequences,
 // V = 10000 42.1 -> 37.4; mixed-width quantiser, 1000 x 128 50 -> 13.8.
 //
 // call() takes the plain forms only (torch.Tensor or Parameter objects with storage, strided, contiguous, of the types that
