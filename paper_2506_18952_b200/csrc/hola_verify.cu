@@ -3303,7 +3303,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     kp.mass_out = sh->mass_out; kp.mass_all = sh->mass_all;
     if (combine) { kp.partials = sh->stats_all; kp.nparts = sh->world; kp.row_stride = 1; kp.part_stride = sh->rec_floats / 4; }
   }
-  const bool vec = rows_of_pieces(a, logits, ldl);
+  const bool vec = rows_of_pieces(a, logits, ldl) && aligned16(q_far);     // (rows read in place are the caller's own)
   const SampleForm f = sample_form(ctx->num_sms, a->B, a->k, a->V, a->q_dtype, a->fallback, vec, phase, sh != nullptr, q_far != nullptr);
   kp.staged = f.staged;
   cudaLaunchConfig_t cfg = {};

@@ -498,6 +498,24 @@ def test_host_entry_reads_missing_rows_in_place_or_copies_them(binding, pinned):
     assert len(set(d.accept_len.tolist())) >= 3              # rows beyond the ones sent ahead are needed
 
 
+@pytest.mark.parametrize("q_dtype,offset", [(torch.bfloat16, 1), (torch.bfloat16, 4), (torch.float32, 1), (torch.float32, 2)])
+def test_rows_read_in_place_may_start_anywhere(binding, q_dtype, offset):
+    """A pinned draft tensor that starts on no 16-byte boundary, in a vocabulary whose rows 16-byte pieces would tile."""
+    w = workloads.gaussian_head("in-place", 21, 4, 128, 5000, seed=79, device=DEV, w_std=0.3, tau=0.0, q_dtype=q_dtype)
+    q = torch.empty(w.draft_q.numel() + offset, dtype=q_dtype).pin_memory()[offset:].view(w.draft_q.shape)
+    q.copy_(w.draft_q)
+    assert q.is_pinned() and q.data_ptr() % 16
+    host = [t.cpu().pin_memory() for t in (w.hidden, w.draft_tok, w.uniforms)]
+    with binding.HolaVerify(w.B, w.k, w.H, w.V) as ctx:
+        ctx.hola_set_option(binding.HOLA_OPT_HOST_ROWS_ON_DEMAND, 1)
+        d = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)
+        torch.cuda.synchronize()
+        h = ctx.hola_verify_host(host[0], w.W_lm, host[1], q, host[2], w.tau)
+    assert torch.equal(h.accept_len, d.accept_len.cpu()) and torch.equal(h.next_tok, d.next_tok.cpu())
+    assert torch.equal(h.entropy, d.entropy.cpu()) and torch.equal(h.logZ, d.logZ.cpu())
+    assert len(set(d.accept_len.tolist())) >= 3              # rows beyond the ones sent ahead are needed
+
+
 @pytest.mark.parametrize("q_dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("gate,fallback", [(0, 0), (0, 1), (1, 0)])
 @pytest.mark.parametrize("tau", [0.0, None, 100.0])
