@@ -3733,9 +3733,9 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
 // hola_verify_host while the target entropy gates.  Of the draft tensor the step then reads k single probabilities
 // per sequence (q_j(x_j), gathered here on the host; the greedy fallback does not look at them) and at most ONE row per
 // sequence: row accept_len, and none when every draft token was kept or the fallback is greedy.  Rows 0 .. ahead-1 of
-// every sequence (as many as the bus carries while the GEMM runs, at least one) are sent ahead on the context's own stream; after the accept test the
-// accept lengths come back and only the rows still missing follow, or the accept/sample kernel reads those in place.  Same
-// arithmetic and so the same results as the whole-tensor copy, with one exception: a launch that reads rows in place keeps
+// every sequence (as many as the bus carries while the GEMM runs, at least one) are sent ahead on the context's own stream;
+// after the accept test the accept lengths come back and only the rows still missing follow, or the accept/sample kernel
+// reads those in place.  Same arithmetic and so the same results as the whole-tensor copy, with one exception: a launch that reads rows in place keeps
 // clusters where the others take one CTA (sample_solo), so that the chunks' masses are summed in another order, in fp64; a
 // token differs only where u R falls within that rounding (some 1e-16) of a boundary.
 constexpr double kHostBusBytesPerSecond = 50e9;          // what a pinned host-to-device copy reaches here
