@@ -2568,8 +2568,8 @@ __global__ void __launch_bounds__(256, 3) quantize_rows_kernel(const uint16_t* W
 // loads per thread at 4096 channels, one barrier.
 constexpr int kHidThreads = 256, kHidKeep = 4;
 template <bool kTwoPlane>
-__global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint4* X, int M, int H, signed char* q,
-                                                                      float* s1, float* s2) {
+__global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint4* X, int M, int H, int q_pitch,
+                                                                      signed char* q, float* s1, float* s2) {
   __shared__ float sh_max[kHidThreads / 32];
   grid_dependency_wait();                                // (no-op unless launched with programmatic serialization)
   // The GEMM kernel may be put in place beside this one (its CTA and several of these fit an SM): its launch and set-up and,
@@ -2581,8 +2581,8 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
   const int row = blockIdx.x;
   const int pieces = H >> 3;
   const size_t row1 = kTwoPlane ? static_cast<size_t>(64) * (row >> 5) + (row & 31) : static_cast<size_t>(row);
-  uint2* q1 = reinterpret_cast<uint2*>(q) + row1 * pieces;
-  uint2* q2 = q1 + static_cast<size_t>(32) * pieces;
+  uint2* q1 = reinterpret_cast<uint2*>(q + row1 * q_pitch);
+  uint2* q2 = reinterpret_cast<uint2*>(q + (row1 + 32) * q_pitch);
   if (row >= M) {
     for (int p = threadIdx.x; p < pieces; p += kHidThreads) { q1[p] = make_uint2(0u, 0u); q2[p] = make_uint2(0u, 0u); }
     return;
@@ -2706,7 +2706,7 @@ struct hola_ctx {
   unsigned* status;         // [1]
   unsigned* pace;           // [kMaxPaceGroups] counters of the groups of pairs when all passes share a launch
   double* hq;               // [max_rows][kHqSlices] slice sums of q ln q over the draft rows
-  signed char* hid8;        // [max_rows][H] int8 hidden rows (8-bit activation mode)
+  signed char* hid8;        // [rows][hidden_pitch8] int8 hidden rows (8-bit activation modes)
   float* hid_scale;         // [max_rows]
   // staging for hola_verify_host
   void* st_hidden; int* st_tok; void* st_q; float* st_u;
@@ -2768,6 +2768,12 @@ struct WsLayout {
   size_t logits, partials, status, pace, hq, hid8, hid_scale, st_hidden, st_tok, st_q, st_u, st_out, st_qtok, st_small_end, total;
 };
 
+// Bytes from one 8-bit hidden row to the next: rows start on 128-byte lines, so that a K block of a row is one line instead of
+// parts of two.  Every CTA pair fetches those rows again, and that traffic out of the L2 is what bounds the 8-bit kind here.  us,
+// rows side by side -> padded, H = 4112: 384 rows, V = 32000 76.1 -> 71.0 (H = 4096: 69.4), 192 rows, V = 128256 170 -> 152 (145),
+// two planes of 96 rows, V = 32000 47.6 -> 43.6; H = 6992, 96 rows, V = 40736 77.0 -> 70.9.
+int hidden_pitch8(int H) { return static_cast<int>(align_up(static_cast<size_t>(H), 128)); }
+
 WsLayout ws_layout(int maxB, int maxK, int H, int V, int num_sms) {
   const size_t rows = static_cast<size_t>(maxB) * (maxK + 1);
   const size_t ldl = align_up(static_cast<size_t>(V), 4);
@@ -2779,7 +2785,7 @@ WsLayout ws_layout(int maxB, int maxK, int H, int V, int num_sms) {
   w.status = take(4);
   w.pace = take(4 * kMaxPaceGroups);
   w.hq = take(rows * kHqSlices * 8);
-  w.hid8 = take(2 * align_up(rows, 32) * static_cast<size_t>(H));     // one or two 8-bit planes of the hidden rows
+  w.hid8 = take(2 * align_up(rows, 32) * hidden_pitch8(H));           // one or two 8-bit planes of the hidden rows
   w.hid_scale = take(2 * rows * 4);                                   // their scales (second plane after the first)
   w.st_hidden = take(rows * H * 2);
   // the three small per-step inputs side by side: hola_verify_host sends them as one copy
@@ -2922,13 +2928,14 @@ const Plan& plan_for(hola_ctx* ctx, int M, int w_dtype) {
 // the 128-byte swizzle that the MMA reads (and that spreads the rows of 8-bit codes over the banks for the converter
 // warps).  `packed4`: rows of cols / 2 bytes holding two 4-bit codes each; box of 64 bytes (128 codes), 64-byte swizzle.
 hola_status encode_map(hola_ctx* ctx, CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
-                       uint32_t box_rows, bool int8 = false, bool packed4 = false, int kpb = 1) {
+                       uint32_t box_rows, bool int8 = false, bool packed4 = false, int kpb = 1, int pitch = 0) {
   if (packed4) { cols /= 2; int8 = true; }
   const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {cols * (int8 ? 1u : 2u)};
+  const cuuint64_t strides[1] = {pitch ? static_cast<cuuint64_t>(pitch) : cols * (int8 ? 1u : 2u)};
   const cuuint32_t box[2] = {static_cast<cuuint32_t>(int8 && !packed4 ? 2 * kBlockK : kBlockK), box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  // `kpb` > 1: the same memory as (element of a K block, row, K block), kpb K blocks per box; needs whole K blocks
+  // `pitch`: bytes from row to row (0: rows side by side).  `kpb` > 1: the same memory as (element of a K block, row, K
+  // block), kpb K blocks per box; needs whole K blocks
   const cuuint64_t dims3[3] = {box[0], rows, cols / box[0]};
   const cuuint64_t strides3[2] = {strides[0], 128};
   const cuuint32_t box3[3] = {box[0], box_rows, static_cast<cuuint32_t>(kpb)};
@@ -3067,7 +3074,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     qc.attrs = qa; qc.numAttrs = 1;
     const cudaError_t qe =
         cudaLaunchKernelEx(&qc, two ? quantize_hidden_kernel<true> : quantize_hidden_kernel<false>,
-                           static_cast<const uint4*>(a->hidden), M, a->H, ctx->hid8, ctx->hid_scale,
+                           static_cast<const uint4*>(a->hidden), M, a->H, hidden_pitch8(a->H), ctx->hid8, ctx->hid_scale,
                            ctx->hid_scale + ctx->max_rows);
     if (qe != cudaSuccess) { set_error(ctx, "launch of the hidden-row quantiser", qe); return HOLA_ERR_CUDA; }
   }
@@ -3085,10 +3092,10 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     me->logits = nullptr;
     if (two)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(2 * round_up(M, 32)), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb);
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hidden_pitch8(a->H));
     else if (i8)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb);
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hidden_pitch8(a->H));
     else
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
                      static_cast<uint32_t>(pl.N / 2), false, false, pl.kpb);
@@ -3103,7 +3110,8 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
         s = encode_map(ctx, &me->tw4, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, i8);
         if (s != HOLA_OK) return s;
         s = encode_map(ctx, &me->tw16, hid_src, static_cast<uint64_t>(two ? 2 * round_up(M, 32) : M),
-                       static_cast<uint64_t>(a->H), static_cast<uint32_t>(pl.N / 2), i8);
+                       static_cast<uint64_t>(a->H), static_cast<uint32_t>(pl.N / 2), i8, false, 1,
+                       i8 ? hidden_pitch8(a->H) : 0);
         if (s != HOLA_OK) return s;
       }
       me->W4 = nullptr; me->W16 = nullptr;
