@@ -156,7 +156,8 @@ struct K1Params {
   int draft_q_dtype, draft_units;   // the first tile's MMAs run; a unit is one slice of one row (draft_rows * kHqSlices)
   double* draft_part;
   int prefetch_blocks;  // K blocks of its first tile a CTA asks into the L2 before it waits for the kernel before
-  unsigned* pace;     // n_pass > 1: one counter per group of pairs (zero at launch), by which the group keeps in step
+  unsigned* pace;     // n_pass > 1, several tiles: two words per group of pairs (zero at launch, and again at the end), by which
+                      // the group keeps in step
 };
 
 struct K3Params {
@@ -413,6 +414,17 @@ __device__ __forceinline__ void keep_pace(unsigned* counter, unsigned target) {
     unsigned seen;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
     if (seen >= target || clock64() - t0 > kPaceLimitCycles) break;
+  }
+}
+// Behind its last tile: the last of the group's `members` leaves both of the group's words at zero for the next launch.
+// (A memset ahead of the launch did so before: an operation of its own in the stream, which also keeps the launch from being put
+// in place early.  us: 660 rows, V = 3920 28.7 -> 23.7, 196 rows of mixed widths, V = 2656 18.5 -> 13.9, which have one tile per
+// pair and no pace at all; 765 8-bit rows, V = 22752 56.6 -> 50.6.)
+__device__ __forceinline__ void leave_pace(unsigned* counter, unsigned members) {
+  __threadfence();
+  if (atomicAdd(counter + kMaxPaceGroups, 1u) == members - 1) {
+    counter[kMaxPaceGroups] = 0u;
+    *counter = 0u;
   }
 }
 
@@ -1024,6 +1036,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
       }
+      if (p.n_pass > 1 && p.pace && my_tiles > 1) leave_pace(p.pace + pair, static_cast<unsigned>(2 * p.n_pass));
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
@@ -2704,7 +2717,7 @@ struct hola_ctx {
   float4* partials;         // [max_rows][part_stride]
   int part_stride;          // CTAs a row may have partials of (the SM count)
   unsigned* status;         // [1]
-  unsigned* pace;           // [kMaxPaceGroups] counters of the groups of pairs when all passes share a launch
+  unsigned* pace;           // [2][kMaxPaceGroups] counters of the groups of pairs when all passes share a launch
   double* hq;               // [max_rows][kHqSlices] slice sums of q ln q over the draft rows
   signed char* hid8;        // [rows][hidden_pitch8] int8 hidden rows (8-bit activation modes)
   float* hid_scale;         // [max_rows]
@@ -2783,7 +2796,7 @@ WsLayout ws_layout(int maxB, int maxK, int H, int V, int num_sms) {
   w.logits = take(rows * ldl * 4);
   w.partials = take(static_cast<size_t>(num_sms) * rows * 16);
   w.status = take(4);
-  w.pace = take(4 * kMaxPaceGroups);
+  w.pace = take(8 * kMaxPaceGroups);
   w.hq = take(rows * kHqSlices * 8);
   w.hid8 = take(2 * align_up(rows, 32) * hidden_pitch8(H));           // one or two 8-bit planes of the hidden rows
   w.hid_scale = take(2 * rows * 4);                                   // their scales (second plane after the first)
@@ -2810,7 +2823,9 @@ int round_up(int x, int a) { return (x + a - 1) / a * a; }
 // Splits M verify rows into passes over W_lm and each pass into one or two MMAs per K step.
 // A pass holds at most 512 rows (two MMAs of N <= 256 fill the tensor memory); N is a multiple of 16.
 // Cost per pass: the slower of streaming W_lm once and the padded rows' tensor time, plus a fixed launch cost.
-Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
+// `want`: number of passes (0: by that cost), vocabulary rows per CTA and tile (0: by the rules below), all passes in one launch.
+struct PlanWish { int passes, tile_rows; bool fuse; };
+Plan plan_as(const hola_ctx* ctx, int M, int w_dtype, const PlanWish& want) {
   const bool mixed = w_dtype == HOLA_W_MIXED;    // vocabulary groups of 4-, 8- and 16-bit rows, expanded on chip
   const bool w8 = w_dtype == HOLA_W_INT8 || mixed;   // int8 W_lm expanded on chip
   const bool two = w_dtype == HOLA_W8A16;        // as W8A8, with two operand rows per verify row
@@ -2822,9 +2837,9 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int max_rows_per_pass = w8 ? kExpandMaxN : two ? kMaxN : kMaxRowsPerPass;
   const int p_min = (rows + max_rows_per_pass - 1) / max_rows_per_pass;
   const double t_hbm = (w8 || i8 ? 1.0 : 2.0) * ctx->V * static_cast<double>(ctx->H) / 6.4e12;
-  const int p_max = ctx->force_passes > p_min + 3 ? ctx->force_passes : p_min + 3;
+  const int p_max = want.passes > p_min + 3 ? want.passes : p_min + 3;
   for (int passes = p_min; passes <= p_max; ++passes) {
-    if (ctx->force_passes && passes != ctx->force_passes && ctx->force_passes >= p_min) continue;
+    if (want.passes && passes != want.passes && want.passes >= p_min) continue;
     const int r = (rows + passes - 1) / passes;
     // up to 256 rows: one MMA, two accumulator buffers; up to 384: three MMAs of N <= 128 on rotating 128-column
     // units; beyond: two MMAs of N <= 256 that fill the tensor memory
@@ -2854,7 +2869,7 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int all_pairs = ctx->num_sms / 2 > 0 ? ctx->num_sms / 2 : 1;
   // Several passes: one launch in which `passes` neighbouring pairs walk the same tiles together, one pass each (W_lm
   // then leaves HBM once, not once per pass), as long as every pass gets a pair.
-  best.fused = (best.passes > 1 && !ctx->no_fuse && all_pairs / best.passes >= 1) ? 1 : 0;
+  best.fused = (best.passes > 1 && want.fuse && all_pairs / best.passes >= 1) ? 1 : 0;
   const int pairs = best.fused ? all_pairs / best.passes : all_pairs;     // pairs that divide the tiles among them
   const int rounds = (ctx->V + pairs * kPairTile - 1) / (pairs * kPairTile);
   // One tile per pair: a tile costs the tensor cores and the traffic of the hidden rows the same whatever its height, and
@@ -2883,6 +2898,7 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   // us: V = 32000, 384 rows (143 tiles of 224 rows -> 125 of 256) 117 -> 113, 8-bit 74.7 -> 72.9; V = 128256 (517 -> 501),
   // 384 rows 434 -> 430, 192 rows at 8 bits (0.87 of the HBM time) 144 -> 140, two planes 221 -> 212.
   if (rounds >= 2 && best.mma_share > 0.8) tile_rows = kLanes;
+  if (want.tile_rows) tile_rows = want.tile_rows;
   if (mixed) tile_rows = kLanes;                 // a pair's tile is one group of 256 rows of one width
   best.tile_rows = tile_rows;
   best.n_ptiles = (ctx->V + 2 * tile_rows - 1) / (2 * tile_rows);
@@ -2909,6 +2925,64 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   if (ctx->force_stages && ctx->force_stages < stages) stages = ctx->force_stages;
   best.stages = stages;
   best.smem_bytes = stages * stage_bytes + kBarrierBytes + trans_bytes + 1024;
+  return best;
+}
+
+// Estimated microseconds of a launch in which every pair has one tile, without what all such launches have in common (some 10).
+// A K block takes the slowest of: its MMAs; its bytes at what one SM gets out of the L2, 61 a cycle (with rows that start on no
+// 128-byte line 48); the bytes of all SMs at what they get together, 6400 a cycle (5100); a turn of the threads that feed the
+// ring; with on-chip expansion a turn of the converters.  All K blocks together take no less than W_lm's way out of HBM.  The
+// read-out takes 1.8 us per chunk of 32 operand rows and epilogue warp.  Fitted to 37 shapes (V = 1200 .. 12000, H = 200 .. 8192,
+// 5 .. 2304 rows, every weight mode) in 2 to 20 splits each: the split it picks was 0.7 % slower than the best one on average, 4 %
+// at worst.
+double one_tile_us(const hola_ctx* ctx, const Plan& pl, int w_dtype) {
+  const bool expand = w_dtype == HOLA_W_INT8 || w_dtype == HOLA_W_MIXED, i8 = w_dtype == HOLA_W8A8 || w_dtype == HOLA_W8A16;
+  const int op_rows = pl.n_sub * pl.N;
+  const double mma = 1.16 * 4.0 * pl.n_sub * (pl.N / 2 > 46 ? pl.N / 2 : 46);
+  const double bytes = pl.tile_rows * (expand ? 64.0 : 128.0) + op_rows * 64.0;
+  const double line = !i8 && ctx->H % kBlockK != 0 ? 0.79 : 1.0;
+  double block = expand ? 326.0 : 180.0;
+  for (const double c : {mma, bytes / (61.0 * line), pl.grid * bytes / (6400.0 * line)})
+    if (c > block) block = c;
+  const double ring = pl.n_kblocks * block / 1900.0, hbm = static_cast<double>(ctx->V) * ctx->H * (expand || i8 ? 1 : 2) / 7.2e6;
+  const int groups = !expand ? kEpiWarps / 4 : op_rows <= 32 ? kW8FewEpiWarps / 4 : kW8EpiWarps / 4;
+  return (ring > hbm ? ring : hbm) + 1.8 * (((op_rows + 31) / 32 + groups - 1) / groups);
+}
+
+// Vocabularies of a tile per pair and fewer leave pairs without work when all rows of a pass go to the same tile's pair.  The
+// rows are then cut into more passes, which share the tiles in one launch, and the tiles into shorter ones, as the estimate has
+// it (half a microsecond less than the split of the general rules, or that one stays).  us, before -> after, bf16: 417 rows,
+// H = 5304, V = 1272 62.4 -> 25.2; 384 rows, H = 4096, V = 8000 45.5 -> 37.0; 384 rows, H = 1024, V = 4000 21.0 -> 14.2; 200 rows,
+// H = 2048, V = 3000 20.6 -> 15.5; 512 rows, H = 512, V = 2000 22.5 -> 12.9; 150 rows, H = 696, V = 6000 15.4 -> 13.7; 8-bit planes,
+// 384 rows, V = 4000 35.1 -> 21.2; two planes, 216 rows, V = 7550 35.6 -> 26.1; mixed widths, 824 rows, V = 1408 43.0 -> 34.8.
+Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
+  PlanWish want = {ctx->force_passes, 0, true};
+  Plan best = plan_as(ctx, M, w_dtype, want);
+  const int pairs = ctx->num_sms / 2;
+  const int p_min = best.passes;
+  if (!ctx->force_passes && best.n_ptiles * p_min <= pairs) {
+    double best_us = one_tile_us(ctx, best, w_dtype) - 0.5;
+    for (int tile_rows = kLanes; tile_rows >= 32; tile_rows -= 32) {
+      if (w_dtype == HOLA_W_MIXED && tile_rows < kLanes) break;
+      const int tiles = (ctx->V + 2 * tile_rows - 1) / (2 * tile_rows);
+      for (int passes = p_min; passes * tiles <= pairs && passes < p_min + 16; ++passes) {
+        if (passes > p_min && M < 32 * passes) break;
+        const PlanWish w = {passes, tile_rows, true};
+        const Plan p = plan_as(ctx, M, w_dtype, w);
+        const double us = one_tile_us(ctx, p, w_dtype);
+        if (p.n_ptiles * p.passes <= pairs && us < best_us) {
+          best = p; best_us = us; want = w;
+          best.est_seconds = us * 1e-6 + 6e-6;
+        }
+      }
+    }
+  }
+  if (ctx->no_fuse && best.passes > 1) {           // the same passes, a launch each
+    const double est = best.est_seconds;
+    want.passes = best.passes; want.fuse = false;
+    best = plan_as(ctx, M, w_dtype, want);
+    best.est_seconds = est;
+  }
   return best;
 }
 
@@ -3222,17 +3296,14 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   kp.prefetch_blocks = 0;
   if (few_before) {
     const int per_tile = w8 ? (pl.n_kblocks + 1) / 2 : pl.n_kblocks - pl.k_tail;
-    const int blocks = static_cast<int>(32e6 / (static_cast<double>(pl.grid) * pl.tile_rows * 128.0));
+    const int ctas = pl.grid / (pl.fused ? pl.passes : 1);                                // that share W_lm among them
+    const int blocks = static_cast<int>(32e6 / (static_cast<double>(ctas) * pl.tile_rows * 128.0));
     kp.prefetch_blocks = (blocks < per_tile ? blocks : per_tile) / pl.kpb * pl.kpb;
   }
   kp.n_pass = pl.fused ? pl.passes : 1;
   kp.rows_per_pass = pl.rows_per_pass;
   kp.pace = nullptr;
-  if (pl.fused && ctx->pace && !ctx->no_pace && pl.grid / (2 * pl.passes) <= kMaxPaceGroups) {
-    kp.pace = ctx->pace;
-    e = cudaMemsetAsync(ctx->pace, 0, sizeof(unsigned) * static_cast<size_t>(pl.grid / (2 * pl.passes)), stream);
-    if (e != cudaSuccess) { set_error(ctx, "reset of the pace counters", e); return HOLA_ERR_CUDA; }
-  }
+  if (pl.fused && ctx->pace && !ctx->no_pace && pl.grid / (2 * pl.passes) <= kMaxPaceGroups) kp.pace = ctx->pace;
   for (int pass = 0; pass < (pl.fused ? 1 : pl.passes); ++pass) {
     kp.row0 = pass * pl.rows_per_pass;
     kp.rows = M - kp.row0 < pl.rows_per_pass ? M - kp.row0 : pl.rows_per_pass;
@@ -3496,6 +3567,7 @@ hola_status hola_create(hola_ctx** out, int device, int maxB, int maxK, int H, i
   ctx->st_out = reinterpret_cast<unsigned char*>(ctx->ws + w.st_out);
   ctx->st_qtok = reinterpret_cast<float*>(ctx->ws + w.st_qtok);
   cudaMemset(ctx->status, 0, 4);
+  cudaMemset(ctx->pace, 0, 8 * kMaxPaceGroups);
   const size_t n_qtok = static_cast<size_t>(maxB) * (maxK > 0 ? maxK : 1);
   void* pinned = nullptr;
   if (cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||

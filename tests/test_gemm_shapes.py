@@ -55,3 +55,30 @@ def check_lm_head(binding, mode, B, k, H, V, seed=0, options=()):
 @pytest.mark.parametrize("B,k,H,V", [(3, 2, 16, 777), (9, 4, 144, 2000), (7, 3, 1040, 5003), (33, 3, 400, 9000), (4, 0, 256, 4097)])
 def test_padded_rows_of_eight_bit_planes(binding, mode, B, k, H, V):
     check_lm_head(binding, mode, B, k, H, V)
+
+
+# Small vocabularies: the rows are cut into several passes over few tiles, all in one launch.  The last pass ends inside a block of
+# rows, or holds a single row; tiles of 32, 64, 96 and 128 rows per CTA; a ragged last tile; a partial last K block; with tiles left
+# over for some pairs (the calls come twice: what the groups of pairs keep step by has to be as it was).
+@pytest.mark.parametrize("mode,B,k,H,V", [
+    ("bf16", 139, 2, 1304, 1272), ("bf16", 128, 3, 512, 2000), ("bf16", 64, 2, 200, 1030), ("bf16", 43, 5, 264, 3001),
+    ("bf16", 256, 8, 128, 1003), ("bf16", 129, 0, 4096, 700), ("int8", 29, 8, 944, 2904), ("int8", 97, 0, 2048, 520),
+    ("w8a8", 64, 5, 1040, 4000), ("w8a8", 200, 1, 512, 700), ("w8a16", 36, 5, 576, 3550), ("w8a16", 41, 2, 2048, 640)])
+def test_rows_of_small_vocabularies_in_several_passes(binding, mode, B, k, H, V):
+    wd = {"bf16": binding.HOLA_W_BF16, "int8": binding.HOLA_W_INT8, "w8a8": binding.HOLA_W8A8, "w8a16": binding.HOLA_W8A16}[mode]
+    plan = binding.hola_plan_for_shape(148, H, V, B * (k + 1), wd)
+    assert plan["passes"] > 1 and plan["kernels_per_call"] == 2
+    check_lm_head(binding, mode, B, k, H, V)
+
+
+@pytest.mark.parametrize("mode,B,k,H,V", [("bf16", 300, 3, 64, 30000), ("w8a8", 200, 4, 128, 40001)])
+def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(binding, mode, B, k, H, V):
+    hidden, W = exact_operands(B, k, H, V, 3)
+    want = (hidden.double().reshape(-1, H) @ W.double().t()).float()
+    scale = None
+    if mode != "bf16":
+        W, scale = binding.hola_quantize_w8(W)
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        for _ in range(3):
+            out = ctx.hola_lm_head_entropy(hidden, W, want_logits=True, w_scale=scale, a8=MODES[mode])
+            assert torch.equal(out.logits.reshape(-1, V), want)
