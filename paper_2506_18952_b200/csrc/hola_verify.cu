@@ -1250,10 +1250,15 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       }
     }
     for (int t = 0; t < my_tiles && ok; ++t) {
-      const int buf = t % p.nbuf;
-      const uint32_t acc_phase = static_cast<uint32_t>(t / p.nbuf) & 1u;
-      if (!mbar_wait_warp(tfull_bar + 8 * buf, acc_phase, abort_flag, p.status)) { ok = false; break; }
-      tc_fence_after();
+      // (one buffer or two.  What depends on the tile alone is worked out, and loaded, ahead of the wait; with 8-bit hidden rows
+      // behind it: there it would be spilled)
+      constexpr bool kAhead = !kI8 || kRot;
+      const int buf = p.nbuf == 2 ? t & 1 : 0;
+      const uint32_t acc_phase = static_cast<uint32_t>(p.nbuf == 2 ? t >> 1 : t) & 1u;
+      if (!kAhead) {
+        if (!mbar_wait_warp(tfull_bar + 8 * buf, acc_phase, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+      }
       const int vbase = (pair + t * npairs) * pair_rows + static_cast<int>(rank) * p.tile_rows;
       const int tile_lane = quarter * 32 + lane;         // lanes at or beyond tile_rows hold nothing
       const int vocab = vbase + tile_lane;
@@ -1268,6 +1273,10 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         w_scale *= width == 8 ? kExpandUnscale8 : (width == 4 ? kExpandUnscale4 : 1.f);
       }
       const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+      if (kAhead) {
+        if (!mbar_wait_warp(tfull_bar + 8 * buf, acc_phase, abort_flag, p.status)) { ok = false; break; }
+        tc_fence_after();
+      }
       if (kTwoPlane) {
         // Two planes: 64 consecutive accumulator columns hold the coarse-plane sums (first 32) and the remainder-plane
         // sums (last 32) of the same 32 verify rows.  Read 16 + 16 columns at a time, add them with their scales, and
@@ -1283,7 +1292,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         for (int slot = 0; slot < 2; ++slot) {
           if (slot < my_pairs) {
             const int pr = group + slot * kGroups;
-            const int sub = (64 * pr) / p.N, col = 64 * pr - sub * p.N;
+            const int sub = 64 * pr >= p.N ? 1 : 0, col = 64 * pr - sub * p.N;      // (at most two MMAs)
             const uint32_t taddr = lane_addr + buf * 256 + sub * 256 + col;
             const int vr0 = row0 + 32 * pr;            // verify row of the pair's first column
             const int n_ok = min(32, p.M - vr0);
@@ -1432,7 +1441,7 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
       for (int slot = 0; slot < kSlots; ++slot) {
         if (slot < my_chunks) {
           const int ch = group + slot * kGroups;
-          const int sub = ch / sub_chunks, j = ch - sub * sub_chunks;
+          const int sub = kI8 ? ch / sub_chunks : ch >= sub_chunks ? 1 : 0, j = ch - sub * sub_chunks;      // (at most two MMAs)
           float v[32];
           __syncwarp();                                  // tcgen05.ld is warp-collective: reconverge first
           tmem_ld32(lane_addr + (kW8 ? buf * p.acc_cols : buf * 256 + sub * 256) + j * 32, v);
@@ -1460,10 +1469,12 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
               } else if (n_ok == 32) {
 #pragma unroll
                 for (int i = 0; i < 32; ++i) dst[static_cast<size_t>(i) * p.ldl] = v[i];
-              } else {
+              } else {                                   // (left at the last row: small batches have few, and wait for this)
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (i < n_ok) store_logit(dst + static_cast<size_t>(i) * p.ldl, v[i], p.stream_logits);
+                for (int i = 0; i < 32; ++i) {
+                  if (!kI8 && i >= n_ok) break;          // (8-bit hidden rows: that, and the selection above, would spill)
+                  if (!kI8 || i < n_ok) store_logit(dst + static_cast<size_t>(i) * p.ldl, v[i], p.stream_logits);
+                }
               }
             }
             if (nv > 0) {
@@ -1659,14 +1670,16 @@ lm_head_entropy_kernel(const __grid_constant__ CUtensorMap tmap_hidden, const __
         x[q] = merge[q * rows_end + r];
         m = fmaxf(m, x[q].x);
       }
+      // (No branches: they kept the eight exponentials from overlapping, 900 cycles at the end of every launch.  With that, the
+      // stores that stop at the last row and what moved ahead of the wait for a tile, us: one sequence, V = 8000 11.66 -> 11.15,
+      // V = 32000 46.9 -> 46.2, mixed widths 34.7 -> 33.8; 4, V = 20000 16.45 -> 16.0; 64, V = 16000 18.3 -> 17.9.)
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         if (x[q].x == m) arg = min(arg, __float_as_int(x[q].w));
-        if (x[q].x != -CUDART_INF_F) {
-          const float d = x[q].x - m, e = __expf(d);
-          sum = fmaf(e, x[q].y, sum);
-          sum_t = fmaf(e, fmaf(d, x[q].y, x[q].z), sum_t);
-        }
+        const bool some = x[q].x != -CUDART_INF_F;
+        const float d = some ? x[q].x - m : 0.f, y = some ? x[q].y : 0.f, z = some ? x[q].z : 0.f, e = __expf(d);
+        sum = fmaf(e, y, sum);
+        sum_t = fmaf(e, fmaf(d, y, z), sum_t);
       }
       p.partials[static_cast<size_t>(row0_end + r) * p.part_stride + 2 * pair_end + (kAnew ? bid & 1 : static_cast<int>(rank))] =
           make_float4(m, sum, sum_t, __int_as_float(arg));
