@@ -98,7 +98,7 @@ constexpr int kK3MaxPerSm = 4;                   // CTAs of the accept/sample ke
 constexpr int kChunk = 128;                      // vocabulary entries per warp step (32 lanes x 4)
 constexpr int kMaxChunks = 4096;                 // => V <= 524288
 constexpr int kMaxK1 = 64;                       // k + 1 <= 64
-constexpr int kK3MaxDynSmem = 200 * 1024;        // rows staged in shared memory, see K3Params::staged
+constexpr int kK3MaxDynSmem = 200 * 1024;        // rows staged in shared memory (kStaged)
 constexpr int kK3Unroll = 4;                     // vocabulary chunks a warp has in flight per step
 
 constexpr int kHqSlices = 8;                     // CTAs that share one draft row in draft_entropy_kernel
@@ -174,8 +174,6 @@ struct K3Params {
   int inputs_settled;           // 1: launched right behind this call's own GEMM kernel, whose CTAs have waited for the
                                 // kernel before the call: tokens, uniforms and draft probabilities may be read
                                 // before this grid's dependency wait.  0: wait first.
-  int staged;                   // 1: this CTA's slice of ALL k + 1 rows is brought into shared memory while the statistics are
-                                // merged and the accept test is made, instead of row n afterwards
   int phase;                    // 0: the whole step; 1: stop after the accept test (accept_len, statistics written);
                                 // vocabulary-parallel form: 3: stop after the masses of row n inside this shard,
                                 // 4: the draw, by the shard that holds the point u * R
@@ -1736,46 +1734,72 @@ __global__ void __launch_bounds__(64, 1) bounded_wait_selftest_kernel(long long 
 // The statistics of one row over all CTAs, by a warp, the same bits in every lane.  Six loads per lane in flight (192
 // partials per round: one round on a 148-SM part; a GEMM launch leaves a row's partials side by side, part_stride 1).  The
 // maximum first (one instruction), so that the exponentials of the partials are independent of one another and only additions
-// remain to be passed round: five shuffles instead of eleven merges of a hundred cycles each.
-__device__ __forceinline__ Stats warp_merge_partials(const float4* partials, int nparts, int row_stride, int part_stride,
-                                                     int row, int lane) {
-  partials += static_cast<size_t>(row) * row_stride;
-  Stats st = stats_empty();
-  for (int base = 0; base < nparts; base += 192) {
-    float4 x[6];
+// remain to be passed round: five shuffles instead of eleven merges of a hundred cycles each.  No branch per partial (an empty one
+// counts as zeros): they kept the exponentials from overlapping.  The arg-max only for whoever reads it.
+constexpr int kPartsPerLane = 6;
+__device__ __forceinline__ void load_partials(const float4* partials, int base, int nparts, int part_stride, int lane,
+                                              float4 x[kPartsPerLane]) {
 #pragma unroll
-    for (int u = 0; u < 6; ++u) {
-      const int i = base + lane + 32 * u;
-      x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride]
-                        : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
-    }
-    const float m = warp_max_f32(fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x)));
-    float s = 0.f, t = 0.f;
-    int arg = 0x7fffffff;
+  for (int u = 0; u < kPartsPerLane; ++u) {
+    const int i = base + lane + 32 * u;
+    x[u] = i < nparts ? partials[static_cast<size_t>(i) * part_stride]
+                      : make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7fffffff));
+  }
+}
+__device__ __forceinline__ Stats merge_loaded(const float4 x[kPartsPerLane], bool want_arg) {
+  const float m = warp_max_f32(fmaxf(max3(x[0].x, x[1].x, x[2].x), max3(x[3].x, x[4].x, x[5].x)));
+  float s = 0.f, t = 0.f;
 #pragma unroll
-    for (int u = 0; u < 6; ++u) {
+  for (int u = 0; u < kPartsPerLane; ++u) {
+    const bool some = x[u].x != -CUDART_INF_F;
+    const float d = some ? x[u].x - m : 0.f, y = some ? x[u].y : 0.f, z = some ? x[u].z : 0.f, e = __expf(d);
+    s = fmaf(e, y, s);
+    t = fmaf(e, fmaf(d, y, z), t);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, off);
+    t += __shfl_xor_sync(0xffffffffu, t, off);
+  }
+  int arg = 0x7fffffff;
+  if (want_arg) {
+#pragma unroll
+    for (int u = 0; u < kPartsPerLane; ++u)
       if (x[u].x == m) arg = min(arg, __float_as_int(x[u].w));
-      if (x[u].x != -CUDART_INF_F) {
-        const float d = x[u].x - m, e = __expf(d);
-        s = fmaf(e, x[u].y, s);
-        t = fmaf(e, fmaf(d, x[u].y, x[u].z), t);
-      }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, off);
-      t += __shfl_xor_sync(0xffffffffu, t, off);
-    }
     arg = __reduce_min_sync(0xffffffffu, arg);
-    st = stats_merge(st, Stats{m, s, t, arg});
+  }
+  return Stats{m, s, t, arg};
+}
+// (x: the first round, loaded)
+__device__ __forceinline__ Stats warp_merge_partials(float4 x[kPartsPerLane], const float4* partials, int nparts, int part_stride,
+                                                     int lane, bool want_arg) {
+  Stats st = merge_loaded(x, want_arg);
+  for (int base = 32 * kPartsPerLane; base < nparts; base += 32 * kPartsPerLane) {
+    load_partials(partials, base, nparts, part_stride, lane, x);
+    st = stats_merge(st, merge_loaded(x, want_arg));
   }
   return st;
 }
+__device__ __forceinline__ Stats warp_merge_row(const float4* partials, int nparts, int row_stride, int row, int lane, bool want_arg) {
+  partials += static_cast<size_t>(row) * row_stride;
+  float4 x[kPartsPerLane];
+  load_partials(partials, 0, nparts, 1, lane, x);
+  return warp_merge_partials(x, partials, nparts, 1, lane, want_arg);
+}
 
+// t / s for 1 <= s <= V: the product with the approximate reciprocal, corrected once by its exact remainder (Newton's step on the
+// quotient), within 2^-23 of a unit in the last place of t / s before its one rounding.  (An IEEE division takes 260 cycles here,
+// of a chain that small batches wait for; this 35.)
+__device__ __forceinline__ float quotient(float t, float s) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s));
+  const float q = t * y;
+  return fmaf(fmaf(-q, s, t), y, q);
+}
 __device__ __forceinline__ void stats_to_outputs(Stats st, float* logZ, float* H) {
   const float ls = logf(st.s);
   *logZ = st.m + ls;
-  *H = fmaxf(0.f, ls - st.t / st.s);
+  *H = fmaxf(0.f, ls - quotient(st.t, st.s));
 }
 
 __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, int nparts, int row_stride, int M,
@@ -1786,7 +1810,7 @@ __global__ void __launch_bounds__(256) finalize_kernel(const float4* partials, i
   const int lane = threadIdx.x & 31;
   grid_dependency_wait();
   if (row >= M) return;
-  Stats st = warp_merge_partials(partials, nparts, row_stride, 1, row, lane);
+  Stats st = warp_merge_row(partials, nparts, row_stride, row, lane, false);
   if (lane == 0) stats_to_outputs(st, &logZ[row], &entropy[row]);
 }
 
@@ -1802,7 +1826,7 @@ __global__ void __launch_bounds__(256) shard_record_kernel(const float4* partial
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= M) return;
-    Stats st = warp_merge_partials(partials, nparts, row_stride, 1, row, lane);
+    Stats st = warp_merge_row(partials, nparts, row_stride, row, lane, true);
     if (lane == 0) {
       const int arg = st.arg == 0x7fffffff ? st.arg : st.arg + v_offset;
       stats_out[row] = make_float4(st.m, st.s, st.t, __int_as_float(arg));
@@ -1873,36 +1897,31 @@ __device__ __forceinline__ void resid4(const float l[4], const float q[4], float
   for (int i = 0; i < 4; ++i) r[i] = fmaxf(0.f, ex2_approx((l[i] - logZ) * kLog2e) - q[i]);
 }
 
-// The residual mass of every chunk of a slice (chunks c_first .. c_first + mine - 1), by the whole CTA of kWarps warps.  In
-// fp32 (128 non-negative terms added pairwise: relative error a few 1e-7), kept as fp64 for the scans that follow.  lrow,
-// qrow: entry 0 of the row, which a staged slice does not hold.  (Inlined once for rows in shared memory and once for rows in
-// global memory, so that each gets loads of its own kind, and once per type of q: us, 50 rows, V = 60000 53.2 -> 52.4, 32 rows,
-// V = 128256 61.0 -> 59.7, 5 rows, V = 32000 46.67 -> 46.46.)
-template <bool kVec, bool kHalf, int kWarps>
-__device__ __forceinline__ void sum_chunks(const float* lrow, const void* qrow, bool residual, int c_first, int mine, int V,
-                                           float logZ, double* csum, int warp, int lane) {
-  for (int c0 = warp; c0 < mine; c0 += kK3Unroll * kWarps) {
-    float l[kK3Unroll][4], q[kK3Unroll][4];
+// The residual masses of up to four chunks, c0 and every kStride-th after it as long as they are among n, by a warp: into csum[],
+// and as the result in lanes 8 i .. 8 i + 7 (0 where there is no i-th).  In fp32 (128 non-negative terms added pairwise: relative error a few 1e-7), kept as fp64 for
+// the sums that follow.  lrow, qrow: entry 0 of the row, which a staged slice does not hold.  (Once per type of q: us, 50 rows,
+// V = 60000 53.2 -> 52.4, 32 rows, V = 128256 61.0 -> 59.7, 5 rows, V = 32000 46.67 -> 46.46.  A form for two chunks, and packed
+// fp32 arithmetic, took fewer instructions and longer.)
+template <bool kVec, bool kHalf, int kStride>
+__device__ __forceinline__ double sum_step(const float* lrow, const void* qrow, bool residual, int c0, int n, int V, float logZ,
+                                           double* csum, int lane) {
+  float l[kK3Unroll][4], q[kK3Unroll][4];
 #pragma unroll
-    for (int i = 0; i < kK3Unroll; ++i) {                // all loads of this step first
-      const int c = c0 + i * kWarps;
-      fetch4<kVec, kHalf>(lrow, qrow, residual, c < mine ? (c_first + c) * kChunk + lane * 4 : V, V, l[i], q[i]);
-    }
-    float part[kK3Unroll];
+  for (int i = 0; i < kK3Unroll; ++i)                    // all loads first
+    fetch4<kVec, kHalf>(lrow, qrow, residual, i * kStride < n ? (c0 + i * kStride) * kChunk + lane * 4 : V, V, l[i], q[i]);
+  float part[kK3Unroll];
 #pragma unroll
-    for (int i = 0; i < kK3Unroll; ++i) {
-      part[i] = 0.f;
-      if (c0 + i * kWarps < mine) {
-        float r[4];
-        resid4(l[i], q[i], logZ, r);
-        part[i] = (r[0] + r[1]) + (r[2] + r[3]);
-      }
+  for (int i = 0; i < kK3Unroll; ++i) {
+    part[i] = 0.f;
+    if (i * kStride < n) {
+      float r[4];
+      resid4(l[i], q[i], logZ, r);
+      part[i] = (r[0] + r[1]) + (r[2] + r[3]);
     }
-    // lanes 0, 8, 16, 24 end up with chunks 0, 1, 2, 3 of this step
-    const float sum = warp_sum4_f32(part, lane);
-    const int c = c0 + (lane >> 3) * kWarps;
-    if ((lane & 7) == 0 && c < mine) csum[c] = static_cast<double>(sum);
   }
+  const double sum = static_cast<double>(warp_sum4_f32(part, lane));
+  if ((lane & 7) == 0 && (lane >> 3) * kStride < n) csum[(lane >> 3) * kStride] = sum;
+  return sum;
 }
 
 // Untiled bulk copy into this CTA's shared memory (addresses and size multiples of 16 bytes), counted on an mbarrier.
@@ -1910,6 +1929,18 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
   asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
                : "memory");
+}
+// A double into a CTA of the cluster (addresses from map_to_cta), counted on a barrier there.
+__device__ __forceinline__ void store_async(uint32_t cluster_addr, double x, uint32_t cluster_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+               ::"r"(cluster_addr), "l"(__double_as_longlong(x)), "r"(cluster_bar)
+               : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n .reg .pred P;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n selp.u32 %0, 1, 0, P;\n}"
+               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return done != 0;
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -1926,14 +1957,14 @@ __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
   return u;
 }
 
-// Waits for the staged rows of this CTA, whose own copies they are.  When the time is up the status word is told at once:
-// the CTA that draws the token, and reports, may be another one of the cluster, whose rows did land (it looks at the status
-// word behind the cluster barrier).  The copies then have as long again before the CTA goes on (and sooner or later leaves
+// Waits for what is counted on a barrier of this CTA: its staged rows, or the masses of all warps of the cluster.  When the time is
+// up the status word is told at once: the CTA that draws the token, and reports, may be another one of the cluster, whose rows did
+// land (it looks at the status word behind the exchange of masses).  The copies then have as long again before the CTA goes on (and sooner or later leaves
 // the memory they write to).  False: gave up.
-__device__ __forceinline__ bool wait_staged_rows(uint32_t bar, unsigned* status, long long limit_cycles) {
+__device__ __forceinline__ bool wait_bulk(uint32_t bar, unsigned* status, long long limit_cycles) {
   const long long t0 = clock64();
   bool late = false;
-  while (!mbar_try_wait(bar, 0u)) {
+  while (!mbar_try_wait_cluster(bar, 0u)) {
     const long long waited = clock64() - t0;
     if (waited > limit_cycles && !late) {
       late = true;
@@ -1957,7 +1988,7 @@ __global__ void __launch_bounds__(64, 1) staged_wait_selftest_kernel(long long l
     if (rank == 0) mbar_arrive(smem_u32(&bar));
   }
   __syncthreads();
-  if (!wait_staged_rows(smem_u32(&bar), status, limit_cycles)) atomicAdd(out + 1, 1u);
+  if (!wait_bulk(smem_u32(&bar), status, limit_cycles)) atomicAdd(out + 1, 1u);
   cluster_sync_all();
   if (rank == 0 && threadIdx.x == 0) {
     K3Params p;
@@ -1967,20 +1998,48 @@ __global__ void __launch_bounds__(64, 1) staged_wait_selftest_kernel(long long l
   atomicAdd(out, 1u);
 }
 
+// Whether the run of accepted drafts ends at a position, and what it flags.
+constexpr unsigned kStop = 1u << 31;
+__device__ __forceinline__ unsigned decide(const K3Params& p, int x, int Vtok, float u, float lx, float qx, float hq, float logZ,
+                                           float H, int amax) {
+  if (x < 0 || x >= Vtok) return HOLA_FLAG_BAD_TOKEN | kStop;
+  if ((p.gate_source == HOLA_GATE_DRAFT_ENTROPY ? hq : H) < p.tau) return 0u;        // entropy gate: fast path keeps the draft token
+  if (p.fallback == HOLA_FALLBACK_GREEDY) return x != amax ? kStop : 0u;             // the verifier's own token, or the run ends here
+  unsigned flags = 0;
+  u = clamp_uniform(u, flags);
+  const float px = expf(lx - logZ);
+  const bool keep = (qx > 0.f) ? (u * qx < px) : (px > 0.f);
+  return flags | (keep ? 0u : kStop);
+}
+
 // One cluster of S CTAs per sequence.  Every CTA derives accept_len on its own (same inputs, same arithmetic,
-// same result), sums the residual mass of its slice of the vocabulary chunk by chunk, and publishes its slice
-// total to all CTAs of the cluster through distributed shared memory.  After one cluster barrier each CTA knows
-// the total mass R and which slice holds the point u*R; that CTA alone finishes the inverse-CDF search.
+// same result), a warp per position from the statistics to the decision, sums the residual mass of its slice of the
+// vocabulary chunk by chunk, and every warp sends what it summed to all CTAs of the cluster through distributed shared memory.
+// Once all of it has arrived each CTA knows the total mass R and which slice holds the point u*R; that CTA alone finishes the
+// inverse-CDF search, with one warp: chunk, lane, entry.
+// On small batches a chain of dependent steps bounds it, a few hundred cycles each (a shuffle is 29, one of a double with its
+// addition 35, a vote 21, an IEEE division 260), and where one SM has 32 warps at it the instructions of all of them: nothing is
+// worked out by more warps than need it, nor ahead of a barrier if one warp can do it behind.  Before, every warp made all
+// decisions behind the first barrier, warp 0 of each CTA scanned its chunks ahead of a cluster barrier, and every warp scanned the
+// slices behind it.  Cycles from entry to token, V = 1000 9030 -> 7090, V = 32000 9890 -> 8820; us, one sequence, V = 1000
+// 9.6 -> 8.7, V = 8000 11.06 -> 10.85, V = 32000 45.8 -> 45.2, mixed widths 33.8 -> 33.2; 8 sequences of 9 positions, V = 30000
+// 18.6 -> 17.9; 200, V = 12000 41.0 -> 39.9; 250, V = 30000 47.4 -> 44.2; 64, V = 16000 18.0 -> 17.9; 8, V = 128256 38.65 -> 38.8.
+// The chunks of a step alternate between the warps: side by side in one warp (so that a warp's mass is that of a run of the
+// vocabulary, and one scan less is needed) rows that start on no line are fetched twice, 60 sequences, V = 50003 33.2 -> 36.9.
 // kAsk: the slice of row n is asked into the L2 as soon as n is known.
 // kSolo: one CTA of 1024 threads instead of the cluster (see sample_solo).
-template <bool kVec, bool kAsk, bool kSolo = false>
+// kStaged: this CTA's slice of ALL k + 1 rows is brought into shared memory while the statistics are merged and the accept test
+// is made, instead of row n afterwards.
+template <bool kVec, bool kAsk, bool kSolo = false, bool kStaged = false>
 __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 : kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
   constexpr int kThreads = kSolo ? kSoloThreads : kK3Threads, kWarps = kThreads / 32;
   extern __shared__ __align__(16) double csum[];                       // per-chunk residual mass of this CTA's slice
-  __shared__ double sh_tot[2][8];                        // slice totals of the whole cluster, per attempt
-  __shared__ float sh_logZ[kMaxK1], sh_H[kMaxK1], sh_lx[kMaxK1], sh_qx[kMaxK1], sh_u[kMaxK1], sh_Hq[kMaxK1];
-  __shared__ int sh_x[kMaxK1], sh_amax[kMaxK1];
+  __shared__ __align__(16) double sh_tot[2][kSolo ? kWarps : 8 * kWarps];      // masses of all warps' runs, per attempt
+  __shared__ float sh_logZ[kMaxK1], sh_uk;
+  __shared__ int sh_amax[kMaxK1];
+  __shared__ unsigned sh_dec[kMaxK1];                    // decide()'s results
   __shared__ __align__(8) uint64_t sh_bar;               // staged rows have landed
+  __shared__ __align__(8) uint64_t sh_all[2];            // all runs' masses have arrived, per attempt
 
   // The next kernel in the stream (normally the next call's GEMM kernel, which waits for this grid before it touches
   // memory) may be scheduled from now on: its launch and prologue then hide behind this kernel.
@@ -1988,42 +2047,57 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
   cg::cluster_group cluster = cg::this_cluster();
   const int S = kSolo ? 1 : static_cast<int>(cluster.num_blocks());
   const int rank = kSolo ? 0 : static_cast<int>(cluster.block_rank());
-  const int b = blockIdx.x / S;
+  const int b = kSolo ? static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x) >> (31 - __clz(S));   // (S is 1, 2, 4 or 8)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k = p.k, V = p.V;
   const int row_first = b * (k + 1);
 
-  // ---- the draft tokens and uniforms, a position per thread (k <= 63 < kK3Threads).  These come from the caller, not from
-  // the GEMM kernel.  Behind this call's own GEMM kernel they are known to be in place (its CTAs waited for whatever ran
-  // before the call) and are asked for before this grid's dependency wait; in every other launch the wait comes first.
-  // Nothing looks at a loaded value before everything that does not depend on it has been asked for: each look costs a
-  // round trip to the L2 (or, where the GEMM kernel's idle warps have not asked ahead, to DRAM).
+  // ---- the draft tokens and uniforms.  The k + 1 positions are dealt to the warps from the last warp down, and lane i of a
+  // warp looks after the warp's i-th position.  These come from the caller, not from the GEMM kernel.  Behind this call's own
+  // GEMM kernel they are known to be in place (its CTAs waited for whatever ran before the call) and are asked for before this
+  // grid's dependency wait; in every other launch the wait comes first.  Nothing looks at a loaded value before everything
+  // that does not depend on it has been asked for: each look costs a round trip to the L2 (or, where the GEMM kernel's idle
+  // warps have not asked ahead, to DRAM).
   if (!p.inputs_settled) grid_dependency_wait();
   const bool shard = p.shard_world > 0;
   const int Vtok = shard ? p.V_global : V;               // range of valid token ids
-  const int j_mine = threadIdx.x;
+  const int j_first = kWarps - 1 - warp, j_mine = j_first + lane * kWarps;
   int x_mine = -1;
   float u_mine = 0.f;
   if (j_mine < k) x_mine = p.tok[b * k + j_mine];
   if (j_mine <= k) u_mine = p.u[b * (k + 1) + j_mine];
   // From here on the GEMM kernel's results are read.
   if (p.inputs_settled) grid_dependency_wait();
+  // (statistics first: what follows looks at the tokens)
+  const float4* row_parts = p.partials + static_cast<size_t>(row_first + j_first) * p.row_stride;
+  float4 x[kPartsPerLane];
+  if (p.combine && j_first <= k) load_partials(row_parts, 0, p.nparts, p.part_stride, lane, x);
+  // (waited for behind the decisions, ahead of the first remote store.  Relaxed: a release here would first wait for the loads)
+  if (!kSolo && S > 1) {
+    if (threadIdx.x == 0) {
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(smem_u32(&sh_all[i]), 1);
+        mbar_expect_tx(smem_u32(&sh_all[i]), S * kWarps * 8u);
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+  }
   const int nchunks = (V + kChunk - 1) / kChunk;
-  const int cpc = (nchunks + S - 1) / S;                 // chunks per CTA
+  const int cpc = kSolo ? nchunks : (nchunks + S - 1) >> (31 - __clz(S));      // chunks per CTA
   const int c_first = rank * cpc;
   const int mine = max(0, min(nchunks, c_first + cpc) - c_first);
   const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
   // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities, each row's
   // slice by one bulk copy, a lane of the first warp per copy, while the other warps merge statistics (with eight rows and more
-  // that one does so too, after its gathers: then the last warp).  (One thread after the
+  // that one does so too: then the last warp).  (One thread after the
   // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows, V = 32000: 46.67 -> 46.31, mixed widths
   // 34.84 -> 34.47.)
-  const bool staged = kVec && !kSolo && p.staged;
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
   char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
   const int here = min(V - c_first * kChunk, mine * kChunk);           // entries of this slice (0 or less: none)
-  if (staged && warp == (k + 1 < kWarps ? 0 : kWarps - 1) && here > 0) {
+  if (kStaged && warp == (k + 1 < kWarps ? 0 : kWarps - 1) && here > 0) {
     const uint32_t bar = smem_u32(&sh_bar), lbytes = here * 4u, qbytes = static_cast<uint32_t>(here * q_elem);
     if (lane == 0) {
       mbar_init(bar, 1);
@@ -2041,7 +2115,7 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
   }
   // the draft token's logit and probability
   float lx = 0.f, hq = 0.f;
-  uint32_t q_bits = 0;                                   // (as loaded: converted when it is stored)
+  uint32_t q_bits = 0;                                   // (as loaded: converted where it is used)
   if (j_mine < k) {
     const int j = j_mine;
     if (x_mine >= 0 && x_mine < Vtok && p.fallback != HOLA_FALLBACK_GREEDY) {     // (greedy: compared by its index alone)
@@ -2063,61 +2137,42 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
       if (rank == 0 && p.draft_entropy) p.draft_entropy[b * k + j] = hq;
     }
   }
-  // ---- softmax statistics of this sequence's k+1 positions
-  if (p.combine) {
-    // (rows are dealt to the warps from the last warp down: warp 0, whose threads are still waiting for the gathers
-    // above, gets a row only when there are as many rows as warps)
-    for (int j = kWarps - 1 - warp; j <= k; j += kWarps) {
-      Stats st = warp_merge_partials(p.partials, p.nparts, p.row_stride, p.part_stride, row_first + j, lane);
-      if (lane == 0) {
-        float lz, h;
-        stats_to_outputs(st, &lz, &h);
-        sh_logZ[j] = lz; sh_H[j] = h; sh_amax[j] = st.arg;
-        if (rank == 0) { p.logZ[row_first + j] = lz; p.entropy[row_first + j] = h; }
+  // ---- softmax statistics of this sequence's k+1 positions; gate and ratio test of each
+  for (int i = 0, j = j_first; j <= k; ++i, j += kWarps) {
+    float lz, h;
+    int amax = 0;
+    if (p.combine) {
+      if (i > 0) {
+        row_parts += static_cast<size_t>(kWarps) * p.row_stride;
+        load_partials(row_parts, 0, p.nparts, p.part_stride, lane, x);
       }
+      const Stats st = warp_merge_partials(x, row_parts, p.nparts, p.part_stride, lane, p.fallback == HOLA_FALLBACK_GREEDY);
+      stats_to_outputs(st, &lz, &h);
+      amax = st.arg;
+    } else {
+      lz = p.logZ[row_first + j];
+      h = p.entropy[row_first + j];
     }
-  } else {
-    for (int j = threadIdx.x; j <= k; j += kThreads) {
-      sh_logZ[j] = p.logZ[row_first + j];
-      sh_H[j] = p.entropy[row_first + j];
+    if (lane == i) {
+      const float qx = __uint_as_float(!p.q_tok && p.q_dtype == HOLA_Q_BF16 ? q_bits << 16 : q_bits);
+      sh_dec[j] = j < k ? decide(p, x_mine, Vtok, u_mine, lx, qx, hq, lz, h, amax) : 0u;
+      sh_logZ[j] = lz; sh_amax[j] = amax;
+      if (j == k) sh_uk = u_mine;
+      if (rank == 0 && p.combine) { p.logZ[row_first + j] = lz; p.entropy[row_first + j] = h; }
     }
-  }
-  if (j_mine <= k) sh_u[j_mine] = u_mine;
-  if (j_mine < k) {
-    sh_x[j_mine] = x_mine; sh_lx[j_mine] = lx; sh_Hq[j_mine] = hq;
-    sh_qx[j_mine] = __uint_as_float(!p.q_tok && p.q_dtype == HOLA_Q_BF16 ? q_bits << 16 : q_bits);
   }
   __syncthreads();
 
-  // ---- gate and ratio test in draft order; the first position that is not accepted ends the run.  A lane per position,
-  // in every warp (same inputs, same result: no second barrier); what a position past the end would flag does not count.
-  unsigned flags = 0;
+  // ---- in draft order, the first position that is not accepted ends the run (what a position past it flags does not count)
+  unsigned flags = 0;                                    // (of the first and the last warp, which report)
   int n = k;
   for (int j0 = 0; j0 < k && n == k; j0 += 32) {
-    const int j = j0 + lane;
-    unsigned fl = 0;
-    bool stop = false;
-    if (j < k) {
-      const int x = sh_x[j];
-      const float gate_value = p.gate_source == HOLA_GATE_DRAFT_ENTROPY ? sh_Hq[j] : sh_H[j];
-      if (x < 0 || x >= Vtok) {
-        fl = HOLA_FLAG_BAD_TOKEN;
-        stop = true;
-      } else if (gate_value < p.tau) {                   // entropy gate: fast path keeps the draft token
-      } else if (p.fallback == HOLA_FALLBACK_GREEDY) {   // the verifier's own token, or the run ends here
-        stop = x != sh_amax[j];
-      } else {
-        const float u = clamp_uniform(sh_u[j], fl);
-        const float px = expf(sh_lx[j] - sh_logZ[j]);
-        const float qx = sh_qx[j];
-        stop = !((qx > 0.f) ? (u * qx < px) : (px > 0.f));
-      }
-    }
-    const unsigned stops = __ballot_sync(0xffffffffu, stop);
+    const unsigned dec = j0 + lane < k ? sh_dec[j0 + lane] : 0u;
+    const unsigned stops = __ballot_sync(0xffffffffu, (dec & kStop) != 0u);
     if (stops) n = j0 + __ffs(stops) - 1;
-    flags |= __reduce_or_sync(0xffffffffu, j <= n ? fl : 0u);
+    if (warp == 0 || warp == kWarps - 1) flags |= __reduce_or_sync(0xffffffffu, j0 + lane <= n ? dec & ~kStop : 0u);
   }
-  if (rank == 0 && threadIdx.x == 0) {
+  if (rank == 0 && threadIdx.x == (kWarps - 1) * 32) {   // (the first warp goes on to the token)
     p.accept_len[b] = n;
     if (p.fallback == HOLA_FALLBACK_GREEDY) {            // greedy: argmax p_n follows the accepted run; no draw
       p.next_tok[b] = min(max(sh_amax[n], 0), Vtok - 1);
@@ -2130,14 +2185,20 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
 
   // ---- this CTA's slice of row n: per-chunk residual mass
   const float logZ = sh_logZ[n];
-  const char* qbase = static_cast<const char*>((p.q_far && n >= p.q_far_from) ? p.q_far : p.q);
-  // (staged: the row as if the slice were the whole of it, entry v at row + v)
-  const float* lstaged = sl + static_cast<size_t>(n) * slice - c_first * kChunk;
-  const char* qstaged = n >= k ? sq : sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem;
-  const float* lrow = p.logits + static_cast<size_t>(row_first + n) * p.ldl;
-  const void* qrow = n >= k ? nullptr : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
+  const char* qbase = static_cast<const char*>(p.q);
+  const float* lrow;
+  const void* qrow;
+  if (kStaged) {                                         // (as if the slice were the whole row, entry v at row + v)
+    lrow = sl + static_cast<size_t>(n) * slice - c_first * kChunk;
+    qrow = n >= k ? sq : sq + static_cast<size_t>(n) * slice * q_elem - c_first * kChunk * q_elem;
+  } else {
+    if (p.q_far && n >= p.q_far_from) qbase = static_cast<const char*>(p.q_far);
+    lrow = p.logits + static_cast<size_t>(row_first + n) * p.ldl;
+    qrow = n >= k ? nullptr : static_cast<const void*>(qbase + (static_cast<size_t>(b) * k + n) * V * q_elem);
+  }
   const bool half = p.q_dtype == HOLA_Q_BF16;
-  if (staged && here > 0) wait_staged_rows(smem_u32(&sh_bar), p.status, kWaitLimitCycles);
+  if (!kSolo && S > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (kStaged && here > 0) wait_bulk(smem_u32(&sh_bar), p.status, kWaitLimitCycles);
   // Several CTAs per SM and short slices (up to 8192 entries): a slice into the L2 by two bulk requests instead of by the loads
   // alone.  us, V = 32000, H = 512, 384 rows 33.2 -> 32.5, 240 rows 25.3 -> 24.7; V = 128256 (16032 entries) no gain.  With a CTA
   // per SM the loads are all out at once, and the code alone costs 0.2 us, hence a kernel without it.
@@ -2149,7 +2210,6 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
       if (q1 > qa) bulk_prefetch_l2(reinterpret_cast<const void*>(qa), static_cast<unsigned>(q1 - qa));
     }
   }
-  const int per_lane = (mine + 31) / 32;
   bool residual = n < k;
 
   // Vocabulary-parallel draw: every rank holds every rank's two masses of row n, so all of them agree on which mass
@@ -2169,7 +2229,7 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
     double total = 0.0;
     for (int r = 0; r < p.shard_world; ++r) total += mass[r * rs + idx];
     unsigned uflags = 0;
-    const double target = static_cast<double>(clamp_uniform(sh_u[k], uflags)) * total;
+    const double target = static_cast<double>(clamp_uniform(sh_uk, uflags)) * total;
     int owner = -1, last_mass = 0;
     double before = 0.0, cum = 0.0;
     for (int r = 0; r < p.shard_world; ++r) {
@@ -2188,51 +2248,38 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
   }
 
   for (int attempt = 0; attempt < 2; ++attempt) {
-    if (staged) {
-      if (half) sum_chunks<kVec, true, kWarps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
-      else sum_chunks<kVec, false, kWarps>(lstaged, qstaged, residual, c_first, mine, V, logZ, csum, warp, lane);
+    double mass = 0.0;
+    for (int c = warp; c < mine; c += kWarps * kK3Unroll) {
+      const int len = mine - c;                          // (a warp's chunks are kWarps apart)
+      mass += half ? sum_step<kVec, true, kWarps>(lrow, qrow, residual, c_first + c, len, V, logZ, csum + c, lane)
+                   : sum_step<kVec, false, kWarps>(lrow, qrow, residual, c_first + c, len, V, logZ, csum + c, lane);
+    }
+    mass += __shfl_xor_sync(0xffffffffu, mass, 8);
+    mass += __shfl_xor_sync(0xffffffffu, mass, 16);
+    if (kSolo || S == 1) {
+      if (lane == 0) sh_tot[attempt][warp] = mass;
     } else {
-      if (half) sum_chunks<kVec, true, kWarps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
-      else sum_chunks<kVec, false, kWarps>(lrow, qrow, residual, c_first, mine, V, logZ, csum, warp, lane);
+      // To all CTAs, counted on a barrier of theirs: half the way of stores and a cluster barrier behind them.
+      if (lane < S)
+        store_async(map_to_cta(smem_u32(&sh_tot[attempt][rank * kWarps + warp]), lane), mass,
+                    map_to_cta(smem_u32(&sh_all[attempt]), lane));
+      if (warp == 0) wait_bulk(smem_u32(&sh_all[attempt]), p.status, kWaitLimitCycles);
     }
-    __syncthreads();
-    // warp 0: scan of the slice; lane L owns chunks [lo, hi)
-    double tot = 0.0, incl = 0.0;
-    const int lo = lane * per_lane, hi = min(mine, lo + per_lane);
-    if (warp == 0) {
-      for (int c = lo; c < hi; ++c) tot += csum[c];
-      incl = tot;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      const double slice_total = __shfl_sync(0xffffffffu, incl, 31);
-      if (kSolo) {
-        if (lane == 0) sh_tot[attempt][0] = slice_total;
-      } else if (lane < S) {
-        *cluster.map_shared_rank(&sh_tot[attempt][rank], lane) = slice_total;
-      }
-    }
-    if (kSolo) __syncthreads();
-    else cluster.sync();
-    // every warp of every CTA: total mass and the slice that holds u * R (identical arithmetic everywhere); lane r has slice r
-    const double slice_mass = lane < S ? sh_tot[attempt][lane] : 0.0;
-    double slice_incl = slice_mass;
-    if (!kSolo) {
-#pragma unroll
-      for (int off = 1; off < 8; off <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, slice_incl, off);
-        if (lane >= off) slice_incl += o;
-      }
-    }
-    const double R = __shfl_sync(0xffffffffu, slice_incl, kSolo ? 0 : 7);
+    __syncthreads();                                     // (and this CTA's chunk masses, for the first warp)
+    // Lane i has masses 2 i and 2 i + 1.  Every warp learns whether there is any; the first one of every CTA goes on.
+    double2 two = make_double2(0.0, 0.0);
+    if (2 * lane < (kSolo ? kWarps : S * kWarps)) two = reinterpret_cast<const double2*>(sh_tot[attempt])[lane];
+    const bool any = __any_sync(0xffffffffu, two.x > 0.0 || two.y > 0.0) &&
+                     !__any_sync(0xffffffffu, two.x != two.x || two.y != two.y);
     if (shard && p.phase == 3) {
       // the shard's masses of row n: of the residual, then (second pass, q taken as 0) of p itself
-      if (rank == 0 && threadIdx.x == 0) {
-        p.mass_out[b * 2 + attempt] = R;
-        if (!residual && attempt == 0) p.mass_out[b * 2 + 1] = R;          // bonus position: both are the mass of p
-        if (attempt == 1 || !residual) report_flags(p, b, flags);
+      if (rank == 0 && warp == 0) {
+        const double R = warp_sum_f64(two.x + two.y);
+        if (lane == 0) {
+          p.mass_out[b * 2 + attempt] = R;
+          if (!residual && attempt == 0) p.mass_out[b * 2 + 1] = R;        // bonus position: both are the mass of p
+          if (attempt == 1 || !residual) report_flags(p, b, flags);
+        }
       }
       if (residual) {
         residual = false;
@@ -2241,81 +2288,109 @@ __global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 :
       }
       return;
     }
-    if (!(R > 0.0) && residual && !shard) {              // p <= q everywhere: draw from p instead
+    if (!any && residual && !shard) {                    // p <= q everywhere: draw from p instead
       residual = false;
       flags |= HOLA_FLAG_R_ZERO;
       __syncthreads();
       continue;
     }
-    const float uk = clamp_uniform(sh_u[k], flags);
-    const double target = shard ? shard_target : static_cast<double>(uk) * R;
-    const unsigned slice_over = __ballot_sync(0xffffffffu, lane < S && slice_incl > target);
-    const unsigned slice_has = __ballot_sync(0xffffffffu, slice_mass > 0.0);
-    const bool take_last_slice = slice_over == 0u;       // rounding left the running sum a hair below u*R
-    const int rstar = slice_over ? __ffs(slice_over) - 1 : (slice_has ? 31 - __clz(slice_has) : 0);
-    const double before_slice = __shfl_sync(0xffffffffu, slice_incl - slice_mass, rstar);
-    bool take_last = take_last_slice;
-    if (rank == rstar && warp == 0) {
-      const unsigned over = __ballot_sync(0xffffffffu, before_slice + incl > target);
-      const unsigned has_mass = __ballot_sync(0xffffffffu, tot > 0.0);
-      int L;
-      if (over && !take_last) L = __ffs(over) - 1;
-      else { L = has_mass ? 31 - __clz(has_mass) : 0; take_last = true; }
-      int cstar = -1;
-      double before = 0.0;
-      if (lane == L) {
-        double cum = before_slice + (incl - tot);
-        int last_pos = lo;
-        for (int c = lo; c < hi; ++c) {
-          if (csum[c] > 0.0) last_pos = c;
-          if (!take_last && cum + csum[c] > target) { cstar = c; before = cum; break; }
-          cum += csum[c];
-        }
-        if (cstar < 0) { cstar = last_pos; before = cum - csum[last_pos]; take_last = true; }
-      }
-      cstar = __shfl_sync(0xffffffffu, cstar, L);
-      before = __shfl_sync(0xffffffffu, before, L);
-      take_last = __shfl_sync(0xffffffffu, take_last ? 1 : 0, L) != 0;
-      // inside the chunk: lane prefix, then the lane's four entries in ascending order
-      const int base = (c_first + cstar) * kChunk + lane * 4;
-      float l4[4], q4[4], r4[4];
-      if (staged) {
-        if (half) fetch4<kVec, true>(lstaged, qstaged, residual, base, V, l4, q4);
-        else fetch4<kVec, false>(lstaged, qstaged, residual, base, V, l4, q4);
-      } else {
-        if (half) fetch4<kVec, true>(lrow, qrow, residual, base, V, l4, q4);
-        else fetch4<kVec, false>(lrow, qrow, residual, base, V, l4, q4);
-      }
-      resid4(l4, q4, logZ, r4);
-      const double mine4 = ((static_cast<double>(r4[0]) + r4[1]) + r4[2]) + r4[3];
-      double lincl = mine4;
+    if (warp != 0) return;
+    const float uk = clamp_uniform(sh_uk, flags);
+    double target = shard_target, before = 0.0;
+    bool take_last = false;                              // rounding left the running sum a hair below u*R
+    if (!kSolo && S > 1) {
+      // the slice that holds u * R, with identical arithmetic in every CTA: lanes 4 r .. 4 r + 3 have slice r
+      constexpr int kPer = kK3Threads / 64;
+      double sum = two.x + two.y;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const double o = __shfl_up_sync(0xffffffffu, lincl, off);
-        if (lane >= off) lincl += o;
+      for (int off = 1; off < kPer; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      double incl = sum;
+      for (int off = kPer; off < kPer * S; off <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += o;
       }
-      double cum = before + (lincl - mine4);
-      int found = -1, last4 = -1;
+      const double R = __shfl_sync(0xffffffffu, incl, kPer * S - 1);
+      if (!shard) target = static_cast<double>(uk) * R;
+      const unsigned over = __ballot_sync(0xffffffffu, sum > 0.0 && incl > target);
+      const unsigned has_mass = __ballot_sync(0xffffffffu, sum > 0.0);
+      take_last = over == 0u;
+      const int at = over ? __ffs(over) - 1 : (has_mass ? 31 - __clz(has_mass) : 0);
+      before = __shfl_sync(0xffffffffu, incl - sum, at);
+      if (at / kPer != rank) return;
+    }
+    // the chunk: lane i has chunks [a, z) of the slice
+    const int per_lane = (cpc + 31) / 32, a = min(mine, lane * per_lane), z = min(mine, a + per_lane);
+    constexpr int kHeld = 4;                             // (that few stay in registers)
+    double m[kHeld], tot = 0.0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        cum += r4[i];
-        if (r4[i] > 0.f) last4 = i;
+    for (int i = 0; i < kHeld; ++i) {
+      m[i] = a + i < z ? csum[a + i] : 0.0;
+      tot += m[i];
+    }
+    for (int c = a + kHeld; c < z; ++c) tot += csum[c];
+    double upto = tot;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const double o = __shfl_up_sync(0xffffffffu, upto, off);
+      if (lane >= off) upto += o;
+    }
+    if ((kSolo || S == 1) && !shard) target = static_cast<double>(uk) * __shfl_sync(0xffffffffu, upto, 31);
+    const unsigned lane_over = __ballot_sync(0xffffffffu, tot > 0.0 && before + upto > target);
+    const unsigned lane_mass = __ballot_sync(0xffffffffu, tot > 0.0);
+    take_last = take_last || lane_over == 0u;
+    const int from = !take_last ? __ffs(lane_over) - 1 : (lane_mass ? 31 - __clz(lane_mass) : 0);
+    int cstar = -1, last = a;
+    double cum = before + (upto - tot), start = cum;
+    auto look = [&](int c, double mc) {                  // (every lane in its own chunks; that of lane `from` counts)
+      if (mc > 0.0) {
+        last = c;
+        if (cstar < 0 && !take_last && cum + mc > target) { cstar = c; start = cum; }
+      }
+      cum += mc;
+    };
+#pragma unroll
+    for (int i = 0; i < kHeld; ++i) look(a + i, m[i]);
+    for (int c = a + kHeld; c < z; ++c) look(c, csum[c]);
+    if (cstar < 0) { cstar = last; take_last = true; }
+    cstar = __shfl_sync(0xffffffffu, cstar, from);
+    before = __shfl_sync(0xffffffffu, start, from);
+    take_last = __shfl_sync(0xffffffffu, take_last ? 1 : 0, from) != 0;
+    // inside the chunk: lane prefix, then the lane's four entries in ascending order
+    const int base = (c_first + cstar) * kChunk + lane * 4;
+    float l4[4], q4[4], r4[4];
+    if (half) fetch4<kVec, true>(lrow, qrow, residual, base, V, l4, q4);
+    else fetch4<kVec, false>(lrow, qrow, residual, base, V, l4, q4);
+    resid4(l4, q4, logZ, r4);
+    const double mine4 = ((static_cast<double>(r4[0]) + r4[1]) + r4[2]) + r4[3];
+    double lincl = mine4;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const double o = __shfl_up_sync(0xffffffffu, lincl, off);
+      if (lane >= off) lincl += o;
+    }
+    cum = before + (lincl - mine4);
+    int found = -1, last4 = -1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      cum += r4[i];
+      if (r4[i] > 0.f) {
+        last4 = i;
         if (found < 0 && !take_last && cum > target) found = i;
       }
-      const unsigned hit = __ballot_sync(0xffffffffu, found >= 0);
-      const unsigned mass = __ballot_sync(0xffffffffu, last4 >= 0);
-      int src, idx;
-      if (hit) { src = __ffs(hit) - 1; idx = found; }
-      else { src = mass ? 31 - __clz(mass) : 0; idx = last4 < 0 ? 0 : last4; }
-      idx = __shfl_sync(0xffffffffu, idx, src);
-      if (lane == 0) {
-        int tokn = (c_first + cstar) * kChunk + src * 4 + idx;
-        if (tokn >= V) tokn = V - 1;
-        p.next_tok[b] = tokn + (shard ? p.v_offset : 0);
-        report_flags(p, b, flags);
-      }
     }
-    break;
+    const unsigned hit = __ballot_sync(0xffffffffu, found >= 0);
+    const unsigned mass4 = __ballot_sync(0xffffffffu, last4 >= 0);
+    int src, idx;
+    if (hit) { src = __ffs(hit) - 1; idx = found; }
+    else { src = mass4 ? 31 - __clz(mass4) : 0; idx = last4 < 0 ? 0 : last4; }
+    idx = __shfl_sync(0xffffffffu, idx, src);
+    if (lane == 0) {
+      int tokn = (c_first + cstar) * kChunk + src * 4 + idx;
+      if (tokn >= V) tokn = V - 1;
+      p.next_tok[b] = tokn + (shard ? p.v_offset : 0);
+      report_flags(p, b, flags);
+    }
+    return;
   }
 }
 
@@ -3397,7 +3472,6 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   }
   const bool vec = rows_of_pieces(a, logits, ldl) && aligned16(q_far);     // (rows read in place are the caller's own)
   const SampleForm f = sample_form(ctx->num_sms, a->B, a->k, a->V, a->q_dtype, a->fallback, vec, phase, sh != nullptr, q_far != nullptr);
-  kp.staged = f.staged;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(a->B * f.S));
   cfg.blockDim = dim3(f.solo ? kSoloThreads : kK3Threads);
@@ -3422,6 +3496,7 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
   }
   const cudaError_t e = f.solo ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, true>, kp)
                                      : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, true>, kp))
+                        : f.staged ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, false, true>, kp)
                         : ask ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, true>, kp)
                         : vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false>, kp)
                               : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false>, kp);
@@ -3476,7 +3551,7 @@ cudaError_t configure_kernels() {
   for (const void* k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(accept_sample_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kK3MaxDynSmem);
+    e = cudaFuncSetAttribute(accept_sample_kernel<true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kK3MaxDynSmem);
   return e;
 }
 
