@@ -22,6 +22,7 @@
 //   quantize_rows_kernel        the Lo-Bi quantiser on W_lm ahead of time: rows at 8 bits, at 4 bits (codes in [-7, 7], one
 //       shared exponent per sub-block of 128 channels) or in groups of mixed width, one launch for the whole head.
 //   quantize_hidden_kernel      the hidden rows of a call as one or two 8-bit planes.
+//   align_hidden_kernel         the hidden rows of a call once more, on 128-byte lines.
 //   bounded_wait_selftest_kernel, staged_wait_selftest_kernel  waits that are made to run out, to exercise the give-up paths
 //       without breaking anything.
 //   draft_entropy_kernel        H(q_j) of the draft rows, for the gate on the draft distribution.
@@ -2750,6 +2751,25 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
   }
 }
 
+// bf16 hidden rows that start on no 128-byte line, once more with a pitch of whole lines (aligns_hidden): a CTA per row, up to
+// four 16-byte loads per thread in flight; latency bounds it (some 2.4 us of a call).
+constexpr int kAlignThreads = 256;
+__global__ void __launch_bounds__(kAlignThreads) align_hidden_kernel(const uint4* X, int pieces, int pitch, uint4* out) {
+  grid_dependency_wait();
+  grid_dependency_release();                             // (as the quantiser does: the GEMM kernel is put in place meanwhile)
+  const uint4* src = X + static_cast<size_t>(blockIdx.x) * pieces;
+  uint4* dst = out + static_cast<size_t>(blockIdx.x) * pitch;
+  for (int p0 = threadIdx.x; p0 < pieces; p0 += 4 * kAlignThreads) {
+    uint4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (p0 + i * kAlignThreads < pieces) x[i] = src[p0 + i * kAlignThreads];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (p0 + i * kAlignThreads < pieces) dst[p0 + i * kAlignThreads] = x[i];
+  }
+}
+
 // ------------------------------------------------------------------------------------------------ draft entropy
 // Grid (rows, kHqSlices): CTA (r, s) leaves slice s of row r in part[r][s]; the accept/sample kernel adds the slices in
 // index order.  Where the GEMM kernel does not make the pass itself: on a side stream under it, hence CTAs of 32 registers
@@ -2807,7 +2827,7 @@ struct hola_ctx {
   unsigned* status;         // [1]
   unsigned* pace;           // [2][kMaxPaceGroups] counters of the groups of pairs when all passes share a launch
   double* hq;               // [max_rows][kHqSlices] slice sums of q ln q over the draft rows
-  signed char* hid8;        // [rows][hidden_pitch8] int8 hidden rows (8-bit activation modes)
+  signed char* hid8;        // [rows][hidden_pitch8] int8 hidden rows (8-bit activation modes), or bf16 rows (aligns_hidden)
   float* hid_scale;         // [max_rows]
   // staging for hola_verify_host
   void* st_hidden; int* st_tok; void* st_q; float* st_u;
@@ -2886,7 +2906,8 @@ WsLayout ws_layout(int maxB, int maxK, int H, int V, int num_sms) {
   w.status = take(4);
   w.pace = take(8 * kMaxPaceGroups);
   w.hq = take(rows * kHqSlices * 8);
-  w.hid8 = take(2 * align_up(rows, 32) * hidden_pitch8(H));           // one or two 8-bit planes of the hidden rows
+  w.hid8 = take(2 * align_up(rows, 32) * hidden_pitch8(H));           // one or two 8-bit planes of the hidden rows, or those
+                                                                      // rows as they are, on whole lines
   w.hid_scale = take(2 * rows * 4);                                   // their scales (second plane after the first)
   w.st_hidden = take(rows * H * 2);
   // the three small per-step inputs side by side: hola_verify_host sends them as one copy
@@ -3198,6 +3219,19 @@ SampleForm sample_form(int num_sms, int B, int k, int V, int q_dtype, int fallba
   return f;
 }
 
+// bf16 rows that start on no 128-byte line make every fetch of a K block of hidden rows two lines instead of one, out of the L2 and
+// for every tile.  From 96 rows on and where rows x K blocks x tiles per pair reach 8000 a copy of the rows on whole lines pays for
+// itself.  us, as they are -> copied: 96 rows, H = 4104, V = 60000 124 -> 109, V = 128256 239 -> 216; 250 rows, H = 4104, V = 30000
+// 96 -> 84.5; 320, V = 60000 213 -> 197; 150, H = 1032, V = 60000 53.8 -> 50.4; 128 47.5 -> 45.8; 384, H = 4104, V = 16000 67 -> 64.8;
+// below the line 92 rows, H = 1032, V = 50003 35.6 -> 37.3; 96, V = 32000 24.8 -> 26.4; 384, H = 520, V = 8000 18.7 -> 22.3.  (With
+// codes expanded on chip: no gain, 160 rows, H = 2064, V = 60000 63.5 -> 65.)
+bool aligns_hidden(const hola_ctx* ctx, const hola_verify_args* a, const Plan& pl) {
+  if (a->w_dtype != HOLA_W_BF16 || a->H % kBlockK == 0 || !ctx->hid8) return false;
+  const int op_rows = pl.n_sub * pl.N, pairs = pl.grid / (2 * (pl.fused ? pl.passes : 1));
+  const double tiles = (pl.n_ptiles + pairs - 1) / pairs;
+  return op_rows >= 96 && tiles * pl.n_kblocks * op_rows >= 8000.0;
+}
+
 // Where the logits of a verify step that does not hand them out go.  The greedy rule reads none (the arg-max travels with the
 // statistics), so none are stored then.  8-bit head and hidden rows, 192 rows, V = 128256 (98 MB of logits beside 525 MB of
 // codes): 137 -> 121 us.
@@ -3223,7 +3257,10 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   const void* w_main = mixed ? (mx->rows8 > 0 ? mx->W8 : (mx->rows4 > 0 ? mx->W4 : mx->W16)) : a->W_lm;
   hola_status s;
   // 8-bit activations: the hidden operand is the context's own buffer of 8-bit planes, filled per call below
-  const void* hid_src = (two || i8) ? static_cast<const void*>(ctx->hid8) : a->hidden;
+  // (as is one that is brought onto whole lines)
+  const bool aligned = aligns_hidden(ctx, a, pl);
+  const void* hid_src = (two || i8 || aligned) ? static_cast<const void*>(ctx->hid8) : a->hidden;
+  const int hid_pitch = (two || i8) ? hidden_pitch8(a->H) : aligned ? round_up(2 * a->H, 128) : 0;
   if ((two || i8) && !ctx->hid8) return HOLA_ERR_INVALID_ARG;   // (the entry point without a context has no room for it)
   if (two || i8) {
     // the same per-row quantiser as for W_lm (one plane), or the two-plane form in blocks of 32 rows
@@ -3240,6 +3277,17 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
                            ctx->hid_scale + ctx->max_rows);
     if (qe != cudaSuccess) { set_error(ctx, "launch of the hidden-row quantiser", qe); return HOLA_ERR_CUDA; }
   }
+  if (aligned) {
+    cudaLaunchConfig_t ac = {};
+    ac.gridDim = dim3(static_cast<unsigned>(M)); ac.blockDim = dim3(kAlignThreads); ac.stream = stream;
+    cudaLaunchAttribute aa[1];
+    aa[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    aa[0].val.programmaticStreamSerializationAllowed = 1;
+    ac.attrs = aa; ac.numAttrs = 1;
+    const cudaError_t ae = cudaLaunchKernelEx(&ac, align_hidden_kernel, static_cast<const uint4*>(a->hidden), a->H / 8, hid_pitch / 16,
+                                              reinterpret_cast<uint4*>(ctx->hid8));
+    if (ae != cudaSuccess) { set_error(ctx, "launch align_hidden_kernel", ae); return HOLA_ERR_CUDA; }
+  }
   MapEntry* me = nullptr;
   for (int i = 0; i < kMapCache; ++i) {
     MapEntry& c = ctx->maps[i];
@@ -3254,13 +3302,13 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
     me->logits = nullptr;
     if (two)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(2 * round_up(M, 32)), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hidden_pitch8(a->H));
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hid_pitch);
     else if (i8)
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hidden_pitch8(a->H));
+                     static_cast<uint32_t>(pl.N / 2), true, false, pl.kpb, hid_pitch);
     else
       s = encode_map(ctx, &me->th, hid_src, static_cast<uint64_t>(M), static_cast<uint64_t>(a->H),
-                     static_cast<uint32_t>(pl.N / 2), false, false, pl.kpb);
+                     static_cast<uint32_t>(pl.N / 2), false, false, pl.kpb, hid_pitch);
     if (s != HOLA_OK) return s;
     const uint32_t trows = static_cast<uint32_t>(pl.tile_rows);
     if (!mixed) {
@@ -3272,8 +3320,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
         s = encode_map(ctx, &me->tw4, a->W_lm, static_cast<uint64_t>(a->V), static_cast<uint64_t>(a->H), trows, i8);
         if (s != HOLA_OK) return s;
         s = encode_map(ctx, &me->tw16, hid_src, static_cast<uint64_t>(two ? 2 * round_up(M, 32) : M),
-                       static_cast<uint64_t>(a->H), static_cast<uint32_t>(pl.N / 2), i8, false, 1,
-                       i8 ? hidden_pitch8(a->H) : 0);
+                       static_cast<uint64_t>(a->H), static_cast<uint32_t>(pl.N / 2), i8, false, 1, hid_pitch);
         if (s != HOLA_OK) return s;
       }
       me->W4 = nullptr; me->W16 = nullptr;
@@ -3307,7 +3354,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   }
   // Rotating units: the logits buffer, where its rows are whole 16-byte pieces; boxes of 16 rows x 32 entries, swizzled like
   // the staging buffers.
-  const bool wide_logits = !pl.rot && pl.N >= 128 && ldl % 4 == 0 && aligned16(logits) && a->V % 4 == 0;
+  const bool wide_logits = !pl.rot && pl.N >= 128 && ldl % 4 == 0 && aligned16(logits);      // (a row's last piece: within ldl)
   const bool bulk_logits = pl.rot && logits && ldl % 4 == 0 && aligned16(logits);
   if (bulk_logits && (me->logits != logits || me->ldl != ldl)) {
     me->logits = nullptr;

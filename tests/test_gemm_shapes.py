@@ -82,3 +82,22 @@ def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(bin
         for _ in range(3):
             out = ctx.hola_lm_head_entropy(hidden, W, want_logits=True, w_scale=scale, a8=MODES[mode])
             assert torch.equal(out.logits.reshape(-1, V), want)
+
+
+# Rows that start on no 128-byte line are copied onto lines where there is enough to do: a partial last K block and several per ring
+# slot, four tiles per pair, several passes, rotating units, two MMAs per K step; the last one stays as it is.  An odd vocabulary:
+# 16-byte stores of logits end within the row's pitch.
+@pytest.mark.parametrize("B,k,H,V", [(24, 3, 5512, 1000), (32, 3, 1032, 60000), (100, 4, 2056, 700), (97, 2, 2008, 20003), (86, 5, 1544, 19001), (24, 3, 5128, 1000)])
+def test_rows_copied_onto_lines(binding, B, k, H, V):
+    check_lm_head(binding, "bf16", B, k, H, V)
+
+
+@pytest.mark.parametrize("B,k,H,V", [(33, 4, 320, 5001), (50, 2, 136, 9002), (64, 2, 64, 20003)])
+def test_statistics_of_an_odd_vocabulary_without_logits(binding, B, k, H, V):
+    hidden, W = exact_operands(B, k, H, V, 5)
+    want = hidden.double().reshape(-1, H) @ W.double().t()
+    with binding.HolaVerify(B, k, H, V) as ctx:
+        out = ctx.hola_lm_head_entropy(hidden, W)
+        torch.cuda.synchronize()
+    assert int(out.status.item()) == 0
+    assert (out.logZ.reshape(-1).double() - torch.logsumexp(want, 1)).abs().max() < 2e-5
