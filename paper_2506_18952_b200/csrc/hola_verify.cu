@@ -95,6 +95,7 @@ constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s of SM clock 
 
 constexpr int kK3Threads = 256;
 constexpr int kSoloThreads = 1024;               // its form with one CTA per sequence
+constexpr int kFewEntries = 8192;                // vocabulary up to which half of them do
 constexpr int kK3MaxPerSm = 4;                   // CTAs of the accept/sample kernel an SM holds (register budget: 64 per thread)
 constexpr int kChunk = 128;                      // vocabulary entries per warp step (32 lanes x 4)
 constexpr int kMaxChunks = 4096;                 // => V <= 524288
@@ -2028,12 +2029,18 @@ __device__ __forceinline__ unsigned decide(const K3Params& p, int x, int Vtok, f
 // The chunks of a step alternate between the warps: side by side in one warp (so that a warp's mass is that of a run of the
 // vocabulary, and one scan less is needed) rows that start on no line are fetched twice, 60 sequences, V = 50003 33.2 -> 36.9.
 // kAsk: the slice of row n is asked into the L2 as soon as n is known.
-// kSolo: one CTA of 1024 threads instead of the cluster (see sample_solo).
+// kSoloWarps: one CTA of 1024 threads instead of the cluster (see sample_solo).  All 32 warps of it take part or, for up to
+// kFewEntries entries and sequences for half of the SMs, the first 16: the others leave at once, and the instructions of the rest
+// find more room.  us, 32 -> 16 warps: V = 2000, 16 sequences 10.5 -> 10.2; V = 3000, 1 9.7 -> 9.5; V = 5000, 2 / 32 10.2 -> 10.0,
+// 12.3 -> 12.1; V = 8000, 1 / 64 / 140 11.0 -> 10.95, 13.3 -> 13.1, 18.45 -> 18.75; V = 8191, 5 12.4 -> 12.2; V = 11000, 16 13.2 -> 13.6;
+// V = 16000, 64 17.7 -> 18.8.
 // kStaged: this CTA's slice of ALL k + 1 rows is brought into shared memory while the statistics are merged and the accept test
 // is made, instead of row n afterwards.
-template <bool kVec, bool kAsk, bool kSolo = false, bool kStaged = false>
-__global__ void __launch_bounds__(kSolo ? kSoloThreads : kK3Threads, kSolo ? 1 : kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
-  constexpr int kThreads = kSolo ? kSoloThreads : kK3Threads, kWarps = kThreads / 32;
+template <bool kVec, bool kAsk, int kSoloWarps = 0, bool kStaged = false>
+__global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloWarps ? 1 : kK3MaxPerSm) accept_sample_kernel(const K3Params p) {
+  constexpr bool kSolo = kSoloWarps > 0;
+  constexpr int kWarps = kSolo ? kSoloWarps : kK3Threads / 32;
+  if (kSolo && threadIdx.x >= kWarps * 32) return;
   extern __shared__ __align__(16) double csum[];                       // per-chunk residual mass of this CTA's slice
   __shared__ __align__(16) double sh_tot[2][kSolo ? kWarps : 8 * kWarps];      // masses of all warps' runs, per attempt
   __shared__ float sh_logZ[kMaxK1], sh_uk;
@@ -3541,9 +3548,12 @@ hola_status run_accept_sample(hola_ctx* ctx, const hola_verify_args* a, const fl
     attr[0] = attr[1];                                   // (no cluster)
     cfg.numAttrs = 1;
   }
-  const cudaError_t e = f.solo ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, true>, kp)
-                                     : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, true>, kp))
-                        : f.staged ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, false, true>, kp)
+  const cudaError_t e = f.solo && a->V <= kFewEntries && 2 * a->B <= ctx->num_sms
+                            ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, 16>, kp)
+                                   : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, 16>, kp))
+                        : f.solo ? (vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, 32>, kp)
+                                        : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false, 32>, kp))
+                        : f.staged ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false, 0, true>, kp)
                         : ask ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, true>, kp)
                         : vec ? cudaLaunchKernelEx(&cfg, accept_sample_kernel<true, false>, kp)
                               : cudaLaunchKernelEx(&cfg, accept_sample_kernel<false, false>, kp);
@@ -3598,7 +3608,7 @@ cudaError_t configure_kernels() {
   for (const void* k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(accept_sample_kernel<true, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kK3MaxDynSmem);
+    e = cudaFuncSetAttribute(accept_sample_kernel<true, false, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kK3MaxDynSmem);
   return e;
 }
 

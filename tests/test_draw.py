@@ -19,7 +19,7 @@ def binding():
 # rows that start on no 16-byte boundary; more positions than warps.
 @pytest.mark.parametrize("B,k,V", [
     (3, 2, 1), (3, 2, 5), (2, 3, 127), (2, 3, 128), (2, 3, 129), (1, 4, 1000), (5, 4, 1921), (40, 2, 3969), (4, 4, 3970), (3, 1, 8064),
-    (3, 1, 8192), (9, 3, 8193), (6, 9, 16384), (6, 4, 16388), (2, 20, 20001), (3, 4, 32768), (3, 4, 32896), (30, 2, 33025), (300, 1, 20000),
+    (3, 1, 8192), (9, 3, 8193), (6, 9, 16384), (80, 2, 8000), (80, 40, 2061), (2, 20, 6000), (6, 4, 16388), (2, 20, 20001), (3, 4, 32768), (3, 4, 32896), (30, 2, 33025), (300, 1, 20000),
     (700, 0, 17000), (600, 1, 33000), (2, 2, 140000)])
 @pytest.mark.parametrize("q_dtype", [torch.float32, torch.bfloat16])
 def test_the_token_is_where_the_cumulative_mass_passes_the_uniform(binding, B, k, V, q_dtype):
