@@ -356,6 +356,12 @@ hola_status hola_selftest_bounded_wait(hola_ctx* ctx, long long limit_cycles, ui
  * HOLA_FLAG_TIMEOUT (what the first CTA reported).  counters is uint32 [3], zeroed by the call. */
 hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
                                       void* cuda_stream);
+/* And for its wait on the sums that the CTAs of a cluster send one another, which ends well there, the second CTA sending behind
+ * its own wait: here the first one gives up on them long before that, and may leave only when they have reached it all the
+ * same.  As above with counters[1] = 96 (64 + the warp that waits for the sums) and counters[3] = 2, the CTAs that hold
+ * both sums when they leave.  counters is uint32 [4], zeroed by the call. */
+hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                    void* cuda_stream);
 
 const char* hola_strerror(hola_status s);
 /* Text of the last CUDA error seen by this context (empty string if none). */

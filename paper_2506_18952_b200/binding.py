@@ -29,7 +29,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -130,7 +130,7 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_profile_begin.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.hola_set_option.restype = ctypes.c_int
     lib.hola_set_option.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
-    for name in ("hola_selftest_bounded_wait", "hola_selftest_staged_wait"):
+    for name in ("hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait"):
         fn = getattr(lib, name)
         fn.restype = ctypes.c_int
         fn.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
@@ -408,6 +408,16 @@ class HolaVerify:
         st = self.lib.hola_selftest_staged_wait(self._ctx, int(limit_cycles), _dptr(status), _dptr(counters),
                                                 _stream_ptr(stream))
         _check(self.lib, self._ctx, st, "hola_selftest_staged_wait")
+        (torch.cuda.current_stream() if stream is None else stream).synchronize()
+        return (int(status.item()), *counters.tolist())
+
+    def hola_selftest_mass_wait(self, limit_cycles: int = 100000, stream=None) -> tuple[int, int, int, int, int]:
+        """Runs the self-test of the wait on the other CTAs' sums; returns (status word, threads that reached the end, waits
+        that gave up, flags that the first CTA reported, CTAs that all sums had reached) after synchronising the stream."""
+        status = torch.zeros(1, dtype=torch.int32, device=self._dev)
+        counters = torch.zeros(4, dtype=torch.int32, device=self._dev)
+        st = self.lib.hola_selftest_mass_wait(self._ctx, int(limit_cycles), _dptr(status), _dptr(counters), _stream_ptr(stream))
+        _check(self.lib, self._ctx, st, "hola_selftest_mass_wait")
         (torch.cuda.current_stream() if stream is None else stream).synchronize()
         return (int(status.item()), *counters.tolist())
 

@@ -1961,8 +1961,8 @@ __device__ __forceinline__ float clamp_uniform(float u, unsigned& flags) {
 
 // Waits for what is counted on a barrier of this CTA: its staged rows, or the masses of all warps of the cluster.  When the time is
 // up the status word is told at once: the CTA that draws the token, and reports, may be another one of the cluster, whose rows did
-// land (it looks at the status word behind the exchange of masses).  The copies then have as long again before the CTA goes on (and sooner or later leaves
-// the memory they write to).  False: gave up.
+// land (it looks at the status word behind the exchange of masses).  What is waited for then has as long again before the CTA goes
+// on (and sooner or later leaves the memory that copies write to).  False: gave up, nothing arrived in that time either.
 __device__ __forceinline__ bool wait_bulk(uint32_t bar, unsigned* status, long long limit_cycles) {
   const long long t0 = clock64();
   bool late = false;
@@ -1972,26 +1972,59 @@ __device__ __forceinline__ bool wait_bulk(uint32_t bar, unsigned* status, long l
       late = true;
       if (status) atomicOr(status, HOLA_FLAG_TIMEOUT);
     }
-    if (waited > 2 * limit_cycles) break;
+    if (waited > 2 * limit_cycles) return false;
   }
-  return !late;
+  return true;
 }
 
-// The way that wait gives up, in miniature: a cluster of two CTAs, of which the second waits on a barrier that nothing ever
-// arrives on.  The first, whose barrier is complete, must find the time-out in the status word when it reports.
+// The exchange of masses: each CTA of the cluster has room for the masses of all, and a barrier that counts their bytes.
+// A warp's mass to every CTA, lane i to CTA i (`lane` < cluster size only).
+__device__ __forceinline__ void send_mass(double* slot, uint64_t* all, double mass, int lane) {
+  store_async(map_to_cta(smem_u32(slot), lane), mass, map_to_cta(smem_u32(all), lane));
+}
+// The wait for them, twice as long as that for staged rows: a CTA whose rows do not land sends what it has behind that wait.
+__device__ __forceinline__ bool wait_masses(uint64_t* all, unsigned* status, long long limit_cycles) {
+  return wait_bulk(smem_u32(all), status, 2 * limit_cycles);
+}
+// The way out for a CTA whose wait gave up (all of its threads).  The others may still be sending to it: it stays until each of
+// them has left (threads that have exited are not waited for) or has come here too, and until what they sent has landed.
+__device__ __forceinline__ void leave_behind_the_others() {
+  cluster_sync_all();
+  __nanosleep(200000);
+}
+
+// The ways those waits give up, in miniature: a cluster of two CTAs, of which the second waits for staged rows that nothing ever
+// brings and sends its mass behind that.  kEarly: the first, whose rows are there, gives up on the second one's mass long before,
+// and has to stay until it has landed; otherwise it gets it, and must find the time-out in the status word when it reports.
 // out[0] counts the threads that reached the end, out[1] the waits that gave up, out[2] is the word of flags that the first
-// CTA leaves.
+// CTA leaves, out[3] (kEarly) counts the CTAs in whose memory both masses have landed when they leave.
+template <bool kEarly>
 __global__ void __launch_bounds__(64, 1) staged_wait_selftest_kernel(long long limit_cycles, unsigned* status, unsigned* out) {
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar, all;
+  __shared__ double masses[2];
+  __shared__ int sh_gave_up;
   const uint32_t rank = cluster_cta_rank();
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&bar), 1);
+    mbar_init(smem_u32(&all), 1);
+    mbar_expect_tx(smem_u32(&all), 2 * 8u);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (rank == 0) mbar_arrive(smem_u32(&bar));
+    masses[0] = masses[1] = 0.0;
+    sh_gave_up = 0;
   }
   __syncthreads();
-  if (!wait_bulk(smem_u32(&bar), status, limit_cycles)) atomicAdd(out + 1, 1u);
   cluster_sync_all();
+  if (!wait_bulk(smem_u32(&bar), status, limit_cycles)) { sh_gave_up = 1; atomicAdd(out + 1, 1u); }
+  if (threadIdx.x < 2) send_mass(&masses[rank], &all, 1.0 + rank, threadIdx.x);
+  if (threadIdx.x < 32 && !wait_masses(&all, status, kEarly && rank == 0 ? limit_cycles / 16 : limit_cycles)) {
+    sh_gave_up = 1;
+    atomicAdd(out + 1, 1u);
+  }
+  __syncthreads();
+  if (sh_gave_up) leave_behind_the_others();
+  if (kEarly && threadIdx.x == 0 && *const_cast<volatile double*>(&masses[0]) == 1.0 && *const_cast<volatile double*>(&masses[1]) == 2.0)
+    atomicAdd(out + 3, 1u);
   if (rank == 0 && threadIdx.x == 0) {
     K3Params p;
     p.status = status; p.flags_out = out + 2;
@@ -2048,6 +2081,7 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
   __shared__ unsigned sh_dec[kMaxK1];                    // decide()'s results
   __shared__ __align__(8) uint64_t sh_bar;               // staged rows have landed
   __shared__ __align__(8) uint64_t sh_all[2];            // all runs' masses have arrived, per attempt
+  __shared__ int sh_gave_up;                             // a wait of this CTA ran out
 
   // The next kernel in the stream (normally the next call's GEMM kernel, which waits for this grid before it touches
   // memory) may be scheduled from now on: its launch and prologue then hide behind this kernel.
@@ -2091,6 +2125,7 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
     }
     asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
   }
+  if (!kSolo && threadIdx.x == 0) sh_gave_up = 0;
   const int nchunks = (V + kChunk - 1) / kChunk;
   const int cpc = kSolo ? nchunks : (nchunks + S - 1) >> (31 - __clz(S));      // chunks per CTA
   const int c_first = rank * cpc;
@@ -2206,7 +2241,8 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
   }
   const bool half = p.q_dtype == HOLA_Q_BF16;
   if (!kSolo && S > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-  if (kStaged && here > 0) wait_bulk(smem_u32(&sh_bar), p.status, kWaitLimitCycles);
+  // (rows that never land: their sums mean nothing, but the other CTAs wait for them)
+  if (kStaged && here > 0 && !wait_bulk(smem_u32(&sh_bar), p.status, kWaitLimitCycles)) sh_gave_up = 1;
   // Several CTAs per SM and short slices (up to 8192 entries): a slice into the L2 by two bulk requests instead of by the loads
   // alone.  us, V = 32000, H = 512, 384 rows 33.2 -> 32.5, 240 rows 25.3 -> 24.7; V = 128256 (16032 entries) no gain.  With a CTA
   // per SM the loads are all out at once, and the code alone costs 0.2 us, hence a kernel without it.
@@ -2268,10 +2304,8 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
       if (lane == 0) sh_tot[attempt][warp] = mass;
     } else {
       // To all CTAs, counted on a barrier of theirs: half the way of stores and a cluster barrier behind them.
-      if (lane < S)
-        store_async(map_to_cta(smem_u32(&sh_tot[attempt][rank * kWarps + warp]), lane), mass,
-                    map_to_cta(smem_u32(&sh_all[attempt]), lane));
-      if (warp == 0) wait_bulk(smem_u32(&sh_all[attempt]), p.status, kWaitLimitCycles);
+      if (lane < S) send_mass(&sh_tot[attempt][rank * kWarps + warp], &sh_all[attempt], mass, lane);
+      if (warp == 0 && !wait_masses(&sh_all[attempt], p.status, kWaitLimitCycles)) sh_gave_up = 1;
     }
     __syncthreads();                                     // (and this CTA's chunk masses, for the first warp)
     // Lane i has masses 2 i and 2 i + 1.  Every warp learns whether there is any; the first one of every CTA goes on.
@@ -2279,6 +2313,15 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
     if (2 * lane < (kSolo ? kWarps : S * kWarps)) two = reinterpret_cast<const double2*>(sh_tot[attempt])[lane];
     const bool any = __any_sync(0xffffffffu, two.x > 0.0 || two.y > 0.0) &&
                      !__any_sync(0xffffffffu, two.x != two.x || two.y != two.y);
+    if (!kSolo && sh_gave_up) {                          // no draw: some token, and the time-out
+      leave_behind_the_others();
+      if (threadIdx.x == 0) {
+        if (shard && p.phase == 3) p.mass_out[b * 2] = p.mass_out[b * 2 + 1] = 0.0;
+        else p.next_tok[b] = shard ? p.v_offset : 0;
+        report_flags(p, b, flags | HOLA_FLAG_TIMEOUT);
+      }
+      return;
+    }
     if (shard && p.phase == 3) {
       // the shard's masses of row n: of the residual, then (second pass, q taken as 0) of p itself
       if (rank == 0 && warp == 0) {
@@ -3850,23 +3893,33 @@ hola_status hola_selftest_bounded_wait(hola_ctx* ctx, long long limit_cycles, ui
   return HOLA_OK;
 }
 
-hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
-                                      void* cuda_stream) {
+static hola_status staged_wait_selftest(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                        void* cuda_stream, bool early) {
   if (!ctx || !status_word || !counters) return HOLA_ERR_INVALID_ARG;
-  if (limit_cycles < 1000 || limit_cycles > 100000000ll) return HOLA_ERR_INVALID_ARG;   // (twice that is waited at most)
+  if (limit_cycles < 1000 || limit_cycles > 100000000ll) return HOLA_ERR_INVALID_ARG;   // (four times that is waited at most)
   DeviceGuard guard(ctx->device);
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(counters, 0, 3 * sizeof(uint32_t), stream) != cudaSuccess) return HOLA_ERR_CUDA;
+  if (cudaMemsetAsync(counters, 0, (early ? 4 : 3) * sizeof(uint32_t), stream) != cudaSuccess) return HOLA_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2); cfg.blockDim = dim3(64); cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, staged_wait_selftest_kernel, limit_cycles,
-                                           static_cast<unsigned*>(status_word), static_cast<unsigned*>(counters));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, early ? staged_wait_selftest_kernel<true> : staged_wait_selftest_kernel<false>,
+                                           limit_cycles, static_cast<unsigned*>(status_word), static_cast<unsigned*>(counters));
   if (e != cudaSuccess) { set_error(ctx, "launch staged_wait_selftest_kernel", e); return HOLA_ERR_CUDA; }
   return HOLA_OK;
+}
+
+hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                      void* cuda_stream) {
+  return staged_wait_selftest(ctx, limit_cycles, status_word, counters, cuda_stream, false);
+}
+
+hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
+                                    void* cuda_stream) {
+  return staged_wait_selftest(ctx, limit_cycles, status_word, counters, cuda_stream, true);
 }
 
 hola_status hola_lm_head_entropy(hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {

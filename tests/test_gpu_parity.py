@@ -1219,6 +1219,12 @@ def test_a_staged_wait_that_runs_out_is_reported_by_the_cta_that_draws(binding):
         for bad in (10, 10 ** 12):
             with pytest.raises(binding.HolaError):
                 ctx.hola_selftest_staged_wait(bad)
+        # a CTA that gives up on the others' sums leaves behind them: the sums still reach its memory
+        for limit in (20000, 100000, 1000000):
+            assert ctx.hola_selftest_mass_wait(limit) == (binding.FLAG_TIMEOUT, 128, 96, binding.FLAG_TIMEOUT, 2)
+        for bad in (10, 10 ** 12):
+            with pytest.raises(binding.HolaError):
+                ctx.hola_selftest_mass_wait(bad)
         got = ctx.hola_verify(w.hidden, w.W_lm, w.draft_tok, w.draft_q, w.uniforms, w.tau)      # (rows staged)
         torch.cuda.synchronize()
         assert int(got.status.item()) == 0
