@@ -303,6 +303,13 @@ def run_dry(args, rank: int, world: int):
     hdist.shutdown()
 
 
+def row_launches(H: int, V: int, rows: int, w_dtype: int, dev) -> int:
+    """Launches per call that put the hidden rows into another form ahead of the LM head."""
+    from paper_2506_18952_b200 import binding
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    return int(binding.hola_hidden_form_for_shape(sms, H, V, rows, w_dtype) != binding.HOLA_HIDDEN_IN_PLACE)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -358,9 +365,9 @@ def main():
     from paper_2506_18952_b200 import binding
     w = workloads.make_config(args.workload, dev, seed_offset=hdist.rank_seed_offset(rank))
     ctx = binding.HolaVerify(w.B, w.k, w.H, w.V, device=local)
-    plan = ctx.hola_plan(w.B, w.k, {"bf16": binding.HOLA_W_BF16, "int8": binding.HOLA_W_INT8,
-                                    "w8a8": binding.HOLA_W8A8, "w8a16": binding.HOLA_W8A16,
-                                    "mixed": binding.HOLA_W_MIXED, "w4": binding.HOLA_W_MIXED}[args.weights])
+    w_dtype = {"bf16": binding.HOLA_W_BF16, "int8": binding.HOLA_W_INT8, "w8a8": binding.HOLA_W8A8,
+               "w8a16": binding.HOLA_W8A16, "mixed": binding.HOLA_W_MIXED, "w4": binding.HOLA_W_MIXED}[args.weights]
+    plan = ctx.hola_plan(w.B, w.k, w_dtype)
     out = ctx.alloc_outputs(w.B, w.k, False)
     global L2_BYTES
     L2_BYTES = int(getattr(torch.cuda.get_device_properties(dev), "L2_cache_size", L2_BYTES)) or L2_BYTES
@@ -483,8 +490,8 @@ def main():
                 "clocks": clocks,
                 "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                         "ms_per_step": e2e_ms, "host_input_bytes": host_bytes},
-                "gpu_launches": (plan["kernels_per_call"] + (1 if gate_source and w.k > 0 else 0) + (1 if a8 else 0))
-                * args.steps,
+                "gpu_launches": (plan["kernels_per_call"] + (1 if gate_source and w.k > 0 else 0)
+                                 + row_launches(w.H, w.V, w.M, w_dtype, dev)) * args.steps,
                 "accepted_tokens_per_s": accepted_all * args.steps / (ms_max * 1e-3),
                 "roofline": roof}
         if world == 1 and not args.no_cpu_baseline:
@@ -581,7 +588,8 @@ def run_vocab_parallel(args, rank: int, world: int, local: int, dev):
                 "clocks": clocks,
                 "e2e": {"value": w.M * args.e2e_steps / (e2e_total * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
                         "d2h_bytes_per_step": d2h, "ms_per_step": e2e_total / args.e2e_steps},
-                "gpu_launches": (sh.ctx.hola_plan(w.B, w.k)["kernels_per_call"] + 2) * args.steps,
+                "gpu_launches": (sh.ctx.hola_plan(w.B, w.k)["kernels_per_call"] + 2
+                                 + row_launches(w.H, sh.V_local, w.M, binding.HOLA_W_BF16, dev)) * args.steps,
                 "accepted_tokens_per_s": accepted * args.steps / (ms_total * 1e-3),
                 "roofline": roof}
         print(json.dumps(line), flush=True)

@@ -314,7 +314,9 @@ hola_status hola_quantize_mixed_widths(const void* W_bf16, int V, int H, const u
                                        float* scale_out, void* cuda_stream);
 
 /* Launch geometry chosen for a shape (for reports): vocabulary rows per tile of a CTA pair, grid size (CTAs),
- * shared-memory ring slots, verify rows per pass, passes over W_lm, kernel launches per hola_verify call. */
+ * shared-memory ring slots, verify rows per pass, passes over W_lm, LM-head and accept/sample launches per hola_verify call
+ * (one more where the hidden rows are put into another form first, see hola_hidden_form_for_shape, or where the pass over the
+ * draft rows that the draft-entropy gate needs has a kernel of its own). */
 typedef struct {
   int32_t tile_v, grid, stages, rows_per_pass, passes, kernels_per_call;
 } hola_plan_info;
@@ -323,6 +325,10 @@ hola_status hola_plan_ex(const hola_ctx* ctx, int B, int k, int w_dtype, hola_pl
 /* The same for a shape alone: no context and no device (host arithmetic only), default tuning options.  num_sms is
  * the SM count the grid is cut for (148 on a B200), rows = B (k + 1) verify rows. */
 hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype, hola_plan_info* out);
+/* What becomes of the hidden rows ahead of the LM-head launch, for a shape as above: read where they are, copied once so that rows
+ * start on 128-byte lines, or turned into 8-bit planes.  (hola_lm_head_entropy_static has no room for copies and makes none.) */
+enum { HOLA_HIDDEN_IN_PLACE = 0, HOLA_HIDDEN_ON_LINES = 1, HOLA_HIDDEN_8BIT = 2 };
+hola_status hola_hidden_form_for_shape(int num_sms, int H, int V, int rows, int w_dtype, int32_t* out);
 /* And for the accept/sample kernel of hola_verify: CTAs per sequence, threads per CTA, and whether the rows go through shared
  * memory (1) or are read where they are (0).  For tensors that start on a 16-byte boundary. */
 typedef struct {

@@ -22,6 +22,7 @@ HOLA_Q_BF16, HOLA_Q_F32 = 0, 1
 HOLA_GATE_TARGET_ENTROPY, HOLA_GATE_DRAFT_ENTROPY = 0, 1
 HOLA_FALLBACK_SAMPLE, HOLA_FALLBACK_GREEDY = 0, 1
 HOLA_W_BF16, HOLA_W_INT8, HOLA_W8A8, HOLA_W8A16, HOLA_W_MIXED = 0, 1, 2, 3, 4
+HOLA_HIDDEN_IN_PLACE, HOLA_HIDDEN_ON_LINES, HOLA_HIDDEN_8BIT = 0, 1, 2
 HOLA_ARG_CLEAR_STATUS = 1
 GROUP_ROWS, SUB_BLOCK = 256, 128
 FLAG_BAD_TOKEN, FLAG_BAD_UNIFORM, FLAG_TIMEOUT, FLAG_R_ZERO = 1, 2, 4, 8
@@ -29,7 +30,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_hidden_form_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -122,6 +123,8 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
     lib.hola_plan.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.POINTER(hola_plan_info)]
     lib.hola_plan_for_shape.restype = ctypes.c_int
     lib.hola_plan_for_shape.argtypes = [ctypes.c_int] * 5 + [ctypes.POINTER(hola_plan_info)]
+    lib.hola_hidden_form_for_shape.restype = ctypes.c_int
+    lib.hola_hidden_form_for_shape.argtypes = [ctypes.c_int] * 5 + [ctypes.POINTER(ctypes.c_int32)]
     lib.hola_sample_plan_for_shape.restype = ctypes.c_int
     lib.hola_sample_plan_for_shape.argtypes = [ctypes.c_int] * 6 + [ctypes.POINTER(hola_sample_info)]
     lib.hola_plan_ex.restype = ctypes.c_int
@@ -621,6 +624,16 @@ def hola_plan_for_shape(num_sms: int, H: int, V: int, rows: int, w_dtype: int = 
     if st != 0:
         raise HolaError(f"hola_plan_for_shape: status {st}")
     return {n: getattr(info, n) for n, _ in hola_plan_info._fields_}
+
+
+def hola_hidden_form_for_shape(num_sms: int, H: int, V: int, rows: int, w_dtype: int = 0) -> int:
+    """HOLA_HIDDEN_IN_PLACE, HOLA_HIDDEN_ON_LINES or HOLA_HIDDEN_8BIT: what becomes of the hidden rows ahead of the LM-head
+    launch (the last two: by a kernel of its own)."""
+    form = ctypes.c_int32()
+    st = load_library().hola_hidden_form_for_shape(int(num_sms), int(H), int(V), int(rows), int(w_dtype), ctypes.byref(form))
+    if st != 0:
+        raise HolaError(f"hola_hidden_form_for_shape: status {st}")
+    return form.value
 
 
 def hola_sample_plan_for_shape(num_sms: int, B: int, k: int, V: int, q_dtype: int = HOLA_Q_BF16,

@@ -3275,8 +3275,8 @@ SampleForm sample_form(int num_sms, int B, int k, int V, int q_dtype, int fallba
 // 96 -> 84.5; 320, V = 60000 213 -> 197; 150, H = 1032, V = 60000 53.8 -> 50.4; 128 47.5 -> 45.8; 384, H = 4104, V = 16000 67 -> 64.8;
 // below the line 92 rows, H = 1032, V = 50003 35.6 -> 37.3; 96, V = 32000 24.8 -> 26.4; 384, H = 520, V = 8000 18.7 -> 22.3.  (With
 // codes expanded on chip: no gain, 160 rows, H = 2064, V = 60000 63.5 -> 65.)
-bool aligns_hidden(const hola_ctx* ctx, const hola_verify_args* a, const Plan& pl) {
-  if (a->w_dtype != HOLA_W_BF16 || a->H % kBlockK == 0 || !ctx->hid8) return false;
+bool aligns_hidden(int w_dtype, int H, const Plan& pl) {
+  if (w_dtype != HOLA_W_BF16 || H % kBlockK == 0) return false;
   const int op_rows = pl.n_sub * pl.N, pairs = pl.grid / (2 * (pl.fused ? pl.passes : 1));
   const double tiles = (pl.n_ptiles + pairs - 1) / pairs;
   return op_rows >= 96 && tiles * pl.n_kblocks * op_rows >= 8000.0;
@@ -3308,7 +3308,7 @@ hola_status run_lm_head(hola_ctx* ctx, const hola_verify_args* a, float* logits,
   hola_status s;
   // 8-bit activations: the hidden operand is the context's own buffer of 8-bit planes, filled per call below
   // (as is one that is brought onto whole lines)
-  const bool aligned = aligns_hidden(ctx, a, pl);
+  const bool aligned = ctx->hid8 && aligns_hidden(a->w_dtype, a->H, pl);
   const void* hid_src = (two || i8 || aligned) ? static_cast<const void*>(ctx->hid8) : a->hidden;
   const int hid_pitch = (two || i8) ? hidden_pitch8(a->H) : aligned ? round_up(2 * a->H, 128) : 0;
   if ((two || i8) && !ctx->hid8) return HOLA_ERR_INVALID_ARG;   // (the entry point without a context has no room for it)
@@ -3801,17 +3801,36 @@ hola_status hola_destroy(hola_ctx* ctx) {
   return HOLA_OK;
 }
 
-hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype, hola_plan_info* out) {
-  if (!out || num_sms < 2 || H <= 0 || V <= 0 || rows <= 0) return HOLA_ERR_INVALID_ARG;
+static hola_status plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype, Plan* pl) {
+  if (num_sms < 2 || H <= 0 || V <= 0 || rows <= 0) return HOLA_ERR_INVALID_ARG;
   if (w_dtype < HOLA_W_BF16 || w_dtype > HOLA_W_MIXED) return HOLA_ERR_INVALID_ARG;
   if (H % 8 != 0 || V > kMaxChunks * kChunk) return HOLA_ERR_UNSUPPORTED_SHAPE;
   hola_ctx* c = static_cast<hola_ctx*>(calloc(1, sizeof(hola_ctx)));     // only the fields make_plan reads
   if (!c) return HOLA_ERR_WORKSPACE;
   c->num_sms = num_sms; c->H = H; c->V = V;
-  const Plan pl = make_plan(c, rows, w_dtype);
+  *pl = make_plan(c, rows, w_dtype);
   free(c);
+  return HOLA_OK;
+}
+
+hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype, hola_plan_info* out) {
+  if (!out) return HOLA_ERR_INVALID_ARG;
+  Plan pl;
+  const hola_status s = plan_for_shape(num_sms, H, V, rows, w_dtype, &pl);
+  if (s != HOLA_OK) return s;
   out->tile_v = 2 * pl.tile_rows; out->grid = pl.grid; out->stages = pl.stages; out->rows_per_pass = pl.rows_per_pass;
   out->passes = pl.passes; out->kernels_per_call = (pl.fused ? 1 : pl.passes) + 1;
+  return HOLA_OK;
+}
+
+hola_status hola_hidden_form_for_shape(int num_sms, int H, int V, int rows, int w_dtype, int32_t* out) {
+  if (!out) return HOLA_ERR_INVALID_ARG;
+  Plan pl;
+  const hola_status s = plan_for_shape(num_sms, H, V, rows, w_dtype, &pl);
+  if (s != HOLA_OK) return s;
+  *out = w_dtype == HOLA_W8A8 || w_dtype == HOLA_W8A16 ? HOLA_HIDDEN_8BIT
+         : aligns_hidden(w_dtype, H, pl)               ? HOLA_HIDDEN_ON_LINES
+                                                       : HOLA_HIDDEN_IN_PLACE;
   return HOLA_OK;
 }
 

@@ -138,3 +138,14 @@ def test_form_of_the_accept_kernel_for_shapes(B, k, V, f32, want):
     for bad in ((1, B, k, V), (148, 0, k, V), (148, B, -1, V), (148, B, 64, V), (148, B, k, 0), (148, B, k, V, 7), (148, B, k, V, 0, 2)):
         with pytest.raises(b.HolaError):
             b.hola_sample_plan_for_shape(*bad)
+
+
+def test_form_of_the_hidden_rows_for_shapes():
+    from paper_2506_18952_b200 import binding as b
+    form = b.hola_hidden_form_for_shape
+    assert form(148, 4096, 128256, 384) == form(148, 1032, 60000, 92) == form(148, 1032, 60000, 128, b.HOLA_W_INT8) == b.HOLA_HIDDEN_IN_PLACE
+    assert form(148, 1032, 60000, 128) == b.HOLA_HIDDEN_ON_LINES
+    assert form(148, 64, 1000, 5, b.HOLA_W8A8) == form(148, 64, 1000, 5, b.HOLA_W8A16) == b.HOLA_HIDDEN_8BIT
+    for bad in ((1, 4096, 32000, 5, 0), (148, 4097, 32000, 5, 0), (148, 4096, 0, 5, 0), (148, 4096, 32000, 0, 0), (148, 4096, 32000, 5, 9)):
+        with pytest.raises(b.HolaError):
+            form(*bad)

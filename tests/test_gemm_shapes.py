@@ -84,12 +84,45 @@ def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(bin
             assert torch.equal(out.logits.reshape(-1, V), want)
 
 
-# Rows that start on no 128-byte line are copied onto lines where there is enough to do: a partial last K block and several per ring
-# slot, four tiles per pair, several passes, rotating units, two MMAs per K step; the last one stays as it is.  An odd vocabulary:
-# 16-byte stores of logits end within the row's pitch.
-@pytest.mark.parametrize("B,k,H,V", [(24, 3, 5512, 1000), (32, 3, 1032, 60000), (100, 4, 2056, 700), (97, 2, 2008, 20003), (86, 5, 1544, 19001), (24, 3, 5128, 1000)])
-def test_rows_copied_onto_lines(binding, B, k, H, V):
+# Rows that start on no 128-byte line are copied onto lines where there is enough to do.  `plan`: rows per tile, ring slots, rows per
+# pass, passes.  All have a partial last K block: in a slot of its own behind slots of two and of four blocks, or one block per slot
+# like the others (rotating units, two MMAs per K step).
+@pytest.mark.parametrize("B,k,H,V,plan,copied", [
+    (32, 3, 1032, 60000, (208, 4, 128, 1), True),                                                   # two blocks per slot
+    (24, 3, 8136, 3000, (64, 4, 96, 1), True), (60, 2, 5320, 1500, (64, 4, 96, 2), True),           # four, in one pass and in two
+    (97, 2, 2008, 20003, (256, 4, 336, 1), True), (86, 5, 1544, 19001, (256, 4, 288, 2), True),     # rotating units
+    (88, 4, 1032, 20003, (256, 4, 448, 1), True), (125, 7, 520, 40001, (256, 4, 512, 2), True),     # two MMAs
+    # too few rows per pass, or too little to do
+    (24, 3, 5512, 1000, (128, 4, 32, 3), False), (100, 4, 2056, 700, (128, 8, 64, 8), False),
+    (23, 3, 1032, 50003, (240, 4, 96, 1), False), (77, 4, 136, 64001, (256, 4, 416, 1), False)])
+def test_rows_copied_onto_lines(binding, B, k, H, V, plan, copied):
+    got = binding.hola_plan_for_shape(148, H, V, B * (k + 1))
+    assert tuple(got[n] for n in ("tile_v", "stages", "rows_per_pass", "passes")) == plan
+    form = binding.hola_hidden_form_for_shape(148, H, V, B * (k + 1))
+    assert form == (binding.HOLA_HIDDEN_ON_LINES if copied else binding.HOLA_HIDDEN_IN_PLACE)
     check_lm_head(binding, "bf16", B, k, H, V)
+
+
+def test_a_copy_of_the_rows_is_a_launch_of_its_own(binding):
+    from cuda.bindings import runtime
+    for B, k, H, V, mode in [(32, 3, 1032, 60000, "bf16"), (23, 3, 1032, 50003, "bf16"), (9, 4, 144, 2000, "w8a8")]:
+        hidden, W = exact_operands(B, k, H, V, 1)
+        scale = None
+        if mode != "bf16":
+            W, scale = binding.hola_quantize_w8(W)
+        tok = torch.zeros((B, k), dtype=torch.int32, device=DEV)
+        q = torch.full((B, k, V), 1.0 / V, device=DEV)
+        u = torch.rand((B, k + 1), device=DEV)
+        code = binding.HOLA_W_BF16 if mode == "bf16" else binding.HOLA_W8A8
+        with binding.HolaVerify(B, k, H, V) as ctx:
+            out = ctx.alloc_outputs(B, k, False)
+            graph = torch.cuda.CUDAGraph(keep_graph=True)
+            with torch.cuda.graph(graph):
+                ctx.hola_verify(hidden, W, tok, q, u, 0.0, out=out, w_scale=scale, a8=MODES[mode])
+            err, _, nodes = runtime.cudaGraphGetNodes(runtime.cudaGraph_t(init_value=graph.raw_cuda_graph()), 64)
+            assert int(err) == 0
+            copied = binding.hola_hidden_form_for_shape(148, H, V, B * (k + 1), code) != binding.HOLA_HIDDEN_IN_PLACE
+            assert nodes == ctx.hola_plan(B, k, code)["kernels_per_call"] + copied
 
 
 @pytest.mark.parametrize("B,k,H,V", [(33, 4, 320, 5001), (50, 2, 136, 9002), (64, 2, 64, 20003)])
