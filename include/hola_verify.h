@@ -369,6 +369,10 @@ hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uin
 hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
                                     void* cuda_stream);
 
+/* Self-test of the division in H = ln s - t / s: out[i] = t[i] / s[i] as the kernels compute it, n values (device pointers).  For
+ * s in [1, 524288] and t = 0 or |t| >= 2^-100: within 0.5 + 2^-20 units in the last place.  Asynchronous on cuda_stream. */
+hola_status hola_selftest_quotient(hola_ctx* ctx, const float* t, const float* s, int n, float* out, void* cuda_stream);
+
 const char* hola_strerror(hola_status s);
 /* Text of the last CUDA error seen by this context (empty string if none). */
 const char* hola_last_cuda_error(const hola_ctx* ctx);

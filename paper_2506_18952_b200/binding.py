@@ -30,7 +30,7 @@ HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HO
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_hidden_form_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_hidden_form_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_selftest_quotient", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -137,6 +137,9 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
         fn = getattr(lib, name)
         fn.restype = ctypes.c_int
         fn.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+    lib.hola_selftest_quotient.restype = ctypes.c_int
+    lib.hola_selftest_quotient.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,
+                                           ctypes.c_void_p]
     lib.hola_shard_record_bytes.restype = ctypes.c_size_t
     lib.hola_shard_record_bytes.argtypes = [ctypes.c_int, ctypes.c_int]
     for name in ("hola_shard_lm_head", "hola_shard_accept", "hola_shard_sample"):
@@ -423,6 +426,16 @@ class HolaVerify:
         _check(self.lib, self._ctx, st, "hola_selftest_mass_wait")
         (torch.cuda.current_stream() if stream is None else stream).synchronize()
         return (int(status.item()), *counters.tolist())
+
+    def hola_selftest_quotient(self, t: torch.Tensor, s: torch.Tensor, stream=None) -> torch.Tensor:
+        """t / s (contiguous fp32 tensors on the context's device) as the kernels divide."""
+        for x in (t, s):
+            if x.dtype != torch.float32 or x.device != self._dev or not x.is_contiguous() or x.numel() != t.numel():
+                raise HolaError("hola_selftest_quotient takes two contiguous fp32 tensors of one size on the context's device")
+        out = torch.empty_like(t)
+        st = self.lib.hola_selftest_quotient(self._ctx, _dptr(t), _dptr(s), t.numel(), _dptr(out), _stream_ptr(stream))
+        _check(self.lib, self._ctx, st, "hola_selftest_quotient")
+        return out
 
     def hola_profile_begin(self, max_calls: int):
         _check(self.lib, self._ctx, self.lib.hola_profile_begin(self._ctx, max_calls), "hola_profile_begin")

@@ -24,7 +24,7 @@
 //   quantize_hidden_kernel      the hidden rows of a call as one or two 8-bit planes.
 //   align_hidden_kernel         the hidden rows of a call once more, on 128-byte lines.
 //   bounded_wait_selftest_kernel, staged_wait_selftest_kernel  waits that are made to run out, to exercise the give-up paths
-//       without breaking anything.
+//       without breaking anything; quotient_selftest_kernel, the division behind every entropy.
 //   draft_entropy_kernel        H(q_j) of the draft rows, for the gate on the draft distribution.
 //   shard_record_kernel         vocabulary-parallel form: a rank's statistics record for the first all-gather.
 //   finalize_kernel             merges the per-CTA statistics:  logZ = m + ln s,  H = ln s - t/s  (entropy
@@ -1789,14 +1789,20 @@ __device__ __forceinline__ Stats warp_merge_row(const float4* partials, int npar
   return warp_merge_partials(x, partials, nparts, 1, lane, want_arg);
 }
 
-// t / s for 1 <= s <= V: the product with the approximate reciprocal, corrected once by its exact remainder (Newton's step on the
-// quotient), within 2^-23 of a unit in the last place of t / s before its one rounding.  (An IEEE division takes 260 cycles here,
-// of a chain that small batches wait for; this 35.)
+// t / s for 1 <= s <= V and t = 0 or |t| >= 2^-100: the product with the approximate reciprocal, corrected once by its remainder
+// (Newton's step on the quotient).  The reciprocal is within 2^-23 (relative), the product then within 1.5 * 2^-23, the corrected
+// quotient within 1.5 * 2^-46, to which the rounding of the remainder adds half of that at most: less than 2^-20 of a unit in the
+// last place ahead of its one rounding, hence t / s rounded or, where that is as close to a tie, its neighbour.  (An IEEE division
+// takes 260 cycles here, of a chain that small batches wait for; this 35.)
 __device__ __forceinline__ float quotient(float t, float s) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s));
   const float q = t * y;
   return fmaf(fmaf(-q, s, t), y, q);
+}
+__global__ void quotient_selftest_kernel(const float* t, const float* s, int n, float* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) out[i] = quotient(t[i], s[i]);
 }
 __device__ __forceinline__ void stats_to_outputs(Stats st, float* logZ, float* H) {
   const float ls = logf(st.s);
@@ -3939,6 +3945,15 @@ hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uin
 hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
                                     void* cuda_stream) {
   return staged_wait_selftest(ctx, limit_cycles, status_word, counters, cuda_stream, true);
+}
+
+hola_status hola_selftest_quotient(hola_ctx* ctx, const float* t, const float* s, int n, float* out, void* cuda_stream) {
+  if (!ctx || !t || !s || !out || n <= 0) return HOLA_ERR_INVALID_ARG;
+  DeviceGuard guard(ctx->device);
+  quotient_selftest_kernel<<<(n - 1) / 256 + 1, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(t, s, n, out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) { set_error(ctx, "launch quotient_selftest_kernel", e); return HOLA_ERR_CUDA; }
+  return HOLA_OK;
 }
 
 hola_status hola_lm_head_entropy(hola_ctx* ctx, const hola_verify_args* a, void* cuda_stream) {

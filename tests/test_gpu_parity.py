@@ -834,6 +834,27 @@ def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable(binding):
     check_against_oracle(binding, w, out=got, want_logits=False)
 
 
+def test_division_behind_the_entropy_is_within_its_bound(binding):
+    """t / s over the statistics' range: sums of V <= 524288 terms e^d and d e^d with the largest d = 0."""
+    g = torch.Generator(device=DEV).manual_seed(11)
+    n = 1 << 22
+    s = torch.exp2(19 * torch.rand(n, generator=g, device=DEV, dtype=torch.float64)).float()
+    s[: n // 4] = 1 + s[: n // 4] / 2 ** 22                                # one term and next to nothing
+    s[n // 4: n // 2] = torch.randint(1, 524289, (n // 4,), generator=g, device=DEV).float()
+    t = -torch.exp2(118 * torch.rand(n, generator=g, device=DEV, dtype=torch.float64) - 100).float()
+    t[: n // 2] = -(s[: n // 2] * 13 * torch.rand(n // 2, generator=g, device=DEV))
+    t[-1000:] = 0.0
+    with binding.HolaVerify(1, 1, 64, 1000) as ctx:
+        got = ctx.hola_selftest_quotient(t, s)
+        torch.cuda.synchronize()
+        with pytest.raises(binding.HolaError):
+            ctx.hola_selftest_quotient(t, s[:5])
+    exact = t.double() / s.double()
+    ulp = torch.exp2(torch.floor(torch.log2(exact.abs().clamp(min=2.0 ** -126))) - 23)
+    assert ((got.double() - exact).abs() <= (0.5 + 2.0 ** -20) * ulp).all()
+    assert torch.equal(got[-1000:].abs(), torch.zeros(1000, device=DEV))
+
+
 def test_inputs_written_by_the_kernel_just_before_the_call_are_seen(binding):
     """Tokens, uniforms and draft probabilities produced on the same stream right before the call (no synchronisation in
     between) must be the ones the step uses: the accept/sample kernel may be scheduled early, but reads its inputs only
