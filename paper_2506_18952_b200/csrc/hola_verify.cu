@@ -2988,6 +2988,25 @@ int round_up(int x, int a) { return (x + a - 1) / a * a; }
 // Splits M verify rows into passes over W_lm and each pass into one or two MMAs per K step.
 // A pass holds at most 512 rows (two MMAs of N <= 256 fill the tensor memory); N is a multiple of 16.
 // Cost per pass: the slower of streaming W_lm once and the padded rows' tensor time, plus a fixed launch cost.
+// How the r verify rows of a pass are laid out as operand rows: MMAs per K step, rows per MMA, verify rows that these hold.
+struct RowSplit { int n_sub, N, rows_per_pass; };
+inline RowSplit split_rows(const hola_ctx* ctx, int r, int w_dtype) {
+  // up to 256 rows: one MMA, two accumulator buffers; up to 384: three MMAs of N <= 128 on rotating 128-column
+  // units; beyond: two MMAs of N <= 256 that fill the tensor memory
+  RowSplit f;
+  if (w_dtype == HOLA_W8A16) {                     // operand rows: 64 per 32 verify rows; one or two MMAs, N % 64 == 0
+    const int r8 = 2 * round_up(r, 32);
+    f.n_sub = r8 > kMaxN ? 2 : 1;
+    f.N = round_up(r8 / f.n_sub, 64);
+    f.rows_per_pass = f.n_sub * f.N / 2;
+    return f;
+  }
+  f.n_sub = (r > 3 * 128 || (ctx->no_rot && r > kMaxN)) ? 2 : (r > kMaxN ? 3 : 1);
+  f.N = round_up((r + f.n_sub - 1) / f.n_sub, w_dtype == HOLA_W8A8 ? 32 : 16);
+  f.rows_per_pass = f.n_sub * f.N;
+  return f;
+}
+
 // `want`: number of passes (0: by that cost), vocabulary rows per CTA and tile (0: by the rules below), all passes in one launch.
 struct PlanWish { int passes, tile_rows; bool fuse; };
 Plan plan_as(const hola_ctx* ctx, int M, int w_dtype, const PlanWish& want) {
@@ -3006,20 +3025,12 @@ Plan plan_as(const hola_ctx* ctx, int M, int w_dtype, const PlanWish& want) {
   for (int passes = p_min; passes <= p_max; ++passes) {
     if (want.passes && passes != want.passes && want.passes >= p_min) continue;
     const int r = (rows + passes - 1) / passes;
-    // up to 256 rows: one MMA, two accumulator buffers; up to 384: three MMAs of N <= 128 on rotating 128-column
-    // units; beyond: two MMAs of N <= 256 that fill the tensor memory
-    int n_sub = (r > 3 * 128 || (ctx->no_rot && r > kMaxN)) ? 2 : (r > kMaxN ? 3 : 1);
-    int N = round_up((r + n_sub - 1) / n_sub, i8 ? 32 : 16);
-    if (two) {                                     // operand rows: 64 per 32 verify rows; one or two MMAs, N % 64 == 0
-      const int r8 = 2 * round_up(r, 32);
-      n_sub = r8 > kMaxN ? 2 : 1;
-      N = round_up(r8 / n_sub, 64);
-    }
-    const double t_mma = 2.0 * n_sub * N * static_cast<double>(ctx->V) * ctx->H / (i8 ? 2.8e15 : 1.4e15);
+    const RowSplit f = split_rows(ctx, r, w_dtype);
+    const double t_mma = 2.0 * f.n_sub * f.N * static_cast<double>(ctx->V) * ctx->H / (i8 ? 2.8e15 : 1.4e15);
     const double cost = passes * ((t_mma > t_hbm ? t_mma : t_hbm) + 6e-6);
     if (cost < best_cost) {
       best_cost = cost;
-      best.n_sub = n_sub; best.N = N; best.rows_per_pass = two ? n_sub * N / 2 : n_sub * N; best.passes = passes;
+      best.n_sub = f.n_sub; best.N = f.N; best.rows_per_pass = f.rows_per_pass; best.passes = passes;
       best.est_seconds = cost;
       best.mma_share = t_mma / t_hbm;
     }
@@ -3100,16 +3111,17 @@ Plan plan_as(const hola_ctx* ctx, int M, int w_dtype, const PlanWish& want) {
 // read-out takes 1.8 us per chunk of 32 operand rows and epilogue warp.  Fitted to 37 shapes (V = 1200 .. 12000, H = 200 .. 8192,
 // 5 .. 2304 rows, every weight mode) in 2 to 20 splits each: the split it picks was 0.7 % slower than the best one on average, 4 %
 // at worst.
-double one_tile_us(const hola_ctx* ctx, const Plan& pl, int w_dtype) {
+inline double one_tile_us(const hola_ctx* ctx, int w_dtype, int n_sub, int N, int tile_rows, int grid) {
   const bool expand = w_dtype == HOLA_W_INT8 || w_dtype == HOLA_W_MIXED, i8 = w_dtype == HOLA_W8A8 || w_dtype == HOLA_W8A16;
-  const int op_rows = pl.n_sub * pl.N;
-  const double mma = 1.16 * 4.0 * pl.n_sub * (pl.N / 2 > 46 ? pl.N / 2 : 46);
-  const double bytes = pl.tile_rows * (expand ? 64.0 : 128.0) + op_rows * 64.0;
+  const int op_rows = n_sub * N;
+  const double mma = 1.16 * 4.0 * n_sub * (N / 2 > 46 ? N / 2 : 46);
+  const double bytes = tile_rows * (expand ? 64.0 : 128.0) + op_rows * 64.0;
   const double line = !i8 && ctx->H % kBlockK != 0 ? 0.79 : 1.0;
   double block = expand ? 326.0 : 180.0;
-  for (const double c : {mma, bytes / (61.0 * line), pl.grid * bytes / (6400.0 * line)})
+  for (const double c : {mma, bytes / (61.0 * line), grid * bytes / (6400.0 * line)})
     if (c > block) block = c;
-  const double ring = pl.n_kblocks * block / 1900.0, hbm = static_cast<double>(ctx->V) * ctx->H * (expand || i8 ? 1 : 2) / 7.2e6;
+  const int n_kblocks = i8 ? (ctx->H + 2 * kBlockK - 1) / (2 * kBlockK) : (ctx->H + kBlockK - 1) / kBlockK;
+  const double ring = n_kblocks * block / 1900.0, hbm = static_cast<double>(ctx->V) * ctx->H * (expand || i8 ? 1 : 2) / 7.2e6;
   const int groups = !expand ? kEpiWarps / 4 : op_rows <= 32 ? kW8FewEpiWarps / 4 : kW8EpiWarps / 4;
   return (ring > hbm ? ring : hbm) + 1.8 * (((op_rows + 31) / 32 + groups - 1) / groups);
 }
@@ -3126,20 +3138,30 @@ Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   const int pairs = ctx->num_sms / 2;
   const int p_min = best.passes;
   if (!ctx->force_passes && best.n_ptiles * p_min <= pairs) {
-    double best_us = one_tile_us(ctx, best, w_dtype) - 0.5;
-    for (int tile_rows = kLanes; tile_rows >= 32; tile_rows -= 32) {
-      if (w_dtype == HOLA_W_MIXED && tile_rows < kLanes) break;
+    // (by the estimate alone, and laid out in full once: a split takes 0.15 to 0.45 us of the host; every try laid out, up to 1.8)
+    constexpr int kTries = 16;
+    struct { RowSplit rows; int passes; } tries[kTries];
+    int n_tries = 0;
+    for (; n_tries < kTries && p_min + n_tries <= pairs; ++n_tries) {
+      const int passes = p_min + n_tries;
+      if (n_tries && M < 32 * passes) break;
+      const RowSplit rows = split_rows(ctx, M > 0 ? (M + passes - 1) / passes : 1, w_dtype);
+      tries[n_tries] = {rows, M > 0 ? (M + rows.rows_per_pass - 1) / rows.rows_per_pass : 1};
+    }
+    double best_us = one_tile_us(ctx, w_dtype, best.n_sub, best.N, best.tile_rows, best.grid) - 0.5;
+    for (int tile_rows = kLanes; tile_rows >= (w_dtype == HOLA_W_MIXED ? kLanes : 32); tile_rows -= 32) {
       const int tiles = (ctx->V + 2 * tile_rows - 1) / (2 * tile_rows);
-      for (int passes = p_min; passes * tiles <= pairs && passes < p_min + 16; ++passes) {
-        if (passes > p_min && M < 32 * passes) break;
-        const PlanWish w = {passes, tile_rows, true};
-        const Plan p = plan_as(ctx, M, w_dtype, w);
-        const double us = one_tile_us(ctx, p, w_dtype);
-        if (p.n_ptiles * p.passes <= pairs && us < best_us) {
-          best = p; best_us = us; want = w;
-          best.est_seconds = us * 1e-6 + 6e-6;
+      for (int i = 0; i < n_tries && (p_min + i) * tiles <= pairs; ++i) {
+        const double us = one_tile_us(ctx, w_dtype, tries[i].rows.n_sub, tries[i].rows.N, tile_rows, 2 * tiles * tries[i].passes);
+        if (us < best_us) {
+          best_us = us;
+          want.passes = p_min + i; want.tile_rows = tile_rows;
         }
       }
+    }
+    if (want.passes) {
+      best = plan_as(ctx, M, w_dtype, want);
+      best.est_seconds = best_us * 1e-6 + 6e-6;
     }
   }
   if (ctx->no_fuse && best.passes > 1) {           // the same passes, a launch each
