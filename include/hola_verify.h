@@ -369,6 +369,11 @@ hola_status hola_selftest_staged_wait(hola_ctx* ctx, long long limit_cycles, uin
 hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint32_t* status_word, uint32_t* counters,
                                     void* cuda_stream);
 
+/* The counters by which the passes of a launch keep in step over several tiles, copied to `words` (device memory).  Every launch
+ * leaves them at zero for the next one.  Asynchronous on cuda_stream. */
+#define HOLA_PACE_WORDS 256
+hola_status hola_selftest_pace(hola_ctx* ctx, uint32_t* words, void* cuda_stream);
+
 /* Self-test of the division in H = ln s - t / s: out[i] = t[i] / s[i] as the kernels compute it, n values (device pointers).  For
  * s in [1, 524288] and t = 0 or |t| >= 2^-100: within 0.5 + 2^-20 units in the last place.  Asynchronous on cuda_stream. */
 hola_status hola_selftest_quotient(hola_ctx* ctx, const float* t, const float* s, int n, float* out, void* cuda_stream);

@@ -24,13 +24,13 @@ HOLA_FALLBACK_SAMPLE, HOLA_FALLBACK_GREEDY = 0, 1
 HOLA_W_BF16, HOLA_W_INT8, HOLA_W8A8, HOLA_W8A16, HOLA_W_MIXED = 0, 1, 2, 3, 4
 HOLA_HIDDEN_IN_PLACE, HOLA_HIDDEN_ON_LINES, HOLA_HIDDEN_8BIT = 0, 1, 2
 HOLA_ARG_CLEAR_STATUS = 1
-GROUP_ROWS, SUB_BLOCK = 256, 128
+GROUP_ROWS, SUB_BLOCK, HOLA_PACE_WORDS = 256, 128, 256
 FLAG_BAD_TOKEN, FLAG_BAD_UNIFORM, FLAG_TIMEOUT, FLAG_R_ZERO = 1, 2, 4, 8
 HOLA_OPT_RING_SLOTS, HOLA_OPT_ROTATING_UNITS, HOLA_OPT_HOST_OVERLAP, HOLA_OPT_HOST_ROWS_ON_DEMAND, HOLA_OPT_PASSES, HOLA_OPT_PAIR_MMA, HOLA_OPT_HOST_IN_PLACE, HOLA_OPT_CONVERTER_GROUP, HOLA_OPT_FUSED_PASSES = 1, 2, 3, 4, 5, 6, 7, 8, 9
 
 EXPORTS = ["hola_create", "hola_destroy", "hola_workspace_bytes", "hola_verify", "hola_verify_host",
            "hola_lm_head_entropy", "hola_accept_sample", "hola_host_traffic", "hola_shard_record_bytes", "hola_shard_lm_head",
-           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_hidden_form_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_selftest_quotient", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
+           "hola_shard_accept", "hola_shard_sample", "hola_lm_head_entropy_static", "hola_quantize_w8", "hola_quantize_w4", "hola_quantize_mixed", "hola_quantize_mixed_widths", "hola_plan", "hola_plan_ex", "hola_plan_for_shape", "hola_hidden_form_for_shape", "hola_sample_plan_for_shape", "hola_set_option", "hola_selftest_bounded_wait", "hola_selftest_staged_wait", "hola_selftest_mass_wait", "hola_selftest_pace", "hola_selftest_quotient", "hola_profile_begin", "hola_profile_end", "hola_strerror", "hola_last_cuda_error",
            "hola_version"]
 
 
@@ -137,6 +137,8 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
         fn = getattr(lib, name)
         fn.restype = ctypes.c_int
         fn.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+    lib.hola_selftest_pace.restype = ctypes.c_int
+    lib.hola_selftest_pace.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     lib.hola_selftest_quotient.restype = ctypes.c_int
     lib.hola_selftest_quotient.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,
                                            ctypes.c_void_p]
@@ -426,6 +428,12 @@ class HolaVerify:
         _check(self.lib, self._ctx, st, "hola_selftest_mass_wait")
         (torch.cuda.current_stream() if stream is None else stream).synchronize()
         return (int(status.item()), *counters.tolist())
+
+    def hola_selftest_pace(self, stream=None) -> torch.Tensor:
+        """The pace counters of launches that hold several passes, behind what is queued on the stream: zeros between calls."""
+        words = torch.empty(HOLA_PACE_WORDS, dtype=torch.int32, device=self._dev)
+        _check(self.lib, self._ctx, self.lib.hola_selftest_pace(self._ctx, _dptr(words), _stream_ptr(stream)), "hola_selftest_pace")
+        return words
 
     def hola_selftest_quotient(self, t: torch.Tensor, s: torch.Tensor, stream=None) -> torch.Tensor:
         """t / s (contiguous fp32 tensors on the context's device) as the kernels divide."""

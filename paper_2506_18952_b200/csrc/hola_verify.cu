@@ -3969,6 +3969,15 @@ hola_status hola_selftest_mass_wait(hola_ctx* ctx, long long limit_cycles, uint3
   return staged_wait_selftest(ctx, limit_cycles, status_word, counters, cuda_stream, true);
 }
 
+hola_status hola_selftest_pace(hola_ctx* ctx, uint32_t* words, void* cuda_stream) {
+  if (!ctx || !words) return HOLA_ERR_INVALID_ARG;
+  static_assert(HOLA_PACE_WORDS == 2 * kMaxPaceGroups, "two words per group");
+  DeviceGuard guard(ctx->device);
+  const cudaError_t e = cudaMemcpyAsync(words, ctx->pace, 4 * HOLA_PACE_WORDS, cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(cuda_stream));
+  if (e != cudaSuccess) { set_error(ctx, "copy of the pace counters", e); return HOLA_ERR_CUDA; }
+  return HOLA_OK;
+}
+
 hola_status hola_selftest_quotient(hola_ctx* ctx, const float* t, const float* s, int n, float* out, void* cuda_stream) {
   if (!ctx || !t || !s || !out || n <= 0) return HOLA_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);

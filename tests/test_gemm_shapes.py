@@ -59,7 +59,7 @@ def test_padded_rows_of_eight_bit_planes(binding, mode, B, k, H, V):
 
 # Small vocabularies: the rows are cut into several passes over few tiles, all in one launch.  The last pass ends inside a block of
 # rows, or holds a single row; tiles of 32, 64, 96 and 128 rows per CTA; a ragged last tile; a partial last K block; with tiles left
-# over for some pairs (the calls come twice: what the groups of pairs keep step by has to be as it was).
+# over for some pairs.
 @pytest.mark.parametrize("mode,B,k,H,V", [
     ("bf16", 139, 2, 1304, 1272), ("bf16", 128, 3, 512, 2000), ("bf16", 64, 2, 200, 1030), ("bf16", 43, 5, 264, 3001),
     ("bf16", 256, 8, 128, 1003), ("bf16", 129, 0, 4096, 700), ("int8", 29, 8, 944, 2904), ("int8", 97, 0, 2048, 520),
@@ -71,17 +71,33 @@ def test_rows_of_small_vocabularies_in_several_passes(binding, mode, B, k, H, V)
     check_lm_head(binding, mode, B, k, H, V)
 
 
-@pytest.mark.parametrize("mode,B,k,H,V", [("bf16", 300, 3, 64, 30000), ("w8a8", 200, 4, 128, 40001)])
+# Passes in one launch keep in step by counters, which every launch has to leave at zero for the next: with other numbers of passes
+# (None: the plan's own), so of groups, on one context.  They are a pace and nothing else, so the logits alone would not show it.
+@pytest.mark.parametrize("mode,B,k,H,V", [
+    ("bf16", 300, 3, 64, 30000), ("bf16", 300, 3, 520, 30001), ("int8", 80, 4, 128, 30000), ("w8a8", 200, 4, 128, 40001),
+    ("w8a16", 150, 3, 256, 40000), ("mixed", 80, 4, 256, 30000)])
 def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(binding, mode, B, k, H, V):
     hidden, W = exact_operands(B, k, H, V, 3)
     want = (hidden.double().reshape(-1, H) @ W.double().t()).float()
     scale = None
-    if mode != "bf16":
+    if mode == "mixed":
+        W = binding.hola_quantize_mixed(W, ([8, 16, 8] * V)[:-(-V // binding.GROUP_ROWS)])
+    elif mode != "bf16":
         W, scale = binding.hola_quantize_w8(W)
+    code = {"bf16": binding.HOLA_W_BF16, "int8": binding.HOLA_W_INT8, "w8a8": binding.HOLA_W8A8, "w8a16": binding.HOLA_W8A16,
+            "mixed": binding.HOLA_W_MIXED}[mode]
     with binding.HolaVerify(B, k, H, V) as ctx:
-        for _ in range(3):
-            out = ctx.hola_lm_head_entropy(hidden, W, want_logits=True, w_scale=scale, a8=MODES[mode])
-            assert torch.equal(out.logits.reshape(-1, V), want)
+        assert not ctx.hola_selftest_pace().any()
+        for passes in (None, 5, 3, 7):
+            if passes:
+                ctx.hola_set_option(binding.HOLA_OPT_PASSES, passes)
+            plan = ctx.hola_plan(B, k, code)
+            groups, tiles = plan["grid"] // (2 * plan["passes"]), -(-V // plan["tile_v"])
+            assert plan["passes"] >= 2 and plan["kernels_per_call"] == 2 and tiles > groups
+            for _ in range(2):
+                out = ctx.hola_lm_head_entropy(hidden, W, want_logits=True, w_scale=scale, a8=MODES.get(mode, False))
+                assert torch.equal(out.logits.reshape(-1, V), want)
+                assert not ctx.hola_selftest_pace().any()
 
 
 # Rows that start on no 128-byte line are copied onto lines where there is enough to do.  `plan`: rows per tile, ring slots, rows per
