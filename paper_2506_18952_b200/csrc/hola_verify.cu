@@ -2807,7 +2807,7 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
   }
 }
 
-// bf16 hidden rows that start on no 128-byte line, once more with a pitch of whole lines (aligns_hidden): a CTA per row, up to
+// bf16 hidden rows that start on no 32-byte sector, once more with a pitch of whole 128-byte lines (aligns_hidden): a CTA per row, up to
 // four 16-byte loads per thread in flight; latency bounds it (some 2.4 us of a call).
 constexpr int kAlignThreads = 256;
 __global__ void __launch_bounds__(kAlignThreads) align_hidden_kernel(const uint4* X, int pieces, int pitch, uint4* out) {
@@ -3297,17 +3297,19 @@ SampleForm sample_form(int num_sms, int B, int k, int V, int q_dtype, int fallba
   return f;
 }
 
-// bf16 rows that start on no 128-byte line make every fetch of a K block of hidden rows two lines instead of one, out of the L2 and
-// for every tile.  From 96 rows on and where rows x K blocks x tiles per pair reach 8000 a copy of the rows on whole lines pays for
-// itself.  us, as they are -> copied: 96 rows, H = 4104, V = 60000 124 -> 109, V = 128256 239 -> 216; 250 rows, H = 4104, V = 30000
-// 96 -> 84.5; 320, V = 60000 213 -> 197; 150, H = 1032, V = 60000 53.8 -> 50.4; 128 47.5 -> 45.8; 384, H = 4104, V = 16000 67 -> 64.8;
-// below the line 92 rows, H = 1032, V = 50003 35.6 -> 37.3; 96, V = 32000 24.8 -> 26.4; 384, H = 520, V = 8000 18.7 -> 22.3.  (With
-// codes expanded on chip: no gain, 160 rows, H = 2064, V = 60000 63.5 -> 65.)
+// bf16 rows of 2 H = 16 bytes more than whole 32-byte sectors make every fetch of a K block of hidden rows five sectors instead of
+// four, out of the L2 and for every tile.  A copy of the rows on whole lines takes some 2.4 us and pays for itself from 96 rows on
+// where rows x K blocks x tiles per pair reach 8000; with one tile per pair and more than 256 rows the MMAs hide the fetches.  us, as
+// they are -> copied (141 shapes were measured both ways): 99 rows, H = 4216, V = 67724 136.6 -> 122.1; 128, 840, 119544 71.2 -> 65.3;
+// 160, 6568, 16524 63.5 -> 55.9; 600, 7240, 29827 336 -> 299; below the lines 92, 1032, 50003 36.0 -> 37.3, 210, 1832, 9089 22.8 ->
+// 24.3; one tile, 480, 2456, 9633 36.1 -> 38.2.  Rows that start on sectors (H a multiple of 16) gain nothing wherever they start
+// in a line (119 shapes): 312, 592, 53988 37.8 -> 40.4; 370, 1312, 10325 31.4 -> 33.1; 365, 2608, 38298 98.8 -> 99.7.  (With codes
+// expanded on chip: no gain, 160 rows, H = 2064, V = 60000 63.5 -> 65.)
 bool aligns_hidden(int w_dtype, int H, const Plan& pl) {
-  if (w_dtype != HOLA_W_BF16 || H % kBlockK == 0) return false;
+  if (w_dtype != HOLA_W_BF16 || H % 16 == 0) return false;
   const int op_rows = pl.n_sub * pl.N, pairs = pl.grid / (2 * (pl.fused ? pl.passes : 1));
-  const double tiles = (pl.n_ptiles + pairs - 1) / pairs;
-  return op_rows >= 96 && tiles * pl.n_kblocks * op_rows >= 8000.0;
+  const int tiles = (pl.n_ptiles + pairs - 1) / pairs;
+  return op_rows >= 96 && (tiles > 1 || op_rows <= 256) && static_cast<double>(tiles) * pl.n_kblocks * op_rows >= 8000.0;
 }
 
 // Where the logits of a verify step that does not hand them out go.  The greedy rule reads none (the arg-max travels with the

@@ -100,7 +100,7 @@ def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(bin
                 assert not ctx.hola_selftest_pace().any()
 
 
-# Rows that start on no 128-byte line are copied onto lines where there is enough to do.  `plan`: rows per tile, ring slots, rows per
+# Rows that start on no 32-byte sector are copied onto lines where there is enough to do.  `plan`: rows per tile, ring slots, rows per
 # pass, passes.  All have a partial last K block: in a slot of its own behind slots of two and of four blocks, or one block per slot
 # like the others (rotating units, two MMAs per K step).
 @pytest.mark.parametrize("B,k,H,V,plan,copied", [
@@ -108,6 +108,9 @@ def test_passes_that_keep_step_over_several_tiles_leave_their_counters_clean(bin
     (24, 3, 8136, 3000, (64, 4, 96, 1), True), (60, 2, 5320, 1500, (64, 4, 96, 2), True),           # four, in one pass and in two
     (97, 2, 2008, 20003, (256, 4, 336, 1), True), (86, 5, 1544, 19001, (256, 4, 288, 2), True),     # rotating units
     (88, 4, 1032, 20003, (256, 4, 448, 1), True), (125, 7, 520, 40001, (256, 4, 512, 2), True),     # two MMAs
+    # rows on sectors (a copy would gain nothing: 37.8 -> 40.4, 31.4 -> 33.1 us); one tile per pair and more than 256 rows
+    (39, 7, 592, 53988, (256, 4, 336, 1), False), (74, 4, 1312, 10325, (256, 4, 384, 1), False),
+    (60, 7, 2456, 9633, (256, 4, 480, 1), False),
     # too few rows per pass, or too little to do
     (24, 3, 5512, 1000, (128, 4, 32, 3), False), (100, 4, 2056, 700, (128, 8, 64, 8), False),
     (23, 3, 1032, 50003, (240, 4, 96, 1), False), (77, 4, 136, 64001, (256, 4, 416, 1), False)])
