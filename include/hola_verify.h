@@ -329,8 +329,9 @@ hola_status hola_plan_for_shape(int num_sms, int H, int V, int rows, int w_dtype
  * start on 128-byte lines, or turned into 8-bit planes.  (hola_lm_head_entropy_static has no room for copies and makes none.) */
 enum { HOLA_HIDDEN_IN_PLACE = 0, HOLA_HIDDEN_ON_LINES = 1, HOLA_HIDDEN_8BIT = 2 };
 hola_status hola_hidden_form_for_shape(int num_sms, int H, int V, int rows, int w_dtype, int32_t* out);
-/* And for the accept/sample kernel of hola_verify: CTAs per sequence, threads per CTA, and whether the rows go through shared
- * memory (1) or are read where they are (0).  For tensors that start on a 16-byte boundary. */
+/* And for the accept/sample kernel of hola_verify: CTAs per sequence, threads per CTA as launched (of 1024 half leave at once
+ * where the vocabulary and the batch are small), and whether the rows go through shared memory (1) or are read where they are
+ * (0).  For tensors that start on a 16-byte boundary. */
 typedef struct {
   int32_t ctas, threads, staged;
 } hola_sample_info;

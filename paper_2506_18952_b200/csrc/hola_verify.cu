@@ -95,7 +95,7 @@ constexpr long long kWaitLimitCycles = 4000000000ll;   // about 2 s of SM clock 
 
 constexpr int kK3Threads = 256;
 constexpr int kSoloThreads = 1024;               // its form with one CTA per sequence
-constexpr int kFewEntries = 8192;                // vocabulary up to which half of them do
+constexpr int kFewEntries = 8192;                // vocabulary up to which half of them stay
 constexpr int kK3MaxPerSm = 4;                   // CTAs of the accept/sample kernel an SM holds (register budget: 64 per thread)
 constexpr int kChunk = 128;                      // vocabulary entries per warp step (32 lanes x 4)
 constexpr int kMaxChunks = 4096;                 // => V <= 524288
@@ -1906,10 +1906,10 @@ __device__ __forceinline__ void resid4(const float l[4], const float q[4], float
 }
 
 // The residual masses of up to four chunks, c0 and every kStride-th after it as long as they are among n, by a warp: into csum[],
-// and as the result in lanes 8 i .. 8 i + 7 (0 where there is no i-th).  In fp32 (128 non-negative terms added pairwise: relative error a few 1e-7), kept as fp64 for
-// the sums that follow.  lrow, qrow: entry 0 of the row, which a staged slice does not hold.  (Once per type of q: us, 50 rows,
-// V = 60000 53.2 -> 52.4, 32 rows, V = 128256 61.0 -> 59.7, 5 rows, V = 32000 46.67 -> 46.46.  A form for two chunks, and packed
-// fp32 arithmetic, took fewer instructions and longer.)
+// and as the result in lanes 8 i .. 8 i + 7 (0 where there is no i-th).  In fp32 (128 non-negative terms added pairwise: relative
+// error a few 1e-7), kept as fp64 for the sums that follow.  lrow, qrow: entry 0 of the row, which a staged slice does not hold.
+// (Once per type of q: us, 50 rows, V = 60000 53.2 -> 52.4, 32 rows, V = 128256 61.0 -> 59.7, 5 rows, V = 32000 46.67 -> 46.46.  A
+// form for two chunks, and packed fp32 arithmetic, took fewer instructions and longer.)
 template <bool kVec, bool kHalf, int kStride>
 __device__ __forceinline__ double sum_step(const float* lrow, const void* qrow, bool residual, int c0, int n, int V, float logZ,
                                            double* csum, int lane) {
@@ -2070,9 +2070,10 @@ __device__ __forceinline__ unsigned decide(const K3Params& p, int x, int Vtok, f
 // kAsk: the slice of row n is asked into the L2 as soon as n is known.
 // kSoloWarps: one CTA of 1024 threads instead of the cluster (see sample_solo).  All 32 warps of it take part or, for up to
 // kFewEntries entries and sequences for half of the SMs, the first 16: the others leave at once, and the instructions of the rest
-// find more room.  us, 32 -> 16 warps: V = 2000, 16 sequences 10.5 -> 10.2; V = 3000, 1 9.7 -> 9.5; V = 5000, 2 / 32 10.2 -> 10.0,
-// 12.3 -> 12.1; V = 8000, 1 / 64 / 140 11.0 -> 10.95, 13.3 -> 13.1, 18.45 -> 18.75; V = 8191, 5 12.4 -> 12.2; V = 11000, 16 13.2 -> 13.6;
-// V = 16000, 64 17.7 -> 18.8.
+// find more room.  us, 32 -> 16 warps: V = 2000, 16 sequences 10.4 -> 10.0; V = 3000, 1 9.7 -> 9.4; V = 5000, 2 / 32 10.15 -> 9.8,
+// 11.55 -> 11.25; V = 8000, 1 / 64 / 75 / 140 10.5 -> 10.25, 13.2 -> 13.0, 15.0 -> 15.0, 18.35 -> 18.45; V = 8191, 5 12.25 -> 11.95;
+// V = 11000, 16 13.2 -> 13.6; V = 16000, 64 17.7 -> 18.8.  (Launched with 512 threads they take 0.05 to 0.15 less again; the
+// launch is one of 1024, as hola_sample_plan_for_shape reports it.)
 // kStaged: this CTA's slice of ALL k + 1 rows is brought into shared memory while the statistics are merged and the accept test
 // is made, instead of row n afterwards.
 template <bool kVec, bool kAsk, int kSoloWarps = 0, bool kStaged = false>
@@ -2139,9 +2140,8 @@ __global__ void __launch_bounds__(kSoloWarps ? kSoloThreads : kK3Threads, kSoloW
   const size_t q_elem = (p.q_dtype == HOLA_Q_BF16) ? 2 : 4;
   // Staged rows, behind the chunk sums: [k + 1][cpc * 128] logits, then [k][cpc * 128] draft probabilities, each row's
   // slice by one bulk copy, a lane of the first warp per copy, while the other warps merge statistics (with eight rows and more
-  // that one does so too: then the last warp).  (One thread after the
-  // other, in a warp that merges as well, they held the merge up by 0.7 us; us, 5 rows, V = 32000: 46.67 -> 46.31, mixed widths
-  // 34.84 -> 34.47.)
+  // that one does so too: then the last warp).  (One thread after the other, in a warp that merges as well, they held the merge
+  // up by 0.7 us; us, 5 rows, V = 32000: 46.67 -> 46.31, mixed widths 34.84 -> 34.47.)
   const int slice = cpc * kChunk;
   float* sl = reinterpret_cast<float*>(csum + (cpc + 1) / 2 * 2);      // (16-byte boundary whatever the number of chunks)
   char* sq = reinterpret_cast<char*>(sl + static_cast<size_t>(k + 1) * slice);
@@ -2730,11 +2730,11 @@ __global__ void __launch_bounds__(kHidThreads) quantize_hidden_kernel(const uint
                                                                       signed char* q, float* s1, float* s2) {
   __shared__ float sh_max[kHidThreads / 32];
   grid_dependency_wait();                                // (no-op unless launched with programmatic serialization)
-  // The GEMM kernel may be put in place beside this one (its CTA and several of these fit an SM): its launch and set-up and,
-  // on small batches, its first requests for W_lm hide behind the quantisation.  It waits for this grid's end before it reads
-  // anything.  us, 8-bit planes, no release / at entry / here / behind the loads: one sequence, V = 32000 33.0 / 30.7 / 30.6 /
-  // 31.9, two planes 33.4 / 30.8 / 31.3 / 31.2; 80 rows, V = 11000 17.5 / 16.5 / 16.2 / 16.3; 300 rows, V = 16000 28.1 / 26.9 /
-  // 26.7 / 28.4.
+  // The GEMM kernel may be put in place while this one runs, on the SMs that have none of its CTAs or no more (side by side they
+  // do not fit: 14336 registers of a CTA here, 10240 that one of the GEMM kernel leaves): its launch and set-up and, on small
+  // batches, its first requests for W_lm hide behind the quantisation.  It waits for this grid's end before it reads anything.
+  // us, 8-bit planes, no release / at entry / here / behind the loads: one sequence, V = 32000 33.0 / 30.7 / 30.6 / 31.9, two
+  // planes 33.4 / 30.8 / 31.3 / 31.2; 80 rows, V = 11000 17.5 / 16.5 / 16.2 / 16.3; 300 rows, V = 16000 28.1 / 26.9 / 26.7 / 28.4.
   grid_dependency_release();
   const int row = blockIdx.x;
   const int pieces = H >> 3;
@@ -2946,9 +2946,10 @@ struct WsLayout {
 };
 
 // Bytes from one 8-bit hidden row to the next: rows start on 128-byte lines, so that a K block of a row is one line instead of
-// parts of two.  Every CTA pair fetches those rows again, and that traffic out of the L2 is what bounds the 8-bit kind here.  us,
-// rows side by side -> padded, H = 4112: 384 rows, V = 32000 76.1 -> 71.0 (H = 4096: 69.4), 192 rows, V = 128256 170 -> 152 (145),
-// two planes of 96 rows, V = 32000 47.6 -> 43.6; H = 6992, 96 rows, V = 40736 77.0 -> 70.9.
+// parts of two, and whole 32-byte sectors.  Every CTA pair fetches those rows again, and that traffic out of the L2 is what bounds
+// the 8-bit kind here.  us, rows side by side -> padded, rows that start on no sector (H = 4112) / on sectors (H = 4128; H = 4096: 67.4):
+// 384 rows, V = 32000 75.5 -> 69.4 / 70.5 -> 68.9; 192 rows, V = 128256 164 -> 150 / 149 -> 147; two planes of 96 rows, V = 32000
+// 48.3 -> 44.0 / 43.6 -> 42.5.
 int hidden_pitch8(int H) { return static_cast<int>(align_up(static_cast<size_t>(H), 128)); }
 
 WsLayout ws_layout(int maxB, int maxK, int H, int V, int num_sms) {
@@ -3052,9 +3053,10 @@ Plan plan_as(const hola_ctx* ctx, int M, int w_dtype, const PlanWish& want) {
   // the statistics of all CTAs have to be merged, so as many pairs as there are is not the best split of a small vocabulary.
   // At least 64 rows per CTA; with more than 96 operand rows a 42nd of the vocabulary per pair, or tiles of 256 rows where that
   // would be more (V > 10752: 43 pairs and up); with more than 256 operand rows tiles of 256 throughout.  42 pairs still stream
-  // W_lm fast enough; the number is the best of those tried at the three sizes below on 74 pairs, not derived.  us, H = 4096: V = 4000, 5 rows 16.6 -> 16.1, 96 rows 20.6 ->
-  // 20.0 (V = 12000 27.6 as it is, 28.4 on 47 pairs); V = 8000, 192 rows 34.6 -> 28.6 (29.6 on 32 pairs), 384 rows 57.4 ->
-  // 45.0, two planes of 192 rows 38.2 -> 35.4; V = 12000, 192 rows 37.4 -> 33.6, 384 rows 61.0 -> 51.4.
+  // W_lm fast enough; the number is the best of those tried at the three sizes below on 74 pairs, not derived.  us, H = 4096:
+  // V = 4000, 5 rows 16.6 -> 16.1, 96 rows 20.6 -> 20.0 (V = 12000 27.6 as it is, 28.4 on 47 pairs); V = 8000, 192 rows 34.6 ->
+  // 28.6 (29.6 on 32 pairs), 384 rows 57.4 -> 45.0, two planes of 192 rows 38.2 -> 35.4; V = 12000, 192 rows 37.4 -> 33.6, 384
+  // rows 61.0 -> 51.4.
   const int op_rows = best.n_sub * best.N;
   int spread = pairs;
   if (rounds == 1 && op_rows > 96) spread = op_rows > 256 ? 1 : (pairs < 42 ? pairs : 42);
@@ -3129,9 +3131,9 @@ inline double one_tile_us(const hola_ctx* ctx, int w_dtype, int n_sub, int N, in
 // Vocabularies of a tile per pair and fewer leave pairs without work when all rows of a pass go to the same tile's pair.  The
 // rows are then cut into more passes, which share the tiles in one launch, and the tiles into shorter ones, as the estimate has
 // it (half a microsecond less than the split of the general rules, or that one stays).  us, before -> after, bf16: 417 rows,
-// H = 5304, V = 1272 62.4 -> 25.2; 384 rows, H = 4096, V = 8000 45.5 -> 37.0; 384 rows, H = 1024, V = 4000 21.0 -> 14.2; 200 rows,
-// H = 2048, V = 3000 20.6 -> 15.5; 512 rows, H = 512, V = 2000 22.5 -> 12.9; 150 rows, H = 696, V = 6000 15.4 -> 13.7; 8-bit planes,
-// 384 rows, V = 4000 35.1 -> 21.2; two planes, 216 rows, V = 7550 35.6 -> 26.1; mixed widths, 824 rows, V = 1408 43.0 -> 34.8.
+// H = 5304, V = 1272 62.3 -> 25.3; 384, 4096, 8000 45.4 -> 36.4; 384, 1024, 4000 20.7 -> 14.1; 200, 2048, 3000 20.9 -> 15.0; 512, 512,
+// 2000 22.1 -> 12.5; 153, 696, 6000 15.4 -> 13.4; 8-bit planes, 384, 4096, 4000 35.0 -> 22.8; two planes, 216, 1024, 7550 25.2 -> 20.1;
+// mixed widths, 824, 1024, 1408 24.6 -> 16.4.
 Plan make_plan(const hola_ctx* ctx, int M, int w_dtype = HOLA_W_BF16) {
   PlanWish want = {ctx->force_passes, 0, true};
   Plan best = plan_as(ctx, M, w_dtype, want);
@@ -3252,19 +3254,18 @@ int sample_cluster(int num_sms, int B, int V, int fallback) {
   return S;
 }
 
-// One CTA of 1024 threads per sequence instead of a cluster of S: no cluster barrier, the statistics of a row merged once, and
+// One CTA of 1024 threads per sequence instead of a cluster of S: no exchange between CTAs, the statistics of a row merged once, and
 // with one sequence per SM most SMs stay free for the next call's GEMM kernel, which then asks for its W_lm while this one runs.
 // Up to 16384 entries (more take one SM too long).  Where clusters would take at most a quarter of the SMs they ask ahead as
 // well, and have their rows staged: then only up to 8192 entries.  Rows of no whole 16-byte pieces are loaded element by element,
 // and one SM is slow at that: only up to 8192 entries, and where clusters would take at most a quarter of the SMs only against
 // clusters of two, or of four whose CTAs have more rows to merge than warps (8).
-// us, cluster -> one CTA, k = 4, H = 1024: V = 3000, 2 / 32 / 100 sequences 11.1 -> 10.6, 15.1 -> 14.5, 26.3 -> 25.1; V = 6000, 1
-// 11.5 -> 11.6; V = 8192, 1 / 4 / 16 / 64 12.3 -> 12.2, 13.1 -> 12.6, 14.5 -> 13.2, 22.5 -> 20.3; k = 30, V = 4000, 1 15.0 -> 11.4;
-// V = 16000, 1 / 8 / 24 / 148 14.3 -> 14.9, 16.6 -> 15.4, 18.1 -> 17.4, 47.2 -> 43.0; V = 16384, 5 / 100 16.6 -> 16.1, 32.0 -> 31.5;
-// V = 24000, 32 26.8 -> 28.2.  No whole pieces: V = 3001, 2 / 12 11.9 -> 11.7, 13.2 -> 13.0; V = 4001, 1 / 7 / 30 11.6 -> 11.9,
-// 12.2 -> 12.6, 16.2 -> 16.2; V = 6001, 2 / 9 12.4 -> 12.7, 13.3 -> 13.7; V = 8191, 1 / 4 / 5 / 16 / 64 12.3 -> 13.1, 13.6 -> 14.2,
-// 14.3 -> 13.9, 15.5 -> 14.9, 24.8 -> 23.8; k = 8, V = 4001 / 6001 / 8191, 1 / 3 / 3 12.4 -> 12.0, 13.9 -> 13.6, 14.1 -> 14.4; k = 20,
-// V = 4001, 1 12.7 -> 11.9; V = 11001, 16 16.7 -> 17.0.  (S = 1, up to 1920 entries: one CTA of 256 threads is enough.)
+// us, cluster -> one CTA, k = 4, H = 1024: V = 3000, 32 / 100 sequences 12.9 -> 12.2, 15.2 -> 14.7; V = 8192, 16 / 64 13.8 -> 13.0,
+// 17.9 -> 17.2; V = 16000, 1 / 8 / 148 12.6 -> 13.9, 15.6 -> 14.9, 41.5 -> 39.9; V = 24000, 32 25.3 -> 27.9; k = 30, V = 4000, 1
+// 15.5 -> 12.6.  No whole pieces: V = 3001, 2 11.2 -> 10.8; V = 6001, 9 12.8 -> 13.0; V = 8191, 1 / 4 / 16 11.8 -> 12.3, 13.0 -> 13.5,
+// 15.1 -> 14.5; k = 8, V = 4001, 1 11.8 -> 11.0.  (S = 1, up to 1920 entries: one CTA of 256 threads is enough.)  The line for few
+// sequences was drawn when a cluster took longer: with k = 4 it is ahead there from some 4000 entries on by now (V = 3000, 2 10.2 -> 10.3;
+// V = 6000, 1 10.6 -> 11.0; V = 8192, 1 / 4 11.2 -> 11.9, 12.1 -> 12.6).
 bool sample_solo(int num_sms, int B, int k, int V, int S, bool vec) {
   const bool many = 4 * B * S > num_sms;
   if (S == 1 || B > num_sms) return false;
@@ -4080,9 +4081,9 @@ hola_status verify_device(hola_ctx* ctx, const hola_verify_args* a, cudaStream_t
 // sequence: row accept_len, and none when every draft token was kept or the fallback is greedy.  Rows 0 .. ahead-1 of
 // every sequence (as many as the bus carries while the GEMM runs, at least one) are sent ahead on the context's own stream;
 // after the accept test the accept lengths come back and only the rows still missing follow, or the accept/sample kernel
-// reads those in place.  Same arithmetic and so the same results as the whole-tensor copy, with one exception: a launch that reads rows in place keeps
-// clusters where the others take one CTA (sample_solo), so that the chunks' masses are summed in another order, in fp64; a
-// token differs only where u R falls within that rounding (some 1e-16) of a boundary.
+// reads those in place.  Same arithmetic and so the same results as the whole-tensor copy, with one exception: a launch that
+// reads rows in place keeps clusters where the others take one CTA (sample_solo), so that the chunks' masses are summed in
+// another order, in fp64; a token differs only where u R falls within that rounding (some 1e-16) of a boundary.
 constexpr double kHostBusBytesPerSecond = 50e9;          // what a pinned host-to-device copy reaches here
 
 // Draft rows per sequence that can cross the bus while the GEMM of this call runs.
