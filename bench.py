@@ -48,8 +48,8 @@ NOMINAL_PEAKS = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}
 # time counters on the full-size launch; their logits are stored with the streaming hint, so most of them reach DRAM
 # inside the kernel; "wide" is the one launch that holds all six passes).  Other workloads, weight modes, gates and
 # fallbacks report null.
-NCU_TRAFFIC = {"batched": 265911680 + 8094490, "large_vocab": 1055523742 + 165214129,
-               "wide": 2598598827 + 1165225941}
+NCU_TRAFFIC = {"batched": 265855104 + 7673344, "large_vocab": 1055257600 + 165534641,
+               "wide": 2702519978 + 1156242816}
 
 
 def ncu_traffic_bytes(w):
